@@ -95,7 +95,7 @@ def parse():
     ap.add_argument("--warmup", type=int, default=5)
     ap.add_argument("--impl", choices=["ours", "reference"], default="ours")
     ap.add_argument("--precision", choices=["f16", "bf16", "bf16x2", "f32"], default="f16",
-                    help="network operands: f16, bf16, bf16x2 (SDF activations split in two bf16 parts), f32 (SIMT)")
+                    help="network operands: f16, bf16, bf16x2 (SDF activations split in two bf16 parts), f32 (operands split in two f16 parts)")
     ap.add_argument("--net-kernel", choices=["auto", "serial", "pipelined"], default="auto",
                     help="tensor-core network kernel; auto: the library's autotuner picks on view 0")
     ap.add_argument("--no-quality", action="store_true")
@@ -498,7 +498,7 @@ def run_ours(args, ws, rank, local):
             step(k)
         torch.cuda.synchronize()
     step_ms = [a.elapsed_time(b) for a, b in evs]
-    mlp_name = "mlp_simt" if prec == "f32" else (
+    mlp_name = "mlp_f32" if prec == "f32" else (
         "mlp_pipe" if T.tsdfs_network_kernel(PREC[prec]) == T.TSDFS_NETKERNEL_PIPELINED else "mlp_tc")
     import ctypes as C
     ms_k, n_k = C.c_double(0), C.c_int64(0)
@@ -532,10 +532,11 @@ def run_ours(args, ws, rank, local):
                     "serial" if mlp_name == "mlp_tc" else ("pipelined-split" if prec == "bf16x2" else "pipelined")]
                 / ALGO_FLOP_PER_SAMPLE}
     else:
-        fp32_peak = 152 * 128 * 2 * 2.07e9 / 1e12  # SMs x FP32 lanes x 2 flop x max SM clock
-        roof = {"bound": "alu", "achieved": achieved, "peak": fp32_peak, "unit": "TFLOP/s",
+        fp32_peak = bf16_burst / 3.0   # each FP32 operand as two FP16 parts, three products per FP32 product
+        roof = {"bound": "tensor", "achieved": achieved, "peak": fp32_peak, "unit": "TFLOP/s",
                 "frac": achieved / fp32_peak, "traffic": None,
-                "peak_kind": "fp32 FMA, 152 SMs x 128 lanes x 2 x 2.07 GHz", "kernel": "mlp_simt"}
+                "peak_kind": f"bf16 dense burst ({peak_src}) / 3: FP32 operands as two FP16 parts, three products",
+                "kernel": "mlp_f32"}
     # the GPU's own bounds of view 0, for the march's roofline line
     bv = T.Bounds(n, device=dev)
     bv.compute(grid, rays[0][0], rays[0][1], bp, mask)
@@ -788,7 +789,7 @@ def run_train(spec, wl, grid, mask, dev, n_rays=8192, iters=5, kind=None, peak_b
         torch.cuda.synchronize()
         ms = e0.elapsed_time(e1) / iters
         split = {}
-        for name in ("mlp_simt", "composite", "train_forward", "train_forward_network", "train_forward_composite",
+        for name in ("mlp_f32", "composite", "train_forward", "train_forward_network", "train_forward_composite",
                      "backward", "backward_forward", "backward_composite", "backward_network", "ray_bounds"):
             t, c = C.c_double(0), C.c_int64(0)
             T.lib().tsdfs_profile_read(name.encode(), C.byref(t), C.byref(c))
@@ -803,7 +804,7 @@ def run_train(spec, wl, grid, mask, dev, n_rays=8192, iters=5, kind=None, peak_b
            "loss": float(loss.item()), "kernel_ms": split,
            "backward": "render_rays_train (layer-major FP32 forward that keeps its activations) + "
                        "render_rays_backward_kept: GEMMs in cuBLAS BF16x9-emulated FP32 on the tensor cores"
-           if gemm else "render_rays (FP32 SIMT) + render_rays_backward (FP32 SIMT, tiles of 8 samples)",
+           if gemm else "render_rays (FP32) + render_rays_backward (FP32 SIMT, tiles of 8 samples)",
            "what": "bounds + render (fp32) + L1 + 0.1 eikonal + backward through both networks"}
     if gemm and "backward_network_ms" in split:
         f = backward_gemm_flops(spec)

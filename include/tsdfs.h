@@ -15,8 +15,9 @@
  *    layer-major backward's first call on a device creates a cuBLAS handle,
  *    whose state cuBLAS allocates).  The render workspaces (render_rays,
  *    render_rays_hier, render_rays_hier_bounded) include about 10 MB for the
- *    tensor-core network kernel, which parks the first tile of each pair of
- *    64-sample tiles there (256 CTAs x 38 KB).
+ *    network kernels: the serial one parks the first tile of each pair of
+ *    64-sample tiles there (256 CTAs x 38 KB), the FP32 one keeps the call's
+ *    split weights there (3 MB).
  *  - Work is enqueued asynchronously on `stream` (a cudaStream_t; NULL = the
  *    legacy default stream); the calls that synchronise say so (the autotuners,
  *    the layer-major backward and training forward, which read the sample
@@ -115,7 +116,9 @@ typedef struct {
 #define TSDFS_OPACITY_VOLSDF 1
 #define TSDFS_ARCH_TINY 0
 #define TSDFS_ARCH_ROOM 1
-#define TSDFS_PREC_F32 0  /* FP32 SIMT networks                                  */
+#define TSDFS_PREC_F32 0  /* FP32 networks: tcgen05 with every operand split into two FP16
+                             * parts (22 bits) and FP32 sums; samples whose operands leave
+                             * the parts' range (|x| > 2000) on FP32 SIMT cores           */
 #define TSDFS_PREC_BF16 1 /* BF16 tcgen05 networks, FP32 accumulate (packed required) */
 #define TSDFS_PREC_F16 2  /* FP16 operands on the same tcgen05 path (packed required)  */
 #define TSDFS_PREC_BF16X2 3 /* BF16 tcgen05 networks with every SDF layer's operand split

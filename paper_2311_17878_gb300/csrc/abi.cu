@@ -7,6 +7,7 @@
 #include <mutex>
 
 #include "common.cuh"
+#include "mlp_f32.cuh"
 
 namespace tsdfs {
 
@@ -164,12 +165,8 @@ static void prof_clear() {
 }
 
 // ---------------------------------------------------------------------------
-// internal launchers (mlp_simt.cu, composite.cu, bounds.cu)
+// internal launchers (composite.cu, bounds.cu, mlp_*.cu)
 // ---------------------------------------------------------------------------
-template <int ARCH>
-int launch_mlp_full_simt(const NetParams& np, const SampleSource& src, SampleRec* rec, int64_t max_samples, cudaStream_t st);
-template <int ARCH>
-int launch_mlp_value_simt(const NetParams& np, const SampleSource& src, float* f_out, cudaStream_t st);
 int launch_composite(const SampleRec* rec, const int32_t* offsets, int per_ray, const uint8_t* status, int64_t n_rays,
                      const int32_t* total_dev, int64_t capacity, Opacity op, float* rgb, float* depth,
                      float* wsum, float* normal, float* eik, cudaStream_t st);
@@ -234,8 +231,14 @@ static NetParams net_params(const tsdfs_mlp* m) {
     return np;
 }
 
-// the network evaluation of every render path; `stash`: the serial tensor-core kernel's parking
-// space in the caller's workspace (mlp_tc_stash_bytes(), 256-byte aligned)
+// scratch of the network kernels in the caller's workspace (256-byte aligned): the serial
+// kernel's parking space, or the single-precision path's redo word and split weights
+static size_t stash_bytes() {
+    const size_t a = mlp_tc_stash_bytes(), b = mlp_f32_stash_bytes();
+    return a > b ? a : b;
+}
+
+// the network evaluation of every render path
 static int run_full_mlp(const tsdfs_mlp* m, const SampleSource& src, SampleRec* rec, int64_t max_samples,
                         uint8_t* stash, cudaStream_t st) {
     if (m->precision != TSDFS_PREC_F32) {
@@ -246,10 +249,30 @@ static int run_full_mlp(const tsdfs_mlp* m, const SampleSource& src, SampleRec* 
         ProfScope ps("mlp_tc", st);
         return launch_mlp_full_tc(m, src, rec, max_samples, stash, st);
     }
-    ProfScope ps("mlp_simt", st);
+    // FP32: the split tensor-core kernel, then the SIMT kernel over the tiles it marked (see
+    // mlp_f32.cu), at every size: one 32-sample tile takes less time than a SIMT tile of 16
+    ProfScope ps("mlp_f32", st);
     const NetParams np = net_params(m);
-    return m->arch == TSDFS_ARCH_TINY ? launch_mlp_full_simt<TSDFS_ARCH_TINY>(np, src, rec, max_samples, st)
-                                      : launch_mlp_full_simt<TSDFS_ARCH_ROOM>(np, src, rec, max_samples, st);
+    const uint32_t* redo = reinterpret_cast<const uint32_t*>(stash);
+    int rc = launch_mlp_full_f32(m, src, rec, max_samples, stash, st);
+    if (rc) return rc;
+    return m->arch == TSDFS_ARCH_TINY ? launch_mlp_full_simt<TSDFS_ARCH_TINY>(np, src, rec, max_samples, redo, st)
+                                      : launch_mlp_full_simt<TSDFS_ARCH_ROOM>(np, src, rec, max_samples, redo, st);
+}
+
+// SDF values only (the samplers' coarse passes)
+static int run_value_mlp(const tsdfs_mlp* m, const SampleSource& src, float* f_out, uint8_t* stash, cudaStream_t st) {
+    if (m->precision != TSDFS_PREC_F32) {
+        ProfScope ps("mlp_value_tc", st);
+        return launch_mlp_value_tc(m, src, f_out, st);
+    }
+    ProfScope ps("mlp_value_f32", st);
+    const NetParams np = net_params(m);
+    const uint32_t* redo = reinterpret_cast<const uint32_t*>(stash);
+    int rc = launch_mlp_value_f32(m, src, f_out, stash, st);
+    if (rc) return rc;
+    return m->arch == TSDFS_ARCH_TINY ? launch_mlp_value_simt<TSDFS_ARCH_TINY>(np, src, f_out, redo, st)
+                                      : launch_mlp_value_simt<TSDFS_ARCH_ROOM>(np, src, f_out, redo, st);
 }
 
 }  // namespace tsdfs
@@ -343,7 +366,7 @@ extern "C" size_t tsdfs_render_workspace_size(const tsdfs_mlp* mlp, int64_t n_ra
     (void)n_rays;
     if (max_samples < 0) return 0;
     return align256((size_t)max_samples * sizeof(SampleRec)) + align256((size_t)max_samples * sizeof(int32_t)) +
-           align256(mlp_tc_stash_bytes()) + 256;
+           align256(stash_bytes()) + 256;
 }
 
 namespace tsdfs {
@@ -388,7 +411,7 @@ extern "C" int render_rays(const tsdfs_mlp* mlp, const float* ray_o, const float
     src.total_dev = offsets + n_rays;
     src.capacity = max_samples;
     if (max_samples > 0) {
-        if (mlp->precision != TSDFS_PREC_F32) {
+        {
             ProfScope ps("sample_ray", st);
             k_sample_ray<<<grid_1d(n_rays, 256), 256, 0, st>>>(offsets, n_rays, max_samples, sample_ray);
             rc = cuda_check(cudaGetLastError(), "sample_ray launch");
@@ -473,7 +496,7 @@ static HierWs hier_layout(void* base, int64_t n, int n_c = 64, int n_f = 32) {
     };
     const size_t n_h = (size_t)(n_c + n_f);
     w.rec = reinterpret_cast<SampleRec*>(take((size_t)n * n_h * sizeof(SampleRec)));
-    w.stash = reinterpret_cast<uint8_t*>(take(mlp_tc_stash_bytes()));
+    w.stash = reinterpret_cast<uint8_t*>(take(stash_bytes()));
     w.t0 = reinterpret_cast<float*>(take((size_t)n * 4));
     w.te = reinterpret_cast<float*>(take((size_t)n * 4));
     w.tc = reinterpret_cast<float*>(take((size_t)n * n_c * 4));
@@ -517,7 +540,6 @@ extern "C" int render_rays_hier(const tsdfs_mlp* mlp, const tsdfs_grid* grid, co
         rc = launch_hier_setup(grid, ray_o, ray_d, n_rays, t_near, t_far, w.t0, w.te, w.status, w.tc, w.dc, n_coarse, st);
     }
     if (rc) return rc;
-    const NetParams np = net_params(mlp);
     SampleSource cs{};
     cs.mode = kExplicit;
     cs.ray_o = ray_o;
@@ -527,14 +549,7 @@ extern "C" int render_rays_hier(const tsdfs_mlp* mlp, const tsdfs_grid* grid, co
     cs.per_ray = n_coarse;
     cs.total_host = n_rays * n_coarse;
     cs.capacity = n_rays * n_coarse;
-    if (mlp->precision != TSDFS_PREC_F32) {
-        ProfScope ps("mlp_value_tc", st);
-        rc = launch_mlp_value_tc(mlp, cs, w.fc, st);
-    } else {
-        ProfScope ps("mlp_value_simt", st);
-        rc = mlp->arch == TSDFS_ARCH_TINY ? launch_mlp_value_simt<TSDFS_ARCH_TINY>(np, cs, w.fc, st)
-                                          : launch_mlp_value_simt<TSDFS_ARCH_ROOM>(np, cs, w.fc, st);
-    }
+    rc = run_value_mlp(mlp, cs, w.fc, w.stash, st);
     if (rc) return rc;
     {
         ProfScope ps("hier_fine", st);
@@ -581,7 +596,7 @@ static BoundedHierWs bounded_hier_layout(void* base, int64_t n, int64_t max_coar
         return q;
     };
     w.rec = reinterpret_cast<SampleRec*>(take((size_t)cap2 * sizeof(SampleRec)));
-    w.stash = reinterpret_cast<uint8_t*>(take(mlp_tc_stash_bytes()));
+    w.stash = reinterpret_cast<uint8_t*>(take(stash_bytes()));
     w.ray_c = reinterpret_cast<int32_t*>(take((size_t)max_coarse * 4));
     w.fc = reinterpret_cast<float*>(take((size_t)max_coarse * 4));
     w.n2 = reinterpret_cast<int32_t*>(take((size_t)n * 4));
@@ -638,15 +653,7 @@ extern "C" int render_rays_hier_bounded(const tsdfs_mlp* mlp, const float* ray_o
             if (rc) return rc;
         }
         cs.sample_ray = w.ray_c;  // the value kernels flag a coarse total above max_coarse
-        if (mlp->precision != TSDFS_PREC_F32) {
-            ProfScope ps("mlp_value_tc", st);
-            rc = launch_mlp_value_tc(mlp, cs, w.fc, st);
-        } else {
-            ProfScope ps("mlp_value_simt", st);
-            const NetParams np = net_params(mlp);
-            rc = mlp->arch == TSDFS_ARCH_TINY ? launch_mlp_value_simt<TSDFS_ARCH_TINY>(np, cs, w.fc, st)
-                                              : launch_mlp_value_simt<TSDFS_ARCH_ROOM>(np, cs, w.fc, st);
-        }
+        rc = run_value_mlp(mlp, cs, w.fc, w.stash, st);
         if (rc) return rc;
     }
     // merged counts, their offsets, then the fine samples and the merged list

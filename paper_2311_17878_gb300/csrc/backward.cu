@@ -18,12 +18,9 @@
 #include <atomic>
 
 #include "backward.cuh"
+#include "mlp_f32.cuh"
 
 namespace tsdfs {
-
-template <int ARCH>
-int launch_mlp_full_simt(const NetParams& np, const SampleSource& src, SampleRec* rec, int64_t max_samples,
-                         cudaStream_t st);
 
 namespace {
 
@@ -693,8 +690,8 @@ extern "C" int render_rays_backward(const tsdfs_mlp* mlp, const float* ray_o, co
     src.total_dev = offsets + n_rays;
     src.capacity = max_samples;
     if (max_samples == 0) return TSDFS_OK;
-    rc = mlp->arch == TSDFS_ARCH_TINY ? launch_mlp_full_simt<TSDFS_ARCH_TINY>(np, src, w.rec, max_samples, st)
-                                      : launch_mlp_full_simt<TSDFS_ARCH_ROOM>(np, src, w.rec, max_samples, st);
+    rc = mlp->arch == TSDFS_ARCH_TINY ? launch_mlp_full_simt<TSDFS_ARCH_TINY>(np, src, w.rec, max_samples, nullptr, st)
+                                      : launch_mlp_full_simt<TSDFS_ARCH_ROOM>(np, src, w.rec, max_samples, nullptr, st);
     if (rc) return rc;
     rc = launch_comp_bwd(w.rec, offsets, status, ray_d, n_rays, mlp, d_rgb, d_depth, d_eik, w.adj, st);
     if (rc) return rc;

@@ -1,0 +1,982 @@
+// Single-precision networks on the tcgen05 tensor cores: every operand as two FP16 parts.
+//
+// An FP32 operand x is carried as hi = fp16(32 x) and lo = fp16(2048 (32 x - hi)): 22
+// significant bits over |x| from 2e-6 to 2047, and an absolute floor of 5e-13 below that (lo is
+// stored scaled, so it stays normal while hi is).  A product sum takes three MMAs per K step,
+// hi hi' into a main accumulator and lo hi' + hi lo' into a correction accumulator that is
+// scaled back by 2^-11 when it is read (lo lo' is below 2^-22 of the product).  Everything
+// between the products is FP32.
+//
+// tcgen05 truncates when it adds into its FP32 accumulator, so the main sum comes out too small
+// by half a unit in the last place per MMA on average: measured against FP64 over random
+// operands of either sign, 2.0e-8 + 1.67e-8 n of the sum after n MMAs with weights of 22 bits and
+// 6 % less with weights of 8 (BF16 values), the same for positive and for signed rows.  The
+// epilogue adds the mean of the two back (kBias0 + n kBias1).  What remains at K = 256 is
+// 2.0e-7 (2-norm), an FP32 FMA chain has 2.9e-7; without the share 3.5e-7 and, worse, of one
+// sign in every layer; with the three products in one accumulator 9.8e-7.  Through the fitted
+// room networks: |grad f| 1.6e-7 off (FP32 FMA chains 3.0e-7; without the share 8.9e-7).
+//
+// Tile: 32 samples = 128 operand rows; TMEM lane quarter q holds samples 8q..8q+7 in four groups
+// of 8 lanes (value, d/dx, d/dy, d/dz rows: forward-mode gradient).  Two parts of 128 x 256
+// operands take 128 KB of shared memory.  A layer runs in phases of at most 128 outputs, each
+// into one of two buffers of TMEM (main and correction, 128 columns each), so the epilogue of a
+// phase runs beside the MMAs of the next.  A layer's operand can be replaced only after its last
+// MMA: the first phase's activations wait in registers (as packed parts), are stored when the
+// second phase is through, and the next layer starts on those 128 columns while the second
+// phase's epilogue fills the others.  The narrow outputs, net_0 (with its gradient) and the
+// three colours, are FP32 dot products that the epilogue of the layer before accumulates: no MMA
+// phase of 16 columns with its hand-offs, and no truncation where |grad f| is near 1 everywhere
+// and the mantissa would make the truncated share differ from its mean for every sample alike.  The weights stream from L2 in items of 64 K columns x
+// 128 outputs (hi and lo, 32 KB) through a ring of two stages; three producer warps copy the
+// items' parts in turn, because one thread's bulk copies do not overlap.
+//
+// The colour network's rows are the value rows only.  Its first layer reads the SDF features
+// where the SDF's operand was and x~, the direction encoding and the unit normal from the first
+// columns of the rows below each value-row group (the d/dx rows' place, dead by then).
+//
+// VALUE: the samplers' coarse pass (SDF value only): 128 samples per tile, one row each, no
+// gradient and no colour network.
+//
+// Range: an operand beyond 2000, a non-finite value or a gradient below 1e-4 marks its tile (the
+// first record of each 16 samples gets pad = 1, a value tile's first results a NaN of a fixed
+// payload) and a launch of the SIMT kernel evaluates the marked tiles again: the split has no
+// exponent range to spare there.  Nothing is marked with networks of ordinary weights.
+//
+// Roles: warps 0-11 epilogue (TMEM lane quarter w % 4, column part w / 4), warp 12 MMA issue,
+// warps 13-15 weight producers.  Every wait is bounded; on timeout the kernel records
+// TSDFS_DEV_TIMEOUT, drains its own copies and MMAs, frees TMEM and returns.
+#include "tc_common.cuh"
+#include "mlp_f32.cuh"
+
+namespace tsdfs {
+
+namespace {
+
+constexpr int kTile = 32;             // samples per tile (four rows each)
+constexpr int kTileV = 128;           // VALUE: samples per tile (one row each)
+constexpr int kEpi = 12;              // epilogue warps: 4 lane quarters x 3 column parts
+constexpr int kParts = 3;
+constexpr int kMma = 12;              // MMA warp
+constexpr int kStages = 2;
+constexpr int kProd = 3;               // weight producers (16 warps in all leave 128 registers a thread)
+constexpr int kThr = 32 * (kMma + 1 + kProd);
+constexpr int kPh = 128;              // outputs per phase
+constexpr int kGrp = 6;               // 8-column groups of a phase per part, at most
+constexpr uint32_t kPartBytes = 64 * 1024;                 // 128 rows x 256 16-bit columns
+constexpr uint32_t kStageBytes = 2 * kPh * kKChunk * 2;    // hi and lo of one item
+constexpr float kUp = 32.0f;          // operand scale
+constexpr float kLoUp = 2048.0f;      // further scale of the low part
+constexpr float kDown = 1.0f / (kUp * kUp), kLoDown = 1.0f / kLoUp;
+constexpr float kLimit = 2000.0f;     // largest operand the high part is trusted with
+constexpr float kBias0 = 1.7e-8f, kBias1 = 1.58e-8f;   // what a main sum of n MMAs lacks: kBias0 + n kBias1
+constexpr float kMinGrad = 1e-4f;
+constexpr float kRsqrt2 = 0.70710678118654752f;
+
+template <int ARCH> struct FArch {
+    using A = Arch<ARCH>;
+    static constexpr int LS = A::kSdfLayers;
+    static constexpr int NL = A::kSdfLayers + A::kRgbLayers;
+    static constexpr int kX = 3 + A::kDirEnc + 3;    // x~, direction encoding, unit normal
+    static constexpr int kXp = pad16(kX);
+    static constexpr int kF = A::kFeat;
+    static constexpr int kFp = pad16(kF);
+    __host__ __device__ static constexpr Layer layer(int L) { return L < LS ? A::sdf(L) : A::rgb(L - LS); }
+    // layers with MMAs: all but the colour output; the SDF output's are the features only.
+    // Operand columns in the main buffers (the colour input: its features), then the rest in its
+    // own chunk; outputs padded to 16
+    __host__ __device__ static constexpr int k_main(int L) { return L == LS ? kFp : pad16(layer(L).in); }
+    __host__ __device__ static constexpr int n_pad(int L) { return L == LS - 1 ? kFp : pad16(layer(L).out); }
+    __host__ __device__ static constexpr int main_chunks(int L) { return (k_main(L) + kKChunk - 1) / kKChunk; }
+    __host__ __device__ static constexpr int chunks(int L) { return main_chunks(L) + (L == LS ? 1 : 0); }
+    __host__ __device__ static constexpr int chunk_k(int L, int c) {
+        return c == main_chunks(L) ? kXp : (k_main(L) - c * kKChunk < kKChunk ? k_main(L) - c * kKChunk : kKChunk);
+    }
+    __host__ __device__ static constexpr int phases(int L) { return (n_pad(L) + kPh - 1) / kPh; }
+    __host__ __device__ static constexpr int phase_n(int L, int p) {
+        return n_pad(L) - p * kPh < kPh ? n_pad(L) - p * kPh : kPh;
+    }
+    __host__ __device__ static constexpr int64_t layer_bytes(int L) {
+        return (int64_t)n_pad(L) * (k_main(L) + (L == LS ? kXp : 0)) * 4;
+    }
+    __host__ __device__ static constexpr int64_t layer_base(int L) {
+        int64_t o = 0;
+        for (int l = 0; l < L; ++l) o += layer_bytes(l);
+        return o;
+    }
+    __host__ __device__ static constexpr int64_t packed_bytes() { return layer_base(NL - 1); }
+    __host__ __device__ static constexpr int items(int L0, int L1) {
+        int n = 0;
+        for (int L = L0; L < L1; ++L) n += phases(L) * chunks(L);
+        return n;
+    }
+    __host__ __device__ static constexpr int bias_base(int L) {
+        int o = 0;
+        for (int l = 0; l < L; ++l) o += n_pad(l);
+        return o;
+    }
+    __host__ __device__ static constexpr int64_t param_offset(int L) {
+        return L < LS ? sdf_layer_offset<ARCH>(L) : rgb_layer_offset<ARCH>(L - LS);
+    }
+    // layer L's source row of padded output n, -1: padding
+    __host__ __device__ static constexpr int src_row(int L, int n) {
+        if (L == LS - 1) return n < kF ? n + 1 : -1;
+        return n < layer(L).out ? n : -1;
+    }
+    // layer L's source column of padded input k (the colour input: features first), -1: padding
+    __host__ __device__ static constexpr int src_col(int L, int k) {
+        if (L == LS) return k < kF ? kX + k : (k >= kFp && k - kFp < kX ? k - kFp : -1);
+        return k < layer(L).in ? k : -1;
+    }
+    template <bool VALUE> __host__ __device__ static constexpr int mma_layers() { return VALUE ? LS - 1 : NL - 1; }
+    template <bool VALUE> __host__ __device__ static constexpr uint32_t table_floats() {
+        return VALUE ? kTileV * (4 + 6 * A::kPeSdf) : kTile * (8 + 6 * (A::kPeSdf + A::kPeDir));
+    }
+    // net_0's weights and partial sums (3 parts x 128 rows); the record's SDF half, the colour
+    // output's weights and partial sums (3 parts x 3 colours x 32 samples)
+    static constexpr int kW0 = pad16(A::sdf(LS - 1).in), kWc = pad16(A::rgb(A::kRgbLayers - 1).in);
+    template <bool VALUE> __host__ __device__ static constexpr uint32_t scratch_floats() {
+        return kW0 + kParts * 128 + (VALUE ? 0 : kTile * 8 + 3 * kWc + kParts * 3 * kTile);
+    }
+    template <bool VALUE> __host__ __device__ static constexpr int n_items() { return items(0, mma_layers<VALUE>()); }
+    template <bool VALUE> __host__ __device__ static constexpr uint32_t bias_floats() {
+        return bias_base(mma_layers<VALUE>());
+    }
+    template <bool VALUE> __host__ __device__ static constexpr size_t smem_bytes() {
+        return 2 * (size_t)kPartBytes + kStages * (size_t)kStageBytes + 4u * bias_floats<VALUE>() +
+               4u * table_floats<VALUE>() + 4u * scratch_floats<VALUE>() + 32u * n_items<VALUE>() + 128;
+    }
+};
+
+// one weight item as the MMA warp and the producers use it
+struct __align__(16) Item {
+    uint32_t off;      // of the hi part in the packed weights (the lo part follows)
+    uint32_t bytes;    // of one part
+    uint32_t a;        // operand offset of its first K step (hi part)
+    uint32_t a_sbo;    // operand row-group stride
+    uint32_t b_sbo;
+    uint32_t idesc;
+    uint16_t steps;    // K steps of 16
+    uint16_t pad[2];
+    uint16_t edge;     // bit 0: first item of a phase, bit 1: last, bit 2 / 3: its operand's columns below /
+                       // from 128 are awaited first
+};
+static_assert(sizeof(Item) == 32, "item record");
+
+struct F32Params {
+    const uint8_t* packed;
+    const float* sdf_w;
+    const float* rgb_w;
+    float center[3];
+    float inv_scale, scale, beta;
+    SampleSource src;
+    SampleRec* rec;      // full evaluation
+    float* f_out;        // VALUE
+    uint32_t* redo;      // set when a tile is marked
+    uint32_t* status;
+    uint32_t spin;
+    int withhold;
+};
+
+__device__ __forceinline__ void wait_ld16(float (&a)[8], float (&b)[8]) {
+    asm volatile("tcgen05.wait::ld.sync.aligned;"
+                 : "+f"(a[0]), "+f"(a[1]), "+f"(a[2]), "+f"(a[3]), "+f"(a[4]), "+f"(a[5]), "+f"(a[6]), "+f"(a[7]),
+                   "+f"(b[0]), "+f"(b[1]), "+f"(b[2]), "+f"(b[3]), "+f"(b[4]), "+f"(b[5]), "+f"(b[6]), "+f"(b[7])
+                 :
+                 : "memory");
+}
+__device__ __forceinline__ void stmat1(uint32_t addr, uint32_t r0) {
+    asm volatile("stmatrix.sync.aligned.m8n8.x1.shared.b16 [%0], {%1};" ::"r"(addr), "r"(r0) : "memory");
+}
+
+// the two FP16 parts of a pair of FP32 operands (see the head of the file)
+__device__ __forceinline__ void split_f32(float a, float b, uint32_t& hi, uint32_t& lo) {
+    a *= kUp;
+    b *= kUp;
+    const __half2 h = __floats2half2_rn(a, b);
+    const float2 f = __half22float2(h);
+    const __half2 l = __floats2half2_rn((a - f.x) * kLoUp, (b - f.y) * kLoUp);
+    hi = *reinterpret_cast<const uint32_t*>(&h);
+    lo = *reinterpret_cast<const uint32_t*>(&l);
+}
+
+// softplus_beta(z) = max(z, 0) + log(1 + e^{-beta |z|}) / beta and its slope sigma(beta z).  The
+// fast exponential and logarithm measure the same errors in f and grad f as expf and an FP32
+// series for the logarithm (|grad f| 6.3e-8 off through the tiny networks either way).
+__device__ __forceinline__ void softplus_slope_f32(float z, float beta, float inv_beta, float& h, float& sg) {
+    const float u = beta * z;
+    const float e = __expf(-fabsf(u)), d = 1.0f + e;
+    const float r = __fdividef(1.0f, d);
+    sg = u >= 0.0f ? r : e * r;
+    h = fmaf(__logf(d), inv_beta, z < 0.0f ? 0.0f : z);
+}
+
+// max(x, 0) that keeps a NaN (so that it is noticed)
+__device__ __forceinline__ float relu_nan(float x) { return x < 0.0f ? 0.0f : x; }
+
+template <int ARCH, bool VALUE>
+__global__ void __launch_bounds__(kThr, 1) k_mlp_f32(F32Params p) {
+    using F = FArch<ARCH>;
+    using A = Arch<ARCH>;
+    constexpr int LS = F::LS, NLr = F::template mma_layers<VALUE>();
+    constexpr int NT = F::template n_items<VALUE>();
+    constexpr int TS = VALUE ? kTileV : kTile;
+    extern __shared__ __align__(1024) uint8_t smem[];
+    uint8_t* a_hi = smem;
+    uint8_t* a_lo = smem + kPartBytes;
+    uint8_t* ring = smem + 2 * kPartBytes;
+    float* s_bias = reinterpret_cast<float*>(ring + kStages * kStageBytes);
+    float* s_x = s_bias + F::template bias_floats<VALUE>();
+    constexpr int kXRow = VALUE ? 4 : 8;       // x~ (3), [direction (3), t, delta]
+    float* s_pe = s_x + TS * kXRow;            // sin, cos of 2^oct x~_a
+    float* s_pd = s_pe + TS * A::kPeSdf * 6;   // of the direction
+    float* s_w0 = s_x + F::template table_floats<VALUE>();
+    float* s_dot = s_w0 + F::kW0;                  // [part][row]
+    float* s_out = s_dot + kParts * 128;           // [sample][8]
+    float* s_wc = s_out + kTile * 8;               // [colour][input]
+    float* s_cdot = s_wc + 3 * F::kWc;             // [part][colour][sample]
+    Item* items = reinterpret_cast<Item*>(s_w0 + F::template scratch_floats<VALUE>());
+    uint64_t* bars = reinterpret_cast<uint64_t*>(items + NT);
+    // bars: full[2], empty[2], acc[2], drained[2], operand[2], epi, end
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 12);
+    volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+    volatile uint32_t* s_mark = tmem_slot + 2;
+    const uint32_t bar_full = smem_u32(bars), bar_empty = smem_u32(bars + kStages);
+    const uint32_t bar_acc = smem_u32(bars + 4), bar_drained = smem_u32(bars + 6), bar_op = smem_u32(bars + 8),
+                   bar_epi = smem_u32(bars + 10), bar_end = smem_u32(bars + 11);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+
+    const int64_t total = sample_total(p.src);
+    if (total > p.src.capacity) {
+        if (blockIdx.x == 0 && threadIdx.x == 0) set_status(p.status, TSDFS_DEV_SAMPLES_OVERFLOW);
+        return;
+    }
+    const int64_t n_tiles = (total + TS - 1) / TS;
+    if ((int64_t)blockIdx.x >= n_tiles) return;
+
+    if (threadIdx.x == 0) {
+        for (int i = 0; i < kStages; ++i) {
+            mbar_init(bar_full + 8 * i, 2);
+            mbar_init(bar_empty + 8 * i, 1);
+            mbar_init(bar_acc + 8 * i, 1);
+            mbar_init(bar_drained + 8 * i, kEpi);
+            mbar_init(bar_op + 8 * i, kEpi);
+        }
+        mbar_init(bar_epi, kEpi);
+        mbar_init(bar_end, 1);
+        *abort_flag = 0;
+        *s_mark = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    // the items in order: layers, phases, chunks; a thread writes one layer's
+    if (threadIdx.x < NLr) {
+        const int L = threadIdx.x;
+        uint32_t off = (uint32_t)F::layer_base(L);
+        int j = F::items(0, L);
+        const uint32_t sbo = (uint32_t)(F::k_main(L) / 8) * 128u;
+        for (int ph = 0; ph < F::phases(L); ++ph) {
+            const int n = F::phase_n(L, ph);
+            for (int c = 0; c < F::chunks(L); ++c) {
+                Item it;
+                const int kc = F::chunk_k(L, c);
+                it.off = off;
+                it.bytes = (uint32_t)(n * kc * 2);
+                off += 2 * it.bytes;
+                // the colour input's extra columns live one row group below the value rows
+                it.a = c < F::main_chunks(L) ? (uint32_t)(c * (kKChunk / 8)) * 128u : sbo;
+                it.a_sbo = sbo;
+                it.b_sbo = (uint32_t)(kc / 8) * 128u;
+                it.idesc = idesc_mma<true>(128, n);
+                it.steps = (uint16_t)(kc / 16);
+                it.pad[0] = it.pad[1] = 0;
+                it.edge = (uint16_t)((c == 0 ? 1 : 0) | (c + 1 == F::chunks(L) ? 2 : 0) | (ph == 0 && c == 0 ? 4 : 0) |
+                                     (ph == 0 && c * kKChunk == kPh ? 8 : 0));
+                items[j++] = it;
+            }
+        }
+    }
+    static_for<0, NLr>([&](auto lc) {
+        constexpr int L = decltype(lc)::value;
+        constexpr Layer ly = F::layer(L);
+        const float* b = (L < LS ? p.sdf_w : p.rgb_w) + F::param_offset(L) + (int64_t)ly.out * ly.in;
+        for (int i = threadIdx.x; i < F::n_pad(L); i += kThr) {
+            const int r = F::src_row(L, i);
+            s_bias[F::bias_base(L) + i] = r >= 0 ? __ldg(b + r) : 0.0f;
+        }
+    });
+    for (int i = threadIdx.x; i < F::kW0; i += kThr) {
+        constexpr int K = A::sdf(LS - 1).in;
+        s_w0[i] = i < K ? __ldg(p.sdf_w + F::param_offset(LS - 1) + i) : 0.0f;
+    }
+    if constexpr (!VALUE) {
+        constexpr int K = A::rgb(A::kRgbLayers - 1).in;
+        for (int i = threadIdx.x; i < 3 * F::kWc; i += kThr) {
+            const int k = i % F::kWc;
+            s_wc[i] = k < K ? __ldg(p.rgb_w + F::param_offset(F::NL - 1) + (i / F::kWc) * K + k) : 0.0f;
+        }
+    }
+    // operand rows the colour network's MMAs read but nothing writes stay finite
+    for (int i = threadIdx.x; i < (int)(2 * kPartBytes / 16); i += kThr)
+        reinterpret_cast<uint4*>(a_hi)[i] = make_uint4(0, 0, 0, 0);
+    if (warp == kMma) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
+                     "r"(512));
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+    }
+    fence_proxy_async();
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = *tmem_slot;
+
+    if (warp > kMma) {
+        // ---------------------------------------- producers: the items' parts in turn
+        if (lane == 0) {
+            const int64_t mine = (n_tiles - blockIdx.x + gridDim.x - 1) / gridDim.x;   // tiles of this CTA
+            const int64_t parts = 2 * mine * NT;
+            int64_t last = -1;       // the last item this thread copied a part of
+            int j = (warp - kMma - 1) / 2;
+            bool ok = true;
+            for (int64_t t = warp - kMma - 1; t < parts; t += kProd) {
+                const int64_t g = t >> 1;
+                const uint32_t stage = (uint32_t)g & 1u, part = (uint32_t)t & 1u;
+                if (p.withhold >= 0 && g >= p.withhold) { ok = false; break; }   // test-only: never issued
+                const uint32_t off = items[j].off, bytes = items[j].bytes;
+                if (!mbar_wait(bar_empty + 8 * stage, ((uint32_t)(g >> 1) & 1u) ^ 1u, abort_flag, p.spin)) { ok = false; break; }
+                mbar_expect_tx(bar_full + 8 * stage, bytes);
+                bulk_g2s(smem_u32(ring) + stage * kStageBytes + part * bytes, p.packed + off + part * bytes, bytes,
+                         bar_full + 8 * stage);
+                last = g;
+                j += (int)(((t + kProd) >> 1) - g);
+                if (j >= NT) j -= NT;
+            }
+            if (!ok && last >= 0) {
+                // a copy of this thread may be in flight: its phase completes once the other part is
+                // there too, so wait (bounded) before the CTA's shared memory goes away
+                for (uint32_t it = 0; it < (1u << 20) && !mbar_try(bar_full + 8 * ((uint32_t)last & 1u), (uint32_t)(last >> 1) & 1u); ++it) {
+                }
+            }
+        }
+    } else if (warp == kMma) {
+        // ---------------------------------------- MMA issue (the warp converged, one lane elected)
+        const uint32_t el = elect_one();
+        const uint32_t ah0 = smem_u32(a_hi), al0 = smem_u32(a_lo), r0 = smem_u32(ring);
+        uint32_t g = 0, ph = 0, op_a = 0, op_b = 0;   // items, phases, waits for either half of an operand
+        bool ok = true;
+        auto wait = [&](uint32_t bar, uint32_t parity) {
+            return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag, p.spin));
+        };
+        for (int64_t tile = blockIdx.x; tile < n_tiles && ok; tile += gridDim.x) {
+            for (int j = 0; j < NT; ++j, ++g) {
+                const Item it = items[j];
+                if ((it.edge & 4u) && !wait(bar_op, op_a++ & 1u)) { ok = false; break; }
+                if ((it.edge & 8u) && !wait(bar_op + 8, op_b++ & 1u)) { ok = false; break; }
+                // the buffer's previous phase has been read
+                if ((it.edge & 1u) && ph >= 2 && !wait(bar_drained + 8 * (ph & 1u), ((ph >> 1) - 1) & 1u)) { ok = false; break; }
+                const uint32_t stage = g & 1u;
+                if (!wait(bar_full + 8 * stage, (g >> 1) & 1u)) { ok = false; break; }
+                tc_fence_after();
+                const uint32_t b = r0 + stage * kStageBytes;
+                uint64_t bh = mdesc(b, 128, it.b_sbo), bl = mdesc(b + it.bytes, 128, it.b_sbo);
+                uint64_t ah = mdesc(ah0 + it.a, 128, it.a_sbo), al = mdesc(al0 + it.a, 128, it.a_sbo);
+                const uint32_t d_main = tmem + (ph & 1u) * (2 * kPh), d_corr = d_main + kPh;
+                uint32_t acc = it.edge & 1u ? 0u : 1u;
+                for (int k = 0; k < it.steps; ++k) {
+                    mma_el(el, d_corr, al, bh, it.idesc, acc);
+                    mma_el(el, d_main, ah, bh, it.idesc, acc);
+                    mma_el(el, d_corr, ah, bl, it.idesc, 1u);
+                    acc = 1u;
+                    ah += 16;
+                    al += 16;
+                    bh += 16;
+                    bl += 16;
+                }
+                commit_el(el, bar_empty + 8 * stage);
+                if (it.edge & 2u) commit_el(el, bar_acc + 8 * (ph++ & 1u));
+            }
+        }
+        if (!ok && el) {
+            mma_commit(bar_end);
+            for (uint32_t it = 0; it < kMaxSpin && !mbar_try(bar_end, 0); ++it) {
+            }
+        }
+    } else {
+        // ---------------------------------------- epilogue
+        const int q = warp & 3, pt = warp >> 2;
+        const int sq = lane >> 2, fc = 2 * (lane & 3);
+        const uint32_t lq = (uint32_t)(32 * q) << 16, lq16 = (uint32_t)(32 * q + 16) << 16;
+        const float inv_beta = 1.0f / p.beta;
+        const float b0 = __ldg(p.sdf_w + F::param_offset(LS - 1) + (int64_t)F::layer(LS - 1).out * F::layer(LS - 1).in);
+        const int et = threadIdx.x;
+        uint32_t phs = 0, epi_ph = 0;            // phases waited for, epilogue barriers
+        uint32_t buf = 0;                         // TMEM column of the phase in hand
+        __half2 big = __float2half2_rn(0.0f);     // largest |operand| (scaled high parts) of this thread, or NaN
+        const __half2 kHuge = __float2half2_rn(65504.0f);
+        bool ok = true;
+        auto epi_sync = [&]() -> bool {
+            __syncwarp();
+            if (lane == 0) mbar_arrive(bar_epi);
+            const bool w = mbar_wait(bar_epi, epi_ph & 1u, abort_flag, p.spin);
+            ++epi_ph;
+            return __all_sync(0xffffffffu, w);
+        };
+        auto wait_acc = [&]() -> bool {
+            const uint32_t b = phs & 1u;
+            const bool w = __all_sync(0xffffffffu, mbar_wait(bar_acc + 8 * b, (phs >> 1) & 1u, abort_flag, p.spin));
+            ++phs;
+            buf = tmem + b * (2 * kPh);
+            tc_fence_after();
+            return w;
+        };
+        // the phase in hand has been read by this warp
+        auto drained = [&]() {
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(bar_drained + 8 * ((phs - 1) & 1u));
+        };
+        // this warp's share of the next operand's columns below (0) or from (1) 128 is stored
+        auto operand_done = [&](int half) {
+            fence_proxy_async();
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(bar_op + 8 * half);
+        };
+        // a phase's raw accumulators of one 8-column group: row groups 0-3 of this thread, two columns
+        auto issue4 = [&](int c, float (&m)[8], float (&cr)[8]) {
+            tmem_ld16x256_x1(buf + lq + c, m);
+            tmem_ld16x256_x1(buf + lq16 + c, m + 4);
+            tmem_ld16x256_x1(buf + lq + kPh + c, cr);
+            tmem_ld16x256_x1(buf + lq16 + kPh + c, cr + 4);
+        };
+        // the value rows only (row group 0): two columns of the phase
+        auto load1 = [&](int c, float share, float (&z)[2]) {
+            float m[4], cr[4];
+            tmem_ld16x256_x1(buf + lq + c, m);
+            tmem_ld16x256_x1(buf + lq + kPh + c, cr);
+            asm volatile("tcgen05.wait::ld.sync.aligned;" : "+f"(m[0]), "+f"(m[1]), "+f"(cr[0]), "+f"(cr[1]) : : "memory");
+#pragma unroll
+            for (int e = 0; e < 2; ++e) z[e] = fmaf(m[e], share, fmaf(cr[e], kLoDown, m[e]));
+        };
+        // row i of the lane quarter (stmatrix: lane i addresses row i) at column 0
+        auto row_at = [&](uint8_t* base, int r, int pitch) { return smem_u32(base) + a_off(32 * q + r, 0, pitch); };
+        // sample (VALUE: its row) that row group r of this thread belongs to
+        auto sample_of = [&](int r) { return VALUE ? 32 * q + 8 * r + sq : 8 * q + sq; };
+        auto enc = [&](int r, int j) {
+            const int s = sample_of(r);
+            return enc_tab(s_x + s * kXRow, s_pe + s * A::kPeSdf * 6, A::kPeSdf, j, VALUE ? 0 : r);
+        };
+        auto split = [&](float a, float b, uint32_t& hi, uint32_t& lo) {
+            split_f32(a, b, hi, lo);
+            big = __hmax2_nan(big, __habs2(*reinterpret_cast<const __half2*>(&hi)));
+        };
+        // split the four row groups' column pairs v
+        auto split4 = [&](const float (&v)[8], uint32_t (&o)[8]) {
+#pragma unroll
+            for (int r = 0; r < 4; ++r) split(v[2 * r], v[2 * r + 1], o[r], o[4 + r]);
+        };
+        // whether a value of this warp is out of the parts' range since the last call
+        auto out_of_range = [&]() {
+            const float2 m = __half22float2(big);
+            big = __float2half2_rn(0.0f);
+            return __any_sync(0xffffffffu, !(fmaxf(m.x, m.y) < kUp * kLimit && m.x == m.x && m.y == m.y)) != 0;
+        };
+        auto store4 = [&](uint32_t rh, uint32_t rl, int c, const uint32_t (&o)[8]) {
+            const uint32_t co = (uint32_t)(c >> 3) * 128u;
+            stmatrix4(rh + co, o[0], o[1], o[2], o[3]);
+            stmatrix4(rl + co, o[4], o[5], o[6], o[7]);
+        };
+        // the tile's table: x~ (and direction, t, delta), then sin / cos of the encodings' octaves
+        auto build_table = [&](int64_t tile) -> bool {
+            if (et < TS) {
+                const int64_t g = tile * TS + et;
+                float t = 0.0f, dl = 0.0f, xs[3] = {0.0f, 0.0f, 0.0f}, ds[3] = {0.0f, 0.0f, 0.0f};
+                if (g < total) {
+                    int64_t ray;
+                    if (p.src.mode == kUniform) {
+                        ray = p.src.sample_ray ? (int64_t)__ldg(p.src.sample_ray + g) : find_ray(p.src.offsets, p.src.n_rays, g);
+                        const int32_t o0 = __ldg(p.src.offsets + ray), o1 = __ldg(p.src.offsets + ray + 1);
+                        const float tn = __ldg(p.src.t_n + ray), tf = __ldg(p.src.t_f + ray);
+                        dl = (tf - tn) / (float)(o1 - o0);
+                        t = tn + ((float)(g - o0) + 0.5f) * dl;
+                    } else {
+                        ray = explicit_ray(p.src, g);
+                        t = __ldg(p.src.t + g);
+                        if constexpr (!VALUE) dl = __ldg(p.src.delta + g);
+                    }
+#pragma unroll
+                    for (int a = 0; a < 3; ++a) {
+                        ds[a] = __ldg(p.src.ray_d + 3 * ray + a);
+                        const float x = __ldg(p.src.ray_o + 3 * ray + a) + t * ds[a];
+                        xs[a] = (x - p.center[a]) * p.inv_scale;
+                    }
+                }
+                float* sx = s_x + et * kXRow;
+#pragma unroll
+                for (int a = 0; a < 3; ++a) {
+                    sx[a] = xs[a];
+                    if constexpr (!VALUE) sx[3 + a] = ds[a];
+                }
+                if constexpr (!VALUE) {
+                    sx[6] = t;
+                    sx[7] = dl;
+                }
+            }
+            if (!epi_sync()) return false;
+            constexpr int nd = VALUE ? 0 : A::kPeDir, per = 3 * (A::kPeSdf + nd);
+            constexpr int div = per > 0 ? per : 1;
+            for (int e = et; e < TS * per; e += kEpi * 32) {
+                const int s = e / div, k = e % div;
+                const bool dir = k >= 3 * A::kPeSdf;
+                const int i = dir ? k - 3 * A::kPeSdf : k;    // octave * 3 + axis
+                float sn, cs;
+                sincosf((float)(1 << (i / 3)) * s_x[s * kXRow + (dir ? 3 : 0) + i % 3], &sn, &cs);
+                float* dst = (dir ? s_pd + s * A::kPeDir * 6 : s_pe + s * A::kPeSdf * 6) + 2 * i;
+                dst[0] = sn;
+                dst[1] = cs;
+            }
+            return epi_sync();
+        };
+        auto write_input0 = [&]() {
+            constexpr int K0 = F::k_main(0);
+            const uint32_t rh = row_at(a_hi, lane, K0), rl = row_at(a_lo, lane, K0);
+            for (int gr = pt; gr < K0 / 8; gr += kParts) {
+                float v[8];
+#pragma unroll
+                for (int r = 0; r < 4; ++r)
+#pragma unroll
+                    for (int e = 0; e < 2; ++e) {
+                        const int j = 8 * gr + fc + e;
+                        v[2 * r + e] = j < A::kEnc ? enc(r, j) : 0.0f;
+                    }
+                uint32_t o[8];
+                split4(v, o);
+                store4(rh, rl, 8 * gr, o);
+            }
+            operand_done(0);
+        };
+
+        ok = build_table(blockIdx.x);
+        if (ok) write_input0();
+        for (int64_t tile = blockIdx.x; tile < n_tiles && ok; tile += gridDim.x) {
+            const float* bias = s_bias;
+            for (int L = 0; L < NLr && ok; bias += F::n_pad(L), ++L) {
+                // a single K step (the 3 raw coordinates and their one-hot derivatives) is exact or nearly so
+                const int n_mma = (F::k_main(L) + (L == LS ? F::kXp : 0)) / 16;
+                const float share = n_mma > 1 ? kBias0 + kBias1 * (float)n_mma : 0.0f;
+                if (L < LS - 1) {
+                    // ---- hidden SDF layer: softplus on value rows, its slope times the tangent rows ----
+                    const int N = F::layer(L).out, Np = F::n_pad(L), Kn = F::k_main(L + 1);
+                    const bool skip = L + 1 == A::kSkip;
+                    const bool last = L == LS - 2;             // net_0's dot products are taken here
+                    const bool store = !(VALUE && last);
+                    float dot[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+                    const float sc = skip ? kRsqrt2 : 1.0f;
+                    const uint32_t rh = row_at(a_hi, lane, Kn), rl = row_at(a_lo, lane, Kn);
+                    // accumulator sums z of operand columns c .. c + 7 -> both parts of the next operand
+                    auto act = [&](int c, const float (&z)[8], uint32_t (&o)[8]) {
+                        float v[8];
+#pragma unroll
+                        for (int e = 0; e < 2; ++e) {
+                            const int col = c + fc + e;
+                            if (col < N) {
+                                const float b = bias[col];
+                                float h, sg;
+                                if constexpr (VALUE) {
+#pragma unroll
+                                    for (int r = 0; r < 4; ++r) {
+                                        softplus_slope_f32(fmaf(z[2 * r + e], kDown, b), p.beta, inv_beta, h, sg);
+                                        v[2 * r + e] = h * sc;
+                                    }
+                                } else {
+                                    softplus_slope_f32(fmaf(z[e], kDown, b), p.beta, inv_beta, h, sg);
+                                    v[e] = h * sc;
+                                    sg *= sc;
+#pragma unroll
+                                    for (int r = 1; r < 4; ++r) v[2 * r + e] = sg * (z[2 * r + e] * kDown);
+                                }
+                                if (last) {
+                                    const float w = s_w0[col];
+#pragma unroll
+                                    for (int r = 0; r < 4; ++r) dot[r] = fmaf(v[2 * r + e], w, dot[r]);
+                                }
+                            } else {
+                                // beyond the outputs: the skip input's encoding, or padding
+                                const bool in = skip && col - N < A::kEnc;
+#pragma unroll
+                                for (int r = 0; r < 4; ++r) v[2 * r + e] = in ? enc(r, col - N) * sc : 0.0f;
+                            }
+                        }
+                        split4(v, o);
+                    };
+                    // a phase's groups of this part in turn, the next one's loads in flight: group i of
+                    // operand column n0 + c to use(i, c, parts); acc: the groups below it have accumulators
+                    auto groups = [&](int n0, int n_acc, int n_all, auto use) {
+                        float m[2][8], cr[2][8];
+                        if (8 * pt < n_acc) issue4(8 * pt, m[0], cr[0]);
+#pragma unroll
+                        for (int i = 0; i < kGrp; ++i) {
+                            const int c = 8 * (pt + i * kParts), cn = c + 8 * kParts;
+                            if (c >= n_all) continue;
+                            float z[8];
+                            if (c < n_acc) {
+                                wait_ld16(m[i & 1], cr[i & 1]);
+                                if (cn < n_acc) issue4(cn, m[(i + 1) & 1], cr[(i + 1) & 1]);
+#pragma unroll
+                                for (int k = 0; k < 8; ++k)
+                                    z[k] = fmaf(m[i & 1][k], share, fmaf(cr[i & 1][k], kLoDown, m[i & 1][k]));
+                            } else {
+#pragma unroll
+                                for (int k = 0; k < 8; ++k) z[k] = 0.0f;
+                            }
+                            uint32_t o[8];
+                            act(n0 + c, z, o);
+                            use(i, c, o);
+                        }
+                    };
+                    uint32_t held[kGrp][8];
+                    const bool two = Np > kPh;
+                    if (two) {
+                        if (!wait_acc()) { ok = false; break; }
+                        groups(0, kPh, kPh, [&](int i, int, const uint32_t (&o)[8]) {
+#pragma unroll
+                            for (int k = 0; k < 8; ++k) held[i][k] = o[k];
+                        });
+                        drained();
+                    }
+                    if (!wait_acc()) { ok = false; break; }
+                    const int n0 = two ? kPh : 0;
+                    if (two && store) {
+#pragma unroll
+                        for (int i = 0; i < kGrp; ++i)
+                            if (pt + i * kParts < kPh / 8) store4(rh, rl, 8 * (pt + i * kParts), held[i]);
+                        operand_done(0);
+                    }
+                    groups(n0, Np - n0, Kn - n0, [&](int, int c, const uint32_t (&o)[8]) {
+                        if (store) store4(rh, rl, n0 + c, o);
+                    });
+                    drained();
+                    if (store) operand_done(two ? 1 : 0);
+                    if (last) {
+#pragma unroll
+                        for (int r = 0; r < 4; ++r) {
+                            dot[r] += __shfl_xor_sync(0xffffffffu, dot[r], 1);
+                            dot[r] += __shfl_xor_sync(0xffffffffu, dot[r], 2);
+                            if ((lane & 3) == 0) s_dot[pt * 128 + 32 * q + 8 * r + sq] = dot[r];
+                        }
+                    }
+                    if constexpr (VALUE) {
+                        if (last) {
+                            // the SDF values, and the next tile's input
+                            if (!epi_sync()) { ok = false; break; }
+                            if (et < TS) {
+                                const float f = p.scale * (s_dot[et] + s_dot[128 + et] + s_dot[256 + et] + b0);
+                                if (!(fabsf(f) < __int_as_float(0x7f800000))) big = kHuge;
+                                if (tile * TS + et < total) p.f_out[tile * TS + et] = f;
+                            }
+                            if (out_of_range() && lane == 0) *s_mark = (uint32_t)(tile + 1);
+                            if (!epi_sync()) { ok = false; break; }
+                            if (et == 0 && *s_mark == (uint32_t)(tile + 1)) {
+                                for (int k = 0; k < TS / 64; ++k)
+                                    if (tile * TS + 64 * k < total) p.f_out[tile * TS + 64 * k] = __uint_as_float(kRedoBits);
+                                atomicExch(p.redo, 1u);
+                            }
+                            if (tile + gridDim.x < n_tiles) {
+                                if (!build_table(tile + gridDim.x)) { ok = false; break; }
+                                write_input0();
+                            }
+                        }
+                    }
+                } else if (L == LS - 1) {
+                    // ---- SDF output: the features; net_0 and its gradient from their dot products ----
+                    if constexpr (!VALUE) {
+                        constexpr int NF = F::phases(LS - 1);
+                        uint32_t held[NF][kGrp][2];
+#pragma unroll
+                        for (int ph = 0; ph < NF; ++ph) {
+                            if (!wait_acc()) { ok = false; break; }
+#pragma unroll
+                            for (int i = 0; i < kGrp; ++i) {
+                                const int c = 8 * (pt + i * kParts);
+                                if (c < F::phase_n(LS - 1, ph)) {
+                                    float z[2];
+                                    load1(c, share, z);
+#pragma unroll
+                                    for (int e = 0; e < 2; ++e) z[e] = fmaf(z[e], kDown, bias[ph * kPh + c + fc + e]);
+                                    split(z[0], z[1], held[ph][i][0], held[ph][i][1]);
+                                }
+                            }
+                            drained();
+                            if (ph > 0) continue;
+                            if (!epi_sync()) { ok = false; break; }
+                            if (et < kTile) {
+                                const int s = et, row = 32 * (s >> 3) + (s & 7);
+                                float n0[4];
+#pragma unroll
+                                for (int r = 0; r < 4; ++r)
+                                    n0[r] = s_dot[row + 8 * r] + s_dot[128 + row + 8 * r] + s_dot[256 + row + 8 * r];
+                                const float f = p.scale * (n0[0] + b0), gx = n0[1], gy = n0[2], gz = n0[3];
+                                const float gn = sqrtf(gx * gx + gy * gy + gz * gz);
+                                const float inv = gn > 0.0f ? 1.0f / gn : 0.0f;
+                                const float* sx = s_x + s * 8;
+                                float* so = s_out + s * 8;
+                                so[0] = f;
+                                so[1] = gx * sx[3] + gy * sx[4] + gz * sx[5];
+                                so[2] = sx[6];
+                                so[3] = sx[7];
+                                so[4] = gn;
+                                so[5] = gx * inv;
+                                so[6] = gy * inv;
+                                so[7] = gz * inv;
+                                const float inf = __int_as_float(0x7f800000);
+                                if ((!(gn >= kMinGrad && gn < inf) || !(fabsf(f) < inf)) && tile * TS + s < total) big = kHuge;
+                            }
+                        }
+                        if (!ok) break;
+                        // the features over the SDF operand's value rows
+                        const uint32_t vh = row_at(a_hi, lane & 7, F::kFp), vl = row_at(a_lo, lane & 7, F::kFp);
+#pragma unroll
+                        for (int ph = 0; ph < NF; ++ph)
+#pragma unroll
+                            for (int i = 0; i < kGrp; ++i) {
+                                const int c = 8 * (pt + i * kParts);
+                                if (c < F::phase_n(LS - 1, ph)) {
+                                    const uint32_t co = (uint32_t)((ph * kPh + c) >> 3) * 128u;
+                                    stmat1(vh + co, held[ph][i][0]);
+                                    stmat1(vl + co, held[ph][i][1]);
+                                }
+                            }
+                        if (!epi_sync()) { ok = false; break; }
+                        // x~, direction encoding, unit normal: one 8-column group of a sample per thread
+                        if (et < kTile * (F::kXp / 8)) {
+                            const int s = et / (F::kXp / 8), c = 8 * (et % (F::kXp / 8));
+                            uint32_t o[8];
+#pragma unroll
+                            for (int k = 0; k < 4; ++k) {
+                                float v[2];
+#pragma unroll
+                                for (int e = 0; e < 2; ++e) {
+                                    const int j = c + 2 * k + e;
+                                    v[e] = 0.0f;
+                                    if (j < 3) v[e] = s_x[s * 8 + j];
+                                    else if (j < 3 + A::kDirEnc)
+                                        v[e] = enc_tab(s_x + s * 8 + 3, s_pd + s * A::kPeDir * 6, A::kPeDir, j - 3, 0);
+                                    else if (j < F::kX) v[e] = s_out[s * 8 + 5 + j - 3 - A::kDirEnc];
+                                }
+                                split(v[0], v[1], o[k], o[4 + k]);
+                            }
+                            // row s of the value rows, one row group below
+                            const uint32_t at = a_off(32 * (s >> 3) + 8 + (s & 7), c, F::kFp);
+                            *reinterpret_cast<uint4*>(a_hi + at) = make_uint4(o[0], o[1], o[2], o[3]);
+                            *reinterpret_cast<uint4*>(a_lo + at) = make_uint4(o[4], o[5], o[6], o[7]);
+                        }
+                        operand_done(0);
+                        if (F::kFp > kPh) operand_done(1);
+                        // this tile's table is read no more: the next tile's, while the colour layers run
+                        if (!epi_sync()) { ok = false; break; }
+                        if (tile + gridDim.x < n_tiles && !build_table(tile + gridDim.x)) { ok = false; break; }
+                    }
+                } else {
+                    // ---- hidden colour layer: ReLU on the value rows ----
+                    const int Kn = F::n_pad(L);
+                    const bool last = L == F::NL - 2;          // the colours' dot products are taken here
+                    const uint32_t vh = row_at(a_hi, lane & 7, Kn), vl = row_at(a_lo, lane & 7, Kn);
+                    constexpr int NP = 2;
+                    uint32_t held[NP][kGrp][2];
+                    float cd[3] = {0.0f, 0.0f, 0.0f};
+                    const int nph = F::phases(L);
+#pragma unroll
+                    for (int ph = 0; ph < NP; ++ph) {
+                        if (ph >= nph) continue;
+                        if (!wait_acc()) { ok = false; break; }
+#pragma unroll
+                        for (int i = 0; i < kGrp; ++i) {
+                            const int c = 8 * (pt + i * kParts);
+                            if (c < F::phase_n(L, ph)) {
+                                float z[2];
+                                load1(c, share, z);
+#pragma unroll
+                                for (int e = 0; e < 2; ++e) {
+                                    const int col = ph * kPh + c + fc + e;
+                                    z[e] = relu_nan(fmaf(z[e], kDown, bias[col]));
+                                    if (last) {
+#pragma unroll
+                                        for (int k = 0; k < 3; ++k) cd[k] = fmaf(z[e], s_wc[k * F::kWc + col], cd[k]);
+                                    }
+                                }
+                                split(z[0], z[1], held[ph][i][0], held[ph][i][1]);
+                            }
+                        }
+                        drained();
+                    }
+                    if (!ok) break;
+                    if (!last) {
+#pragma unroll
+                        for (int ph = 0; ph < NP; ++ph)
+#pragma unroll
+                            for (int i = 0; i < kGrp; ++i) {
+                                const int c = 8 * (pt + i * kParts);
+                                if (ph < nph && c < F::phase_n(L, ph)) {
+                                    const uint32_t co = (uint32_t)((ph * kPh + c) >> 3) * 128u;
+                                    stmat1(vh + co, held[ph][i][0]);
+                                    stmat1(vl + co, held[ph][i][1]);
+                                }
+                            }
+                        operand_done(0);
+                        if (Kn > kPh) operand_done(1);
+                        continue;
+                    }
+                    // ---- the next tile's layer-0 input (every MMA of this one is complete), the records ----
+#pragma unroll
+                    for (int k = 0; k < 3; ++k) {
+                        cd[k] += __shfl_xor_sync(0xffffffffu, cd[k], 1);
+                        cd[k] += __shfl_xor_sync(0xffffffffu, cd[k], 2);
+                        if ((lane & 3) == 0) s_cdot[(pt * 3 + k) * kTile + 8 * q + sq] = cd[k];
+                    }
+                    if (out_of_range() && lane == 0) *s_mark = (uint32_t)(tile + 1);
+                    if (!epi_sync()) { ok = false; break; }
+                    if (tile + gridDim.x < n_tiles) write_input0();
+                    if (et < kTile) {
+                        const float* bc = p.rgb_w + F::param_offset(F::NL - 1) + 3 * F::layer(F::NL - 1).in;
+                        float c3[3];
+                        bool bad = *s_mark == (uint32_t)(tile + 1);
+#pragma unroll
+                        for (int k = 0; k < 3; ++k) {
+                            c3[k] = s_cdot[k * kTile + et] + s_cdot[(3 + k) * kTile + et] + s_cdot[(6 + k) * kTile + et] + __ldg(bc + k);
+                            bad = bad || !(fabsf(c3[k]) < __int_as_float(0x7f800000));
+                        }
+                        const bool mark = __any_sync(0xffffffffu, bad) != 0;
+                        const int64_t g = tile * kTile + et;
+                        const float4* so = reinterpret_cast<const float4*>(s_out + et * 8);
+                        const float4 s0 = so[0], s1 = so[1];
+                        if (g < total) {
+                            float4* R4 = reinterpret_cast<float4*>(p.rec + g);
+                            R4[0] = s0;
+                            R4[1] = make_float4(1.0f / (1.0f + expf(-c3[0])), 1.0f / (1.0f + expf(-c3[1])),
+                                                1.0f / (1.0f + expf(-c3[2])), s1.x);
+                            R4[2] = make_float4(s1.y, s1.z, s1.w, mark && (g % 16) == 0 ? 1.0f : 0.0f);
+                        }
+                        if (mark && et == 0) atomicExch(p.redo, 1u);
+                    }
+                }
+            }
+        }
+        if (!ok) set_status(p.status, TSDFS_DEV_TIMEOUT);
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    if (warp == kMma) {
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512));
+    }
+}
+
+// Split the parameters into the items' hi and lo images (8 x 8 core matrices, K-major), one
+// 8-column row piece per thread; clears the redo word.  3 MB for the room networks, every call:
+// the parameters may have changed since the last one.
+template <int ARCH>
+__global__ void k_split_weights(const float* __restrict__ sdf_w, const float* __restrict__ rgb_w,
+                                uint8_t* __restrict__ packed, uint32_t* __restrict__ redo) {
+    using F = FArch<ARCH>;
+    if (blockIdx.x == 0 && threadIdx.x == 0) *redo = 0;
+    constexpr int64_t n8 = F::packed_bytes() / 32;   // 8 columns x 2 parts x 2 bytes
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n8; i += (int64_t)gridDim.x * blockDim.x) {
+        int L = 0;
+        while (L + 2 < F::NL && F::layer_base(L + 1) <= i * 32) ++L;
+        const Layer ly = F::layer(L);
+        int64_t r = i - F::layer_base(L) / 32;     // within the layer, in items' order
+        const int kt = (F::k_main(L) + (L == F::LS ? F::kXp : 0)) / 8;
+        int ph = 0, n_first = 0;
+        while (r >= (int64_t)F::phase_n(L, ph) * kt) {
+            r -= (int64_t)F::phase_n(L, ph) * kt;
+            n_first += F::phase_n(L, ph++);
+        }
+        const int n_ph = F::phase_n(L, ph);
+        int c = 0, k_first = 0;
+        while (r >= (int64_t)n_ph * (F::chunk_k(L, c) / 8)) {
+            r -= (int64_t)n_ph * (F::chunk_k(L, c) / 8);
+            k_first += F::chunk_k(L, c++);
+        }
+        const int kc8 = F::chunk_k(L, c) / 8;
+        const int n = (int)(r / kc8), k8 = (int)(r % kc8);
+        const int row = F::src_row(L, n_first + n);
+        const float* W = (L < F::LS ? sdf_w : rgb_w) + F::param_offset(L);
+        uint32_t o[8];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            float v[2];
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                const int col = F::src_col(L, k_first + 8 * k8 + 2 * j + e);
+                v[e] = row >= 0 && col >= 0 ? __ldg(W + (int64_t)row * ly.in + col) : 0.0f;
+            }
+            split_f32(v[0], v[1], o[j], o[4 + j]);
+        }
+        // the item's hi image starts after the phases and chunks before it
+        uint8_t* item = packed + F::layer_base(L) + (int64_t)n_first * kt * 32 + (int64_t)n_ph * (k_first / 8) * 32;
+        const uint32_t at = (uint32_t)(((n >> 3) * kc8 + k8) * 128 + (n & 7) * 16);
+        *reinterpret_cast<uint4*>(item + at) = make_uint4(o[0], o[1], o[2], o[3]);
+        *reinterpret_cast<uint4*>(item + (int64_t)n_ph * kc8 * 16 + at) = make_uint4(o[4], o[5], o[6], o[7]);
+    }
+}
+
+template <int ARCH, bool VALUE>
+int launch_f32(const tsdfs_mlp* m, const SampleSource& src, SampleRec* rec, float* f_out, int64_t max_samples,
+               uint8_t* stash, cudaStream_t st) {
+    using F = FArch<ARCH>;
+    constexpr size_t smem = F::template smem_bytes<VALUE>();
+    static_assert(smem <= 232448, "k_mlp_f32 shared memory exceeds 227 KB");
+    static std::mutex mu;
+    static bool set[64] = {};
+    int dev = 0, sms = 152;
+    int rc = cuda_check(cudaGetDevice(&dev), "mlp_f32 device");
+    if (rc) return rc;
+    {
+        std::lock_guard<std::mutex> lk(mu);
+        if (dev < 0 || dev >= 64 || !set[dev]) {
+            rc = cuda_check(cudaFuncSetAttribute(k_mlp_f32<ARCH, VALUE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                 (int)smem),
+                            "mlp_f32 smem attribute");
+            if (rc) return rc;
+            if (dev >= 0 && dev < 64) set[dev] = true;
+        }
+    }
+    F32Params p{};
+    p.packed = stash + kRedoBytes;
+    p.redo = reinterpret_cast<uint32_t*>(stash);
+    p.sdf_w = m->sdf_w;
+    p.rgb_w = m->rgb_w;
+    for (int a = 0; a < 3; ++a) p.center[a] = m->center[a];
+    p.scale = m->scale;
+    p.inv_scale = 1.0f / m->scale;
+    p.beta = m->beta;
+    p.src = src;
+    p.rec = rec;
+    p.f_out = f_out;
+    p.status = device_status_word();
+    p.spin = test_spin_limit(kMaxSpin);
+    p.withhold = test_withhold_chunk();
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const int64_t ts = VALUE ? kTileV : kTile, tiles = (max_samples + ts - 1) / ts;
+    const unsigned blocks = (unsigned)(tiles < sms ? (tiles < 1 ? 1 : tiles) : sms);
+    k_split_weights<ARCH><<<grid_1d(F::packed_bytes() / 32, 256), 256, 0, st>>>(m->sdf_w, m->rgb_w,
+                                                                               stash + kRedoBytes, p.redo);
+    k_mlp_f32<ARCH, VALUE><<<blocks, kThr, smem, st>>>(p);
+    return cuda_check(cudaGetLastError(), "mlp_f32 launch");
+}
+
+}  // namespace
+
+size_t mlp_f32_stash_bytes() { return kRedoBytes + (size_t)FArch<TSDFS_ARCH_ROOM>::packed_bytes(); }
+
+int launch_mlp_full_f32(const tsdfs_mlp* m, const SampleSource& src, SampleRec* rec, int64_t max_samples,
+                        uint8_t* stash, cudaStream_t st) {
+    return m->arch == TSDFS_ARCH_TINY ? launch_f32<TSDFS_ARCH_TINY, false>(m, src, rec, nullptr, max_samples, stash, st)
+                                      : launch_f32<TSDFS_ARCH_ROOM, false>(m, src, rec, nullptr, max_samples, stash, st);
+}
+
+int launch_mlp_value_f32(const tsdfs_mlp* m, const SampleSource& src, float* f_out, uint8_t* stash, cudaStream_t st) {
+    const int64_t n = sample_bound(src);
+    return m->arch == TSDFS_ARCH_TINY ? launch_f32<TSDFS_ARCH_TINY, true>(m, src, nullptr, f_out, n, stash, st)
+                                      : launch_f32<TSDFS_ARCH_ROOM, true>(m, src, nullptr, f_out, n, stash, st);
+}
+
+}  // namespace tsdfs

@@ -9,6 +9,7 @@
 // K-chunk tile in shared memory.  Results go to a per-sample record consumed
 // by the compositing kernel.
 #include "common.cuh"
+#include "mlp_f32.cuh"
 
 namespace tsdfs {
 
@@ -231,10 +232,11 @@ __device__ void rgb_network(Smem& sm, const NetParams& np, int& cur) {
 // Full evaluation: f, grad f, colour for each sample -> records.
 template <int ARCH>
 __global__ void __launch_bounds__(kThreads, 1) k_mlp_full(NetParams np, SampleSource src, SampleRec* __restrict__ rec,
-                                                          uint32_t* dev_status) {
+                                                          const uint32_t* redo, uint32_t* dev_status) {
     using A = Arch<ARCH>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     Smem& sm = *reinterpret_cast<Smem*>(smem_raw);
+    if (redo && *redo == 0) return;
     int64_t total = sample_total(src);
     if (total > src.capacity) {
         if (blockIdx.x == 0 && threadIdx.x == 0) set_status(dev_status, TSDFS_DEV_SAMPLES_OVERFLOW);
@@ -243,6 +245,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_mlp_full(NetParams np, SampleSo
     const int64_t n_tiles = (total + kTS - 1) / kTS;
     for (int64_t tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
         __syncthreads();
+        if (redo && rec[tile * kTS].pad == 0.0f) continue;   // not marked
         if (threadIdx.x < kTS) {
             const int s = threadIdx.x;
             const int64_t g = tile * kTS + s;
@@ -361,10 +364,11 @@ __global__ void __launch_bounds__(kThreads, 1) k_mlp_full(NetParams np, SampleSo
 // SDF values only (hierarchical coarse pass): 4*kTS samples per tile, one row each.
 template <int ARCH>
 __global__ void __launch_bounds__(kThreads, 1) k_mlp_value(NetParams np, SampleSource src, float* __restrict__ f_out,
-                                                           uint32_t* dev_status) {
+                                                           const uint32_t* redo, uint32_t* dev_status) {
     using A = Arch<ARCH>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     Smem& sm = *reinterpret_cast<Smem*>(smem_raw);
+    if (redo && *redo == 0) return;
     const int64_t total = sample_total(src);
     if (total > src.capacity) {
         if (blockIdx.x == 0 && threadIdx.x == 0) set_status(dev_status, TSDFS_DEV_SAMPLES_OVERFLOW);
@@ -374,6 +378,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_mlp_value(NetParams np, SampleS
     const int64_t n_tiles = (total + TS - 1) / TS;
     for (int64_t tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
         __syncthreads();
+        if (redo && __float_as_uint(f_out[tile * TS]) != kRedoBits) continue;   // not marked
         if (threadIdx.x < TS) {
             const int s = threadIdx.x;
             const int64_t g = tile * TS + s;
@@ -450,26 +455,29 @@ static unsigned persistent_blocks(int64_t tiles) {
 // max_samples: host-side bound on the sample total (sizes the persistent grid)
 template <int ARCH>
 int launch_mlp_full_simt(const NetParams& np, const SampleSource& src, SampleRec* rec, int64_t max_samples,
-                         cudaStream_t st) {
+                         const uint32_t* redo, cudaStream_t st) {
     int rc = ensure_attrs<ARCH>();
     if (rc) return rc;
     k_mlp_full<ARCH><<<persistent_blocks((max_samples + kTS - 1) / kTS), kThreads, sizeof(Smem), st>>>(
-        np, src, rec, device_status_word());
+        np, src, rec, redo, device_status_word());
     return cuda_check(cudaGetLastError(), "mlp launch");
 }
 
 template <int ARCH>
-int launch_mlp_value_simt(const NetParams& np, const SampleSource& src, float* f_out, cudaStream_t st) {
+int launch_mlp_value_simt(const NetParams& np, const SampleSource& src, float* f_out, const uint32_t* redo,
+                          cudaStream_t st) {
     int rc = ensure_attrs<ARCH>();
     if (rc) return rc;
     k_mlp_value<ARCH><<<persistent_blocks((sample_bound(src) + 4 * kTS - 1) / (4 * kTS)), kThreads, sizeof(Smem), st>>>(
-        np, src, f_out, device_status_word());
+        np, src, f_out, redo, device_status_word());
     return cuda_check(cudaGetLastError(), "mlp value launch");
 }
 
-template int launch_mlp_full_simt<TSDFS_ARCH_TINY>(const NetParams&, const SampleSource&, SampleRec*, int64_t, cudaStream_t);
-template int launch_mlp_full_simt<TSDFS_ARCH_ROOM>(const NetParams&, const SampleSource&, SampleRec*, int64_t, cudaStream_t);
-template int launch_mlp_value_simt<TSDFS_ARCH_TINY>(const NetParams&, const SampleSource&, float*, cudaStream_t);
-template int launch_mlp_value_simt<TSDFS_ARCH_ROOM>(const NetParams&, const SampleSource&, float*, cudaStream_t);
+template int launch_mlp_full_simt<TSDFS_ARCH_TINY>(const NetParams&, const SampleSource&, SampleRec*, int64_t, const uint32_t*,
+                                                    cudaStream_t);
+template int launch_mlp_full_simt<TSDFS_ARCH_ROOM>(const NetParams&, const SampleSource&, SampleRec*, int64_t, const uint32_t*,
+                                                    cudaStream_t);
+template int launch_mlp_value_simt<TSDFS_ARCH_TINY>(const NetParams&, const SampleSource&, float*, const uint32_t*, cudaStream_t);
+template int launch_mlp_value_simt<TSDFS_ARCH_ROOM>(const NetParams&, const SampleSource&, float*, const uint32_t*, cudaStream_t);
 
 }  // namespace tsdfs
