@@ -29,113 +29,280 @@ __global__ void k_grid_init(void* V, int f16, uint8_t* W, int64_t n) {
     }
 }
 
-// One thread per voxel; the camera table of all views is staged in shared
-// memory (16 floats per view: c2w[12], fx, fy, cx, cy).
+// Projective fusion, brick by brick.  A camera inside a room sees about a tenth of its voxels, and
+// what a voxel-view costs is the projection's IEEE divisions and square root (~170 instructions in
+// all).  So:
+//  - a block takes a brick of 8 x 8 x 8 voxels and first tests every view against it (a view per
+//    thread; the image's four side planes and the camera plane as linear functions over a box); only
+//    the views that may see it are run per voxel, in their order, and a brick that no view sees is not
+//    read.  A view is left out only if every voxel of the brick fails the per-voxel tests: a plane's
+//    bound is widened by 1e-5 of the sum of its terms' magnitudes, some 20 times the FP32 rounding
+//    of the per-voxel arithmetic, and a NaN keeps the view;
+//  - the pixel comes from an approximate reciprocal wherever u and v are not within its error of a
+//    whole number, and from the divisions elsewhere (the same pixel either way);
+//  - a depth that is more than D_T (and the rounding) in front of or behind the voxel needs no
+//    projection onto the ray: the voxel is skipped, or s is D_T and s / D_T is 1; and a voxel whose
+//    mean is 1 keeps it.
+// The camera table of all views is staged in shared memory once per block (20 floats per view:
+// c2w[12], fx, fy, cx, cy and what the tests use), the list of the brick's views after it.  256^3
+// voxels, 100 views of the room: 2816 us without any of it, 950 with bricks of 32 x 4 x 4 alone.
+constexpr int kBX = 8, kBY = 8, kBZ = 8;
+constexpr int kBrickVoxels = kBX * kBY * kBZ;
+constexpr int kCam = 20;
+
+// whether view P can see a voxel centre within h[3] of c[3]
+__device__ __forceinline__ bool brick_visible(const float* P, const float c[3], const float h[3], float fW, float fH) {
+    float x = 0.0f, y = 0.0f, z = 0.0f;          // camera coordinates of the centre
+    float ax = 0.0f, ay = 0.0f, az = 0.0f;       // sums of their terms' magnitudes over the brick
+    float d[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        d[k] = c[k] - P[4 * k + 3];
+        const float m = fabsf(c[k]) + fabsf(P[4 * k + 3]) + h[k];
+        x += P[4 * k] * d[k];
+        y += P[4 * k + 1] * d[k];
+        z += P[4 * k + 2] * d[k];
+        ax += fabsf(P[4 * k]) * m;
+        ay += fabsf(P[4 * k + 1]) * m;
+        az += fabsf(P[4 * k + 2]) * m;
+    }
+    const float fx = P[12], fy = P[13], cx = P[14], cy = P[15];
+    float rz = 0.0f, rl = 0.0f, rr = 0.0f, rt = 0.0f, rb = 0.0f;   // half ranges over the brick
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        rz += fabsf(P[4 * k + 2]) * h[k];
+        rl += fabsf(fx * P[4 * k] + cx * P[4 * k + 2]) * h[k];
+        rr += fabsf(fx * P[4 * k] + (cx - fW) * P[4 * k + 2]) * h[k];
+        rt += fabsf(fy * P[4 * k + 1] + cy * P[4 * k + 2]) * h[k];
+        rb += fabsf(fy * P[4 * k + 1] + (cy - fH) * P[4 * k + 2]) * h[k];
+    }
+    constexpr float kSlack = 1e-5f;
+    const float su = kSlack * (fabsf(fx) * ax + (fabsf(cx) + fW) * az), sv = kSlack * (fabsf(fy) * ay + (fabsf(cy) + fH) * az);
+    if (z + rz + kSlack * az < 0.0f) return false;                        // behind the camera
+    if (fx * x + cx * z + rl + su < 0.0f) return false;                   // u < 0 throughout
+    if (fx * x + (cx - fW) * z - rr - su > 0.0f) return false;            // u > W
+    if (fy * y + cy * z + rt + sv < 0.0f) return false;
+    if (fy * y + (cy - fH) * z - rb - sv > 0.0f) return false;
+    return true;
+}
+
 __global__ void __launch_bounds__(kFuseBlock) k_integrate(int nx, int ny, int nz, float ox, float oy, float oz,
                                                           float vs, float trunc, void* V, int f16, uint8_t* W,
                                                           const float* __restrict__ depth, int nv, int H, int Wd,
                                                           const float* __restrict__ Kc, const float* __restrict__ c2w) {
     extern __shared__ float cam[];
-    for (int i = threadIdx.x; i < nv * 16; i += blockDim.x) {
-        int v = i >> 4, c = i & 15;
-        cam[i] = c < 12 ? c2w[v * 12 + c] : Kc[v * 4 + (c - 12)];
+    uint16_t* list = reinterpret_cast<uint16_t*>(cam + nv * kCam);
+    __shared__ int s_warp[kFuseBlock / 32];
+    for (int v = threadIdx.x; v < nv; v += blockDim.x) {
+        float* P = cam + v * kCam;
+        for (int c = 0; c < 12; ++c) P[c] = c2w[v * 12 + c];
+        for (int c = 0; c < 4; ++c) P[12 + c] = Kc[v * 4 + c];
+        // the voxel's range times cos(angle to its pixel's ray) is the projection: the pixel's half
+        // diagonal bounds the angle, 1e-5 the rounding
+        const float hx = 0.5f / P[12], hy = 0.5f / P[13];
+        P[16] = 1.0f - 1.1f * (hx * hx + hy * hy) - 1e-5f;     // least (projection / range)^2
+        P[17] = 1e-5f * fabsf(P[14]) + 1e-4f;                  // error of the approximate u, v: plus 1e-5 of them
+        P[18] = 1e-5f * fabsf(P[15]) + 1e-4f;
     }
-    __syncthreads();
-    const int64_t n = (int64_t)nx * ny * nz;
+    const int bx = (nx + kBX - 1) / kBX, by = (ny + kBY - 1) / kBY, bz = (nz + kBZ - 1) / kBZ;
+    const int64_t bricks = (int64_t)bx * by * bz;
     const float fW = (float)Wd, fH = (float)H;
-    for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < n; q += (int64_t)gridDim.x * blockDim.x) {
-        const int i = (int)(q % nx);
-        const int j = (int)((q / nx) % ny);
-        const int k = (int)(q / ((int64_t)nx * ny));
-        const float cx = __fadd_rn(ox, __fmul_rn(__fadd_rn((float)i, 0.5f), vs));
-        const float cy = __fadd_rn(oy, __fmul_rn(__fadd_rn((float)j, 0.5f), vs));
-        const float cz = __fadd_rn(oz, __fmul_rn(__fadd_rn((float)k, 0.5f), vs));
-        float Vv = load_v(V, f16, q);
-        int Wv = W[q];
-        for (int view = 0; view < nv; ++view) {
-            const float* P = cam + view * 16;
-            const float dx = __fsub_rn(cx, P[3]), dy = __fsub_rn(cy, P[7]), dz = __fsub_rn(cz, P[11]);
-            const float zc = __fadd_rn(__fadd_rn(__fmul_rn(P[2], dx), __fmul_rn(P[6], dy)), __fmul_rn(P[10], dz));
-            if (!(zc > 0.0f)) continue;
-            const float xc = __fadd_rn(__fadd_rn(__fmul_rn(P[0], dx), __fmul_rn(P[4], dy)), __fmul_rn(P[8], dz));
-            const float yc = __fadd_rn(__fadd_rn(__fmul_rn(P[1], dx), __fmul_rn(P[5], dy)), __fmul_rn(P[9], dz));
-            const float fx = P[12], fy = P[13], ccx = P[14], ccy = P[15];
-            const float u = __fadd_rn(__fmul_rn(fx, __fdiv_rn(xc, zc)), ccx);
-            const float v = __fadd_rn(__fmul_rn(fy, __fdiv_rn(yc, zc)), ccy);
-            if (!(u >= 0.0f && u < fW && v >= 0.0f && v < fH)) continue;
-            int px = (int)floorf(u), py = (int)floorf(v);
-            px = px >= Wd ? Wd - 1 : px;
-            py = py >= H ? H - 1 : py;
-            const float D = __ldg(depth + ((int64_t)view * H + py) * Wd + px);
-            const float a = __fdiv_rn(__fsub_rn(__fadd_rn((float)px, 0.5f), ccx), fx);
-            const float b = __fdiv_rn(__fsub_rn(__fadd_rn((float)py, 0.5f), ccy), fy);
-            const float nrm = __fsqrt_rn(__fadd_rn(__fadd_rn(__fmul_rn(a, a), __fmul_rn(b, b)), 1.0f));
-            const float proj = __fdiv_rn(__fadd_rn(__fadd_rn(__fmul_rn(a, xc), __fmul_rn(b, yc)), zc), nrm);
-            float s = __fsub_rn(D, proj);
-            if (s > trunc) s = trunc;
-            if (s < -trunc) s = -trunc;
-            if (s > -trunc) {
-                const float sn = __fdiv_rn(s, trunc);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int64_t br = blockIdx.x; br < bricks; br += gridDim.x) {
+        const int i0 = (int)(br % bx) * kBX, j0 = (int)((br / bx) % by) * kBY, k0 = (int)(br / ((int64_t)bx * by)) * kBZ;
+        const float h[3] = {0.5f * kBX * vs, 0.5f * kBY * vs, 0.5f * kBZ * vs};
+        const float c[3] = {ox + ((float)i0 + 0.5f * kBX) * vs, oy + ((float)j0 + 0.5f * kBY) * vs,
+                            oz + ((float)k0 + 0.5f * kBZ) * vs};
+        // the brick's views, in order
+        int n_list = 0;
+        for (int v0 = 0; v0 < nv; v0 += kFuseBlock) {
+            __syncthreads();   // the table; the last brick's list; s_warp
+            const int v = v0 + (int)threadIdx.x;
+            const bool keep = v < nv && brick_visible(cam + v * kCam, c, h, fW, fH);
+            const unsigned m = __ballot_sync(0xffffffffu, keep);
+            if (lane == 0) s_warp[warp] = __popc(m);
+            __syncthreads();
+            int before = n_list, all = 0;
+#pragma unroll
+            for (int w = 0; w < kFuseBlock / 32; ++w) {
+                const int n = s_warp[w];
+                before += w < warp ? n : 0;
+                all += n;
+            }
+            if (keep) list[before + __popc(m & ((1u << lane) - 1u))] = (uint16_t)v;
+            n_list += all;
+        }
+        if (n_list == 0) continue;
+        __syncthreads();
+        for (int e = threadIdx.x; e < kBrickVoxels; e += kFuseBlock) {
+            const int i = i0 + (e % kBX), j = j0 + (e / kBX) % kBY, k = k0 + e / (kBX * kBY);
+            if (i >= nx || j >= ny || k >= nz) continue;
+            const int64_t q = ((int64_t)k * ny + j) * nx + i;
+            const float cx = __fadd_rn(ox, __fmul_rn(__fadd_rn((float)i, 0.5f), vs));
+            const float cy = __fadd_rn(oy, __fmul_rn(__fadd_rn((float)j, 0.5f), vs));
+            const float cz = __fadd_rn(oz, __fmul_rn(__fadd_rn((float)k, 0.5f), vs));
+            float Vv = load_v(V, f16, q);
+            int Wv = W[q];
+            for (int l = 0; l < n_list; ++l) {
+                const int view = list[l];
+                const float* P = cam + view * kCam;
+                const float dx = __fsub_rn(cx, P[3]), dy = __fsub_rn(cy, P[7]), dz = __fsub_rn(cz, P[11]);
+                const float zc = __fadd_rn(__fadd_rn(__fmul_rn(P[2], dx), __fmul_rn(P[6], dy)), __fmul_rn(P[10], dz));
+                if (!(zc > 0.0f)) continue;
+                const float xc = __fadd_rn(__fadd_rn(__fmul_rn(P[0], dx), __fmul_rn(P[4], dy)), __fmul_rn(P[8], dz));
+                const float yc = __fadd_rn(__fadd_rn(__fmul_rn(P[1], dx), __fmul_rn(P[5], dy)), __fmul_rn(P[9], dz));
+                const float fx = P[12], fy = P[13], ccx = P[14], ccy = P[15];
+                // the pixel: floor(u), floor(v)
+                const float rz = __fdividef(1.0f, zc);
+                const float ua = fmaf(fx * xc, rz, ccx), va = fmaf(fy * yc, rz, ccy);
+                float fu = floorf(ua), fv = floorf(va);
+                const float eu = fmaf(1e-5f, fabsf(ua), P[17]), ev = fmaf(1e-5f, fabsf(va), P[18]);
+                const float ru = ua - fu, rv = va - fv;
+                if (!(ru > eu && ru < 1.0f - eu && rv > ev && rv < 1.0f - ev)) {
+                    const float u = __fadd_rn(__fmul_rn(fx, __fdiv_rn(xc, zc)), ccx);
+                    const float v = __fadd_rn(__fmul_rn(fy, __fdiv_rn(yc, zc)), ccy);
+                    if (!(u >= 0.0f && u < fW && v >= 0.0f && v < fH)) continue;
+                    fu = floorf(u);
+                    fv = floorf(v);
+                }
+                if (!(fu >= 0.0f && fu < fW && fv >= 0.0f && fv < fH)) continue;
+                const int px = min((int)fu, Wd - 1), py = min((int)fv, H - 1);
+                const float D = __ldg(depth + ((int64_t)view * H + py) * Wd + px);
+                // far behind the surface: proj >= range * cos > D + D_T
+                const float range2 = fmaf(xc, xc, fmaf(yc, yc, zc * zc)), reach = D + trunc;
+                if (reach >= 0.0f && reach * reach < range2 * P[16]) continue;
+                float sn = 1.0f;
+                // far before it: proj <= range < D - D_T, so s is cut to D_T
+                const float room = D - trunc;
+                if (!(room > 0.0f && room * room > range2 * 1.00001f)) {
+                    const float a = __fdiv_rn(__fsub_rn(__fadd_rn((float)px, 0.5f), ccx), fx);
+                    const float b = __fdiv_rn(__fsub_rn(__fadd_rn((float)py, 0.5f), ccy), fy);
+                    const float nrm = __fsqrt_rn(__fadd_rn(__fadd_rn(__fmul_rn(a, a), __fmul_rn(b, b)), 1.0f));
+                    const float proj = __fdiv_rn(__fadd_rn(__fadd_rn(__fmul_rn(a, xc), __fmul_rn(b, yc)), zc), nrm);
+                    float s = __fsub_rn(D, proj);
+                    if (s > trunc) s = trunc;
+                    if (s < -trunc) s = -trunc;
+                    if (!(s > -trunc)) continue;
+                    sn = __fdiv_rn(s, trunc);
+                }
                 const float Wf = (float)Wv;
-                Vv = __fdiv_rn(__fadd_rn(__fmul_rn(Wf, Vv), sn), __fadd_rn(Wf, 1.0f));
+                // (W + 1) / (W + 1)
+                if (!(sn == 1.0f && Vv == 1.0f))
+                    Vv = __fdiv_rn(__fadd_rn(__fmul_rn(Wf, Vv), sn), __fadd_rn(Wf, 1.0f));
                 if (Wv < 255) ++Wv;
             }
+            store_v(V, f16, q, Vv);
+            W[q] = (uint8_t)Wv;
         }
-        store_v(V, f16, q, Vv);
-        W[q] = (uint8_t)Wv;
     }
 }
 
-// K2: inside bit of voxel X = all voxels within Chebyshev radius r have V < 0,
-// computed as a separable running maximum over a shared-memory halo tile.
-constexpr int kMTX = 32, kMTY = 4, kMTZ = 4, kMaxR = 4;
+// K2: inside bit of voxel X = all voxels within Chebyshev radius r have V < 0.
+//
+// Only the signs matter, so the erosion runs on words of 32 voxels: a warp reads 32 voxels of a
+// row and one ballot makes their word; an x erosion is an AND of the word's shifts (with the
+// neighbour words' bits), the y and z erosions ANDs of whole words.  A block takes kMW words x
+// kMY x kMZ rows with a halo of r rows (and, at a tile's end inside the grid, one word); the volume is
+// read once from memory, the halo (1.9 x at r = 2) from L2.  Bound: the instructions of those reads.
+// 256^3 FP32, r = 2: 592 us as a running maximum of values over shared-memory tiles.  A NaN voxel
+// counts as negative unless its whole neighbourhood is NaN (a maximum of the values ignores a NaN):
+// a tile that has one goes through its neighbourhoods again.  Rows that are no multiple of 32 voxels
+// long put their words into the bit array with two atomic ORs each.
+constexpr int kMW = 8, kMY = 8, kMZ = 16, kMaxR = 4;
+constexpr int kMThreads = 256;
 
-__global__ void __launch_bounds__(kMTX * kMTY) k_inside_mask(const void* __restrict__ V, int f16, int nx, int ny,
-                                                             int nz, int r, uint32_t* __restrict__ bits,
-                                                             int aligned_rows) {
-    constexpr int HX = kMTX + 2 * kMaxR, HY = kMTY + 2 * kMaxR, HZ = kMTZ + 2 * kMaxR;
-    __shared__ float a[HZ][HY][HX];
-    __shared__ float bx[HZ][HY][kMTX];
-    __shared__ float by[HZ][kMTY][kMTX];
-    const int x0 = blockIdx.x * kMTX, y0 = blockIdx.y * kMTY, z0 = blockIdx.z * kMTZ;
-    const int hx = kMTX + 2 * r, hy = kMTY + 2 * r, hz = kMTZ + 2 * r;
-    const int tid = threadIdx.x + threadIdx.y * kMTX;
-    const int nthr = kMTX * kMTY;
-    for (int e = tid; e < hx * hy * hz; e += nthr) {
-        int lx = e % hx, ly = (e / hx) % hy, lz = e / (hx * hy);
-        int gx = x0 + lx - r, gy = y0 + ly - r, gz = z0 + lz - r;
-        float v = -1.0f;  // out of grid = unseen
-        if (gx >= 0 && gy >= 0 && gz >= 0 && gx < nx && gy < ny && gz < nz) v = load_v(V, f16, ((int64_t)gz * ny + gy) * nx + gx);
-        a[lz][ly][lx] = v;
+__global__ void __launch_bounds__(kMThreads) k_inside_mask(const void* __restrict__ V, int f16, int nx, int ny, int nz,
+                                                           int r, uint32_t* __restrict__ bits, int aligned_rows) {
+    constexpr int RY = kMY + 2 * kMaxR, RZ = kMZ + 2 * kMaxR;
+    __shared__ uint32_t s_neg[RZ * RY][kMW + 2];   // not (V >= 0): word w - 1 of the tile's row; then its x erosion
+    const int w0 = blockIdx.x * kMW, y0 = blockIdx.y * kMY, z0 = blockIdx.z * kMZ;
+    const int words = (nx + 31) / 32;
+    const int hy = kMY + 2 * r, hz = kMZ + 2 * r;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const bool left = w0 > 0, right = w0 + kMW < words;   // words beyond the tile inside the grid
+    bool nan = false;
+    int ly = warp % hy, lz = warp / hy;
+    for (int row = warp; row < hy * hz; row += kMThreads / 32) {
+        const int gy = y0 + ly - r, gz = z0 + lz - r;
+        const bool in = gy >= 0 && gz >= 0 && gy < ny && gz < nz;
+        const int64_t base = in ? ((int64_t)gz * ny + gy) * nx : 0;
+        const int x0 = w0 * 32 + lane;
+        float v[kMW], vl = -1.0f, vr = -1.0f;   // out of grid = unseen
+#pragma unroll
+        for (int w = 0; w < kMW; ++w) {
+            v[w] = -1.0f;
+            if (in && x0 + 32 * w < nx) v[w] = load_v(V, f16, base + x0 + 32 * w);
+        }
+        if (in && left && lane >= 32 - r) vl = load_v(V, f16, base + x0 - 32);
+        if (in && right && lane < r && x0 + 32 * kMW < nx) vr = load_v(V, f16, base + x0 + 32 * kMW);
+        nan = nan || vl != vl || vr != vr;
+        uint32_t mine = 0xffffffffu;
+#pragma unroll
+        for (int w = 0; w < kMW; ++w) {
+            nan = nan || v[w] != v[w];
+            const unsigned neg = __ballot_sync(0xffffffffu, !(v[w] >= 0.0f));
+            if (lane == w + 1) mine = neg;
+        }
+        const unsigned nl = __ballot_sync(0xffffffffu, !(vl >= 0.0f)), nr = __ballot_sync(0xffffffffu, !(vr >= 0.0f));
+        if (lane == 0) mine = nl;
+        if (lane == kMW + 1) mine = nr;
+        if (lane < kMW + 2) s_neg[row][lane] = mine;
+        ly += kMThreads / 32;
+        while (ly >= hy) {
+            ly -= hy;
+            ++lz;
+        }
+    }
+    const bool any_nan = __syncthreads_or(nan);
+    // x erosion: each thread keeps its words in registers, then they replace the rows' words
+    constexpr int kPer = (RZ * RY * kMW + kMThreads - 1) / kMThreads;
+    uint32_t ew[kPer];
+#pragma unroll
+    for (int i = 0; i < kPer; ++i) {
+        const int e = threadIdx.x + i * kMThreads, row = e / kMW, w = e % kMW;
+        ew[i] = 0;
+        if (row >= hy * hz) continue;
+        const uint32_t l = s_neg[row][w], c = s_neg[row][w + 1], h = s_neg[row][w + 2];
+        uint32_t m = c;
+        for (int d = 1; d <= r; ++d) m &= __funnelshift_l(l, c, d) & __funnelshift_r(c, h, d);
+        ew[i] = m;
     }
     __syncthreads();
-    for (int e = tid; e < kMTX * hy * hz; e += nthr) {
-        int lx = e % kMTX, ly = (e / kMTX) % hy, lz = e / (kMTX * hy);
-        float m = a[lz][ly][lx];
-        for (int d = 1; d <= 2 * r; ++d) m = fmaxf(m, a[lz][ly][lx + d]);
-        bx[lz][ly][lx] = m;
+#pragma unroll
+    for (int i = 0; i < kPer; ++i) {
+        const int e = threadIdx.x + i * kMThreads, row = e / kMW, w = e % kMW;
+        if (row < hy * hz) s_neg[row][w] = ew[i];
     }
     __syncthreads();
-    for (int e = tid; e < kMTX * kMTY * hz; e += nthr) {
-        int lx = e % kMTX, ly = (e / kMTX) % kMTY, lz = e / (kMTX * kMTY);
-        float m = bx[lz][ly][lx];
-        for (int d = 1; d <= 2 * r; ++d) m = fmaxf(m, bx[lz][ly + d][lx]);
-        by[lz][ly][lx] = m;
-    }
-    __syncthreads();
-    const int lx = threadIdx.x, ly = threadIdx.y;
-    for (int lz = 0; lz < kMTZ; ++lz) {
-        float m = by[lz][ly][lx];
-        for (int d = 1; d <= 2 * r; ++d) m = fmaxf(m, by[lz + d][ly][lx]);
-        const int gx = x0 + lx, gy = y0 + ly, gz = z0 + lz;
-        const bool valid = gx < nx && gy < ny && gz < nz;
-        const bool inside = valid && m < 0.0f;
-        const int64_t idx = ((int64_t)gz * ny + gy) * nx + gx;
+    for (int e = threadIdx.x; e < kMW * kMY * kMZ; e += kMThreads) {
+        const int w = e % kMW, ty = (e / kMW) % kMY, tz = e / (kMW * kMY);
+        const int gw = w0 + w, gy = y0 + ty, gz = z0 + tz;
+        if (gw >= words || gy >= ny || gz >= nz) continue;
+        uint32_t m = 0xffffffffu;
+        for (int dz = 0; dz <= 2 * r; ++dz)
+            for (int dy = 0; dy <= 2 * r; ++dy) m &= s_neg[(tz + dz) * hy + ty + dy][w];
+        const int rest = nx - gw * 32;   // voxels of this word inside the row
+        if (rest < 32) m &= (1u << rest) - 1u;
+        if (any_nan) {
+            // drop voxels whose neighbourhood holds no V < 0 (it is all NaN then)
+            for (uint32_t todo = m; todo; todo &= todo - 1) {
+                const int b = __ffs(todo) - 1, gx = gw * 32 + b;
+                bool lt = false;
+                for (int z = gz - r; z <= gz + r && !lt; ++z)
+                    for (int y = gy - r; y <= gy + r && !lt; ++y)
+                        for (int x = gx - r; x <= gx + r && !lt; ++x)
+                            lt = x < 0 || y < 0 || z < 0 || x >= nx || y >= ny || z >= nz ||
+                                 load_v(V, f16, ((int64_t)z * ny + y) * nx + x) < 0.0f;
+                if (!lt) m &= ~(1u << b);
+            }
+        }
+        const int64_t idx = ((int64_t)gz * ny + gy) * nx + (int64_t)gw * 32;
         if (aligned_rows) {
-            unsigned word = __ballot_sync(0xffffffffu, inside);
-            if (lx == 0 && gy < ny && gz < nz) bits[idx >> 5] = word;
-        } else if (inside) {
-            atomicOr(bits + (idx >> 5), 1u << (idx & 31));
+            bits[idx >> 5] = m;
+        } else if (m) {
+            const int sh = (int)(idx & 31);
+            atomicOr(bits + (idx >> 5), m << sh);
+            if (sh && (m >> (32 - sh))) atomicOr(bits + (idx >> 5) + 1, m >> (32 - sh));
         }
     }
 }
@@ -252,15 +419,15 @@ extern "C" int tsdf_integrate(const tsdfs_grid* g, const float* depth, int32_t n
     if (n_views == 0) return TSDFS_OK;
     if (n_views > 2048) return fail(TSDFS_E_INVALID, "at most 2048 views per call (split larger sets)");
     if (!depth || !K || !c2w) return fail(TSDFS_E_INVALID, "depth, K and c2w must be non-NULL");
-    int64_t n = (int64_t)g->nx * g->ny * g->nz;
-    size_t smem = (size_t)n_views * 16 * sizeof(float);
+    const int64_t bricks = (int64_t)((g->nx + kBX - 1) / kBX) * ((g->ny + kBY - 1) / kBY) * ((g->nz + kBZ - 1) / kBZ);
+    size_t smem = (size_t)n_views * (kCam * sizeof(float) + sizeof(uint16_t));
     if (smem > 48 * 1024) {
         rc = cuda_check(cudaFuncSetAttribute(k_integrate, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem),
                         "tsdf_integrate smem attribute");
         if (rc) return rc;
     }
     ProfScope ps("integrate", (cudaStream_t)stream);
-    k_integrate<<<grid_1d(n, kFuseBlock, 152 * 8), kFuseBlock, smem, (cudaStream_t)stream>>>(
+    k_integrate<<<grid_1d(bricks, 1, 152 * 8), kFuseBlock, smem, (cudaStream_t)stream>>>(
         g->nx, g->ny, g->nz, g->origin[0], g->origin[1], g->origin[2], g->voxel_size, g->trunc, g->tsdf,
         g->dtype == TSDFS_F16, g->weight, depth, n_views, H, W, K, c2w);
     return cuda_check(cudaGetLastError(), "tsdf_integrate launch");
@@ -320,10 +487,10 @@ extern "C" int tsdfs_inside_mask(const tsdfs_grid* g, int32_t r, uint32_t* bits,
                         "tsdfs_inside_mask memset");
         if (rc) return rc;
     }
-    dim3 grid((g->nx + kMTX - 1) / kMTX, (g->ny + kMTY - 1) / kMTY, (g->nz + kMTZ - 1) / kMTZ);
+    dim3 grid((g->nx + 32 * kMW - 1) / (32 * kMW), (g->ny + kMY - 1) / kMY, (g->nz + kMZ - 1) / kMZ);
     if (grid.y > 65535 || grid.z > 65535) return fail(TSDFS_E_INVALID, "grid too large for the mask kernel");
     ProfScope ps("inside_mask", (cudaStream_t)stream);
-    k_inside_mask<<<grid, dim3(kMTX, kMTY), 0, (cudaStream_t)stream>>>(g->tsdf, g->dtype == TSDFS_F16, g->nx, g->ny,
+    k_inside_mask<<<grid, kMThreads, 0, (cudaStream_t)stream>>>(g->tsdf, g->dtype == TSDFS_F16, g->nx, g->ny,
                                                                        g->nz, r, bits, aligned);
     return cuda_check(cudaGetLastError(), "tsdfs_inside_mask launch");
 }
