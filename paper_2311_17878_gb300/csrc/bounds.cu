@@ -1,12 +1,13 @@
 // K3: TSDF sample bounds of Alg. 1 + the adaptive count of Sec. 3.4.
 // K4: exclusive scan of the counts into ragged offsets.
 //
-// One thread per ray; the voxel walk recomputes every crossing parameter from
+// One thread per ray, or a warp for few rays.  The voxel walk recomputes every crossing parameter from
 // its integer boundary, so the walk is exact to the voxel no matter how long.
 // fp32, round-to-nearest, no contraction (intrinsics + --fmad=false), in the
 // operation order of the oracle's fp32-exact mode, so t_n, t_f, counts and
 // status are identical bit for bit.
 #include <mutex>
+#include <type_traits>
 
 #include "common.cuh"
 #include "march.cuh"
@@ -28,6 +29,7 @@ struct BoundsDev {
     int max_steps;   // voxel steps a walk may take (0: nx + ny + nz + 8, more than any walk needs)
 };
 
+template <bool SMALL>
 __device__ __forceinline__ float trilinear(const GridDev& g, const float p[3]) {
     int i0[3];
     float fr[3];
@@ -50,7 +52,7 @@ __device__ __forceinline__ float trilinear(const GridDev& g, const float p[3]) {
                 const int ii = min(max(i0[0] + dx, 0), g.n[0] - 1);
                 const int jj = min(max(i0[1] + dy, 0), g.n[1] - 1);
                 const int kk = min(max(i0[2] + dz, 0), g.n[2] - 1);
-                c[dz][dy][dx] = gval(g, ii, jj, kk);
+                c[dz][dy][dx] = vat(g, vidx<SMALL>(g, ii, jj, kk));
             }
     const float x00 = __fadd_rn(c[0][0][0], __fmul_rn(fr[0], __fsub_rn(c[0][0][1], c[0][0][0])));
     const float x01 = __fadd_rn(c[0][1][0], __fmul_rn(fr[0], __fsub_rn(c[0][1][1], c[0][1][0])));
@@ -61,134 +63,373 @@ __device__ __forceinline__ float trilinear(const GridDev& g, const float p[3]) {
     return __fadd_rn(y0, __fmul_rn(fr[2], __fsub_rn(y1, y0)));
 }
 
-__device__ __forceinline__ bool all_negative(const GridDev& g, const int X[3], int r) {
-    for (int dz = -r; dz <= r; ++dz)
-        for (int dy = -r; dy <= r; ++dy)
-            for (int dx = -r; dx <= r; ++dx)
-                if (!(gval(g, X[0] + dx, X[1] + dy, X[2] + dz) < 0.0f)) return false;
+// The far phase's test without the precomputed mask: every voxel of [lo, hi] has V < 0 (out of
+// grid = unseen = -1).  A plane at a time, its loads in flight together.
+__device__ __forceinline__ bool box_negative(const GridDev& g, const int lo[3], const int hi[3]) {
+    const int x0 = max(lo[0], 0), x1 = min(hi[0], g.n[0] - 1), y0 = max(lo[1], 0), y1 = min(hi[1], g.n[1] - 1);
+    const int z0 = max(lo[2], 0), z1 = min(hi[2], g.n[2] - 1);
+    for (int z = z0; z <= z1; ++z) {
+        bool neg = true;
+        const int64_t plane = (int64_t)z * g.n[1];
+#pragma unroll 5
+        for (int y = y0; y <= y1; ++y) {
+            const int64_t row = (plane + y) * g.n[0];
+#pragma unroll 5
+            for (int x = x0; x <= x1; ++x) {
+                const float v = g.f16 ? __half2float(__ldg(reinterpret_cast<const __half*>(g.V) + row + x))
+                                      : __ldg(reinterpret_cast<const float*>(g.V) + row + x);
+                neg = neg && v < 0.0f;
+            }
+        }
+        if (!neg) return false;
+    }
     return true;
 }
+__device__ __forceinline__ bool all_negative(const GridDev& g, const int X[3], int r) {
+    const int lo[3] = {X[0] - r, X[1] - r, X[2] - r}, hi[3] = {X[0] + r, X[1] + r, X[2] + r};
+    return box_negative(g, lo, hi);
+}
+// the same for a voxel whose predecessor along `axis` passed: only the leading face is new
+__device__ __forceinline__ bool face_negative(const GridDev& g, const int X[3], int r, int axis, int step) {
+    int lo[3], hi[3];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        lo[a] = X[a] + (a == axis && step > 0 ? r : -r);
+        hi[a] = X[a] + (a == axis && step < 0 ? -r : r);
+    }
+    return box_negative(g, lo, hi);
+}
 
-__device__ __forceinline__ bool inside_bit(const uint32_t* __restrict__ mask, const GridDev& g, const int X[3]) {
-    const int64_t idx = ((int64_t)X[2] * g.n[1] + X[1]) * g.n[0] + X[0];
+__device__ __forceinline__ bool inside_bit(const uint32_t* __restrict__ mask, int64_t idx) {
     return (__ldg(mask + (idx >> 5)) >> (idx & 31)) & 1u;
 }
 
-__global__ void __launch_bounds__(kBoundsMaxBlock) k_ray_bounds(GridDev g, const uint32_t* __restrict__ mask,
-                                                             const float* __restrict__ ray_o,
-                                                             const float* __restrict__ ray_d, int64_t n_rays,
-                                                             BoundsDev p, float* __restrict__ t_n_out,
-                                                             float* __restrict__ t_f_out, int32_t* __restrict__ n_out,
-                                                             float* __restrict__ t_zero_out,
-                                                             uint8_t* __restrict__ status_out, uint32_t* dev_status) {
-    const float kInf = __int_as_float(0x7f800000);
+// clamp(ceil((t_f - t_n) / step), 1, n_max) (Sec. 3.4)
+__device__ __forceinline__ int adaptive_count(float tn, float tf, const BoundsDev& p) {
+    const float q = __fdiv_rn(__fsub_rn(tf, tn), p.step);
+    int cnt;
+    if (!(q > 1.0f)) cnt = 1;
+    else if (q >= (float)p.n_max) cnt = p.n_max;
+    else cnt = (int)ceilf(q);
+    return cnt > p.n_max ? p.n_max : cnt;
+}
+
+// A thread per ray.  Bound by instruction issue (80 % of the slots of a 640 x 480 view): voxels known
+// to lie in the grid are not checked again, the walk converts nothing (march.cuh), and every loop is
+// left by the whole warp together: rays that end a phase at different steps otherwise go through the
+// next one apart (a view took half as long again).
+template <bool SMALL>
+__global__ void __launch_bounds__(kBoundsMaxBlock, 3) k_ray_bounds(GridDev g, const uint32_t* __restrict__ mask,
+                                                                const float* __restrict__ ray_o,
+                                                                const float* __restrict__ ray_d, int64_t n_rays,
+                                                                BoundsDev p, float* __restrict__ t_n_out,
+                                                                float* __restrict__ t_f_out, int32_t* __restrict__ n_out,
+                                                                float* __restrict__ t_zero_out,
+                                                                uint8_t* __restrict__ status_out, uint32_t* dev_status) {
     const float kNaN = __int_as_float(0x7fffffff);
+    const unsigned kAll = 0xffffffffu;
     const float ds_norm = __fdiv_rn(p.d_s, g.trunc);
     const int max_steps = p.max_steps > 0 ? p.max_steps : g.n[0] + g.n[1] + g.n[2] + 8;
-    for (int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; r < n_rays; r += (int64_t)gridDim.x * blockDim.x) {
+    const bool search = t_zero_out != nullptr;   // nobody asks for t_zero: its samples are not taken
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x, n_warps_rays = (n_rays + 31) / 32 * 32;
+    for (int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; r < n_warps_rays; r += stride) {
+        const bool valid = r < n_rays;
+        const int64_t rr = valid ? r : n_rays - 1;
+        float o[3], d[3];
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            o[a] = __ldg(ray_o + 3 * rr + a);
+            d[a] = __ldg(ray_d + 3 * rr + a);
+        }
+        // ---- clip to the grid box ("RenderingCube") ----
+        float t0, t_end;
+        const bool hit = clip_box(g, o, d, p.t_near, p.t_far, t0, t_end) && valid;
+        // ---- voxel walk init ----
+        Walk<SMALL> s;
+        s.start(g, o, d, t0);
+        // ---- near phase: first voxel with V(centre) <= D_s ----
+        // The walk does not depend on the values: the next kAhead voxels are stepped and
+        // their values requested before the current one is tested, so the loads are in
+        // flight together; the voxels, their order and every test are unchanged.
+        constexpr int kAhead = 4;
+        float tq[kAhead], vq[kAhead];
+        std::conditional_t<SMALL, uint32_t, int64_t> iq[kAhead], at = 0;
+        bool okq[kAhead];     // the loop condition of that step: still in the grid, t < t_end
+        bool live = hit;      // the walk has not left the grid
+#pragma unroll
+        for (int i = 0; i < kAhead; ++i) {
+            if (i > 0) {
+                const bool in = s.next(g);
+                live = live && in;
+            }
+            tq[i] = s.t;
+            iq[i] = s.idx;
+            okq[i] = live && s.t < t_end;
+            vq[i] = live ? vat(g, s.idx) : 0.0f;
+        }
+        bool found = false;
+        float t_before = t0, tn = 0.0f;
+        int steps = 0;
+        for (bool run = hit;;) {
+            run = run && okq[0];
+            if (!__any_sync(kAll, run)) break;
+            if (run) {
+                if (++steps > max_steps) {
+                    set_status(dev_status, TSDFS_DEV_MARCH_CAP);
+                    run = false;
+                } else if (vq[0] <= ds_norm) {
+                    found = true;
+                    tn = tq[0];
+                    at = iq[0];
+                    run = false;
+                } else {
+                    t_before = tq[0];
+                }
+            }
+#pragma unroll
+            for (int i = 0; i + 1 < kAhead; ++i) {
+                tq[i] = tq[i + 1];
+                iq[i] = iq[i + 1];
+                vq[i] = vq[i + 1];
+                okq[i] = okq[i + 1];
+            }
+            const bool in = s.next(g);
+            live = live && run && in;
+            tq[kAhead - 1] = s.t;
+            iq[kAhead - 1] = s.idx;
+            okq[kAhead - 1] = live && s.t < t_end;
+            vq[kAhead - 1] = live ? vat(g, s.idx) : 0.0f;
+        }
+        // ---- zero-crossing search, starting at the entry of the voxel before ----
+        float tf = t_end, tz = kNaN, t_prev = tn, v_prev = 0.0f;
+        if (found) {
+            // back from the voxels looked ahead at
+            int X[3];
+            const int64_t row = SMALL ? (int64_t)((uint32_t)at / (uint32_t)g.n[0]) : (int64_t)at / g.n[0];
+            X[0] = (int)((int64_t)at - row * g.n[0]);
+            X[2] = SMALL ? (int)((uint32_t)row / (uint32_t)g.n[1]) : (int)(row / g.n[1]);
+            X[1] = (int)(row - (int64_t)X[2] * g.n[1]);
+            s.place(g, X, tn);
+            float pp[3];
+            point_at(o, d, t_before, pp);
+            const float vb = trilinear<SMALL>(g, pp);
+            point_at(o, d, tn, pp);
+            v_prev = trilinear<SMALL>(g, pp);
+            if (tn > t_before && vb > 0.0f && v_prev <= 0.0f)
+                tz = __fadd_rn(t_before, __fmul_rn(__fsub_rn(tn, t_before), __fdiv_rn(vb, __fsub_rn(vb, v_prev))));
+        }
+        // ---- far phase: consecutive voxels whose neighbourhood is all negative ----
+        int m = 0, axis = 0;
+        for (bool run = found;;) {
+            run = run && s.t < t_end;
+            if (!__any_sync(kAll, run)) break;
+            if (run && ++steps > max_steps) {
+                set_status(dev_status, TSDFS_DEV_MARCH_CAP);
+                run = false;
+            }
+            if (run) {
+                bool inside;
+                if (mask) {
+                    inside = inside_bit(mask, s.idx);
+                } else {
+                    int X[3];
+                    s.voxel(X);
+                    inside = m > 0 ? face_negative(g, X, p.nb_radius, axis, axis == 0 ? s.st[0] : (axis == 1 ? s.st[1] : s.st[2]))
+                                   : all_negative(g, X, p.nb_radius);
+                }
+                m = inside ? m + 1 : 0;
+            }
+            const bool in = s.next(g, axis);
+            if (run) {
+                const float tc = s.t < t_end ? s.t : t_end;
+                if (search && tz != tz) {
+                    float pp[3];
+                    point_at(o, d, tc, pp);
+                    const float vc = trilinear<SMALL>(g, pp);
+                    if (v_prev > 0.0f && vc <= 0.0f)
+                        tz = __fadd_rn(t_prev, __fmul_rn(__fsub_rn(tc, t_prev), __fdiv_rn(v_prev, __fsub_rn(v_prev, vc))));
+                    v_prev = vc;
+                    t_prev = tc;
+                }
+                if (m == p.m_confirm) {
+                    tf = tc;
+                    run = false;
+                }
+                run = run && in;
+            }
+        }
+        if (!valid) continue;
+        const bool miss = !hit;
+        t_n_out[r] = found ? tn : (miss ? 0.0f : t0);
+        t_f_out[r] = found ? tf : (miss ? 0.0f : t_end);
+        n_out[r] = found ? adaptive_count(tn, tf, p) : (miss ? 0 : p.n_fallback);
+        status_out[r] = found ? TSDFS_BOUNDED : (miss ? TSDFS_MISS : TSDFS_FALLBACK);
+        if (t_zero_out) t_zero_out[r] = tz;
+    }
+}
+
+// A warp per ray, for few rays, where a thread's chain of steps and loads is all there is to wait for
+// (500 rays in a 64^3 grid without the inside mask: 616 us with a thread per ray, 34 us).  The walk does not
+// depend on the values, so every lane walks the next 32 voxels and keeps the one of its number;
+// the values, the far phase's neighbourhoods and the trilinear samples of 32 voxels are then loaded
+// together, and the first event in their order is taken: the same voxels, tests and results.
+template <bool SMALL>
+__global__ void __launch_bounds__(kBoundsMaxBlock, 2) k_ray_bounds_warp(GridDev g, const uint32_t* __restrict__ mask,
+                                                                  const float* __restrict__ ray_o,
+                                                                  const float* __restrict__ ray_d, int64_t n_rays,
+                                                                  BoundsDev p, float* __restrict__ t_n_out,
+                                                                  float* __restrict__ t_f_out, int32_t* __restrict__ n_out,
+                                                                  float* __restrict__ t_zero_out,
+                                                                  uint8_t* __restrict__ status_out, uint32_t* dev_status) {
+    const float kNaN = __int_as_float(0x7fffffff);
+    const unsigned kAll = 0xffffffffu;
+    const float ds_norm = __fdiv_rn(p.d_s, g.trunc);
+    const int max_steps = p.max_steps > 0 ? p.max_steps : g.n[0] + g.n[1] + g.n[2] + 8;
+    const int lane = threadIdx.x & 31;
+    const bool search = t_zero_out != nullptr;
+    const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
+    for (int64_t r = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5); r < n_rays; r += warps) {
         float o[3], d[3];
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
             o[a] = __ldg(ray_o + 3 * r + a);
             d[a] = __ldg(ray_d + 3 * r + a);
         }
-        // ---- clip to the grid box ("RenderingCube") ----
+        auto put = [&](float tn, float tf, int n, int status, float tz) {
+            if (lane != 0) return;
+            t_n_out[r] = tn; t_f_out[r] = tf; n_out[r] = n; status_out[r] = (uint8_t)status;
+            if (t_zero_out) t_zero_out[r] = tz;
+        };
         float t0, t_end;
         if (!clip_box(g, o, d, p.t_near, p.t_far, t0, t_end)) {
-            t_n_out[r] = 0.0f; t_f_out[r] = 0.0f; n_out[r] = 0; status_out[r] = TSDFS_MISS;
-            if (t_zero_out) t_zero_out[r] = kNaN;
+            put(0.0f, 0.0f, 0, TSDFS_MISS, kNaN);
             continue;
         }
-        // ---- voxel walk init ----
-        Dda s;
-        dda_init(s, g, o, d, t0);
-        // ---- near phase: first voxel with V(centre) <= D_s ----
-        // The walk does not depend on the values: the next kAhead voxels are stepped and
-        // their values requested before the current one is tested, so the loads are in
-        // flight together; the voxels, their order and every test are unchanged.
-        constexpr int kAhead = 4;
-        Dda wq[kAhead];
-        float qv[kAhead];
-        bool qok[kAhead];   // the loop condition of that step: still in the grid, t < t_end
-        bool live = true;   // the walk has not left the grid
-        wq[0] = s;
-        qok[0] = s.t < t_end;
-        qv[0] = gval(g, s.X[0], s.X[1], s.X[2]);
-#pragma unroll
-        for (int i = 1; i < kAhead; ++i) {
-            wq[i] = wq[i - 1];
-            live = live && dda_next(wq[i], g, o);
-            qok[i] = live && wq[i].t < t_end;
-            qv[i] = live ? gval(g, wq[i].X[0], wq[i].X[1], wq[i].X[2]) : 0.0f;
-        }
-        bool found = false, in_grid = true;
-        float t_before = t0;
-        int steps = 0;
-        while (qok[0]) {
-            if (++steps > max_steps) { set_status(dev_status, TSDFS_DEV_MARCH_CAP); in_grid = false; break; }
-            if (qv[0] <= ds_norm) { found = true; break; }
-            t_before = wq[0].t;
-            Dda nx = wq[kAhead - 1];
-#pragma unroll
-            for (int i = 0; i + 1 < kAhead; ++i) {
-                wq[i] = wq[i + 1];
-                qv[i] = qv[i + 1];
-                qok[i] = qok[i + 1];
+        Walk<SMALL> s;
+        s.start(g, o, d, t0);
+        bool in = true;             // s is in the grid
+        int steps = 0;              // voxels visited
+        // the lane's voxel: position, entry parameter, whether the walk visits it, and the next one's entry
+        int64_t idx;
+        float t, t_next;
+        bool ok;
+        auto walk = [&]() {
+            ok = false;
+            t = t_next = 0.0f;
+            idx = 0;
+            for (int k = 0; k < 32 && in && s.t < t_end; ++k) {
+                if (lane == k) {
+                    idx = s.idx;
+                    t = s.t;
+                    ok = true;
+                }
+                in = s.next(g);
+                if (lane == k) t_next = s.t;
             }
-            live = live && dda_next(nx, g, o);
-            wq[kAhead - 1] = nx;
-            qok[kAhead - 1] = live && nx.t < t_end;
-            qv[kAhead - 1] = live ? gval(g, nx.X[0], nx.X[1], nx.X[2]) : 0.0f;
+        };
+        // ---- near phase ----
+        bool found = false;
+        float tn = 0.0f, t_before = t0;
+        int first = 0;              // the found voxel's lane in the batch in hand
+        while (true) {
+            walk();
+            const unsigned oks = __ballot_sync(kAll, ok);
+            if (oks == 0) break;
+            const unsigned hits = __ballot_sync(kAll, ok && vat(g, idx) <= ds_norm);
+            first = hits ? __ffs(hits) - 1 : 32;
+            const int visited = first < 32 ? first + 1 : __popc(oks);
+            if (steps + visited > max_steps) {
+                if (lane == 0) set_status(dev_status, TSDFS_DEV_MARCH_CAP);
+                break;
+            }
+            steps += visited;
+            if (first < 32) {
+                found = true;
+                tn = __shfl_sync(kAll, t, first);
+                const float tb = __shfl_sync(kAll, t, first > 0 ? first - 1 : 0);
+                if (first > 0) t_before = tb;
+                break;
+            }
+            t_before = __shfl_sync(kAll, t, __popc(oks) - 1);
         }
-        s = wq[0];
         if (!found) {
-            t_n_out[r] = t0; t_f_out[r] = t_end; n_out[r] = p.n_fallback; status_out[r] = TSDFS_FALLBACK;
-            if (t_zero_out) t_zero_out[r] = kNaN;
+            put(t0, t_end, p.n_fallback, TSDFS_FALLBACK, kNaN);
             continue;
         }
-        const float tn = s.t;
-        float tf = t_end;
-        // ---- zero-crossing search, starting at the entry of the voxel before ----
-        float tz = kNaN, t_prev = t_before, v_prev;
+        float tf = t_end, tz = kNaN, t_prev = tn, v_prev;
         {
             float pp[3];
             point_at(o, d, t_before, pp);
-            v_prev = trilinear(g, pp);
+            const float vb = trilinear<SMALL>(g, pp);
             point_at(o, d, tn, pp);
-            const float vn = trilinear(g, pp);
-            if (tn > t_before && v_prev > 0.0f && vn <= 0.0f)
-                tz = __fadd_rn(t_prev, __fmul_rn(__fsub_rn(tn, t_prev), __fdiv_rn(v_prev, __fsub_rn(v_prev, vn))));
-            v_prev = vn;
-            t_prev = tn;
+            v_prev = trilinear<SMALL>(g, pp);
+            if (tn > t_before && vb > 0.0f && v_prev <= 0.0f)
+                tz = __fadd_rn(t_before, __fmul_rn(__fsub_rn(tn, t_before), __fdiv_rn(vb, __fsub_rn(vb, v_prev))));
         }
-        // ---- far phase: consecutive voxels whose neighbourhood is all negative ----
+        // ---- far phase: the rest of the batch in hand (from lane `first`), then whole batches ----
         int m = 0;
-        while (in_grid && s.t < t_end) {
-            if (++steps > max_steps) { set_status(dev_status, TSDFS_DEV_MARCH_CAP); break; }
-            const bool inside = mask ? inside_bit(mask, g, s.X) : all_negative(g, s.X, p.nb_radius);
-            m = inside ? m + 1 : 0;
-            in_grid = dda_next(s, g, o);
-            const float tc = s.t < t_end ? s.t : t_end;
-            if (tz != tz) {
-                float pp[3];
-                point_at(o, d, tc, pp);
-                const float vc = trilinear(g, pp);
-                if (v_prev > 0.0f && vc <= 0.0f)
-                    tz = __fadd_rn(t_prev, __fmul_rn(__fsub_rn(tc, t_prev), __fdiv_rn(v_prev, __fsub_rn(v_prev, vc))));
-                v_prev = vc;
-                t_prev = tc;
+        while (true) {
+            unsigned oks = __ballot_sync(kAll, ok && lane >= first);
+            if (oks == 0) {
+                if (!(in && s.t < t_end)) break;
+                first = 0;
+                walk();
+                oks = __ballot_sync(kAll, ok);
             }
-            if (m == p.m_confirm) { tf = tc; break; }
+            const int n_ok = __popc(oks);             // lanes first .. first + n_ok - 1
+            const int allowed = max_steps - steps;    // voxels before the step cap
+            const int n_vis = n_ok < allowed ? n_ok : allowed;
+            const bool vis = lane >= first && lane < first + n_vis;
+            bool inside = false;
+            if (vis) {
+                if (mask) {
+                    inside = inside_bit(mask, idx);
+                } else {
+                    const int64_t row = idx / g.n[0];
+                    const int X[3] = {(int)(idx - row * g.n[0]), (int)(row % g.n[1]), (int)(row / g.n[1])};
+                    inside = all_negative(g, X, p.nb_radius);
+                }
+            }
+            const unsigned ins = __ballot_sync(kAll, inside);
+            // consecutive inside voxels up to this lane's
+            const unsigned out = ~ins & ((2u << lane) - 1u) & ~((1u << first) - 1u);
+            const int run = out ? lane - (31 - __clz(out)) : m + lane - first + 1;
+            const unsigned conf = __ballot_sync(kAll, vis && inside && run == p.m_confirm);
+            const int last = conf ? __ffs(conf) - 1 : first + n_vis - 1;   // the last voxel visited
+            const float tc = t_next < t_end ? t_next : t_end;
+            if (search && tz != tz && n_vis > 0) {
+                float vc = 0.0f;
+                if (vis) {
+                    float pp[3];
+                    point_at(o, d, tc, pp);
+                    vc = trilinear<SMALL>(g, pp);
+                }
+                float vp = __shfl_up_sync(kAll, vc, 1), tp = __shfl_up_sync(kAll, tc, 1);
+                if (lane == first) {
+                    vp = v_prev;
+                    tp = t_prev;
+                }
+                const unsigned cross = __ballot_sync(kAll, vis && lane <= last && vp > 0.0f && vc <= 0.0f);
+                if (cross) {
+                    const float z = __fadd_rn(tp, __fmul_rn(__fsub_rn(tc, tp), __fdiv_rn(vp, __fsub_rn(vp, vc))));
+                    tz = __shfl_sync(kAll, z, __ffs(cross) - 1);
+                }
+                v_prev = __shfl_sync(kAll, vc, last);
+                t_prev = __shfl_sync(kAll, tc, last);
+            }
+            if (conf) {
+                tf = __shfl_sync(kAll, tc, last);
+                break;
+            }
+            if (n_vis < n_ok) {
+                if (lane == 0) set_status(dev_status, TSDFS_DEV_MARCH_CAP);
+                break;
+            }
+            steps += n_vis;
+            m = __shfl_sync(kAll, inside ? run : 0, last);
+            ok = false;
         }
-        // ---- adaptive count (Sec. 3.4) ----
-        const float q = __fdiv_rn(__fsub_rn(tf, tn), p.step);
-        int cnt;
-        if (!(q > 1.0f)) cnt = 1;
-        else if (q >= (float)p.n_max) cnt = p.n_max;
-        else cnt = (int)ceilf(q);
-        if (cnt > p.n_max) cnt = p.n_max;
-        t_n_out[r] = tn; t_f_out[r] = tf; n_out[r] = cnt; status_out[r] = TSDFS_BOUNDED;
-        if (t_zero_out) t_zero_out[r] = tz;
+        put(tn, tf, adaptive_count(tn, tf, p), TSDFS_BOUNDED, tz);
     }
 }
 
@@ -216,84 +457,93 @@ __global__ void __launch_bounds__(kBoundsMaxBlock) k_recovery_bounds(GridDev g, 
     }
 }
 
-// ---- K4: three-phase exclusive scan (chunk sums, scan of sums, chunk scan) ----
-__device__ __forceinline__ int block_exclusive_scan(int v, int* sh, int& total) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    int x = v;
+// ---- K4: exclusive scan of the counts, in chunks of 8192: one launch for one chunk; two
+// (the chunks' sums; each chunk's scan, which adds up the sums before it itself) for up to 1024;
+// else a third between them that scans the sums.  What it costs is the launches: 307 200 counts
+// took 12 us in three, their 2.5 MB take under 1.
+__device__ __forceinline__ int warp_inclusive(int x) {
+    const int lane = threadIdx.x & 31;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
-        int y = __shfl_up_sync(0xffffffffu, x, o);
+        const int y = __shfl_up_sync(0xffffffffu, x, o);
         if (lane >= o) x += y;
     }
-    if (lane == 31) sh[warp] = x;
+    return x;
+}
+// sum of v over the block's 32 warps, and the sum over the warps before this one
+__device__ __forceinline__ int block_sums(int warp_total, int* sh, int& total) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     __syncthreads();
-    if (warp == 0) {
-        int w = lane < (int)(blockDim.x >> 5) ? sh[lane] : 0;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            int y = __shfl_up_sync(0xffffffffu, w, o);
-            if (lane >= o) w += y;
-        }
-        sh[lane] = w;  // inclusive warp prefix
-    }
+    if (lane == 0) sh[warp] = warp_total;
     __syncthreads();
-    total = sh[(blockDim.x >> 5) - 1];
-    const int excl = x - v + (warp > 0 ? sh[warp - 1] : 0);
-    __syncthreads();
-    return excl;
+    const int incl = warp_inclusive(sh[lane]);
+    total = __shfl_sync(0xffffffffu, incl, 31);
+    return __shfl_sync(0xffffffffu, incl, warp) - sh[warp];
 }
 
 __global__ void __launch_bounds__(kScanBlock) k_chunk_sums(const int32_t* __restrict__ cnt, int64_t n,
                                                            int32_t* __restrict__ sums) {
     __shared__ int sh[32];
-    const int64_t base = (int64_t)blockIdx.x * kScanChunk + (int64_t)threadIdx.x * kScanItems;
+    const int64_t base = (int64_t)blockIdx.x * kScanChunk + threadIdx.x;
     int v = 0;
 #pragma unroll
     for (int i = 0; i < kScanItems; ++i)
-        if (base + i < n) v += cnt[base + i];
+        if (base + i * kScanBlock < n) v += cnt[base + i * kScanBlock];
     int total;
-    block_exclusive_scan(v, sh, total);
+    block_sums(__reduce_add_sync(0xffffffffu, v), sh, total);
     if (threadIdx.x == 0) sums[blockIdx.x] = total;
 }
 
-__global__ void __launch_bounds__(kScanBlock) k_scan_sums(int32_t* __restrict__ sums, int64_t n_chunks,
-                                                          int32_t* __restrict__ offsets_last, int64_t n_rays) {
+__global__ void __launch_bounds__(kScanBlock) k_scan_sums(int32_t* __restrict__ sums, int64_t n_chunks) {
     __shared__ int sh[32];
     const int per = (int)((n_chunks + kScanBlock - 1) / kScanBlock);
     const int64_t base = (int64_t)threadIdx.x * per;
     int v = 0;
     for (int i = 0; i < per; ++i)
         if (base + i < n_chunks) v += sums[base + i];
+    const int incl = warp_inclusive(v);
     int total;
-    int run = block_exclusive_scan(v, sh, total);
+    int run = block_sums(__shfl_sync(0xffffffffu, incl, 31), sh, total) + incl - v;
     for (int i = 0; i < per; ++i)
         if (base + i < n_chunks) {
-            int c = sums[base + i];
+            const int c = sums[base + i];
             sums[base + i] = run;
             run += c;
         }
-    if (threadIdx.x == 0) offsets_last[n_rays] = total;
 }
 
+// sums: the chunks' sums (SCANNED: their exclusive scan); the last chunk writes the total
+template <bool SCANNED>
 __global__ void __launch_bounds__(kScanBlock) k_chunk_scan(const int32_t* __restrict__ cnt, int64_t n,
                                                            const int32_t* __restrict__ sums,
                                                            int32_t* __restrict__ offsets) {
     __shared__ int sh[32];
-    const int64_t base = (int64_t)blockIdx.x * kScanChunk + (int64_t)threadIdx.x * kScanItems;
-    int v[kScanItems];
-    int s = 0;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    // a warp's 256 counts as 8 rows of 32
+    const int64_t base = (int64_t)blockIdx.x * kScanChunk + warp * (32 * kScanItems) + lane;
+    int v[kScanItems], x[kScanItems], carry = 0;
+#pragma unroll
+    for (int i = 0; i < kScanItems; ++i) v[i] = base + 32 * i < n ? cnt[base + 32 * i] : 0;
+    int before = 0;
+    if (SCANNED) {
+        before = sums[blockIdx.x];
+    } else if (gridDim.x > 1) {
+        const int s = (int)threadIdx.x < (int)blockIdx.x ? sums[threadIdx.x] : 0;
+        block_sums(__reduce_add_sync(0xffffffffu, s), sh, before);
+    }
 #pragma unroll
     for (int i = 0; i < kScanItems; ++i) {
-        v[i] = base + i < n ? cnt[base + i] : 0;
-        s += v[i];
+        const int incl = warp_inclusive(v[i]);
+        x[i] = carry + incl - v[i];
+        carry += __shfl_sync(0xffffffffu, incl, 31);
     }
     int total;
-    int run = block_exclusive_scan(s, sh, total) + sums[blockIdx.x];
+    before += block_sums(carry, sh, total) ;
 #pragma unroll
     for (int i = 0; i < kScanItems; ++i)
-        if (base + i < n) {
-            offsets[base + i] = run;
-            run += v[i];
+        if (base + 32 * i < n) {
+            offsets[base + 32 * i] = before + x[i];
+            if (base + 32 * i == n - 1) offsets[n] = before + x[i] + v[i];
         }
 }
 
@@ -332,15 +582,29 @@ int exclusive_scan(const int32_t* cnt, int64_t n, int32_t* offsets, int32_t* sum
     if (n == 0) return cuda_check(cudaMemsetAsync(offsets, 0, sizeof(int32_t), st), "scan memset");
     if (chunks > (int64_t)kScanBlock * 64) return fail(TSDFS_E_INVALID, "too many rays for the scan (%lld)", (long long)n);
     ProfScope ps("scan", st);
-    k_chunk_sums<<<(unsigned)chunks, kScanBlock, 0, st>>>(cnt, n, sums);
-    k_scan_sums<<<1, kScanBlock, 0, st>>>(sums, chunks, offsets, n);
-    k_chunk_scan<<<(unsigned)chunks, kScanBlock, 0, st>>>(cnt, n, sums, offsets);
+    if (chunks > 1) k_chunk_sums<<<(unsigned)chunks, kScanBlock, 0, st>>>(cnt, n, sums);
+    if (chunks > kScanBlock) {
+        k_scan_sums<<<1, kScanBlock, 0, st>>>(sums, chunks);
+        k_chunk_scan<true><<<(unsigned)chunks, kScanBlock, 0, st>>>(cnt, n, sums, offsets);
+    } else {
+        k_chunk_scan<false><<<(unsigned)chunks, kScanBlock, 0, st>>>(cnt, n, sums, offsets);
+    }
     return cuda_check(cudaGetLastError(), "scan launch");
 }
 
 }  // namespace tsdfs
 
 using namespace tsdfs;
+
+namespace tsdfs {
+namespace {
+// A warp per ray up to these many rays, with and without the inside mask.  Measured (us, warp /
+// thread, rays of a room view in 256^3 and of a sphere view in 64^3): with the mask 1728 rays 22 / 35 and
+// 20 / 78, 4800 39 / 35 and 25 / 78; without it 4800 80 / 190 and 47 / 550, 10 800 144 / 192 and 70 / 550;
+// a thread per ray takes the same up to 30 000 rays.
+constexpr int64_t kWarpRaysMask = 4096, kWarpRays = 16384;
+}  // namespace
+}  // namespace tsdfs
 
 extern "C" size_t tsdfs_bounds_workspace_size(int64_t n_rays) {
     if (n_rays < 0) return 0;
@@ -369,6 +633,7 @@ extern "C" int tsdf_ray_bounds(const tsdfs_grid* g, const uint32_t* mask, const 
     if (!offsets) return fail(TSDFS_E_INVALID, "offsets is NULL");
     if (ws_bytes < tsdfs_bounds_workspace_size(n_rays) || !ws) return fail(TSDFS_E_WORKSPACE, "bounds workspace too small");
     cudaStream_t st = (cudaStream_t)stream;
+    int32_t* sums = reinterpret_cast<int32_t*>((reinterpret_cast<uintptr_t>(ws) + 255) & ~uintptr_t(255));
     if (n_rays > 0) {
         GridDev gd{g->tsdf, g->dtype == TSDFS_F16, {g->nx, g->ny, g->nz}, {g->origin[0], g->origin[1], g->origin[2]},
                    g->voxel_size, g->trunc};
@@ -376,12 +641,14 @@ extern "C" int tsdf_ray_bounds(const tsdfs_grid* g, const uint32_t* mask, const 
                      test_march_cap()};
         const MarchShape sh = march_shape();
         ProfScope ps("ray_bounds", st);
-        k_ray_bounds<<<march_grid(n_rays, sh), sh.block, 0, st>>>(gd, mask, ray_o, ray_d, n_rays, bd, t_n, t_f,
-                                                                  n_samples, t_zero, status, device_status_word());
+        const bool warp = n_rays <= (mask ? kWarpRaysMask : kWarpRays), small = small_grid(gd.n);
+        auto march = warp ? (small ? k_ray_bounds_warp<true> : k_ray_bounds_warp<false>)
+                          : (small ? k_ray_bounds<true> : k_ray_bounds<false>);
+        march<<<march_grid(warp ? n_rays * 32 : n_rays, sh), sh.block, 0, st>>>(
+            gd, mask, ray_o, ray_d, n_rays, bd, t_n, t_f, n_samples, t_zero, status, device_status_word());
         rc = cuda_check(cudaGetLastError(), "tsdf_ray_bounds launch");
         if (rc) return rc;
     }
-    int32_t* sums = reinterpret_cast<int32_t*>((reinterpret_cast<uintptr_t>(ws) + 255) & ~uintptr_t(255));
     return exclusive_scan(n_samples, n_rays, offsets, sums, st);
 }
 
