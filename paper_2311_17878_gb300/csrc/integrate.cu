@@ -335,8 +335,8 @@ __global__ void __launch_bounds__(kFuseBlock) k_raycast_view(GridDev g, const fl
     const int max_steps = g.n[0] + g.n[1] + g.n[2] + 8;
     const int lane = threadIdx.x & 31;
     const int tx = (Wd + kRayW - 1) / kRayW, ty = (H + kRayH - 1) / kRayH;
-    const int64_t tiles = (int64_t)tx * ty, warps = (int64_t)gridDim.x * (kFuseBlock / 32);
-    for (int64_t q = blockIdx.x * (int64_t)(kFuseBlock / 32) + (threadIdx.x >> 5); q < tiles; q += warps) {
+    const int64_t tiles = (int64_t)tx * ty, warps = (int64_t)gridDim.x * (blockDim.x / 32);
+    for (int64_t q = blockIdx.x * (int64_t)(blockDim.x / 32) + (threadIdx.x >> 5); q < tiles; q += warps) {
         const int px = (int)(q % tx) * kRayW + lane % kRayW, py = (int)(q / tx) * kRayH + lane / kRayW;
         bool act = px < Wd && py < H;
         const float a = __fdiv_rn(__fsub_rn(__fadd_rn((float)px, 0.5f), cx), fx);
@@ -507,9 +507,11 @@ extern "C" int tsdf_integrate_raycast(const tsdfs_grid* g, const float* depth, i
                g->voxel_size, g->trunc};
     const int f16 = g->dtype == TSDFS_F16;
     const int64_t tiles = (int64_t)((W + kRayW - 1) / kRayW) * ((H + kRayH - 1) / kRayH);
+    // few warps: one to a block, so that each has an SM's issue slots for its chain of steps
+    const int block = tiles < 152 * 16 ? 32 : kFuseBlock;
     for (int v = 0; v < n_views; ++v) {
         auto view = small_grid(gd.n) ? k_raycast_view<true> : k_raycast_view<false>;
-        view<<<grid_1d(tiles * 32, kFuseBlock, 152 * 16), kFuseBlock, 0, st>>>(gd, depth, H, W, K, c2w, v, lack, cnt);
+        view<<<grid_1d(tiles * 32, block, 152 * 16), block, 0, st>>>(gd, depth, H, W, K, c2w, v, lack, cnt);
         k_raycast_apply<<<grid_1d((n + 7) / 8, 256, 152 * 8), 256, 0, st>>>(g->tsdf, f16, g->weight, lack, cnt, n);
     }
     return cuda_check(cudaGetLastError(), "tsdf_integrate_raycast launch");
