@@ -32,7 +32,7 @@
 // stream weight chunks, one per slot (two ring stages, and a slot in the free part of A1 while
 // the colour layers run): bulk copies issued by one thread towards different mbarriers do not
 // overlap (measured), so each slot has a thread of its own.  The value kernel (the
-// comparator's coarse pass) has 8 epilogue warps, one MMA warp and one producer warp per ring
+// samplers' coarse pass) has the same epilogue and MMA warps and one producer warp per ring
 // stage.  All hand-offs are mbarriers; every wait is bounded and on timeout the kernel
 // records TSDFS_DEV_TIMEOUT, drains its own copies / MMAs and returns.
 #include <type_traits>
@@ -49,9 +49,6 @@ namespace {
 constexpr int kTileS = 64;        // samples per tile
 constexpr int kStages = 2;        // weight chunks in flight (ring depth), one producer warp each
 constexpr uint32_t kBarBytes = 256;  // mbarriers, TMEM slot and abort flag
-constexpr int kEpiThreads = 256;  // warps 0-7
-constexpr int kMmaWarp = 8;
-constexpr int kThreads = 32 * (kMmaWarp + 1 + kStages);
 // the full kernel: kEpiWarpsF epilogue warps (kPartsF per TMEM lane quarter, each writing one
 // column part of the next operand), then the MMA warp, then one producer warp per stage
 constexpr int kEpiWarpsF = 12;
@@ -141,6 +138,69 @@ constexpr uint32_t kRecPar = 1u << 10;       // parity of the slot's use within 
 constexpr uint32_t kRecFlip = 1u << 11;      // the slot's uses per pair of tiles are odd
 constexpr uint32_t kRecRestore = 1u << 12;   // first colour chunk: the pair's first tile is back in place
 
+// The chunk schedule of a pair of tiles (the first tile's SDF layers, the second's, then the colour
+// layers once): SDF chunks alternate over the ring stages, colour chunks cycle over the ring stages and
+// the free part of A1.  Made at compile time and handed to the kernel as an argument: derived in
+// the kernel by one thread it took as long as a tile (136 tiles: 145 us with it and a pair of tiles to
+// half the CTAs, 51 us without and a tile to each).
+struct PairEntry {
+    uint32_t off, bytes;     // in the packed weights
+    uint32_t a;              // operand offset of the chunk's first K step
+    uint32_t a_sbo;          // operand row-group stride
+    uint16_t np, kc;         // outputs, K columns
+    uint16_t flags;          // kRec* without the K steps
+    uint16_t a_in_a1;        // the (first) operand is in A1 instead of A0
+};
+template <int ARCH> struct PairTab {
+    using TA = TcFull<ARCH>;
+    static constexpr int kLS = TA::kLS, kN = TA::pair_chunks();
+    static constexpr int kColSlots = kA1Slots ? kStages + TA::a1_slots() : kStages;
+    PairEntry e[kN];
+    uint32_t first_pass;     // bit s: the first tile's SDF layers use slot s an odd number of times
+};
+template <int ARCH> constexpr PairTab<ARCH> make_pair_tab() {
+    using T = PairTab<ARCH>;
+    using TA = TcFull<ARCH>;
+    PairTab<ARCH> t{};
+    int uses[kSlots] = {};
+    int j = 0, sdf_j = 0, col_j = 0;
+    for (int u = 0; u < 2 * T::kLS + (TA::kLayers - T::kLS); ++u) {
+        const int L = u < 2 * T::kLS ? u % T::kLS : u - T::kLS;
+        const TcLayer ly = TA::layer(L);
+        if (u == T::kLS)
+            for (int i = 0; i < kSlots; ++i) t.first_pass |= (uint32_t)(uses[i] & 1) << i;
+        uint32_t off = (uint32_t)TA::packed_offset(L, 0);
+        for (int c = 0; c < TA::chunks(L); ++c, ++j) {
+            const uint32_t sl = L < T::kLS ? (uint32_t)(sdf_j++ % kStages) : (uint32_t)(col_j % T::kColSlots);
+            const bool keep = L >= T::kLS && sl >= (uint32_t)kStages && col_j + T::kColSlots >= TA::rgb_chunks();
+            if (L >= T::kLS) ++col_j;
+            PairEntry& e = t.e[j];
+            const int k0 = c * kKChunk;
+            e.off = off;
+            e.bytes = (uint32_t)TA::chunk_bytes(L, c);
+            off += e.bytes;
+            e.np = (uint16_t)ly.Np;
+            e.kc = (uint16_t)TA::chunk_k(L, c);
+            // the folded colour input: its h chunks are the last SDF layer's input rows in A0 (that
+            // layer's layout), its x~ / direction / normal chunk starts A1
+            const bool fold = !ly.sdf && ly.idx == 0;
+            e.a_in_a1 = fold && k0 >= TA::kH;
+            e.a = (uint32_t)((e.a_in_a1 ? k0 - TA::kH : k0) / 8) * 128u;
+            e.a_sbo = (uint32_t)((fold ? (e.a_in_a1 ? TA::kXp : TA::kH) : ly.Kp) / 8) * 128u;
+            // the A1 slots are released after the second tile's SDF MMAs (the last to read A1)
+            e.flags = (uint16_t)((ly.sdf ? kRecTwo : 0u) | (keep ? kRecKeep : 0u) | (c == 0 ? kRecFirst : 0u) |
+                                 (c + 1 == TA::chunks(L) ? kRecLast : 0u) |
+                                 (c + 1 == TA::chunks(L) && u == 2 * T::kLS - 1 ? kRecRelA1 : 0u) |
+                                 (c == 0 && u == 2 * T::kLS ? kRecRestore : 0u) | (sl << kRecSlotShift) |
+                                 ((uses[sl] & 1) ? kRecPar : 0u));
+            ++uses[sl];
+        }
+    }
+    for (int i = 0; i < T::kN; ++i)
+        if (uses[(t.e[i].flags >> kRecSlotShift) & 3u] & 1) t.e[i].flags |= kRecFlip;
+    return t;
+}
+
 // most CTAs of one launch of the full kernel, and the parking space of each in the caller's
 // workspace: the first tile of a pair keeps its last SDF layer's input value rows and its
 // folded colour input extras there while the second tile's SDF layers use the operand
@@ -172,7 +232,7 @@ struct TcParams {
 };
 
 template <int ARCH, bool F16>
-__global__ void __launch_bounds__(kThreadsF, 1) k_mlp_tc(TcParams p) {
+__global__ void __launch_bounds__(kThreadsF, 1) k_mlp_tc(TcParams p, const __grid_constant__ PairTab<ARCH> tab) {
     using TA = TcFull<ARCH>;
     using A = Arch<ARCH>;
     constexpr int NL = TA::kLayers;
@@ -217,10 +277,20 @@ __global__ void __launch_bounds__(kThreadsF, 1) k_mlp_tc(TcParams p) {
         return;
     }
     const int64_t n_tiles = (total + kTileS - 1) / kTileS;
-    // pair k: tiles 2k and 2k + 1 (the second past n_tiles when the count is odd: its samples
-    // are all invalid, its table zero and its records not written)
-    const int64_t n_pairs = (n_tiles + 1) / 2;
-    if ((int64_t)blockIdx.x >= n_pairs) return;
+    // Rounds of one pair of tiles per CTA, then the rest: one tile per CTA where that is enough (a
+    // tile alone takes a good half of a pair's time), else pairs again.  A pair's second tile may be
+    // past n_tiles: its samples are all invalid, its table zero and its records not written.  A tile
+    // alone runs as a pair's second tile: the first pass is left out.
+    const int64_t rounds = n_tiles / (2 * (int64_t)gridDim.x), rest = n_tiles - rounds * 2 * gridDim.x;
+    const bool rest_single = rest <= (int64_t)gridDim.x;
+    // first tile of the CTA's unit w, -1: it has none
+    auto unit = [&](int64_t w) -> int64_t {
+        if (w > rounds) return -1;
+        const int64_t t = w * 2 * (int64_t)gridDim.x + (w < rounds || !rest_single ? 2 * (int64_t)blockIdx.x : (int64_t)blockIdx.x);
+        return t < n_tiles ? t : -1;
+    };
+    auto single = [&](int64_t w) { return w == rounds && rest_single; };
+    if (unit(0) < 0) return;
 
     if (threadIdx.x == 0) {
         for (int i = 0; i < kSlots; ++i) {
@@ -234,66 +304,31 @@ __global__ void __launch_bounds__(kThreadsF, 1) k_mlp_tc(TcParams p) {
         mbar_init(bar_rest, 1);
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        // the pair's chunk schedule (the first tile's SDF layers, the second's, then the colour
-        // layers once), computed once: SDF chunks alternate over the ring stages, colour chunks
-        // cycle over the ring stages and the free part of A1 (the producers and the MMA warp
-        // read it instead of re-deriving offsets and slots in their loops)
-        static_assert(TA::layer(LS - 1).Np <= 256, "the SDF output layer fits one MMA per accumulator");
-        {
-            int uses[kSlots];
-            for (int i = 0; i < kSlots; ++i) uses[i] = 0;
-            const uint32_t a0 = smem_u32(A0), a1 = smem_u32(A1);
-            int j = 0, sdf_j = 0, col_j = 0;
-            for (int u = 0; u < 2 * LS + (NL - LS); ++u) {
-                const int L = u < 2 * LS ? u % LS : u - LS;
-                const TcLayer ly = TA::layer(L);
-                const uint32_t a_sbo = (uint32_t)(ly.Kp / 8) * 128u;
-                for (int c = 0; c < TA::chunks(L); ++c, ++j) {
-                    const uint32_t sl = L < LS ? (uint32_t)(sdf_j++ % kStages) : (uint32_t)(col_j % kColSlots);
-                    const bool keep = L >= LS && sl >= (uint32_t)kStages && col_j + kColSlots >= TA::rgb_chunks();
-                    if (L >= LS) ++col_j;
-                    const int kc = TA::chunk_k(L, c);
-                    s_chunks[j] = ChunkInfo{(uint32_t)TA::packed_offset(L, c), (uint32_t)TA::chunk_bytes(L, c), (uint16_t)sl,
-                                            (uint16_t)(kc | (keep ? 0x8000 : 0))};
-                    const int k0 = c * kKChunk;
-                    MmaRec r;
-                    r.bd = mdesc(slot_addr(sl), 128, (uint32_t)(kc / 8) * 128u);
-                    r.ad0 = mdesc(a0 + (uint32_t)(k0 / 8) * 128u, 128, a_sbo);
-                    // the folded colour input: its h chunks are the last SDF layer's input rows in
-                    // A0 (that layer's layout), its x~ / direction / normal chunk starts A1
-                    if (!ly.sdf && ly.idx == 0)
-                        r.ad0 = k0 < TA::kH ? mdesc(a0 + (uint32_t)(k0 / 8) * 128u, 128, (TA::kH / 8) * 128u)
-                                            : mdesc(a1 + (uint32_t)((k0 - TA::kH) / 8) * 128u, 128, (TA::kXp / 8) * 128u);
-                    r.ad1 = mdesc(a1 + (uint32_t)(k0 / 8) * 128u, 128, a_sbo);
-                    r.id = idesc_mma<F16>(128, ly.Np);
-                    // the A1 slots are released after the second tile's SDF MMAs (the last to read A1)
-                    r.flags = (uint32_t)(kc / 16) | (ly.sdf ? kRecTwo : 0u) | (keep ? kRecKeep : 0u) |
-                              (c == 0 ? kRecFirst : 0u) | (c + 1 == TA::chunks(L) ? kRecLast : 0u) |
-                              (c + 1 == TA::chunks(L) && u == 2 * LS - 1 ? kRecRelA1 : 0u) |
-                              (c == 0 && u == 2 * LS ? kRecRestore : 0u) | (sl << kRecSlotShift) |
-                              ((uses[sl] & 1) ? kRecPar : 0u);
-                    ++uses[sl];
-                    s_mma[j] = r;
-                }
-            }
-            for (int jj = 0; jj < kPC; ++jj)
-                if (uses[s_chunks[jj].slot] & 1) s_mma[jj].flags |= kRecFlip;
-        }
+    }
+    static_assert(TA::layer(LS - 1).Np <= 256, "the SDF output layer fits one MMA per accumulator");
+    for (int j = threadIdx.x; j < kPC; j += kThreadsF) {
+        const PairEntry e = tab.e[j];
+        const uint32_t sl = (e.flags >> kRecSlotShift) & 3u;
+        s_chunks[j] = ChunkInfo{e.off, e.bytes, (uint16_t)sl, (uint16_t)(e.kc | (e.flags & kRecKeep ? 0x8000 : 0))};
+        const uint32_t a0 = smem_u32(A0), a1 = smem_u32(A1);
+        MmaRec r;
+        r.bd = mdesc(slot_addr(sl), 128, (uint32_t)(e.kc / 8) * 128u);
+        r.ad0 = mdesc((e.a_in_a1 ? a1 : a0) + e.a, 128, e.a_sbo);
+        r.ad1 = mdesc(a1 + e.a, 128, e.a_sbo);
+        r.id = idesc_mma<F16>(128, e.np);
+        r.flags = e.flags | (uint32_t)(e.kc / 16);
+        s_mma[j] = r;
     }
     // all biases of both networks, staged once (the two folded layers' from the packed buffer)
-    for (int i = threadIdx.x; i < TA::bias_total(); i += kThreadsF) {
-        int L = 0;
-        while (L + 1 < NL && TA::bias_offset(L + 1) <= i) ++L;
-        const TcLayer ly = TA::layer(L);
-        const int j = i - TA::bias_offset(L);
-        if (TA::folded(L)) {
-            const float* fb = reinterpret_cast<const float*>(p.packed + TA::fold_bias_offset());
-            sbias[i] = __ldg(fb + (L == LS ? TA::layer(LS - 1).Np : 0) + j);
-        } else {
-            const float* W = (ly.sdf ? p.sdf_w : p.rgb_w) + TA::param_offset(L);
-            sbias[i] = j < ly.N ? __ldg(W + (int64_t)ly.N * ly.K + j) : 0.0f;
-        }
-    }
+    static_for<0, NL>([&](auto lc) {
+        constexpr int L = decltype(lc)::value;
+        constexpr TcLayer ly = TA::layer(L);
+        const float* b = TA::folded(L) ? reinterpret_cast<const float*>(p.packed + TA::fold_bias_offset()) +
+                                             (L == LS ? TA::layer(LS - 1).Np : 0)
+                                       : (ly.sdf ? p.sdf_w : p.rgb_w) + TA::param_offset(L) + (int64_t)ly.N * ly.K;
+        for (int j = threadIdx.x; j < ly.Np; j += kThreadsF)
+            sbias[TA::bias_offset(L) + j] = TA::folded(L) || j < ly.N ? __ldg(b + j) : 0.0f;
+    });
     if (warp == kMmaWarpF) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
                      "r"(512));
@@ -315,12 +350,13 @@ __global__ void __launch_bounds__(kThreadsF, 1) k_mlp_tc(TcParams p) {
             uint32_t issued = 0;
             bool ok = true;
             const uint32_t dst = slot_addr(own);
-            for (int64_t pr = blockIdx.x; pr < n_pairs && ok; pr += gridDim.x) {
-                for (int j = 0; j < kPC; ++j) {
+            for (int64_t w = 0; ok && unit(w) >= 0; ++w) {
+                const int j0 = single(w) ? TA::sdf_chunks() : 0;
+                for (int j = j0; j < kPC; ++j) {
                     const ChunkInfo ci = s_chunks[j];
                     if (ci.slot != own) continue;
-                    // test-only: stop before the withheld chunk of the first pair
-                    if (pr == blockIdx.x && j == p.withhold) { ok = false; break; }
+                    // test-only: stop before the withheld chunk of the first pair (or tile)
+                    if (w == 0 && p.withhold >= 0 && j - j0 >= p.withhold) { ok = false; break; }
                     if (!mbar_wait(bar_empty0 + 8 * own, (issued & 1u) ^ first, abort_flag, p.spin)) { ok = false; break; }
                     mbar_expect_tx(bar_full0 + 8 * own, ci.bytes);
                     bulk_g2s(dst, p.packed + ci.off, ci.bytes, bar_full0 + 8 * own);
@@ -342,15 +378,17 @@ __global__ void __launch_bounds__(kThreadsF, 1) k_mlp_tc(TcParams p) {
             const uint32_t el = elect_one();
             uint32_t lc = 0, tpar = 0;
             bool ok = true;
-            for (int64_t pr = blockIdx.x; pr < n_pairs && ok; pr += gridDim.x, tpar ^= 1u) {
-                MmaRec cr = s_mma[0];
-                for (int j = 0; j < kPC; ++j) {
+            for (int64_t w = 0; ok && unit(w) >= 0; ++w, tpar ^= 1u) {
+                const bool one = single(w);
+                const uint32_t skipped = one ? tab.first_pass : 0u;   // slot uses of the pass left out
+                MmaRec cr = s_mma[one ? TA::sdf_chunks() : 0];
+                for (int j = one ? TA::sdf_chunks() : 0; j < kPC; ++j) {
                     const uint32_t f = cr.flags;
                     if (f & kRecFirst) {
                         if (!__all_sync(0xffffffffu, mbar_wait(bar_a, lc & 1u, abort_flag, p.spin))) { ok = false; break; }
                         // the colour layers' first input rows also hold the pair's first tile, back
                         // from its parking space
-                        if ((f & kRecRestore) &&
+                        if ((f & kRecRestore) && !one &&
                             !__all_sync(0xffffffffu, mbar_wait(bar_rest, tpar, abort_flag, p.spin))) {
                             ok = false;
                             break;
@@ -358,7 +396,7 @@ __global__ void __launch_bounds__(kThreadsF, 1) k_mlp_tc(TcParams p) {
                         tc_fence_after();
                     }
                     const uint32_t s = (f >> kRecSlotShift) & 3u;
-                    const uint32_t ph = ((f & kRecPar) ? 1u : 0u) ^ ((f & kRecFlip) ? tpar : 0u);
+                    const uint32_t ph = ((f & kRecPar) ? 1u : 0u) ^ ((f & kRecFlip) ? tpar : 0u) ^ ((skipped >> s) & 1u);
                     if (!__all_sync(0xffffffffu, mbar_wait(bar_full0 + 8 * s, ph, abort_flag, p.spin))) { ok = false; break; }
                     tc_fence_after();
                     const MmaRec nx = s_mma[j + 1 < kPC ? j + 1 : 0];
@@ -553,12 +591,14 @@ __global__ void __launch_bounds__(kThreadsF, 1) k_mlp_tc(TcParams p) {
                 ++tab_ph;
             return true;
         };
-        ok = build_table(2 * (int64_t)blockIdx.x, false);
-        for (int64_t pr = blockIdx.x; pr < n_pairs && ok; pr += gridDim.x) {
+        ok = build_table(unit(0), false);
+        for (int64_t w = 0; ok && unit(w) >= 0; ++w) {
+            const bool one = single(w);
+            const int64_t tile0 = unit(w), tile1 = one ? tile0 : tile0 + 1;
             // ---- the SDF layers of the pair's two tiles ----
-            for (int pass = 0; pass < 2 && ok; ++pass) {
-                const int64_t tile = 2 * pr + pass;
-                if (pass == 1 && !build_table(tile, true)) {
+            for (int pass = one ? 1 : 0; pass < 2 && ok; ++pass) {
+                const int64_t tile = pass ? tile1 : tile0;
+                if (pass == 1 && !one && !build_table(tile, true)) {
                     ok = false;
                     break;
                 }
@@ -583,7 +623,7 @@ __global__ void __launch_bounds__(kThreadsF, 1) k_mlp_tc(TcParams p) {
                     tc_fence_after();
                     const float* bias = sbias + boff;
                     boff += ly.Np;
-                    if (pass == 1 && L == LS - 1 && stasher) {
+                    if (pass == 1 && !one && L == LS - 1 && stasher) {
                         // the second tile's SDF MMAs are done: bring the first tile back into
                         // the tangent-row groups of A0 and of A1's extras block
                         bulk_wait();
@@ -873,8 +913,8 @@ __global__ void __launch_bounds__(kThreadsF, 1) k_mlp_tc(TcParams p) {
                     float x0[16];
                     tmem_ld16(tmem + lane_addr, x0);
                     tmem_wait_ld();
-                    const int64_t g = (2 * pr + (lane < 16 ? 1 : 0)) * kTileS + 16 * q + (lane & 15);
-                    if (g < total) {
+                    const int64_t g = (lane < 16 ? tile1 : tile0) * kTileS + 16 * q + (lane & 15);
+                    if (g < total && (lane < 16 || !one)) {
                         float* R = reinterpret_cast<float*>(p.rec + g);
                         R[4] = __fdividef(1.0f, 1.0f + __expf(-(x0[0] + bias[0])));
                         R[5] = __fdividef(1.0f, 1.0f + __expf(-(x0[1] + bias[1])));
@@ -889,7 +929,7 @@ __global__ void __launch_bounds__(kThreadsF, 1) k_mlp_tc(TcParams p) {
                 // the next pair's first table, while the colour layers' MMAs run: every warp
                 // has left the second tile's SDF output layer (the last reader of its table)
                 // once colour layer 0's accumulator is complete
-                if (L == LS && pr + gridDim.x < n_pairs && !build_table(2 * (pr + gridDim.x), false)) {
+                if (L == LS && unit(w + 1) >= 0 && !build_table(unit(w + 1), false)) {
                     ok = false;
                     break;
                 }
@@ -906,22 +946,73 @@ __global__ void __launch_bounds__(kThreadsF, 1) k_mlp_tc(TcParams p) {
     }
 }
 
-// ---- SDF values only (the hierarchical comparator's coarse pass) ----------
-// Tile: 128 samples, one value row each (no tangents); one accumulator
-// (TMEM columns 0..255); SDF layers only; the output layer needs column 0.
-constexpr int kTileV = 128;
+// ---- SDF values only (the samplers' coarse passes) ----------
+// Tile: 256 samples, one value row each, 128 to either operand region and accumulator, so that
+// a weight chunk's MMAs serve both; SDF layers only; of the output layer the 16 rows with net_0.
+// 12 epilogue warps (TMEM lane quarter w % 4, column part w / 4), one row per thread and
+// region, 16 columns a TMEM load, the next load in flight while the current columns are computed.
+// A layer is 4.1 k cycles of MMAs and then the softplus of 65 536 values, about 12 instructions
+// each, 6 k cycles of issue.  307 200 coarse samples of the room networks: 472 us; 1421 us with tiles
+// of 128, eight warps and the encodings by one sincos per column.
+constexpr int kTileV = 256;
+constexpr int kThreadsV = 32 * (kMmaWarpF + 1 + kStages);
+
+template <int ARCH> struct TcValue : TcArch<ARCH> {
+    using Base = TcArch<ARCH>;
+    static constexpr int LS = Base::kLS;
+    // the output layer's chunks are cut to their first 16 rows
+    __host__ __device__ static constexpr uint32_t bytes(int L, int c) {
+        return (uint32_t)((L == LS - 1 ? 16 : Base::layer(L).Np) * Base::chunk_k(L, c) * 2);
+    }
+    __host__ __device__ static constexpr uint32_t stage() {
+        uint32_t m = 0;
+        for (int l = 0; l < LS; ++l)
+            for (int c = 0; c < Base::chunks(l); ++c) m = bytes(l, c) > m ? bytes(l, c) : m;
+        return m;
+    }
+    __host__ __device__ static constexpr size_t smem_bytes() {
+        return 2 * (size_t)kABytes + kStages * (size_t)stage() + Base::bias_offset(LS) * 4 + kBarBytes +
+               (size_t)Base::sdf_chunks() * sizeof(ValRec);
+    }
+};
+struct ValEntry {
+    uint32_t off, bytes, a, a_sbo;
+    uint16_t n, kc, flags, pad;
+};
+template <int ARCH> struct ValTab {
+    ValEntry e[TcArch<ARCH>::sdf_chunks()];
+};
+template <int ARCH> constexpr ValTab<ARCH> make_val_tab() {
+    using TA = TcValue<ARCH>;
+    ValTab<ARCH> t{};
+    int j = 0;
+    for (int L = 0; L < TA::LS; ++L)
+        for (int c = 0; c < TA::chunks(L); ++c, ++j) {
+            ValEntry& e = t.e[j];
+            e.off = (uint32_t)TA::packed_offset(L, c);
+            e.bytes = TA::bytes(L, c);
+            e.a = (uint32_t)(c * kKChunk / 8) * 128u;
+            e.a_sbo = (uint32_t)(TA::layer(L).Kp / 8) * 128u;
+            e.n = (uint16_t)(L == TA::LS - 1 ? 16 : TA::layer(L).Np);
+            e.kc = (uint16_t)TA::chunk_k(L, c);
+            e.flags = (uint16_t)((c == 0 ? kRecFirst : 0u) | (c + 1 == TA::chunks(L) ? kRecLast : 0u));
+        }
+    return t;
+}
 
 template <int ARCH, bool F16>
-__global__ void __launch_bounds__(kThreads, 1) k_mlp_tc_value(TcParams p, float* __restrict__ f_out) {
-    using TA = TcArch<ARCH>;
+__global__ void __launch_bounds__(kThreadsV, 1) k_mlp_tc_value(TcParams p, const __grid_constant__ ValTab<ARCH> tab,
+                                                               float* __restrict__ f_out) {
+    using TA = TcValue<ARCH>;
     using A = Arch<ARCH>;
     constexpr int LS = A::kSdfLayers;
-    constexpr uint32_t kStage = TA::stage_bytes();
+    constexpr uint32_t kStage = TA::stage();
     extern __shared__ __align__(1024) uint8_t smem[];
     uint8_t* A0 = smem;
+    uint8_t* A1 = smem + kABytes;
     uint8_t* stage_base = smem + 2 * kABytes;
     float* sbias = reinterpret_cast<float*>(stage_base + kStages * kStage);
-    uint64_t* bars = reinterpret_cast<uint64_t*>(stage_base + kStages * kStage + TA::bias_bytes());
+    uint64_t* bars = reinterpret_cast<uint64_t*>(sbias + TA::bias_offset(LS));
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * kStages + 3);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
     const uint32_t bar_full0 = smem_u32(bars + 0), bar_empty0 = smem_u32(bars + kStages);
@@ -943,42 +1034,31 @@ __global__ void __launch_bounds__(kThreads, 1) k_mlp_tc_value(TcParams p, float*
             mbar_init(bar_empty0 + 8 * i, 1);
         }
         mbar_init(bar_acc, 1);
-        mbar_init(bar_a, kEpiThreads);
+        mbar_init(bar_a, kEpiWarpsF);
         mbar_init(bar_drain, 1);
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        // per-chunk records (offsets and descriptors computed here once instead of per chunk
-        // and tile in the producers' and the MMA warp's loops)
-        uint32_t off = 0;
-        for (int L = 0, j = 0; L < LS; ++L) {
-            const TcLayer ly = TA::layer(L);
-            const uint32_t a_sbo = (uint32_t)(ly.Kp / 8) * 128u;
-            const int n_mma = L == LS - 1 ? 16 : ly.Np;
-            for (int c = 0; c < TA::chunks(L); ++c, ++j) {
-                const int kc = TA::chunk_k(L, c);
-                const int k0 = c * kKChunk;
-                ValRec r;
-                r.bd0 = mdesc(smem_u32(stage_base), 128, (uint32_t)(kc / 8) * 128u);
-                r.ad = mdesc(smem_u32(A0) + (uint32_t)(k0 / 8) * 128u, 128, a_sbo);
-                r.id = idesc_mma<F16>(128, n_mma);
-                r.flags = (uint32_t)(kc / 16) | (c == 0 ? kRecFirst : 0u) | (c + 1 == TA::chunks(L) ? kRecLast : 0u);
-                r.off = off;
-                r.bytes = (uint32_t)TA::chunk_bytes(L, c);
-                off += r.bytes;
-                s_rec[j] = r;
-            }
-        }
     }
-    for (int i = threadIdx.x; i < TA::bias_offset(LS); i += kThreads) {
-        int L = 0;
-        while (L + 1 < LS && TA::bias_offset(L + 1) <= i) ++L;
-        const TcLayer ly = TA::layer(L);
-        const int j = i - TA::bias_offset(L);
-        sbias[i] = j < ly.N ? __ldg(p.sdf_w + TA::param_offset(L) + (int64_t)ly.N * ly.K + j) : 0.0f;
+    for (int j = threadIdx.x; j < kChunksV; j += kThreadsV) {
+        const ValEntry e = tab.e[j];
+        ValRec r;
+        r.bd0 = mdesc(smem_u32(stage_base), 128, (uint32_t)(e.kc / 8) * 128u);
+        r.ad = mdesc(smem_u32(A0) + e.a, 128, e.a_sbo);
+        r.id = idesc_mma<F16>(128, e.n);
+        r.flags = e.flags | (uint32_t)(e.kc / 16);
+        r.off = e.off;
+        r.bytes = e.bytes;
+        s_rec[j] = r;
     }
-    if (warp == kMmaWarp) {
+    static_for<0, LS>([&](auto lc) {
+        constexpr int L = decltype(lc)::value;
+        constexpr TcLayer ly = TA::layer(L);
+        const float* b = p.sdf_w + TA::param_offset(L) + (int64_t)ly.N * ly.K;
+        for (int j = threadIdx.x; j < ly.Np; j += kThreadsV) sbias[TA::bias_offset(L) + j] = j < ly.N ? __ldg(b + j) : 0.0f;
+    });
+    if (warp == kMmaWarpF) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
-                     "r"(256));
+                     "r"(512));
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
     }
     tc_fence_before();
@@ -986,15 +1066,15 @@ __global__ void __launch_bounds__(kThreads, 1) k_mlp_tc_value(TcParams p, float*
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
 
-    if (warp > kMmaWarp) {
+    if (warp > kMmaWarpF) {
         if (lane == 0) {
-            const uint32_t own = (uint32_t)(warp - kMmaWarp - 1);
+            const uint32_t own = (uint32_t)(warp - kMmaWarpF - 1);
             uint32_t seq = 0, issued = 0;
             bool ok = true;
             for (int64_t tile = blockIdx.x; tile < n_tiles && ok; tile += gridDim.x) {
                 for (int j = 0; j < kChunksV; ++j, ++seq) {
                     if (seq % kStages != own) continue;
-                    if (tile == blockIdx.x && (int)seq == p.withhold) { ok = false; break; }
+                    if (tile == blockIdx.x && p.withhold >= 0 && (int)seq >= p.withhold) { ok = false; break; }
                     const ValRec& r = s_rec[j];
                     const uint32_t ph = (seq / kStages) & 1u;
                     if (!mbar_wait(bar_empty0 + 8 * own, ph ^ 1u, abort_flag, p.spin)) { ok = false; break; }
@@ -1008,7 +1088,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_mlp_tc_value(TcParams p, float*
                 }
             }
         }
-    } else if (warp == kMmaWarp) {
+    } else if (warp == kMmaWarpF) {
         // the whole warp runs the issue loop (converged: the descriptors stay warp-uniform),
         // one elected lane issues the MMAs and commits
         {
@@ -1029,11 +1109,12 @@ __global__ void __launch_bounds__(kThreads, 1) k_mlp_tc_value(TcParams p, float*
                     const ValRec nx = s_rec[j + 1 < kChunksV ? j + 1 : 0];
                     // descriptors of the chunk's first K step (the weights' moved to stage s:
                     // kStage / 16 in the address field, which stays below 2^14), advanced by 16
-                    // (256 bytes) per K step
+                    // (256 bytes) per K step; A1 is kABytes further on
                     uint64_t ad = cr.ad, bd = cr.bd0 + (uint64_t)(s * (kStage >> 4));
                     uint32_t acc = (f & kRecFirst) ? 0u : 1u;
                     for (int kk = 0; kk < (int)(f & kRecNk); ++kk) {
                         mma_el(el, tmem, ad, bd, cr.id, acc);
+                        mma_el(el, tmem + 256, ad + (kABytes >> 4), bd, cr.id, acc);
                         acc = 1u;
                         ad += 16;
                         bd += 16;
@@ -1053,45 +1134,68 @@ __global__ void __launch_bounds__(kThreads, 1) k_mlp_tc_value(TcParams p, float*
             }
         }
     } else {
-        const int q = warp & 3, hf = warp >> 2;
-        const int r = 32 * q + lane;  // row = sample within the tile
+        const int q = warp & 3, pt = warp >> 2;   // lane quarter, column part
+        const int r = 32 * q + lane;              // row in either region
         const uint32_t lane_addr = (uint32_t)(32 * q) << 16;
         const float half_beta = 0.5f * p.beta, inv_beta = 1.0f / p.beta;
         constexpr float kInvSqrt2 = 0.70710678118654752f;
+        constexpr int kOct = A::kPeSdf, kOctPart = (kOct + kPartsF - 1) / kPartsF;   // octaves of a part
         uint32_t lc = 0;
         bool ok = true;
-        for (int64_t tile = blockIdx.x; tile < n_tiles && ok; tile += gridDim.x) {
-            const int64_t g = tile * kTileV + r;
-            const bool valid = g < total;
-            int64_t ray = 0;
-            float t = 0.0f;
-            if (valid) {
-                if (p.src.mode == kUniform) {
-                    ray = __ldg(p.src.sample_ray + g);
-                    const int32_t o0 = __ldg(p.src.offsets + ray), o1 = __ldg(p.src.offsets + ray + 1);
-                    const float tn = __ldg(p.src.t_n + ray), tf = __ldg(p.src.t_f + ray);
-                    const float dl = (tf - tn) / (float)(o1 - o0);
-                    t = tn + ((float)(g - o0) + 0.5f) * dl;
-                } else {
-                    ray = explicit_ray(p.src, g);
-                    t = __ldg(p.src.t + g);
-                }
-            }
-            float xt[3];
-#pragma unroll
-            for (int a = 0; a < 3; ++a)
-                xt[a] = (__ldg(p.src.ray_o + 3 * ray + a) + t * __ldg(p.src.ray_d + 3 * ray + a) - p.center[a]) * p.inv_scale;
-            {
-                constexpr int Kp0 = TA::layer(0).Kp;
-                for (int k0 = hf * (Kp0 / 2); k0 < (hf + 1) * (Kp0 / 2); k0 += 8) {
-                    float v0[8];
-#pragma unroll
-                    for (int j = 0; j < 8; ++j) v0[j] = k0 + j < A::kEnc ? enc_val(xt, k0 + j, A::kPeSdf, 0, false) : 0.0f;
-                    st_row8<F16>(A0, r, k0, Kp0, v0);
-                }
-            }
+        auto arrive = [&]() {
             fence_proxy_async();
-            mbar_arrive(bar_a);
+            __syncwarp();
+            if (lane == 0) mbar_arrive(bar_a);
+        };
+        auto put = [&](uint8_t* base, int c, int Kp, float v) {
+            *reinterpret_cast<uint16_t*>(base + a_off(r, c, Kp)) = (uint16_t)(pack2<F16>(v, 0.0f) & 0xffffu);
+        };
+        // this part's share of the encoding at columns c0 .. of both rows, times sc: the coordinates
+        // and the padding up to Kp (part 0), then its octaves
+        auto encode = [&](const float (&xt)[2][3], int c0, int Kp, float sc) {
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                uint8_t* base = h ? A1 : A0;
+                if (pt == 0) {
+#pragma unroll
+                    for (int a = 0; a < 3; ++a) put(base, c0 + a, Kp, xt[h][a] * sc);
+                    for (int c = c0 + A::kEnc; c < Kp; ++c) put(base, c, Kp, 0.0f);
+                }
+                for (int o = pt * kOctPart; o < (pt + 1) * kOctPart && o < kOct; ++o)
+#pragma unroll
+                    for (int a = 0; a < 3; ++a) {
+                        float sn, cs;
+                        sincosf((float)(1 << o) * xt[h][a], &sn, &cs);
+                        put(base, c0 + 3 + 6 * o + a, Kp, sn * sc);
+                        put(base, c0 + 6 + 6 * o + a, Kp, cs * sc);
+                    }
+            }
+        };
+        for (int64_t tile = blockIdx.x; tile < n_tiles && ok; tile += gridDim.x) {
+            float xt[2][3];
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int64_t g = tile * kTileV + 128 * h + r;
+                int64_t ray = 0;
+                float t = 0.0f;
+                if (g < total) {
+                    if (p.src.mode == kUniform) {
+                        ray = __ldg(p.src.sample_ray + g);
+                        const int32_t o0 = __ldg(p.src.offsets + ray), o1 = __ldg(p.src.offsets + ray + 1);
+                        const float tn = __ldg(p.src.t_n + ray), tf = __ldg(p.src.t_f + ray);
+                        const float dl = (tf - tn) / (float)(o1 - o0);
+                        t = tn + ((float)(g - o0) + 0.5f) * dl;
+                    } else {
+                        ray = explicit_ray(p.src, g);
+                        t = __ldg(p.src.t + g);
+                    }
+                }
+#pragma unroll
+                for (int a = 0; a < 3; ++a)
+                    xt[h][a] = (__ldg(p.src.ray_o + 3 * ray + a) + t * __ldg(p.src.ray_d + 3 * ray + a) - p.center[a]) * p.inv_scale;
+            }
+            encode(xt, 0, TA::layer(0).Kp, 1.0f);
+            arrive();
             int boff = 0;
             for (int L = 0; L < LS; ++L, ++lc) {
                 const TcLayer ly = TA::layer(L);
@@ -1102,39 +1206,61 @@ __global__ void __launch_bounds__(kThreads, 1) k_mlp_tc_value(TcParams p, float*
                 boff += ly.Np;
                 if (L < LS - 1) {
                     const int Kn = TA::layer(L + 1).Kp;
-                    const float sc = ly.idx + 1 == A::kSkip ? kInvSqrt2 : 1.0f;
-                    for (int c0 = half_lo(Kn, hf); c0 < half_hi(Kn, hf); c0 += 16) {
-                        float x0[16], o[16];
-                        if (c0 < ly.Np) {
-                            tmem_ld16(tmem + lane_addr + c0, x0);
-                            tmem_wait_ld();
-                        }
+                    const bool skip = ly.idx + 1 == A::kSkip;
+                    const float sc = skip ? kInvSqrt2 : 1.0f;
+                    // this part's 16-column blocks that hold hidden units, region A0 then A1
+                    const int lo = part_lo(Kn, pt, kPartsF), hi0 = part_hi(Kn, pt, kPartsF);
+                    const int hi = hi0 < ly.Np ? hi0 : ly.Np;
+                    const int nb = hi > lo ? (hi - lo) / 16 : 0;
+                    auto block = [&](int b, const float (&x)[16]) {
+                        uint8_t* base = b < nb ? A0 : A1;
+                        const int c0 = lo + 16 * (b < nb ? b : b - nb);
+                        float o[16];
 #pragma unroll
                         for (int j = 0; j < 16; ++j) {
-                            const int col = c0 + j;
-                            if (col < ly.N) {
-                                float h, sg;
-                                softplus_slope_tanh(x0[j] + bias[col], half_beta, inv_beta, h, sg);
-                                o[j] = h * sc;
+                            float h, sg;
+                            softplus_slope_tanh(x[j] + bias[c0 + j], half_beta, inv_beta, h, sg);
+                            o[j] = h * sc;
+                        }
+#pragma unroll
+                        for (int g8 = 0; g8 < 2; ++g8) {
+                            const int c = c0 + 8 * g8;
+                            if (c + 8 <= ly.N) {
+                                st_row8<F16>(base, r, c, Kn, o + 8 * g8);
                             } else {
-                                const int e = col - ly.N;
-                                o[j] = e < A::kEnc ? enc_val(xt, e, A::kPeSdf, 0, false) * sc : 0.0f;
+                                // hidden units below N; the rest of the group is padding, or the skip
+                                // input's encoding, which others write
+#pragma unroll
+                                for (int j = 0; j < 8; ++j) {
+                                    if (c + j < ly.N) put(base, c + j, Kn, o[8 * g8 + j]);
+                                    else if (!skip && c + j < Kn) put(base, c + j, Kn, 0.0f);
+                                }
                             }
                         }
-                        st_row8<F16>(A0, r, c0, Kn, o);
-                        st_row8<F16>(A0, r, c0 + 8, Kn, o + 8);
+                    };
+                    auto addr = [&](int b) { return tmem + lane_addr + (b < nb ? 0 : 256) + lo + 16 * (b < nb ? b : b - nb); };
+                    float xa[16], xb[16];
+                    if (nb > 0) {
+                        tmem_ld16(addr(0), xa);
+                        for (int b = 0; b < 2 * nb; b += 2) {
+                            tmem_wait_ld16(xa);
+                            tmem_ld16(addr(b + 1), xb);
+                            block(b, xa);
+                            tmem_wait_ld16(xb);
+                            if (b + 2 < 2 * nb) tmem_ld16(addr(b + 2), xa);
+                            block(b + 1, xb);
+                        }
                     }
-                } else if (hf == 0) {
+                    if (skip) encode(xt, ly.N, Kn, kInvSqrt2);
+                } else if (pt < 2) {
                     float x0[16];
-                    tmem_ld16(tmem + lane_addr, x0);
-                    tmem_wait_ld();
-                    if (valid) f_out[g] = p.scale * (x0[0] + bias[0]);
+                    tmem_ld16(tmem + lane_addr + 256 * pt, x0);
+                    tmem_wait_ld16(x0);
+                    const int64_t g = tile * kTileV + 128 * pt + r;
+                    if (g < total) f_out[g] = p.scale * (x0[0] + bias[0]);
                 }
                 tc_fence_before();
-                if (L < LS - 1) {
-                    fence_proxy_async();
-                    mbar_arrive(bar_a);
-                }
+                if (L < LS - 1) arrive();
             }
         }
         if (!ok) set_status(p.status, TSDFS_DEV_TIMEOUT);
@@ -1142,16 +1268,15 @@ __global__ void __launch_bounds__(kThreads, 1) k_mlp_tc_value(TcParams p, float*
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    if (warp == kMmaWarp) {
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(256));
+    if (warp == kMmaWarpF) {
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512));
     }
 }
 
 template <int ARCH, bool F16>
 int launch_tc_value(const tsdfs_mlp* m, const SampleSource& src, float* f_out, cudaStream_t st) {
-    using TA = TcArch<ARCH>;
-    const size_t smem = 2 * kABytes + kStages * (size_t)TA::stage_bytes() + TA::bias_bytes() + kBarBytes +
-                        (size_t)TA::sdf_chunks() * sizeof(ValRec);
+    constexpr size_t smem = TcValue<ARCH>::smem_bytes();
+    static_assert(smem <= 232448, "k_mlp_tc_value shared memory exceeds 227 KB");
     static bool attr[2] = {false, false};
     if (!attr[ARCH]) {
         int rc = cuda_check(cudaFuncSetAttribute(k_mlp_tc_value<ARCH, F16>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -1178,7 +1303,8 @@ int launch_tc_value(const tsdfs_mlp* m, const SampleSource& src, float* f_out, c
     if (src.mode == kUniform && !src.sample_ray) return fail(TSDFS_E_INVALID, "value pass needs the sample ray index");
     const int64_t tiles = (sample_bound(src) + kTileV - 1) / kTileV;
     const unsigned blocks = (unsigned)(tiles < sms ? (tiles < 1 ? 1 : tiles) : sms);
-    k_mlp_tc_value<ARCH, F16><<<blocks, kThreads, smem, st>>>(p, f_out);
+    static constexpr ValTab<ARCH> tab = make_val_tab<ARCH>();
+    k_mlp_tc_value<ARCH, F16><<<blocks, kThreadsV, smem, st>>>(p, tab, f_out);
     return cuda_check(cudaGetLastError(), "mlp_tc_value launch");
 }
 
@@ -1323,11 +1449,12 @@ int launch_tc(const tsdfs_mlp* m, const SampleSource& src, SampleRec* rec, int64
     int dev = 0, sms = 152;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const int64_t pairs = ((max_samples + kTileS - 1) / kTileS + 1) / 2;
-    int64_t blocks = pairs < sms ? pairs : sms;
+    const int64_t tiles = (max_samples + kTileS - 1) / kTileS;
+    int64_t blocks = tiles < sms ? tiles : sms;
     if (blocks > kPairCtas) blocks = kPairCtas;
     if (blocks < 1) blocks = 1;
-    k_mlp_tc<ARCH, F16><<<(unsigned)blocks, kThreadsF, smem, st>>>(p);
+    static constexpr PairTab<ARCH> tab = make_pair_tab<ARCH>();
+    k_mlp_tc<ARCH, F16><<<(unsigned)blocks, kThreadsF, smem, st>>>(p, tab);
     return cuda_check(cudaGetLastError(), "mlp_tc launch");
 }
 
