@@ -30,9 +30,14 @@
 // 128 outputs (hi and lo, 32 KB) through a ring of two stages; three producer warps copy the
 // items' parts in turn, because one thread's bulk copies do not overlap.
 //
-// The colour network's rows are the value rows only.  Its first layer reads the SDF features
-// where the SDF's operand was and x~, the direction encoding and the unit normal from the first
-// columns of the rows below each value-row group (the d/dx rows' place, dead by then).
+// The colour network has value rows only, a quarter of a tile's: so its layers run once for up to
+// kUnit tiles, on all 128 rows.  Each tile's colour input (the SDF features, and x~, the
+// direction encoding and the unit normal) is parked in global memory (L2) in operand layout, tile j
+// in row group j of every lane quarter; bulk copies bring the features back as the operand, and
+// the other columns through the weight ring as an item of their own before their weights.  (One
+// tile at a time the colour layers were 38 of a tile's 96 items.)  61 915 samples of the room
+// networks: SIMT kernel 13.8 ms, this one with the colour layers per tile 1.20 ms, per unit 1.10 ms,
+// and with the epilogue's groups two at a time 1.03 ms.
 //
 // VALUE: the samplers' coarse pass (SDF value only): 128 samples per tile, one row each, no
 // gradient and no colour network.
@@ -64,12 +69,14 @@ constexpr int kPh = 128;              // outputs per phase
 constexpr int kGrp = 6;               // 8-column groups of a phase per part, at most
 constexpr uint32_t kPartBytes = 64 * 1024;                 // 128 rows x 256 16-bit columns
 constexpr uint32_t kStageBytes = 2 * kPh * kKChunk * 2;    // hi and lo of one item
+constexpr int kUnit = 4;              // tiles per pass of the colour layers
 constexpr float kUp = 32.0f;          // operand scale
 constexpr float kLoUp = 2048.0f;      // further scale of the low part
 constexpr float kDown = 1.0f / (kUp * kUp), kLoDown = 1.0f / kLoUp;
 constexpr float kLimit = 2000.0f;     // largest operand the high part is trusted with
 constexpr float kBias0 = 1.7e-8f, kBias1 = 1.58e-8f;   // what a main sum of n MMAs lacks: kBias0 + n kBias1
 constexpr float kMinGrad = 1e-4f;
+constexpr int kMaxCtas = 192;         // CTAs with a place to park
 constexpr float kRsqrt2 = 0.70710678118654752f;
 
 template <int ARCH> struct FArch {
@@ -132,12 +139,20 @@ template <int ARCH> struct FArch {
         return VALUE ? kTileV * (4 + 6 * A::kPeSdf) : kTile * (8 + 6 * (A::kPeSdf + A::kPeDir));
     }
     // net_0's weights and partial sums (3 parts x 128 rows); the record's SDF half, the colour
-    // output's weights and partial sums (3 parts x 3 colours x 32 samples)
+    // output's weights and partial sums (3 parts x 3 colours x 128 rows)
     static constexpr int kW0 = pad16(A::sdf(LS - 1).in), kWc = pad16(A::rgb(A::kRgbLayers - 1).in);
     template <bool VALUE> __host__ __device__ static constexpr uint32_t scratch_floats() {
-        return kW0 + kParts * 128 + (VALUE ? 0 : kTile * 8 + 3 * kWc + kParts * 3 * kTile);
+        return kW0 + kParts * 128 + (VALUE ? 0 : kTile * 8 + 3 * kWc + kParts * 3 * 128);
     }
-    template <bool VALUE> __host__ __device__ static constexpr int n_items() { return items(0, mma_layers<VALUE>()); }
+    // items of a tile's SDF layers, and of a unit's colour layers (the first one's phases take one
+    // more each, the operand columns beyond the features)
+    template <bool VALUE> __host__ __device__ static constexpr int sdf_items() { return items(0, VALUE ? LS - 1 : LS); }
+    template <bool VALUE> __host__ __device__ static constexpr int n_items() {
+        return VALUE ? sdf_items<true>() : items(0, NL - 1) + phases(LS);
+    }
+    // the parked colour inputs of a unit: the features' operand image (hi, lo), then the others'
+    static constexpr uint32_t kParkF = 16u * (kFp / 8) * 128u, kParkX = 16u * (kXp / 8) * 128u;
+    __host__ __device__ static constexpr size_t park_bytes() { return 2 * (size_t)(kParkF + kParkX); }
     template <bool VALUE> __host__ __device__ static constexpr uint32_t bias_floats() {
         return bias_base(mma_layers<VALUE>());
     }
@@ -158,7 +173,8 @@ struct __align__(16) Item {
     uint16_t steps;    // K steps of 16
     uint16_t pad[2];
     uint16_t edge;     // bit 0: first item of a phase, bit 1: last, bit 2 / 3: its operand's columns below /
-                       // from 128 are awaited first
+                       // from 128 are awaited first, bit 4: the parked features are, bit 5: an operand item
+                       // (parked columns, no MMAs), bit 6: its operand is the item before
 };
 static_assert(sizeof(Item) == 32, "item record");
 
@@ -172,6 +188,7 @@ struct F32Params {
     SampleRec* rec;      // full evaluation
     float* f_out;        // VALUE
     uint32_t* redo;      // set when a tile is marked
+    uint8_t* park;       // FArch::park_bytes() per CTA
     uint32_t* status;
     uint32_t spin;
     int withhold;
@@ -184,14 +201,10 @@ __device__ __forceinline__ void wait_ld16(float (&a)[8], float (&b)[8]) {
                  :
                  : "memory");
 }
-__device__ __forceinline__ void stmat1(uint32_t addr, uint32_t r0) {
-    asm volatile("stmatrix.sync.aligned.m8n8.x1.shared.b16 [%0], {%1};" ::"r"(addr), "r"(r0) : "memory");
-}
-
-// the two FP16 parts of a pair of FP32 operands (see the head of the file)
+// global-memory writes of this thread before bulk copies that read them
+__device__ __forceinline__ void fence_async_global() { asm volatile("fence.proxy.async;" ::: "memory"); }
+// the two FP16 parts of a pair of FP32 operands times kUp (see the head of the file)
 __device__ __forceinline__ void split_f32(float a, float b, uint32_t& hi, uint32_t& lo) {
-    a *= kUp;
-    b *= kUp;
     const __half2 h = __floats2half2_rn(a, b);
     const float2 f = __half22float2(h);
     const __half2 l = __floats2half2_rn((a - f.x) * kLoUp, (b - f.y) * kLoUp);
@@ -233,16 +246,17 @@ __global__ void __launch_bounds__(kThr, 1) k_mlp_f32(F32Params p) {
     float* s_dot = s_w0 + F::kW0;                  // [part][row]
     float* s_out = s_dot + kParts * 128;           // [sample][8]
     float* s_wc = s_out + kTile * 8;               // [colour][input]
-    float* s_cdot = s_wc + 3 * F::kWc;             // [part][colour][sample]
+    float* s_cdot = s_wc + 3 * F::kWc;             // [part][colour][row]
     Item* items = reinterpret_cast<Item*>(s_w0 + F::template scratch_floats<VALUE>());
     uint64_t* bars = reinterpret_cast<uint64_t*>(items + NT);
-    // bars: full[2], empty[2], acc[2], drained[2], operand[2], epi, end
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 12);
+    // bars: full[2], empty[2], acc[2], drained[2], operand[2], epi, end, parked, back
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 14);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
     volatile uint32_t* s_mark = tmem_slot + 2;
     const uint32_t bar_full = smem_u32(bars), bar_empty = smem_u32(bars + kStages);
     const uint32_t bar_acc = smem_u32(bars + 4), bar_drained = smem_u32(bars + 6), bar_op = smem_u32(bars + 8),
-                   bar_epi = smem_u32(bars + 10), bar_end = smem_u32(bars + 11);
+                   bar_epi = smem_u32(bars + 10), bar_end = smem_u32(bars + 11), bar_park = smem_u32(bars + 12),
+                   bar_back = smem_u32(bars + 13);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
     const int64_t total = sample_total(p.src);
@@ -263,6 +277,8 @@ __global__ void __launch_bounds__(kThr, 1) k_mlp_f32(F32Params p) {
         }
         mbar_init(bar_epi, kEpi);
         mbar_init(bar_end, 1);
+        mbar_init(bar_park, kEpi);
+        mbar_init(bar_back, 1);
         *abort_flag = 0;
         *s_mark = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -271,25 +287,33 @@ __global__ void __launch_bounds__(kThr, 1) k_mlp_f32(F32Params p) {
     if (threadIdx.x < NLr) {
         const int L = threadIdx.x;
         uint32_t off = (uint32_t)F::layer_base(L);
-        int j = F::items(0, L);
+        int j = F::items(0, L) + (L > LS ? F::phases(LS) : 0);
         const uint32_t sbo = (uint32_t)(F::k_main(L) / 8) * 128u;
         for (int ph = 0; ph < F::phases(L); ++ph) {
             const int n = F::phase_n(L, ph);
             for (int c = 0; c < F::chunks(L); ++c) {
                 Item it;
                 const int kc = F::chunk_k(L, c);
+                const bool extra = c == F::main_chunks(L);   // the colour input's columns beyond the features
                 it.off = off;
                 it.bytes = (uint32_t)(n * kc * 2);
                 off += 2 * it.bytes;
-                // the colour input's extra columns live one row group below the value rows
-                it.a = c < F::main_chunks(L) ? (uint32_t)(c * (kKChunk / 8)) * 128u : sbo;
-                it.a_sbo = sbo;
+                it.a = extra ? 0u : (uint32_t)(c * (kKChunk / 8)) * 128u;
+                it.a_sbo = extra ? (uint32_t)(F::kXp / 8) * 128u : sbo;
                 it.b_sbo = (uint32_t)(kc / 8) * 128u;
                 it.idesc = idesc_mma<true>(128, n);
                 it.steps = (uint16_t)(kc / 16);
                 it.pad[0] = it.pad[1] = 0;
-                it.edge = (uint16_t)((c == 0 ? 1 : 0) | (c + 1 == F::chunks(L) ? 2 : 0) | (ph == 0 && c == 0 ? 4 : 0) |
-                                     (ph == 0 && c * kKChunk == kPh ? 8 : 0));
+                const bool back = L == LS && ph == 0 && c == 0;
+                it.edge = (uint16_t)((c == 0 ? 1 : 0) | (c + 1 == F::chunks(L) ? 2 : 0) | (L != LS && ph == 0 && c == 0 ? 4 : 0) |
+                                     (L != LS && ph == 0 && c * kKChunk == kPh ? 8 : 0) | (back ? 16 : 0) | (extra ? 64 : 0));
+                if (extra) {
+                    Item x = it;
+                    x.off = 2 * F::kParkF;
+                    x.bytes = F::kParkX;
+                    x.edge = 32;
+                    items[j++] = x;
+                }
                 items[j++] = it;
             }
         }
@@ -314,9 +338,6 @@ __global__ void __launch_bounds__(kThr, 1) k_mlp_f32(F32Params p) {
             s_wc[i] = k < K ? __ldg(p.rgb_w + F::param_offset(F::NL - 1) + (i / F::kWc) * K + k) : 0.0f;
         }
     }
-    // operand rows the colour network's MMAs read but nothing writes stay finite
-    for (int i = threadIdx.x; i < (int)(2 * kPartBytes / 16); i += kThr)
-        reinterpret_cast<uint4*>(a_hi)[i] = make_uint4(0, 0, 0, 0);
     if (warp == kMma) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
                      "r"(512));
@@ -327,27 +348,42 @@ __global__ void __launch_bounds__(kThr, 1) k_mlp_f32(F32Params p) {
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
+    // this CTA's tiles: blockIdx.x + k gridDim.x, k < mine; units of kUnit of them (VALUE: one)
+    const int64_t mine = (n_tiles - blockIdx.x + gridDim.x - 1) / gridDim.x;
+    constexpr int kU = VALUE ? 1 : kUnit, NS = F::template sdf_items<VALUE>();
+    auto tile_of = [&](int64_t k) { return blockIdx.x + k * gridDim.x; };
+    uint8_t* park = VALUE ? nullptr : p.park + (size_t)blockIdx.x * F::park_bytes();
 
     if (warp > kMma) {
         // ---------------------------------------- producers: the items' parts in turn
         if (lane == 0) {
-            const int64_t mine = (n_tiles - blockIdx.x + gridDim.x - 1) / gridDim.x;   // tiles of this CTA
-            const int64_t parts = 2 * mine * NT;
-            int64_t last = -1;       // the last item this thread copied a part of
-            int j = (warp - kMma - 1) / 2;
+            int64_t last = -1, g = 0;       // the last item this thread copied a part of, the item in hand
+            int turn = warp - kMma - 1;     // parts until this thread's next one
+            uint32_t parked = 0;            // units up to the one in hand
             bool ok = true;
-            for (int64_t t = warp - kMma - 1; t < parts; t += kProd) {
-                const int64_t g = t >> 1;
-                const uint32_t stage = (uint32_t)g & 1u, part = (uint32_t)t & 1u;
-                if (p.withhold >= 0 && g >= p.withhold) { ok = false; break; }   // test-only: never issued
-                const uint32_t off = items[j].off, bytes = items[j].bytes;
-                if (!mbar_wait(bar_empty + 8 * stage, ((uint32_t)(g >> 1) & 1u) ^ 1u, abort_flag, p.spin)) { ok = false; break; }
-                mbar_expect_tx(bar_full + 8 * stage, bytes);
-                bulk_g2s(smem_u32(ring) + stage * kStageBytes + part * bytes, p.packed + off + part * bytes, bytes,
-                         bar_full + 8 * stage);
-                last = g;
-                j += (int)(((t + kProd) >> 1) - g);
-                if (j >= NT) j -= NT;
+            auto item = [&](int j) {
+                const bool operand = (items[j].edge & 32u) != 0;
+                for (uint32_t part = 0; part < 2; ++part, --turn) {
+                    if (turn != 0) continue;
+                    turn = kProd;
+                    const uint32_t stage = (uint32_t)g & 1u;
+                    if (p.withhold >= 0 && g >= p.withhold) { ok = false; return; }   // test-only: never issued
+                    const uint32_t off = items[j].off, bytes = items[j].bytes;
+                    if (operand && !mbar_wait(bar_park, (parked - 1) & 1u, abort_flag, p.spin)) { ok = false; return; }
+                    if (!mbar_wait(bar_empty + 8 * stage, ((uint32_t)(g >> 1) & 1u) ^ 1u, abort_flag, p.spin)) { ok = false; return; }
+                    mbar_expect_tx(bar_full + 8 * stage, bytes);
+                    bulk_g2s(smem_u32(ring) + stage * kStageBytes + part * bytes, (operand ? park : p.packed) + off + part * bytes,
+                             bytes, bar_full + 8 * stage);
+                    last = g;
+                }
+                ++g;
+            };
+            for (int64_t k = 0; k < mine && ok; k += kU) {
+                const int nt = mine - k < kU ? (int)(mine - k) : kU;
+                for (int i = 0; i < nt && ok; ++i)
+                    for (int j = 0; j < NS && ok; ++j) item(j);
+                ++parked;
+                for (int j = NS; j < NT && ok; ++j) item(j);
             }
             if (!ok && last >= 0) {
                 // a copy of this thread may be in flight: its phase completes once the other part is
@@ -365,19 +401,25 @@ __global__ void __launch_bounds__(kThr, 1) k_mlp_f32(F32Params p) {
         auto wait = [&](uint32_t bar, uint32_t parity) {
             return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag, p.spin));
         };
-        for (int64_t tile = blockIdx.x; tile < n_tiles && ok; tile += gridDim.x) {
-            for (int j = 0; j < NT; ++j, ++g) {
+        uint32_t back = 0;
+        auto run = [&](int j0, int j1) {
+            for (int j = j0; j < j1; ++j, ++g) {
                 const Item it = items[j];
-                if ((it.edge & 4u) && !wait(bar_op, op_a++ & 1u)) { ok = false; break; }
-                if ((it.edge & 8u) && !wait(bar_op + 8, op_b++ & 1u)) { ok = false; break; }
-                // the buffer's previous phase has been read
-                if ((it.edge & 1u) && ph >= 2 && !wait(bar_drained + 8 * (ph & 1u), ((ph >> 1) - 1) & 1u)) { ok = false; break; }
                 const uint32_t stage = g & 1u;
-                if (!wait(bar_full + 8 * stage, (g >> 1) & 1u)) { ok = false; break; }
+                if (it.edge & 32u) continue;   // an operand: the next item waits for it
+                if ((it.edge & 4u) && !wait(bar_op, op_a++ & 1u)) return false;
+                if ((it.edge & 8u) && !wait(bar_op + 8, op_b++ & 1u)) return false;
+                if ((it.edge & 16u) && !wait(bar_back, back++ & 1u)) return false;
+                // the buffer's previous phase has been read
+                if ((it.edge & 1u) && ph >= 2 && !wait(bar_drained + 8 * (ph & 1u), ((ph >> 1) - 1) & 1u)) return false;
+                if ((it.edge & 64u) && !wait(bar_full + 8 * (stage ^ 1u), ((g - 1) >> 1) & 1u)) return false;
+                if (!wait(bar_full + 8 * stage, (g >> 1) & 1u)) return false;
                 tc_fence_after();
                 const uint32_t b = r0 + stage * kStageBytes;
                 uint64_t bh = mdesc(b, 128, it.b_sbo), bl = mdesc(b + it.bytes, 128, it.b_sbo);
-                uint64_t ah = mdesc(ah0 + it.a, 128, it.a_sbo), al = mdesc(al0 + it.a, 128, it.a_sbo);
+                const uint32_t ax = r0 + (stage ^ 1u) * kStageBytes;
+                uint64_t ah = mdesc(it.edge & 64u ? ax : ah0 + it.a, 128, it.a_sbo);
+                uint64_t al = mdesc(it.edge & 64u ? ax + F::kParkX : al0 + it.a, 128, it.a_sbo);
                 const uint32_t d_main = tmem + (ph & 1u) * (2 * kPh), d_corr = d_main + kPh;
                 uint32_t acc = it.edge & 1u ? 0u : 1u;
                 for (int k = 0; k < it.steps; ++k) {
@@ -390,9 +432,16 @@ __global__ void __launch_bounds__(kThr, 1) k_mlp_f32(F32Params p) {
                     bh += 16;
                     bl += 16;
                 }
+                if (it.edge & 64u) commit_el(el, bar_empty + 8 * (stage ^ 1u));
                 commit_el(el, bar_empty + 8 * stage);
                 if (it.edge & 2u) commit_el(el, bar_acc + 8 * (ph++ & 1u));
             }
+            return true;
+        };
+        for (int64_t k = 0; k < mine && ok; k += kU) {
+            const int nt = mine - k < kU ? (int)(mine - k) : kU;
+            for (int i = 0; i < nt && ok; ++i) ok = run(0, NS);
+            if (ok) ok = run(NS, NT);
         }
         if (!ok && el) {
             mma_commit(bar_end);
@@ -407,7 +456,7 @@ __global__ void __launch_bounds__(kThr, 1) k_mlp_f32(F32Params p) {
         const float inv_beta = 1.0f / p.beta;
         const float b0 = __ldg(p.sdf_w + F::param_offset(LS - 1) + (int64_t)F::layer(LS - 1).out * F::layer(LS - 1).in);
         const int et = threadIdx.x;
-        uint32_t phs = 0, epi_ph = 0;            // phases waited for, epilogue barriers
+        uint32_t phs = 0, epi_ph = 0, backs = 0;   // phases waited for, epilogue barriers, units fetched back
         uint32_t buf = 0;                         // TMEM column of the phase in hand
         __half2 big = __float2half2_rn(0.0f);     // largest |operand| (scaled high parts) of this thread, or NaN
         const __half2 kHuge = __float2half2_rn(65504.0f);
@@ -447,14 +496,10 @@ __global__ void __launch_bounds__(kThr, 1) k_mlp_f32(F32Params p) {
             tmem_ld16x256_x1(buf + lq + kPh + c, cr);
             tmem_ld16x256_x1(buf + lq16 + kPh + c, cr + 4);
         };
-        // the value rows only (row group 0): two columns of the phase
-        auto load1 = [&](int c, float share, float (&z)[2]) {
-            float m[4], cr[4];
+        // rows 0-15 only: the value rows' registers are 0 and 1
+        auto issue1 = [&](int c, float (&m)[4], float (&cr)[4]) {
             tmem_ld16x256_x1(buf + lq + c, m);
             tmem_ld16x256_x1(buf + lq + kPh + c, cr);
-            asm volatile("tcgen05.wait::ld.sync.aligned;" : "+f"(m[0]), "+f"(m[1]), "+f"(cr[0]), "+f"(cr[1]) : : "memory");
-#pragma unroll
-            for (int e = 0; e < 2; ++e) z[e] = fmaf(m[e], share, fmaf(cr[e], kLoDown, m[e]));
         };
         // row i of the lane quarter (stmatrix: lane i addresses row i) at column 0
         auto row_at = [&](uint8_t* base, int r, int pitch) { return smem_u32(base) + a_off(32 * q + r, 0, pitch); };
@@ -468,7 +513,7 @@ __global__ void __launch_bounds__(kThr, 1) k_mlp_f32(F32Params p) {
             split_f32(a, b, hi, lo);
             big = __hmax2_nan(big, __habs2(*reinterpret_cast<const __half2*>(&hi)));
         };
-        // split the four row groups' column pairs v
+        // split the four row groups' column pairs v (operands times kUp)
         auto split4 = [&](const float (&v)[8], uint32_t (&o)[8]) {
 #pragma unroll
             for (int r = 0; r < 4; ++r) split(v[2 * r], v[2 * r + 1], o[r], o[4 + r]);
@@ -545,7 +590,7 @@ __global__ void __launch_bounds__(kThr, 1) k_mlp_f32(F32Params p) {
 #pragma unroll
                     for (int e = 0; e < 2; ++e) {
                         const int j = 8 * gr + fc + e;
-                        v[2 * r + e] = j < A::kEnc ? enc(r, j) : 0.0f;
+                        v[2 * r + e] = j < A::kEnc ? enc(r, j) * kUp : 0.0f;
                     }
                 uint32_t o[8];
                 split4(v, o);
@@ -554,11 +599,63 @@ __global__ void __launch_bounds__(kThr, 1) k_mlp_f32(F32Params p) {
             operand_done(0);
         };
 
+        // a phase's 8-column groups of this part, two at a time.  What a group takes is a chain of some
+        // 40 dependent instructions, and three warps to a scheduler do not hide it: two groups wholly
+        // below n_fast go through act(c, z, o) as one straight run of code that interleaves, and only
+        // the others branch per column, through edge(c, z, o).  (One group at a time, with the branches:
+        // 1330 cycles a group and warp.)  put(i, c, o) takes the results; accumulators end at n_acc
+        // (zero sums beyond), groups at n_all.
+        auto groups = [&](float share, int n_fast, int n_acc, int n_all, auto act, auto edge, auto put) {
+#pragma unroll
+            for (int i = 0; i < kGrp; i += 2) {
+                const int c0 = 8 * (pt + i * kParts), c1 = c0 + 8 * kParts;
+                if (c0 >= n_all) continue;
+                float z0[8], z1[8], r0[8], r1[8];
+                uint32_t o0[8], o1[8];
+                const bool ld0 = c0 < n_acc, ld1 = c1 < n_acc;
+                if (ld0) issue4(c0, z0, r0);
+                if (ld1) issue4(c1, z1, r1);
+                wait_ld16(z0, r0);
+                wait_ld16(z1, r1);
+#pragma unroll
+                for (int k = 0; k < 8; ++k) {
+                    z0[k] = fmaf(z0[k], share, fmaf(r0[k], kLoDown, z0[k]));
+                    z1[k] = fmaf(z1[k], share, fmaf(r1[k], kLoDown, z1[k]));
+                }
+                if (c1 + 8 <= n_fast) {
+                    act(c0, z0, o0);
+                    act(c1, z1, o1);
+                    put(i, c0, o0);
+                    put(i + 1, c1, o1);
+                } else {
+                    if (c0 + 8 <= n_fast) act(c0, z0, o0);
+                    else {
+                        if (!ld0) {
+#pragma unroll
+                            for (int k = 0; k < 8; ++k) z0[k] = 0.0f;
+                        }
+                        edge(c0, z0, o0);
+                    }
+                    put(i, c0, o0);
+                    if (c1 < n_all) {
+                        if (!ld1) {
+#pragma unroll
+                            for (int k = 0; k < 8; ++k) z1[k] = 0.0f;
+                        }
+                        edge(c1, z1, o1);
+                        put(i + 1, c1, o1);
+                    }
+                }
+            }
+        };
         ok = build_table(blockIdx.x);
         if (ok) write_input0();
-        for (int64_t tile = blockIdx.x; tile < n_tiles && ok; tile += gridDim.x) {
+        for (int64_t kt = 0; kt < mine && ok; ++kt) {
+            const int64_t tile = tile_of(kt);
+            const int slot = (int)(kt % kU);                        // of its unit
+            const bool unit_end = slot == kU - 1 || kt + 1 == mine;
             const float* bias = s_bias;
-            for (int L = 0; L < NLr && ok; bias += F::n_pad(L), ++L) {
+            for (int L = 0; L < (unit_end ? NLr : (NLr < LS ? NLr : LS)) && ok; bias += F::n_pad(L), ++L) {
                 // a single K step (the 3 raw coordinates and their one-hot derivatives) is exact or nearly so
                 const int n_mma = (F::k_main(L) + (L == LS ? F::kXp : 0)) / 16;
                 const float share = n_mma > 1 ? kBias0 + kBias1 * (float)n_mma : 0.0f;
@@ -571,8 +668,37 @@ __global__ void __launch_bounds__(kThr, 1) k_mlp_f32(F32Params p) {
                     float dot[4] = {0.0f, 0.0f, 0.0f, 0.0f};
                     const float sc = skip ? kRsqrt2 : 1.0f;
                     const uint32_t rh = row_at(a_hi, lane, Kn), rl = row_at(a_lo, lane, Kn);
-                    // accumulator sums z of operand columns c .. c + 7 -> both parts of the next operand
+                    // accumulator sums z of operand columns c .. c + 7 -> both parts of the next operand; the
+                    // scales are powers of two (but sc), so where they are applied changes no bit
                     auto act = [&](int c, const float (&z)[8], uint32_t (&o)[8]) {
+                        float v[8];
+                        const float2 b = *reinterpret_cast<const float2*>(bias + c + fc);
+#pragma unroll
+                        for (int e = 0; e < 2; ++e) {
+                            float h, sg;
+                            if constexpr (VALUE) {
+#pragma unroll
+                                for (int r = 0; r < 4; ++r) {
+                                    softplus_slope_f32(fmaf(z[2 * r + e], kDown, e ? b.y : b.x), p.beta, inv_beta, h, sg);
+                                    v[2 * r + e] = h * (sc * kUp);
+                                }
+                            } else {
+                                softplus_slope_f32(fmaf(z[e], kDown, e ? b.y : b.x), p.beta, inv_beta, h, sg);
+                                v[e] = h * (sc * kUp);
+                                sg *= sc * kUp * kDown;
+#pragma unroll
+                                for (int r = 1; r < 4; ++r) v[2 * r + e] = sg * z[2 * r + e];
+                            }
+                        }
+                        if (last) {
+                            const float2 w = *reinterpret_cast<const float2*>(s_w0 + c + fc);
+#pragma unroll
+                            for (int r = 0; r < 4; ++r) dot[r] = fmaf(v[2 * r + 1], w.y, fmaf(v[2 * r], w.x, dot[r]));
+                        }
+                        split4(v, o);
+                    };
+                    // some of the columns are beyond the outputs: the skip input's encoding, or padding
+                    auto edge = [&](int c, const float (&z)[8], uint32_t (&o)[8]) {
                         float v[8];
 #pragma unroll
                         for (int e = 0; e < 2; ++e) {
@@ -580,18 +706,15 @@ __global__ void __launch_bounds__(kThr, 1) k_mlp_f32(F32Params p) {
                             if (col < N) {
                                 const float b = bias[col];
                                 float h, sg;
-                                if constexpr (VALUE) {
 #pragma unroll
-                                    for (int r = 0; r < 4; ++r) {
-                                        softplus_slope_f32(fmaf(z[2 * r + e], kDown, b), p.beta, inv_beta, h, sg);
-                                        v[2 * r + e] = h * sc;
-                                    }
-                                } else {
-                                    softplus_slope_f32(fmaf(z[e], kDown, b), p.beta, inv_beta, h, sg);
-                                    v[e] = h * sc;
-                                    sg *= sc;
+                                for (int r = 0; r < (VALUE ? 4 : 1); ++r) {
+                                    softplus_slope_f32(fmaf(z[2 * r + e], kDown, b), p.beta, inv_beta, h, sg);
+                                    v[2 * r + e] = h * (sc * kUp);
+                                }
+                                if constexpr (!VALUE) {
+                                    sg *= sc * kUp * kDown;
 #pragma unroll
-                                    for (int r = 1; r < 4; ++r) v[2 * r + e] = sg * (z[2 * r + e] * kDown);
+                                    for (int r = 1; r < 4; ++r) v[2 * r + e] = sg * z[2 * r + e];
                                 }
                                 if (last) {
                                     const float w = s_w0[col];
@@ -599,44 +722,18 @@ __global__ void __launch_bounds__(kThr, 1) k_mlp_f32(F32Params p) {
                                     for (int r = 0; r < 4; ++r) dot[r] = fmaf(v[2 * r + e], w, dot[r]);
                                 }
                             } else {
-                                // beyond the outputs: the skip input's encoding, or padding
                                 const bool in = skip && col - N < A::kEnc;
 #pragma unroll
-                                for (int r = 0; r < 4; ++r) v[2 * r + e] = in ? enc(r, col - N) * sc : 0.0f;
+                                for (int r = 0; r < 4; ++r) v[2 * r + e] = in ? enc(r, col - N) * (sc * kUp) : 0.0f;
                             }
                         }
                         split4(v, o);
-                    };
-                    // a phase's groups of this part in turn, the next one's loads in flight: group i of
-                    // operand column n0 + c to use(i, c, parts); acc: the groups below it have accumulators
-                    auto groups = [&](int n0, int n_acc, int n_all, auto use) {
-                        float m[2][8], cr[2][8];
-                        if (8 * pt < n_acc) issue4(8 * pt, m[0], cr[0]);
-#pragma unroll
-                        for (int i = 0; i < kGrp; ++i) {
-                            const int c = 8 * (pt + i * kParts), cn = c + 8 * kParts;
-                            if (c >= n_all) continue;
-                            float z[8];
-                            if (c < n_acc) {
-                                wait_ld16(m[i & 1], cr[i & 1]);
-                                if (cn < n_acc) issue4(cn, m[(i + 1) & 1], cr[(i + 1) & 1]);
-#pragma unroll
-                                for (int k = 0; k < 8; ++k)
-                                    z[k] = fmaf(m[i & 1][k], share, fmaf(cr[i & 1][k], kLoDown, m[i & 1][k]));
-                            } else {
-#pragma unroll
-                                for (int k = 0; k < 8; ++k) z[k] = 0.0f;
-                            }
-                            uint32_t o[8];
-                            act(n0 + c, z, o);
-                            use(i, c, o);
-                        }
                     };
                     uint32_t held[kGrp][8];
                     const bool two = Np > kPh;
                     if (two) {
                         if (!wait_acc()) { ok = false; break; }
-                        groups(0, kPh, kPh, [&](int i, int, const uint32_t (&o)[8]) {
+                        groups(share, kPh, kPh, kPh, act, edge, [&](int i, int, const uint32_t (&o)[8]) {
 #pragma unroll
                             for (int k = 0; k < 8; ++k) held[i][k] = o[k];
                         });
@@ -650,9 +747,12 @@ __global__ void __launch_bounds__(kThr, 1) k_mlp_f32(F32Params p) {
                             if (pt + i * kParts < kPh / 8) store4(rh, rl, 8 * (pt + i * kParts), held[i]);
                         operand_done(0);
                     }
-                    groups(n0, Np - n0, Kn - n0, [&](int, int c, const uint32_t (&o)[8]) {
-                        if (store) store4(rh, rl, n0 + c, o);
-                    });
+                    groups(share, N - n0, Np - n0, Kn - n0,
+                           [&](int c, const float (&z)[8], uint32_t (&o)[8]) { act(n0 + c, z, o); },
+                           [&](int c, const float (&z)[8], uint32_t (&o)[8]) { edge(n0 + c, z, o); },
+                           [&](int, int c, const uint32_t (&o)[8]) {
+                               if (store) store4(rh, rl, n0 + c, o);
+                           });
                     drained();
                     if (store) operand_done(two ? 1 : 0);
                     if (last) {
@@ -660,7 +760,7 @@ __global__ void __launch_bounds__(kThr, 1) k_mlp_f32(F32Params p) {
                         for (int r = 0; r < 4; ++r) {
                             dot[r] += __shfl_xor_sync(0xffffffffu, dot[r], 1);
                             dot[r] += __shfl_xor_sync(0xffffffffu, dot[r], 2);
-                            if ((lane & 3) == 0) s_dot[pt * 128 + 32 * q + 8 * r + sq] = dot[r];
+                            if ((lane & 3) == 0) s_dot[pt * 128 + 32 * q + 8 * r + sq] = dot[r] * (1.0f / kUp);
                         }
                     }
                     if constexpr (VALUE) {
@@ -679,8 +779,8 @@ __global__ void __launch_bounds__(kThr, 1) k_mlp_f32(F32Params p) {
                                     if (tile * TS + 64 * k < total) p.f_out[tile * TS + 64 * k] = __uint_as_float(kRedoBits);
                                 atomicExch(p.redo, 1u);
                             }
-                            if (tile + gridDim.x < n_tiles) {
-                                if (!build_table(tile + gridDim.x)) { ok = false; break; }
+                            if (kt + 1 < mine) {
+                                if (!build_table(tile_of(kt + 1))) { ok = false; break; }
                                 write_input0();
                             }
                         }
@@ -689,19 +789,42 @@ __global__ void __launch_bounds__(kThr, 1) k_mlp_f32(F32Params p) {
                     // ---- SDF output: the features; net_0 and its gradient from their dot products ----
                     if constexpr (!VALUE) {
                         constexpr int NF = F::phases(LS - 1);
-                        uint32_t held[NF][kGrp][2];
+                        // value row sq of quarter q goes to row group `slot` of it; a warp's 8 rows x 8
+                        // columns are one core matrix, 128 bytes in lane order
+                        uint8_t* pf = park + (4 * q + slot) * (F::kFp / 8) * 128 + 4 * lane;
 #pragma unroll
                         for (int ph = 0; ph < NF; ++ph) {
                             if (!wait_acc()) { ok = false; break; }
+                            constexpr int kAt = kGrp / 2;   // groups whose loads are in flight together
 #pragma unroll
-                            for (int i = 0; i < kGrp; ++i) {
-                                const int c = 8 * (pt + i * kParts);
-                                if (c < F::phase_n(LS - 1, ph)) {
+                            for (int i0 = 0; i0 < kGrp; i0 += kAt) {
+                                float m[kAt][4], cr[kAt][4];
+#pragma unroll
+                                for (int i = 0; i < kAt; ++i) {
+                                    const int c = 8 * (pt + (i0 + i) * kParts);
+                                    if (c < F::phase_n(LS - 1, ph)) issue1(c, m[i], cr[i]);
+                                }
+#pragma unroll
+                                for (int i = 0; i < kAt; ++i)
+                                    asm volatile("tcgen05.wait::ld.sync.aligned;"
+                                                 : "+f"(m[i][0]), "+f"(m[i][1]), "+f"(cr[i][0]), "+f"(cr[i][1])
+                                                 :
+                                                 : "memory");
+#pragma unroll
+                                for (int i = 0; i < kAt; ++i) {
+                                    const int c = 8 * (pt + (i0 + i) * kParts);
+                                    if (c >= F::phase_n(LS - 1, ph)) continue;
                                     float z[2];
-                                    load1(c, share, z);
 #pragma unroll
-                                    for (int e = 0; e < 2; ++e) z[e] = fmaf(z[e], kDown, bias[ph * kPh + c + fc + e]);
-                                    split(z[0], z[1], held[ph][i][0], held[ph][i][1]);
+                                    for (int e = 0; e < 2; ++e) {
+                                        z[e] = fmaf(m[i][e], share, fmaf(cr[i][e], kLoDown, m[i][e]));
+                                        z[e] = fmaf(z[e], kDown, bias[ph * kPh + c + fc + e]) * kUp;
+                                    }
+                                    uint32_t hi, lo;
+                                    split(z[0], z[1], hi, lo);
+                                    uint32_t* at = reinterpret_cast<uint32_t*>(pf + (ph * kPh + c) / 8 * 128);
+                                    at[0] = hi;
+                                    at[F::kParkF / 4] = lo;
                                 }
                             }
                             drained();
@@ -718,32 +841,21 @@ __global__ void __launch_bounds__(kThr, 1) k_mlp_f32(F32Params p) {
                                 const float inv = gn > 0.0f ? 1.0f / gn : 0.0f;
                                 const float* sx = s_x + s * 8;
                                 float* so = s_out + s * 8;
-                                so[0] = f;
-                                so[1] = gx * sx[3] + gy * sx[4] + gz * sx[5];
-                                so[2] = sx[6];
-                                so[3] = sx[7];
-                                so[4] = gn;
-                                so[5] = gx * inv;
-                                so[6] = gy * inv;
-                                so[7] = gz * inv;
-                                const float inf = __int_as_float(0x7f800000);
-                                if ((!(gn >= kMinGrad && gn < inf) || !(fabsf(f) < inf)) && tile * TS + s < total) big = kHuge;
+                                so[0] = gx * inv;
+                                so[1] = gy * inv;
+                                so[2] = gz * inv;
+                                const int64_t g = tile * kTile + s;
+                                if (g < total) {
+                                    float4* R4 = reinterpret_cast<float4*>(p.rec + g);
+                                    R4[0] = make_float4(f, gx * sx[3] + gy * sx[4] + gz * sx[5], sx[6], sx[7]);
+                                    R4[2] = make_float4(so[0], so[1], so[2], 0.0f);
+                                    p.rec[g].gnorm = gn;
+                                    const float inf = __int_as_float(0x7f800000);
+                                    if (!(gn >= kMinGrad && gn < inf) || !(fabsf(f) < inf)) big = kHuge;
+                                }
                             }
                         }
                         if (!ok) break;
-                        // the features over the SDF operand's value rows
-                        const uint32_t vh = row_at(a_hi, lane & 7, F::kFp), vl = row_at(a_lo, lane & 7, F::kFp);
-#pragma unroll
-                        for (int ph = 0; ph < NF; ++ph)
-#pragma unroll
-                            for (int i = 0; i < kGrp; ++i) {
-                                const int c = 8 * (pt + i * kParts);
-                                if (c < F::phase_n(LS - 1, ph)) {
-                                    const uint32_t co = (uint32_t)((ph * kPh + c) >> 3) * 128u;
-                                    stmat1(vh + co, held[ph][i][0]);
-                                    stmat1(vl + co, held[ph][i][1]);
-                                }
-                            }
                         if (!epi_sync()) { ok = false; break; }
                         // x~, direction encoding, unit normal: one 8-column group of a sample per thread
                         if (et < kTile * (F::kXp / 8)) {
@@ -759,107 +871,125 @@ __global__ void __launch_bounds__(kThr, 1) k_mlp_f32(F32Params p) {
                                     if (j < 3) v[e] = s_x[s * 8 + j];
                                     else if (j < 3 + A::kDirEnc)
                                         v[e] = enc_tab(s_x + s * 8 + 3, s_pd + s * A::kPeDir * 6, A::kPeDir, j - 3, 0);
-                                    else if (j < F::kX) v[e] = s_out[s * 8 + 5 + j - 3 - A::kDirEnc];
+                                    else if (j < F::kX) v[e] = s_out[s * 8 + j - 3 - A::kDirEnc];
                                 }
-                                split(v[0], v[1], o[k], o[4 + k]);
+                                split(v[0] * kUp, v[1] * kUp, o[k], o[4 + k]);
                             }
-                            // row s of the value rows, one row group below
-                            const uint32_t at = a_off(32 * (s >> 3) + 8 + (s & 7), c, F::kFp);
-                            *reinterpret_cast<uint4*>(a_hi + at) = make_uint4(o[0], o[1], o[2], o[3]);
-                            *reinterpret_cast<uint4*>(a_lo + at) = make_uint4(o[4], o[5], o[6], o[7]);
+                            uint8_t* at = park + 2 * F::kParkF + a_off(32 * (s >> 3) + 8 * slot + (s & 7), c, F::kXp);
+                            *reinterpret_cast<uint4*>(at) = make_uint4(o[0], o[1], o[2], o[3]);
+                            *reinterpret_cast<uint4*>(at + F::kParkX) = make_uint4(o[4], o[5], o[6], o[7]);
                         }
-                        operand_done(0);
-                        if (F::kFp > kPh) operand_done(1);
-                        // this tile's table is read no more: the next tile's, while the colour layers run
+                        fence_async_global();
+                        __syncwarp();
+                        if (unit_end && lane == 0) mbar_arrive(bar_park);
                         if (!epi_sync()) { ok = false; break; }
-                        if (tile + gridDim.x < n_tiles && !build_table(tile + gridDim.x)) { ok = false; break; }
+                        if (unit_end && et == 0) {
+                            // the unit's features as the operand (the SDF MMAs are complete)
+                            fence_async_global();
+                            mbar_expect_tx(bar_back, 2 * F::kParkF);
+                            ++backs;
+                            bulk_g2s(smem_u32(a_hi), park, F::kParkF, bar_back);
+                            bulk_g2s(smem_u32(a_lo), park + F::kParkF, F::kParkF, bar_back);
+                        }
+                        // this tile's table is read no more: the next tile's (while the colour layers run, at
+                        // a unit's end)
+                        if (kt + 1 < mine && !build_table(tile_of(kt + 1))) { ok = false; break; }
+                        if (!unit_end) write_input0();
                     }
                 } else {
-                    // ---- hidden colour layer: ReLU on the value rows ----
-                    const int Kn = F::n_pad(L);
+                    // ---- hidden colour layer: ReLU, all rows (row group j: tile j of the unit) ----
+                    const int Np = F::n_pad(L);
                     const bool last = L == F::NL - 2;          // the colours' dot products are taken here
-                    const uint32_t vh = row_at(a_hi, lane & 7, Kn), vl = row_at(a_lo, lane & 7, Kn);
-                    constexpr int NP = 2;
-                    uint32_t held[NP][kGrp][2];
-                    float cd[3] = {0.0f, 0.0f, 0.0f};
-                    const int nph = F::phases(L);
+                    const uint32_t rh = row_at(a_hi, lane, Np), rl = row_at(a_lo, lane, Np);
+                    float cd[3][4] = {};
+                    auto act = [&](int c, const float (&z)[8], uint32_t (&o)[8]) {
+                        float v[8];
+                        const float2 b = *reinterpret_cast<const float2*>(bias + c + fc);
 #pragma unroll
-                    for (int ph = 0; ph < NP; ++ph) {
-                        if (ph >= nph) continue;
-                        if (!wait_acc()) { ok = false; break; }
-#pragma unroll
-                        for (int i = 0; i < kGrp; ++i) {
-                            const int c = 8 * (pt + i * kParts);
-                            if (c < F::phase_n(L, ph)) {
-                                float z[2];
-                                load1(c, share, z);
-#pragma unroll
-                                for (int e = 0; e < 2; ++e) {
-                                    const int col = ph * kPh + c + fc + e;
-                                    z[e] = relu_nan(fmaf(z[e], kDown, bias[col]));
-                                    if (last) {
-#pragma unroll
-                                        for (int k = 0; k < 3; ++k) cd[k] = fmaf(z[e], s_wc[k * F::kWc + col], cd[k]);
-                                    }
-                                }
-                                split(z[0], z[1], held[ph][i][0], held[ph][i][1]);
-                            }
+                        for (int r = 0; r < 4; ++r) {
+                            v[2 * r] = relu_nan(fmaf(z[2 * r], kDown * kUp, b.x * kUp));
+                            v[2 * r + 1] = relu_nan(fmaf(z[2 * r + 1], kDown * kUp, b.y * kUp));
+                            // rows of tiles the unit does not have are nobody's
+                            if (r > slot) v[2 * r] = v[2 * r + 1] = 0.0f;
                         }
+                        if (last) {
+#pragma unroll
+                            for (int k = 0; k < 3; ++k) {
+                                const float2 w = *reinterpret_cast<const float2*>(s_wc + k * F::kWc + c + fc);
+#pragma unroll
+                                for (int r = 0; r < 4; ++r) cd[k][r] = fmaf(v[2 * r + 1], w.y, fmaf(v[2 * r], w.x, cd[k][r]));
+                            }
+                        } else {
+                            split4(v, o);
+                        }
+                    };
+                    uint32_t held[kGrp][8];
+                    const bool two = Np > kPh;
+                    if (two) {
+                        if (!wait_acc()) { ok = false; break; }
+                        groups(share, kPh, kPh, kPh, act, act, [&](int i, int, const uint32_t (&o)[8]) {
+#pragma unroll
+                            for (int k = 0; k < 8; ++k) held[i][k] = o[k];
+                        });
                         drained();
                     }
-                    if (!ok) break;
-                    if (!last) {
+                    if (!wait_acc()) { ok = false; break; }
+                    const int n0 = two ? kPh : 0;
+                    if (two && !last) {
 #pragma unroll
-                        for (int ph = 0; ph < NP; ++ph)
-#pragma unroll
-                            for (int i = 0; i < kGrp; ++i) {
-                                const int c = 8 * (pt + i * kParts);
-                                if (ph < nph && c < F::phase_n(L, ph)) {
-                                    const uint32_t co = (uint32_t)((ph * kPh + c) >> 3) * 128u;
-                                    stmat1(vh + co, held[ph][i][0]);
-                                    stmat1(vl + co, held[ph][i][1]);
-                                }
-                            }
+                        for (int i = 0; i < kGrp; ++i)
+                            if (pt + i * kParts < kPh / 8) store4(rh, rl, 8 * (pt + i * kParts), held[i]);
                         operand_done(0);
-                        if (Kn > kPh) operand_done(1);
+                    }
+                    auto rest = [&](int c, const float (&z)[8], uint32_t (&o)[8]) { act(n0 + c, z, o); };
+                    groups(share, Np - n0, Np - n0, Np - n0, rest, rest, [&](int, int c, const uint32_t (&o)[8]) {
+                        if (!last) store4(rh, rl, n0 + c, o);
+                    });
+                    drained();
+                    if (!last) {
+                        operand_done(two ? 1 : 0);
                         continue;
                     }
-                    // ---- the next tile's layer-0 input (every MMA of this one is complete), the records ----
+                    // ---- the next unit's first layer-0 input (every MMA of this one is complete), the colours ----
 #pragma unroll
-                    for (int k = 0; k < 3; ++k) {
-                        cd[k] += __shfl_xor_sync(0xffffffffu, cd[k], 1);
-                        cd[k] += __shfl_xor_sync(0xffffffffu, cd[k], 2);
-                        if ((lane & 3) == 0) s_cdot[(pt * 3 + k) * kTile + 8 * q + sq] = cd[k];
-                    }
+                    for (int k = 0; k < 3; ++k)
+#pragma unroll
+                        for (int r = 0; r < 4; ++r) {
+                            cd[k][r] += __shfl_xor_sync(0xffffffffu, cd[k][r], 1);
+                            cd[k][r] += __shfl_xor_sync(0xffffffffu, cd[k][r], 2);
+                            if ((lane & 3) == 0) s_cdot[(pt * 3 + k) * 128 + 32 * q + 8 * r + sq] = cd[k][r] * (1.0f / kUp);
+                        }
                     if (out_of_range() && lane == 0) *s_mark = (uint32_t)(tile + 1);
                     if (!epi_sync()) { ok = false; break; }
-                    if (tile + gridDim.x < n_tiles) write_input0();
-                    if (et < kTile) {
+                    if (kt + 1 < mine) write_input0();
+                    if (et < 128) {
                         const float* bc = p.rgb_w + F::param_offset(F::NL - 1) + 3 * F::layer(F::NL - 1).in;
-                        float c3[3];
-                        bool bad = *s_mark == (uint32_t)(tile + 1);
+                        const int j = (et >> 3) & 3;                       // tile of the unit
+                        const int64_t g = tile_of(kt - slot + j) * kTile + 8 * (et >> 5) + (et & 7);
+                        if (j <= slot && g < total) {
+                            bool bad = false;
+                            float* R = reinterpret_cast<float*>(p.rec + g);
 #pragma unroll
-                        for (int k = 0; k < 3; ++k) {
-                            c3[k] = s_cdot[k * kTile + et] + s_cdot[(3 + k) * kTile + et] + s_cdot[(6 + k) * kTile + et] + __ldg(bc + k);
-                            bad = bad || !(fabsf(c3[k]) < __int_as_float(0x7f800000));
+                            for (int k = 0; k < 3; ++k) {
+                                const float* sd = s_cdot + k * 128 + et;
+                                const float c3 = sd[0] + sd[3 * 128] + sd[6 * 128] + __ldg(bc + k);
+                                bad = bad || !(fabsf(c3) < __int_as_float(0x7f800000));
+                                R[4 + k] = 1.0f / (1.0f + expf(-c3));
+                            }
+                            if (bad || (*s_mark == (uint32_t)(tile + 1) && (g % 16) == 0)) {
+                                p.rec[g / 16 * 16].pad = 1.0f;
+                                atomicExch(p.redo, 1u);
+                            }
                         }
-                        const bool mark = __any_sync(0xffffffffu, bad) != 0;
-                        const int64_t g = tile * kTile + et;
-                        const float4* so = reinterpret_cast<const float4*>(s_out + et * 8);
-                        const float4 s0 = so[0], s1 = so[1];
-                        if (g < total) {
-                            float4* R4 = reinterpret_cast<float4*>(p.rec + g);
-                            R4[0] = s0;
-                            R4[1] = make_float4(1.0f / (1.0f + expf(-c3[0])), 1.0f / (1.0f + expf(-c3[1])),
-                                                1.0f / (1.0f + expf(-c3[2])), s1.x);
-                            R4[2] = make_float4(s1.y, s1.z, s1.w, mark && (g % 16) == 0 ? 1.0f : 0.0f);
-                        }
-                        if (mark && et == 0) atomicExch(p.redo, 1u);
                     }
                 }
             }
         }
         if (!ok) set_status(p.status, TSDFS_DEV_TIMEOUT);
+        if (!ok && backs > 0) {   // this thread's copies may be in flight
+            for (uint32_t it = 0; it < kMaxSpin && !mbar_try(bar_back, (backs - 1) & 1u); ++it) {
+            }
+        }
     }
     tc_fence_before();
     __syncthreads();
@@ -908,7 +1038,7 @@ __global__ void k_split_weights(const float* __restrict__ sdf_w, const float* __
                 const int col = F::src_col(L, k_first + 8 * k8 + 2 * j + e);
                 v[e] = row >= 0 && col >= 0 ? __ldg(W + (int64_t)row * ly.in + col) : 0.0f;
             }
-            split_f32(v[0], v[1], o[j], o[4 + j]);
+            split_f32(v[0] * kUp, v[1] * kUp, o[j], o[4 + j]);
         }
         // the item's hi image starts after the phases and chunks before it
         uint8_t* item = packed + F::layer_base(L) + (int64_t)n_first * kt * 32 + (int64_t)n_ph * (k_first / 8) * 32;
@@ -941,6 +1071,7 @@ int launch_f32(const tsdfs_mlp* m, const SampleSource& src, SampleRec* rec, floa
     }
     F32Params p{};
     p.packed = stash + kRedoBytes;
+    p.park = stash + kRedoBytes + F::packed_bytes();
     p.redo = reinterpret_cast<uint32_t*>(stash);
     p.sdf_w = m->sdf_w;
     p.rgb_w = m->rgb_w;
@@ -956,6 +1087,7 @@ int launch_f32(const tsdfs_mlp* m, const SampleSource& src, SampleRec* rec, floa
     p.withhold = test_withhold_chunk();
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const int64_t ts = VALUE ? kTileV : kTile, tiles = (max_samples + ts - 1) / ts;
+    if (sms > kMaxCtas) sms = kMaxCtas;
     const unsigned blocks = (unsigned)(tiles < sms ? (tiles < 1 ? 1 : tiles) : sms);
     k_split_weights<ARCH><<<grid_1d(F::packed_bytes() / 32, 256), 256, 0, st>>>(m->sdf_w, m->rgb_w,
                                                                                stash + kRedoBytes, p.redo);
@@ -965,7 +1097,10 @@ int launch_f32(const tsdfs_mlp* m, const SampleSource& src, SampleRec* rec, floa
 
 }  // namespace
 
-size_t mlp_f32_stash_bytes() { return kRedoBytes + (size_t)FArch<TSDFS_ARCH_ROOM>::packed_bytes(); }
+size_t mlp_f32_stash_bytes() {
+    using F = FArch<TSDFS_ARCH_ROOM>;
+    return kRedoBytes + (size_t)F::packed_bytes() + kMaxCtas * F::park_bytes();
+}
 
 int launch_mlp_full_f32(const tsdfs_mlp* m, const SampleSource& src, SampleRec* rec, int64_t max_samples,
                         uint8_t* stash, cudaStream_t st) {

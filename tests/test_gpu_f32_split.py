@@ -122,3 +122,19 @@ def test_coarse_pass(scene, n_rays, big):
     compare(got, {k: ref[k].detach().numpy() for k in got}, depth_rel=DEPTH_REL_F32)
     rc, bits = T.tsdfs_sync_status()
     assert rc == 0, bits
+
+
+@pytest.mark.parametrize("scene", ["tiny", "room"])
+@pytest.mark.parametrize("counts,huge", [([64] * 304, False), ([64] * 304 + [33], False), ([50] * 250, True)],
+                         ids=["full", "one-over", "marked"])
+def test_colour_layers_over_several_tiles(scene, counts, huge):
+    """Totals at which a CTA's colour layers take four tiles, four and one, and three with marks."""
+    o, d, b = rays(scene, counts, seed=63)
+    spec = spec_of(scene)
+    if huge:
+        spec = scaled(spec, "rgb", 1, 4e5, True)
+    got = gpu_render(spec, o, d, b)
+    ref, _ = oracle_render(spec, o, d, b)
+    compare(got, ref, depth_rel=DEPTH_REL_F32)
+    rc, bits = T.tsdfs_sync_status()
+    assert rc == 0, bits
