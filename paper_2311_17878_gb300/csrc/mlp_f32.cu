@@ -2,9 +2,12 @@
 //
 // An FP32 operand x is carried as hi = fp16(32 x) and lo = fp16(2048 (32 x - hi)): 22
 // significant bits over |x| from 2e-6 to 2047, and an absolute floor of 5e-13 below that (lo is
-// stored scaled, so it stays normal while hi is).  A product sum takes three MMAs per K step,
+// stored scaled, so it stays normal while hi is).  A product sum takes three products per K step,
 // hi hi' into a main accumulator and lo hi' + hi lo' into a correction accumulator that is
-// scaled back by 2^-11 when it is read (lo lo' is below 2^-22 of the product).  Everything
+// scaled back by 2^-11 when it is read (lo lo' is below 2^-22 of the product).  Main and correction
+// columns adjoin in TMEM and hi' and lo' rows in shared memory, so hi hi' and hi lo' are one MMA of
+// twice the outputs: the hi operand is read once for both (20 instead of 24 KB of shared memory per K
+// step; at 128 bytes a cycle the three MMAs alone took what the tensor cores need for them).  Everything
 // between the products is FP32.
 //
 // tcgen05 truncates when it adds into its FP32 accumulator, so the main sum comes out too small
@@ -19,7 +22,7 @@
 // Tile: 32 samples = 128 operand rows; TMEM lane quarter q holds samples 8q..8q+7 in four groups
 // of 8 lanes (value, d/dx, d/dy, d/dz rows: forward-mode gradient).  Two parts of 128 x 256
 // operands take 128 KB of shared memory.  A layer runs in phases of at most 128 outputs, each
-// into one of two buffers of TMEM (main and correction, 128 columns each), so the epilogue of a
+// into one of two buffers of TMEM (main and correction, up to 128 columns each), so the epilogue of a
 // phase runs beside the MMAs of the next.  A layer's operand can be replaced only after its last
 // MMA: the first phase's activations wait in registers (as packed parts), are stored when the
 // second phase is through, and the next layer starts on those 128 columns while the second
@@ -37,7 +40,9 @@
 // the other columns through the weight ring as an item of their own before their weights.  (One
 // tile at a time the colour layers were 38 of a tile's 96 items.)  61 915 samples of the room
 // networks: SIMT kernel 13.8 ms, this one with the colour layers per tile 1.20 ms, per unit 1.10 ms,
-// and with the epilogue's groups two at a time 1.03 ms.
+// with the epilogue's groups two at a time 1.03 ms, one MMA for hi hi' and hi lo' 1.00 ms, and an
+// item's MMAs as straight code 0.95 ms.  Of a tile's 145 k cycles the epilogue works for 86 k and
+// the MMAs take 53 k at the tensor cores' rate; a layer's two phases overlap them in part.
 //
 // VALUE: the samplers' coarse pass (SDF value only): 128 samples per tile, one row each, no
 // gradient and no colour network.
@@ -171,7 +176,8 @@ struct __align__(16) Item {
     uint32_t b_sbo;
     uint32_t idesc;
     uint16_t steps;    // K steps of 16
-    uint16_t pad[2];
+    uint16_t n;        // outputs
+    uint16_t pad;
     uint16_t edge;     // bit 0: first item of a phase, bit 1: last, bit 2 / 3: its operand's columns below /
                        // from 128 are awaited first, bit 4: the parked features are, bit 5: an operand item
                        // (parked columns, no MMAs), bit 6: its operand is the item before
@@ -303,7 +309,8 @@ __global__ void __launch_bounds__(kThr, 1) k_mlp_f32(F32Params p) {
                 it.b_sbo = (uint32_t)(kc / 8) * 128u;
                 it.idesc = idesc_mma<true>(128, n);
                 it.steps = (uint16_t)(kc / 16);
-                it.pad[0] = it.pad[1] = 0;
+                it.n = (uint16_t)n;
+                it.pad = 0;
                 const bool back = L == LS && ph == 0 && c == 0;
                 it.edge = (uint16_t)((c == 0 ? 1 : 0) | (c + 1 == F::chunks(L) ? 2 : 0) | (L != LS && ph == 0 && c == 0 ? 4 : 0) |
                                      (L != LS && ph == 0 && c * kKChunk == kPh ? 8 : 0) | (back ? 16 : 0) | (extra ? 64 : 0));
@@ -416,22 +423,20 @@ __global__ void __launch_bounds__(kThr, 1) k_mlp_f32(F32Params p) {
                 if (!wait(bar_full + 8 * stage, (g >> 1) & 1u)) return false;
                 tc_fence_after();
                 const uint32_t b = r0 + stage * kStageBytes;
-                uint64_t bh = mdesc(b, 128, it.b_sbo), bl = mdesc(b + it.bytes, 128, it.b_sbo);
+                uint64_t bh = mdesc(b, 128, it.b_sbo);
                 const uint32_t ax = r0 + (stage ^ 1u) * kStageBytes;
                 uint64_t ah = mdesc(it.edge & 64u ? ax : ah0 + it.a, 128, it.a_sbo);
                 uint64_t al = mdesc(it.edge & 64u ? ax + F::kParkX : al0 + it.a, 128, it.a_sbo);
-                const uint32_t d_main = tmem + (ph & 1u) * (2 * kPh), d_corr = d_main + kPh;
-                uint32_t acc = it.edge & 1u ? 0u : 1u;
-                for (int k = 0; k < it.steps; ++k) {
-                    mma_el(el, d_corr, al, bh, it.idesc, acc);
-                    mma_el(el, d_main, ah, bh, it.idesc, acc);
-                    mma_el(el, d_corr, ah, bl, it.idesc, 1u);
-                    acc = 1u;
-                    ah += 16;
-                    al += 16;
-                    bh += 16;
-                    bl += 16;
-                }
+                const uint32_t d_main = tmem + (ph & 1u) * (2 * kPh), d_corr = d_main + it.n;
+                const uint32_t idesc2 = idesc_mma<true>(128, 2 * it.n);   // both parts of the weights
+                const uint32_t acc = it.edge & 1u ? 0u : 1u;
+                auto step = [&](int k) {
+                    mma_el(el, d_main, ah + 16 * k, bh + 16 * k, idesc2, k > 0 ? 1u : acc);
+                    mma_el(el, d_corr, al + 16 * k, bh + 16 * k, it.idesc, 1u);
+                };
+                if (it.steps == kKChunk / 16) static_for<0, kKChunk / 16>([&](auto k) { step(decltype(k)::value); });
+                else
+                    for (int k = 0; k < it.steps; ++k) step(k);
                 if (it.edge & 64u) commit_el(el, bar_empty + 8 * (stage ^ 1u));
                 commit_el(el, bar_empty + 8 * stage);
                 if (it.edge & 2u) commit_el(el, bar_acc + 8 * (ph++ & 1u));
@@ -457,7 +462,7 @@ __global__ void __launch_bounds__(kThr, 1) k_mlp_f32(F32Params p) {
         const float b0 = __ldg(p.sdf_w + F::param_offset(LS - 1) + (int64_t)F::layer(LS - 1).out * F::layer(LS - 1).in);
         const int et = threadIdx.x;
         uint32_t phs = 0, epi_ph = 0, backs = 0;   // phases waited for, epilogue barriers, units fetched back
-        uint32_t buf = 0;                         // TMEM column of the phase in hand
+        uint32_t buf = 0, cor = 0;                // TMEM columns of the phase in hand: main, correction
         __half2 big = __float2half2_rn(0.0f);     // largest |operand| (scaled high parts) of this thread, or NaN
         const __half2 kHuge = __float2half2_rn(65504.0f);
         bool ok = true;
@@ -468,11 +473,12 @@ __global__ void __launch_bounds__(kThr, 1) k_mlp_f32(F32Params p) {
             ++epi_ph;
             return __all_sync(0xffffffffu, w);
         };
-        auto wait_acc = [&]() -> bool {
+        auto wait_acc = [&](int n) -> bool {       // n: the phase's outputs
             const uint32_t b = phs & 1u;
             const bool w = __all_sync(0xffffffffu, mbar_wait(bar_acc + 8 * b, (phs >> 1) & 1u, abort_flag, p.spin));
             ++phs;
             buf = tmem + b * (2 * kPh);
+            cor = buf + n;
             tc_fence_after();
             return w;
         };
@@ -493,13 +499,13 @@ __global__ void __launch_bounds__(kThr, 1) k_mlp_f32(F32Params p) {
         auto issue4 = [&](int c, float (&m)[8], float (&cr)[8]) {
             tmem_ld16x256_x1(buf + lq + c, m);
             tmem_ld16x256_x1(buf + lq16 + c, m + 4);
-            tmem_ld16x256_x1(buf + lq + kPh + c, cr);
-            tmem_ld16x256_x1(buf + lq16 + kPh + c, cr + 4);
+            tmem_ld16x256_x1(cor + lq + c, cr);
+            tmem_ld16x256_x1(cor + lq16 + c, cr + 4);
         };
         // rows 0-15 only: the value rows' registers are 0 and 1
         auto issue1 = [&](int c, float (&m)[4], float (&cr)[4]) {
             tmem_ld16x256_x1(buf + lq + c, m);
-            tmem_ld16x256_x1(buf + lq + kPh + c, cr);
+            tmem_ld16x256_x1(cor + lq + c, cr);
         };
         // row i of the lane quarter (stmatrix: lane i addresses row i) at column 0
         auto row_at = [&](uint8_t* base, int r, int pitch) { return smem_u32(base) + a_off(32 * q + r, 0, pitch); };
@@ -732,15 +738,15 @@ __global__ void __launch_bounds__(kThr, 1) k_mlp_f32(F32Params p) {
                     uint32_t held[kGrp][8];
                     const bool two = Np > kPh;
                     if (two) {
-                        if (!wait_acc()) { ok = false; break; }
+                        if (!wait_acc(kPh)) { ok = false; break; }
                         groups(share, kPh, kPh, kPh, act, edge, [&](int i, int, const uint32_t (&o)[8]) {
 #pragma unroll
                             for (int k = 0; k < 8; ++k) held[i][k] = o[k];
                         });
                         drained();
                     }
-                    if (!wait_acc()) { ok = false; break; }
                     const int n0 = two ? kPh : 0;
+                    if (!wait_acc(Np - n0)) { ok = false; break; }
                     if (two && store) {
 #pragma unroll
                         for (int i = 0; i < kGrp; ++i)
@@ -794,7 +800,7 @@ __global__ void __launch_bounds__(kThr, 1) k_mlp_f32(F32Params p) {
                         uint8_t* pf = park + (4 * q + slot) * (F::kFp / 8) * 128 + 4 * lane;
 #pragma unroll
                         for (int ph = 0; ph < NF; ++ph) {
-                            if (!wait_acc()) { ok = false; break; }
+                            if (!wait_acc(F::phase_n(LS - 1, ph))) { ok = false; break; }
                             constexpr int kAt = kGrp / 2;   // groups whose loads are in flight together
 #pragma unroll
                             for (int i0 = 0; i0 < kGrp; i0 += kAt) {
@@ -926,15 +932,15 @@ __global__ void __launch_bounds__(kThr, 1) k_mlp_f32(F32Params p) {
                     uint32_t held[kGrp][8];
                     const bool two = Np > kPh;
                     if (two) {
-                        if (!wait_acc()) { ok = false; break; }
+                        if (!wait_acc(kPh)) { ok = false; break; }
                         groups(share, kPh, kPh, kPh, act, act, [&](int i, int, const uint32_t (&o)[8]) {
 #pragma unroll
                             for (int k = 0; k < 8; ++k) held[i][k] = o[k];
                         });
                         drained();
                     }
-                    if (!wait_acc()) { ok = false; break; }
                     const int n0 = two ? kPh : 0;
+                    if (!wait_acc(Np - n0)) { ok = false; break; }
                     if (two && !last) {
 #pragma unroll
                         for (int i = 0; i < kGrp; ++i)
