@@ -186,7 +186,8 @@ int launch_mlp_full_tc(const tsdfs_mlp* mlp, const SampleSource& src, SampleRec*
                        uint8_t* stash, cudaStream_t st);
 size_t mlp_tc_stash_bytes();
 int launch_mlp_value_tc(const tsdfs_mlp* mlp, const SampleSource& src, float* f_out, cudaStream_t st);
-int launch_mlp_pipe(const tsdfs_mlp* mlp, const SampleSource& src, SampleRec* rec, int64_t max_samples,
+size_t mlp_pipe_stash_bytes();
+int launch_mlp_pipe(const tsdfs_mlp* mlp, const SampleSource& src, SampleRec* rec, int64_t max_samples, uint8_t* stash,
                     cudaStream_t st);
 
 // network kernel per precision (tsdfs_set_network_kernel), index = TSDFS_PREC_*
@@ -231,11 +232,11 @@ static NetParams net_params(const tsdfs_mlp* m) {
     return np;
 }
 
-// scratch of the network kernels in the caller's workspace (256-byte aligned): the serial
-// kernel's parking space, or the single-precision path's redo word and split weights
+// scratch of the network kernels in the caller's workspace (256-byte aligned): the kernels'
+// parking space, the single-precision path's redo word and split weights
 static size_t stash_bytes() {
-    const size_t a = mlp_tc_stash_bytes(), b = mlp_f32_stash_bytes();
-    return a > b ? a : b;
+    const size_t a = mlp_tc_stash_bytes(), b = mlp_f32_stash_bytes(), c = mlp_pipe_stash_bytes();
+    return a > b ? (a > c ? a : c) : (b > c ? b : c);
 }
 
 // the network evaluation of every render path
@@ -244,7 +245,7 @@ static int run_full_mlp(const tsdfs_mlp* m, const SampleSource& src, SampleRec* 
     if (m->precision != TSDFS_PREC_F32) {
         if (netkernel_of(m->precision) == TSDFS_NETKERNEL_PIPELINED) {
             ProfScope ps("mlp_pipe", st);
-            return launch_mlp_pipe(m, src, rec, max_samples, st);
+            return launch_mlp_pipe(m, src, rec, max_samples, stash, st);
         }
         ProfScope ps("mlp_tc", st);
         return launch_mlp_full_tc(m, src, rec, max_samples, stash, st);

@@ -45,7 +45,8 @@ __global__ void k_grid_init(void* V, int f16, uint8_t* W, int64_t n) {
 //    mean is 1 keeps it.
 // The camera table of all views is staged in shared memory once per block (20 floats per view:
 // c2w[12], fx, fy, cx, cy and what the tests use), the list of the brick's views after it.  256^3
-// voxels, 100 views of the room: 2816 us without any of it, 950 with bricks of 32 x 4 x 4 alone.
+// voxels, 100 views of the room: 2816 us without any of it, 950 with bricks of 32 x 4 x 4, 844 as it
+// is; what is left is the ~40 instructions of a voxel-view and the divisions near the surface.
 constexpr int kBX = 8, kBY = 8, kBZ = 8;
 constexpr int kBrickVoxels = kBX * kBY * kBZ;
 constexpr int kCam = 20;
@@ -204,7 +205,7 @@ __global__ void __launch_bounds__(kFuseBlock) k_integrate(int nx, int ny, int nz
 // neighbour words' bits), the y and z erosions ANDs of whole words.  A block takes kMW words x
 // kMY x kMZ rows with a halo of r rows (and, at a tile's end inside the grid, one word); the volume is
 // read once from memory, the halo (1.9 x at r = 2) from L2.  Bound: the instructions of those reads.
-// 256^3 FP32, r = 2: 592 us as a running maximum of values over shared-memory tiles.  A NaN voxel
+// 256^3 FP32, r = 2: 592 us as a running maximum of values over shared-memory tiles, 37 us so.  A NaN voxel
 // counts as negative unless its whole neighbourhood is NaN (a maximum of the values ignores a NaN):
 // a tile that has one goes through its neighbourhoods again.  Rows that are no multiple of 32 voxels
 // long put their words into the bit array with two atomic ORs each.
@@ -318,7 +319,8 @@ __global__ void __launch_bounds__(kMThreads) k_inside_mask(const void* __restric
 // for each.  Nearly all of them are in free space, where s / D_T is exactly 1: so the sum is kept
 // as what is missing to the count, 2^32 - s / D_T 2^32, which is 0 there and needs no atomic.  And
 // rays of neighbouring pixels cross the same voxels in step: a warp takes 8 x 4 pixels, and
-// lanes in one voxel at the same step add their counts with one atomic.
+// lanes in one voxel at the same step add their counts with one atomic.  144 us a view so; what is
+// left is the walk.
 constexpr double kFix = 4294967296.0;   // 2^32
 constexpr int kRayW = 8, kRayH = 4;     // pixels of a warp
 

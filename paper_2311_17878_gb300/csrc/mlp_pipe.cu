@@ -23,6 +23,14 @@
 // hidden layer's activations with its weight row, accumulated by the epilogue
 // that writes those activations.
 //
+// The colour layers need the value rows only, a quarter of a tile's.  So they run once for up to
+// kPUnit tiles, on all 128 rows: each tile's colour input is parked in global memory (L2) in
+// operand layout, tile j in row group j of every lane quarter, and bulk copies bring the unit's back
+// as the operand.  A unit of one tile (few samples, or a CTA's last) stays in shared memory, and its
+// colour layers start block by block behind the output layer's epilogue.  Room networks, split
+// operands, the chunk of a 160 x 120 view: 1494 us with the colour layers per tile, 1344 us per unit,
+// 1313 us with a 64-column chunk's MMAs as straight code; the results are the same bits.
+//
 // Warps 0-11 are the epilogue (warp w: TMEM lane quarter w % 4, column part
 // w / 4; parts take the 8-column groups g with g % 3 == part, so every 64-column
 // block fills at the same pace), warp 12 allocates TMEM and issues the MMAs
@@ -45,6 +53,8 @@ constexpr int kPMaxBlocks = 5;        // 64-column operand blocks of the widest 
 constexpr uint32_t kPABytes = 64 * 1024;        // 128 rows x 256 16-bit columns
 constexpr uint32_t kPXMax = 128 * 64 * 2;       // the colour input beyond column 256 (<= 64 columns)
 constexpr uint32_t kPBarBytes = 256;
+constexpr int kPUnit = 4;             // tiles per pass of the colour layers
+constexpr int kPMaxCtas = 192;        // CTAs with a place to park
 constexpr int kPBatch = 4;            // 8-column groups an epilogue thread loads and computes together
 
 template <int MODE> struct PipeMode {
@@ -77,7 +87,16 @@ template <int ARCH> struct PipeArch : TcArch<ARCH> {
     __host__ __device__ static constexpr uint32_t table_bytes() {
         return (uint32_t)(kPTile * (8 + 6 * (A::kPeSdf + A::kPeDir)) * 4);
     }
-    // per-sample outputs kept for the record (8 floats), col 0 of the output rows (4 floats),
+    // a unit's parked colour input: the operand's main columns, then those beyond column 256
+    static constexpr uint32_t kParkMain = 16u * (uint32_t)(pitch_main(LS) / 8) * 128u;
+    static constexpr uint32_t kParkX = 16u * (uint32_t)(kPitchX / 8) * 128u;
+    // sums over the SDF layers' chunks only
+    __host__ __device__ static constexpr int sdf_chunks() {
+        int n = 0;
+        for (int l = 0; l < LS; ++l) n += TcArch<ARCH>::chunks(l);
+        return n;
+    }
+    // the unit normal of each sample (8 floats), col 0 of the output rows (4 floats),
     // the partial dot products of the extra column (3 parts) and its weight row
     __host__ __device__ static constexpr uint32_t scratch_bytes() {
         return (uint32_t)((kPTile * 8 + 128 + kPParts * kPTile + (kExtraCol ? 256 : 0)) * 4);
@@ -112,6 +131,7 @@ struct PipeParams {
     SampleRec* rec;
     uint32_t* status;
     uint32_t spin;   // polls of a bounded wait before it gives up
+    uint8_t* park;   // kParkMain + kParkX bytes per CTA
     int withhold;    // test-only: weight chunk of the first tile whose copy is never issued (-1: none)
 };
 
@@ -129,6 +149,8 @@ __device__ __forceinline__ void tmem_ld32x4(uint32_t taddr, float (&v)[4]) {
 #pragma unroll
     for (int j = 0; j < 4; ++j) v[j] = __uint_as_float(r[j]);
 }
+// global-memory writes of this thread before bulk copies that read them
+__device__ __forceinline__ void fence_async_all() { asm volatile("fence.proxy.async;" ::: "memory"); }
 // one 8x8 16-bit matrix: threads 0-7 give the row addresses; thread t's register holds
 // row t / 4, columns 2 (t % 4) and 2 (t % 4) + 1
 __device__ __forceinline__ void stmatrix1(uint32_t addr, uint32_t r0) {
@@ -164,7 +186,7 @@ __global__ void __launch_bounds__(PipeMode<MODE>::kThreads, 1) k_mlp_pipe(PipePa
     constexpr int NL = TA::kLayers;
     constexpr int LS = A::kSdfLayers;
     constexpr uint32_t kStage = TA::stage_bytes();
-    constexpr int kNT = TA::total_chunks();
+    constexpr int kNT = TA::total_chunks(), kNS = TA::sdf_chunks();
     static_assert(TA::template valid<MODE>(), "network shape outside the pipelined kernel's layout");
     extern __shared__ __align__(1024) uint8_t smem[];
     uint8_t* A_hi = smem;
@@ -181,14 +203,14 @@ __global__ void __launch_bounds__(PipeMode<MODE>::kThreads, 1) k_mlp_pipe(PipePa
     float* s_w255 = s_f255 + kPParts * kPTile;
     PChunk* s_chunks = reinterpret_cast<PChunk*>(reinterpret_cast<uint8_t*>(s_out) + TA::scratch_bytes());
     uint64_t* bars = reinterpret_cast<uint64_t*>(reinterpret_cast<uint8_t*>(s_chunks) + TA::chunk_tab_bytes());
-    // bars: full[kStages], empty[kStages], accf[2], ablk[kPMaxBlocks], epi, drain
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * kStages + 2 + kPMaxBlocks + 2);
+    // bars: full[kStages], empty[kStages], accf[2], ablk[kPMaxBlocks], epi, drain, back
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * kStages + 2 + kPMaxBlocks + 3);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
     const uint32_t bar_full0 = smem_u32(bars), bar_empty0 = smem_u32(bars + kStages);
     const uint32_t bar_accf0 = smem_u32(bars + 2 * kStages);
     const uint32_t bar_blk0 = smem_u32(bars + 2 * kStages + 2);
     const uint32_t bar_epi = smem_u32(bars + 2 * kStages + 2 + kPMaxBlocks);
-    const uint32_t bar_drain = bar_epi + 8;
+    const uint32_t bar_drain = bar_epi + 8, bar_back = bar_epi + 16;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
     const int64_t total = sample_total(p.src);
@@ -209,6 +231,7 @@ __global__ void __launch_bounds__(PipeMode<MODE>::kThreads, 1) k_mlp_pipe(PipePa
         for (int b = 0; b < kPMaxBlocks; ++b) mbar_init(bar_blk0 + 8 * b, kPEpiWarps);
         mbar_init(bar_epi, kPEpiWarps);
         mbar_init(bar_drain, 1);
+        mbar_init(bar_back, 1);
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         uint32_t off = 0;
@@ -232,15 +255,6 @@ __global__ void __launch_bounds__(PipeMode<MODE>::kThreads, 1) k_mlp_pipe(PipePa
         for (int i = threadIdx.x; i < 256; i += PM::kThreads)
             s_w255[i] = i < lo.K ? __ldg(p.sdf_w + TA::param_offset(LS - 1) + (int64_t)256 * lo.K + i) : 0.0f;
     }
-    if constexpr (!kSplit) {
-        // the tangent rows of the colour input beyond column 256 are never written: clear them
-        // once so that the rows the colour MMAs compute and the epilogue ignores stay finite
-        for (int i = threadIdx.x; i < (int)(kPXMax / 16); i += PM::kThreads)
-            reinterpret_cast<uint4*>(X)[i] = make_uint4(0, 0, 0, 0);
-    } else {
-        for (int i = threadIdx.x; i < (int)(kPABytes / 16); i += PM::kThreads)
-            reinterpret_cast<uint4*>(A_lo)[i] = make_uint4(0, 0, 0, 0);
-    }
     if (warp == kPMmaWarp) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
                      "r"(512));
@@ -251,6 +265,11 @@ __global__ void __launch_bounds__(PipeMode<MODE>::kThreads, 1) k_mlp_pipe(PipePa
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
+    // this CTA's tiles: blockIdx.x + k gridDim.x, k < mine; the colour layers follow every kPUnit-th
+    // and the last
+    const int64_t mine = (n_tiles - blockIdx.x + gridDim.x - 1) / gridDim.x;
+    auto unit_end = [&](int64_t k) { return k % kPUnit == kPUnit - 1 || k + 1 == mine; };
+    uint8_t* park = p.park + (size_t)blockIdx.x * (TA::kParkMain + TA::kParkX);
 
     if (warp > kPMmaWarp) {
         // ------------------------------------------------ producers, one per ring stage
@@ -259,10 +278,11 @@ __global__ void __launch_bounds__(PipeMode<MODE>::kThreads, 1) k_mlp_pipe(PipePa
             const uint32_t dst = smem_u32(stage_base + own * kStage);
             uint32_t issued = 0;
             bool ok = true;
-            for (int64_t tile = blockIdx.x; tile < n_tiles && ok; tile += gridDim.x) {
-                for (int j = (int)own; j < kNT; j += kStages) {
-                    // test-only: stop before the withheld chunk of the first tile
-                    if (tile == blockIdx.x && j == p.withhold) { ok = false; break; }
+            for (int64_t k = 0; k < mine && ok; ++k) {
+                const int n_j = unit_end(k) ? kNT : kNS;
+                for (int j = (int)own; j < n_j; j += kStages) {
+                    // test-only: stop before the withheld chunk of the first tile (or unit)
+                    if (k < kPUnit && j == p.withhold) { ok = false; break; }
                     const PChunk ci = s_chunks[j];
                     if (!mbar_wait(bar_empty0 + 8 * own, (issued & 1u) ^ 1u, abort_flag, p.spin)) { ok = false; break; }
                     mbar_expect_tx(bar_full0 + 8 * own, ci.bytes);
@@ -286,23 +306,30 @@ __global__ void __launch_bounds__(PipeMode<MODE>::kThreads, 1) k_mlp_pipe(PipePa
             for (int i = 0; i < kStages; ++i) full_uses[i] = 0;
 #pragma unroll
             for (int i = 0; i < kPMaxBlocks; ++i) blk_uses[i] = 0;
-            uint32_t lc = 0;
+            uint32_t lc = 0, back = 0;
             bool ok = true;
             const uint32_t a_hi = smem_u32(A_hi), a_lo = smem_u32(A_lo), a_x = smem_u32(X);
-            for (int64_t tile = blockIdx.x; tile < n_tiles && ok; tile += gridDim.x) {
+            for (int64_t k = 0; k < mine && ok; ++k) {
                 int j = 0;
-                for (int L = 0; L < NL && ok; ++L, ++lc) {
+                const bool parked = k % kPUnit != 0;   // the unit has more than one tile
+                const int n_l = unit_end(k) ? NL : LS;
+                for (int L = 0; L < n_l && ok; ++L, ++lc) {
                     const TcLayer ly = TA::layer(L);
                     const uint32_t d_tmem = tmem + (lc & 1u) * 256u;
                     const uint32_t idesc = idesc_mma<F16>(128, TA::n_mma(L));
                     const uint32_t a_sbo = (uint32_t)(TA::pitch_main(L) / 8) * 128u;
                     const bool two = kSplit && ly.sdf;
                     for (int c = 0; c < TA::chunks(L); ++c, ++j) {
-                        uint32_t bph = 0;
+                        uint32_t bph = 0, bar = bar_blk0 + 8 * c;
+                        if (L == LS && parked) {
+                            bar = bar_back;
+                            bph = back & 1u;
+                        } else {
 #pragma unroll
-                        for (int i = 0; i < kPMaxBlocks; ++i)
-                            if (i == c) bph = blk_uses[i]++ & 1u;
-                        if (!__all_sync(0xffffffffu, mbar_wait(bar_blk0 + 8 * c, bph, abort_flag, p.spin))) { ok = false; break; }
+                            for (int i = 0; i < kPMaxBlocks; ++i)
+                                if (i == c) bph = blk_uses[i]++ & 1u;
+                        }
+                        if (!__all_sync(0xffffffffu, mbar_wait(bar, bph, abort_flag, p.spin))) { ok = false; break; }
                         const PChunk ci = s_chunks[j];
                         uint32_t fph = 0;
 #pragma unroll
@@ -318,14 +345,14 @@ __global__ void __launch_bounds__(PipeMode<MODE>::kThreads, 1) k_mlp_pipe(PipePa
                         uint64_t bd = mdesc(b0, 128, b_sbo);
                         if (k0 < 256) {
                             const uint32_t ko = (uint32_t)(k0 / 8) * 128u;
-                            uint64_t ah = mdesc(a_hi + ko, 128, a_sbo), al = mdesc(a_lo + ko, 128, a_sbo);
-                            for (int kk = 0; kk < ci.kc / 16; ++kk) {
-                                mma_el(el, d_tmem, ah, bd, idesc, (k0 | kk) != 0 ? 1u : 0u);
-                                if (two) mma_el(el, d_tmem, al, bd, idesc, 1u);
-                                ah += 16;
-                                al += 16;
-                                bd += 16;
-                            }
+                            const uint64_t ah = mdesc(a_hi + ko, 128, a_sbo), al = mdesc(a_lo + ko, 128, a_sbo);
+                            auto step = [&](int kk) {
+                                mma_el(el, d_tmem, ah + 16 * kk, bd + 16 * kk, idesc, (k0 | kk) != 0 ? 1u : 0u);
+                                if (two) mma_el(el, d_tmem, al + 16 * kk, bd + 16 * kk, idesc, 1u);
+                            };
+                            if (ci.kc == kKChunk) static_for<0, kKChunk / 16>([&](auto kk) { step(decltype(kk)::value); });
+                            else
+                                for (int kk = 0; kk < ci.kc / 16; ++kk) step(kk);
                         } else {
                             uint64_t ax = mdesc(a_x + (uint32_t)((k0 - 256) / 8) * 128u, 128, (uint32_t)(TA::kPitchX / 8) * 128u);
                             for (int kk = 0; kk < ci.kc / 16; ++kk) {
@@ -338,6 +365,7 @@ __global__ void __launch_bounds__(PipeMode<MODE>::kThreads, 1) k_mlp_pipe(PipePa
                     }
                     if (!ok) break;
                     commit_el(el, bar_accf0 + 8 * (lc & 1u));
+                    if (L == LS && parked) ++back;
                 }
             }
             if (!ok && el) {
@@ -357,7 +385,7 @@ __global__ void __launch_bounds__(PipeMode<MODE>::kThreads, 1) k_mlp_pipe(PipePa
         const SoftplusH2 spk = softplus_h2_consts(half_beta, inv_beta);
         const __half2 inv_sqrt2_h2 = __float2half2_rn(kInvSqrt2);
         const int et = threadIdx.x;
-        uint32_t acc_uses[2] = {0, 0}, epi_ph = 0, lc = 0;
+        uint32_t acc_uses[2] = {0, 0}, epi_ph = 0, lc = 0, backs = 0;
         bool ok = true;
         auto epi_sync = [&]() -> bool {
             __syncwarp();
@@ -465,9 +493,12 @@ __global__ void __launch_bounds__(PipeMode<MODE>::kThreads, 1) k_mlp_pipe(PipePa
 
         ok = build_table(blockIdx.x);
         if (ok) write_input0();
-        for (int64_t tile = blockIdx.x; tile < n_tiles && ok; tile += gridDim.x) {
+        for (int64_t kt = 0; kt < mine && ok; ++kt) {
+            const int64_t tile = blockIdx.x + kt * gridDim.x;
+            const int slot = (int)(kt % kPUnit);   // of its unit
+            const bool end = unit_end(kt), parked = !end || slot > 0;
             int boff = 0;
-            for (int L = 0; L < NL; ++L, ++lc) {
+            for (int L = 0; L < (end ? NL : LS); ++L, ++lc) {
                 const TcLayer ly = TA::layer(L);
                 const uint32_t hsel = lc & 1u;
                 const bool w_ok = mbar_wait(bar_accf0 + 8 * hsel, acc_uses[hsel] & 1u, abort_flag, p.spin);
@@ -604,7 +635,10 @@ __global__ void __launch_bounds__(PipeMode<MODE>::kThreads, 1) k_mlp_pipe(PipePa
                 } else if (ly.sdf) {
                     // ---- SDF output layer: f, grad f and the features -> colour input rows ----
                     constexpr int kD = TA::kD;
-                    constexpr int Kc = TA::layer(LS).Kp;
+                    constexpr int Kc = TA::layer(LS).Kp, kPm = TA::pitch_main(LS);
+                    // generic pointers: the operand itself, or the unit's parking place
+                    uint8_t* main_at = parked ? park : A_hi;
+                    uint8_t* x_at = parked ? park + TA::kParkMain : X;
                     if (pt == 0) {
                         // column 0 of all 128 rows: f (value rows), then the three gradient rows
                         float c0;
@@ -620,16 +654,18 @@ __global__ void __launch_bounds__(PipeMode<MODE>::kThreads, 1) k_mlp_pipe(PipePa
                             const float inv = gn > 0.0f ? 1.0f / gn : 0.0f;
                             const float* sx = s_x + sm * 8;
                             float* so = s_out + sm * 8;
-                            so[0] = p.scale * (c0 + bias[0]);
-                            so[1] = gx * sx[3] + gy * sx[4] + gz * sx[5];
-                            so[2] = sx[6];
-                            so[3] = sx[7];
-                            so[4] = gn;
                             so[5] = gx * inv;
                             so[6] = gy * inv;
                             so[7] = gz * inv;
+                            const int64_t g = tile * kPTile + sm;
+                            if (g < total) {
+                                float4* R4 = reinterpret_cast<float4*>(p.rec + g);
+                                R4[0] = make_float4(p.scale * (c0 + bias[0]), gx * sx[3] + gy * sx[4] + gz * sx[5], sx[6], sx[7]);
+                                R4[2] = make_float4(so[5], so[6], so[7], 0.0f);
+                                p.rec[g].gnorm = gn;
+                            }
                             // colour prefix: x~, direction encoding, normal (columns 0 .. kD - 1)
-                            const uint32_t row = 32 * q + lane;
+                            const int row = 32 * q + 8 * slot + lane;
                             for (int c8 = 0; c8 < kD; c8 += 8) {
                                 float o[8];
 #pragma unroll
@@ -642,15 +678,16 @@ __global__ void __launch_bounds__(PipeMode<MODE>::kThreads, 1) k_mlp_pipe(PipePa
                                     else if (col < kD + 1) val = so[5 + col - 3 - A::kDirEnc];
                                     o[jj] = val;
                                 }
-                                st_row8<F16>(A_hi, row, c8, TA::pitch_main(LS), o);
+                                st_row8<F16>(main_at, row, c8, kPm, o);
                             }
                         }
                     }
                     if (!epi_sync()) { ok = false; break; }
                     // features: colour group cg = output group cg - kD / 8; column kD holds n_z
                     constexpr int ncg = Kc / 8;
-                    const uint32_t rv_hi = smem_u32(A_hi) + a_off(32 * q + (lane & 7), 0, TA::pitch_main(LS));
-                    const uint32_t rv_x = smem_u32(X) + a_off(32 * q + (lane & 7), 0, TA::kPitchX > 0 ? TA::kPitchX : 8);
+                    // a warp's 8 rows x 8 columns are one core matrix: 128 bytes in lane order
+                    uint8_t* rv_main = main_at + (4 * q + slot) * (kPm / 8) * 128 + 4 * lane;
+                    uint8_t* rv_x = x_at + (4 * q + slot) * (TA::kPitchX / 8) * 128 + 4 * lane;
                     for (int b = 0; b * 8 < ncg; ++b) {
                         const int g0 = b * 8 < kD / 8 ? kD / 8 : b * 8;
                         const int gf = g0 + ((pt - g0) % kPParts + kPParts) % kPParts;
@@ -681,63 +718,97 @@ __global__ void __launch_bounds__(PipeMode<MODE>::kThreads, 1) k_mlp_pipe(PipePa
                                 o[e] = val;
                             }
                             const int kc = 8 * cg;
-                            if (kc < 256) stmatrix1(rv_hi + (uint32_t)(kc >> 3) * 128u, pack2<F16>(o[0], o[1]));
-                            else stmatrix1(rv_x + (uint32_t)((kc - 256) >> 3) * 128u, pack2<F16>(o[0], o[1]));
+                            *reinterpret_cast<uint32_t*>(kc < 256 ? rv_main + (kc >> 3) * 128 : rv_x + ((kc - 256) >> 3) * 128) =
+                                pack2<F16>(o[0], o[1]);
                         }
-                        block_done(b);
+                        if (!parked) block_done(b);
                     }
-                    // the next tile's table (this tile's is no longer read)
-                    if (tile + gridDim.x < n_tiles && !build_table(tile + gridDim.x)) { ok = false; break; }
+                    if (parked) {
+                        fence_async_all();
+                        if (!epi_sync()) { ok = false; break; }
+                        if (end && et == 0) {
+                            // the unit's colour input as the operand (the SDF MMAs are complete)
+                            fence_async_all();
+                            mbar_expect_tx(bar_back, TA::kParkMain + TA::kParkX);
+                            bulk_g2s(smem_u32(A_hi), park, TA::kParkMain, bar_back);
+                            if (TA::kParkX > 0) bulk_g2s(smem_u32(X), park + TA::kParkMain, TA::kParkX, bar_back);
+                            ++backs;
+                        }
+                    }
+                    // the next tile's table (this tile's is no longer read), and its layer-0 input if that
+                    // is next
+                    if (kt + 1 < mine && !build_table(tile + gridDim.x)) { ok = false; break; }
+                    if (!end) write_input0();
                 } else if (L < NL - 1) {
-                    // ---- hidden colour layer (ReLU), value rows only ----
+                    // ---- hidden colour layer (ReLU): row group j holds tile j of the unit ----
                     const int Kn = TA::layer(L + 1).Kp;
-                    const uint32_t rv = smem_u32(A_hi) + a_off(32 * q + (lane & 7), 0, Kn);
                     const int ng = Kn / 8;
-                    for (int b = 0; b * 8 < ng; ++b) {
-                        // this part's (at most three) groups of the block: loads together, one wait
-                        const int gf = 8 * b + ((pt - 8 * b) % kPParts + kPParts) % kPParts;
-                        float d[3][4];
+                    auto colour = [&](auto nr) {
+                        constexpr int NR = decltype(nr)::value;   // row groups: 1 or all 4
+                        const uint32_t rv = smem_u32(A_hi) + a_off(32 * q + (NR == 1 ? lane & 7 : lane), 0, Kn);
+                        for (int b = 0; b * 8 < ng; ++b) {
+                            // this part's (at most three) groups of the block: loads together, one wait
+                            const int gf = 8 * b + ((pt - 8 * b) % kPParts + kPParts) % kPParts;
+                            float d[3][8];
 #pragma unroll
-                        for (int i = 0; i < 3; ++i) {
-                            const int c = 8 * (gf + i * kPParts);
-                            if (c < 8 * (8 * b + 8) && c < 8 * ng && c < ly.Np) tmem_ld16x256_x1(th + lq + c, d[i]);
-                            else d[i][0] = d[i][1] = d[i][2] = d[i][3] = 0.0f;
-                        }
+                            for (int i = 0; i < 3; ++i) {
+                                const int c = 8 * (gf + i * kPParts);
+                                if (c < 8 * (8 * b + 8) && c < 8 * ng && c < ly.Np) {
+                                    tmem_ld16x256_x1(th + lq + c, d[i]);
+                                    if (NR > 1) tmem_ld16x256_x1(th + lq16 + c, d[i] + 4);
+                                } else {
 #pragma unroll
-                        for (int i = 0; i < 3; ++i) tmem_wait_ld4(d[i]);
-#pragma unroll
-                        for (int i = 0; i < 3; ++i) {
-                            const int g = gf + i * kPParts;
-                            if (g >= 8 * b + 8 || g >= ng) continue;
-                            const int c = 8 * g;
-                            float o[2];
-#pragma unroll
-                            for (int e = 0; e < 2; ++e) {
-                                const int col = c + fc + e;
-                                o[e] = col < ly.N ? fmaxf(d[i][e] + bias[col], 0.0f) : 0.0f;
+                                    for (int k = 0; k < 8; ++k) d[i][k] = 0.0f;
+                                }
                             }
-                            stmatrix1(rv + (uint32_t)(c >> 3) * 128u, pack2<F16>(o[0], o[1]));
+#pragma unroll
+                            for (int i = 0; i < 3; ++i) tmem_wait_ld8(d[i]);
+#pragma unroll
+                            for (int i = 0; i < 3; ++i) {
+                                const int g = gf + i * kPParts;
+                                if (g >= 8 * b + 8 || g >= ng) continue;
+                                const int c = 8 * g;
+                                uint32_t o[4];
+#pragma unroll
+                                for (int r = 0; r < NR; ++r) {
+                                    float v[2];
+#pragma unroll
+                                    for (int e = 0; e < 2; ++e) {
+                                        const int col = c + fc + e;
+                                        v[e] = col < ly.N ? fmaxf(d[i][2 * r + e] + bias[col], 0.0f) : 0.0f;
+                                    }
+                                    o[r] = pack2<F16>(v[0], v[1]);
+                                }
+                                const uint32_t at = rv + (uint32_t)(c >> 3) * 128u;
+                                if constexpr (NR == 1) {
+                                    stmatrix1(at, o[0]);
+                                } else {
+                                    stmatrix4(at, o[0], o[1], o[2], o[3]);
+                                }
+                            }
+                            block_done(b);
                         }
-                        block_done(b);
+                    };
+                    if (slot == 0) {
+                        colour(std::integral_constant<int, 1>{});
+                    } else {
+                        colour(std::integral_constant<int, 4>{});
                     }
                 } else {
                     // ---- colour output: the next tile's layer-0 input first (its MMAs run
                     // under this epilogue; every MMA of this tile is complete), then the record ----
-                    if (tile + gridDim.x < n_tiles) write_input0();
+                    if (kt + 1 < mine) write_input0();
                     if (pt == 0) {
                         float x0[4];
                         tmem_ld32x4(th + lq, x0);
                         tmem_wait_ld();
-                        const int64_t g = tile * kPTile + 8 * q + lane;
-                        if (lane < 8 && g < total) {
-                            const float* so = s_out + (8 * q + lane) * 8;
-                            const float cr = __fdividef(1.0f, 1.0f + __expf(-(x0[0] + bias[0])));
-                            const float cgc = __fdividef(1.0f, 1.0f + __expf(-(x0[1] + bias[1])));
-                            const float cb = __fdividef(1.0f, 1.0f + __expf(-(x0[2] + bias[2])));
-                            float4* R4 = reinterpret_cast<float4*>(p.rec + g);
-                            R4[0] = make_float4(so[0], so[1], so[2], so[3]);
-                            R4[1] = make_float4(cr, cgc, cb, so[4]);
-                            R4[2] = make_float4(so[5], so[6], so[7], 0.0f);
+                        const int jt = lane >> 3;   // the lane's tile of the unit
+                        const int64_t g = (tile + (int64_t)(jt - slot) * gridDim.x) * kPTile + 8 * q + (lane & 7);
+                        if (jt <= slot && g < total) {
+                            float* R = reinterpret_cast<float*>(p.rec + g) + 4;
+                            R[0] = __fdividef(1.0f, 1.0f + __expf(-(x0[0] + bias[0])));
+                            R[1] = __fdividef(1.0f, 1.0f + __expf(-(x0[1] + bias[1])));
+                            R[2] = __fdividef(1.0f, 1.0f + __expf(-(x0[2] + bias[2])));
                         }
                     }
                 }
@@ -745,6 +816,10 @@ __global__ void __launch_bounds__(PipeMode<MODE>::kThreads, 1) k_mlp_pipe(PipePa
             }
         }
         if (!ok) set_status(p.status, TSDFS_DEV_TIMEOUT);
+        if (!ok && backs > 0) {   // this thread's copies may be in flight
+            for (uint32_t it = 0; it < kMaxSpin && !mbar_try(bar_back, (backs - 1) & 1u); ++it) {
+            }
+        }
     }
     tc_fence_before();
     __syncthreads();
@@ -755,7 +830,8 @@ __global__ void __launch_bounds__(PipeMode<MODE>::kThreads, 1) k_mlp_pipe(PipePa
 }
 
 template <int ARCH, int MODE>
-int launch_pipe(const tsdfs_mlp* m, const SampleSource& src, SampleRec* rec, int64_t max_samples, cudaStream_t st) {
+int launch_pipe(const tsdfs_mlp* m, const SampleSource& src, SampleRec* rec, int64_t max_samples, uint8_t* stash,
+                cudaStream_t st) {
     using TA = PipeArch<ARCH>;
     constexpr size_t smem = TA::template smem_bytes<MODE>();
     static_assert(smem <= 232448, "k_mlp_pipe shared memory exceeds 227 KB");
@@ -782,30 +858,38 @@ int launch_pipe(const tsdfs_mlp* m, const SampleSource& src, SampleRec* rec, int
     p.status = device_status_word();
     p.spin = test_spin_limit(kMaxSpin);
     p.withhold = test_withhold_chunk();
+    p.park = stash;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const int64_t tiles = (max_samples + kPTile - 1) / kPTile;
+    if (sms > kPMaxCtas) sms = kPMaxCtas;
     const unsigned blocks = (unsigned)(tiles < sms ? (tiles < 1 ? 1 : tiles) : sms);
     k_mlp_pipe<ARCH, MODE><<<blocks, PipeMode<MODE>::kThreads, smem, st>>>(p);
     return cuda_check(cudaGetLastError(), "mlp_pipe launch");
 }
 
 template <int ARCH>
-int launch_pipe_arch(const tsdfs_mlp* m, const SampleSource& src, SampleRec* rec, int64_t max_samples,
+int launch_pipe_arch(const tsdfs_mlp* m, const SampleSource& src, SampleRec* rec, int64_t max_samples, uint8_t* stash,
                      cudaStream_t st) {
     switch (m->precision) {
-        case TSDFS_PREC_F16: return launch_pipe<ARCH, TSDFS_PREC_F16>(m, src, rec, max_samples, st);
-        case TSDFS_PREC_BF16: return launch_pipe<ARCH, TSDFS_PREC_BF16>(m, src, rec, max_samples, st);
-        case TSDFS_PREC_BF16X2: return launch_pipe<ARCH, TSDFS_PREC_BF16X2>(m, src, rec, max_samples, st);
+        case TSDFS_PREC_F16: return launch_pipe<ARCH, TSDFS_PREC_F16>(m, src, rec, max_samples, stash, st);
+        case TSDFS_PREC_BF16: return launch_pipe<ARCH, TSDFS_PREC_BF16>(m, src, rec, max_samples, stash, st);
+        case TSDFS_PREC_BF16X2: return launch_pipe<ARCH, TSDFS_PREC_BF16X2>(m, src, rec, max_samples, stash, st);
         default: return fail(TSDFS_E_INVALID, "pipelined network kernel: unsupported precision %d", m->precision);
     }
 }
 
 }  // namespace
 
-int launch_mlp_pipe(const tsdfs_mlp* m, const SampleSource& src, SampleRec* rec, int64_t max_samples, cudaStream_t st) {
+size_t mlp_pipe_stash_bytes() {
+    using TA = PipeArch<TSDFS_ARCH_ROOM>;
+    return (size_t)kPMaxCtas * (TA::kParkMain + TA::kParkX);
+}
+
+int launch_mlp_pipe(const tsdfs_mlp* m, const SampleSource& src, SampleRec* rec, int64_t max_samples, uint8_t* stash,
+                    cudaStream_t st) {
     if ((reinterpret_cast<uintptr_t>(m->packed) & 15u) != 0) return fail(TSDFS_E_INVALID, "packed weights must be 16-byte aligned");
-    if (m->arch == TSDFS_ARCH_TINY) return launch_pipe_arch<TSDFS_ARCH_TINY>(m, src, rec, max_samples, st);
-    if (m->arch == TSDFS_ARCH_ROOM) return launch_pipe_arch<TSDFS_ARCH_ROOM>(m, src, rec, max_samples, st);
+    if (m->arch == TSDFS_ARCH_TINY) return launch_pipe_arch<TSDFS_ARCH_TINY>(m, src, rec, max_samples, stash, st);
+    if (m->arch == TSDFS_ARCH_ROOM) return launch_pipe_arch<TSDFS_ARCH_ROOM>(m, src, rec, max_samples, stash, st);
     return fail(TSDFS_E_UNSUPPORTED, "pipelined network kernel: unknown arch %d", m->arch);
 }
 

@@ -65,3 +65,27 @@ def test_coarse_tiles(scene, precision):
     assert np.isfinite(whole.cpu().numpy()).all()
     rc, bits = T.tsdfs_sync_status()
     assert rc == 0, bits
+
+
+@pytest.mark.parametrize("scene,precision", [("room", T.TSDFS_PREC_BF16X2), ("tiny", T.TSDFS_PREC_BF16X2),
+                                             ("room", T.TSDFS_PREC_F16)])
+def test_pipelined_colour_layers_over_several_tiles(scene, precision):
+    """The pipelined kernel runs the colour layers for up to four 32-sample tiles of a CTA at a time
+    (here two tiles per ray): the bits of the rays in parts of one tile to a CTA."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    o, d = (torch.tensor(a).cuda() for a in synth.room_heldout_rays(0))
+    half = sms // 2
+    idx = torch.tensor(synth.sub_sample(len(o), 7 * half, seed=4)).cuda()
+    o, d = o[idx].contiguous(), d[idx].contiguous()
+    mlp = T.Mlp(synth.scene_mlp(scene), precision)
+    before = T.tsdfs_network_kernel(precision)
+    T.tsdfs_set_network_kernel(precision, T.TSDFS_NETKERNEL_PIPELINED)
+    try:
+        parts = torch.cat([render(mlp, half, 64, o[r:], d[r:]) for r in range(0, 7 * half, half)])
+        # tiles per CTA: 1 and 2, 2, 4, 4 and 5, 5, 6, 7
+        for n in (half + 1, 2 * half, 4 * half, 4 * half + 1, 5 * half, 6 * half, 7 * half):
+            assert torch.equal(render(mlp, n, 64, o, d), parts[:n]), n
+    finally:
+        T.tsdfs_set_network_kernel(precision, before)
+    rc, bits = T.tsdfs_sync_status()
+    assert rc == 0, bits
