@@ -46,10 +46,16 @@ __global__ void k_grid_init(void* V, int f16, uint8_t* W, int64_t n) {
 // The camera table of all views is staged in shared memory once per block (20 floats per view:
 // c2w[12], fx, fy, cx, cy and what the tests use), the list of the brick's views after it.  256^3
 // voxels, 100 views of the room: 2816 us without any of it, 950 with bricks of 32 x 4 x 4, 844 as it
-// is; what is left is the ~40 instructions of a voxel-view and the divisions near the surface.
+// is in 152 x 8 blocks and 645 in kFuseBlocks; what is left is the ~40 instructions of a voxel-view and
+// the divisions near the surface.
 constexpr int kBX = 8, kBY = 8, kBZ = 8;
 constexpr int kBrickVoxels = kBX * kBY * kBZ;
 constexpr int kCam = 20;
+// Blocks at most.  Five are resident on an SM, and bricks differ in their views: 152 x 8 blocks are
+// 1.6 rounds of equal shares (the SMs idle for 15 % of the time), 20 rounds even out, and staging the
+// table once per block still costs less than that.  256^3, 100 views / 300 x 225 x 121, 3 views: 152 x 5
+// blocks 770 / 102 us, x 8 846 / 72, x 32 680 / 56, x 108 645 / 56, x 216 648 / 56.
+constexpr int kFuseBlocks = 152 * 5 * 20;
 
 // whether view P can see a voxel centre within h[3] of c[3]
 __device__ __forceinline__ bool brick_visible(const float* P, const float c[3], const float h[3], float fW, float fH) {
@@ -471,7 +477,7 @@ extern "C" int tsdf_integrate(const tsdfs_grid* g, const float* depth, int32_t n
         if (rc) return rc;
     }
     ProfScope ps("integrate", (cudaStream_t)stream);
-    k_integrate<<<grid_1d(bricks, 1, 152 * 8), kFuseBlock, smem, (cudaStream_t)stream>>>(
+    k_integrate<<<grid_1d(bricks, 1, kFuseBlocks), kFuseBlock, smem, (cudaStream_t)stream>>>(
         g->nx, g->ny, g->nz, g->origin[0], g->origin[1], g->origin[2], g->voxel_size, g->trunc, g->tsdf,
         g->dtype == TSDFS_F16, g->weight, depth, n_views, H, W, K, c2w);
     return cuda_check(cudaGetLastError(), "tsdf_integrate launch");
