@@ -170,6 +170,11 @@ static void prof_clear() {
 int launch_composite(const SampleRec* rec, const int32_t* offsets, int per_ray, const uint8_t* status, int64_t n_rays,
                      const int32_t* total_dev, int64_t capacity, Opacity op, float* rgb, float* depth,
                      float* wsum, float* normal, float* eik, cudaStream_t st);
+int launch_composite_again(const SampleRec* rec, const int32_t* offsets, int per_ray, const uint8_t* status,
+                           int64_t n_rays, const int32_t* total_dev, int64_t capacity, Opacity op, float* rgb,
+                           float* depth, float* wsum, float* normal, float* eik, const uint32_t* again, cudaStream_t st);
+int launch_mark_thin(SampleRec* rec, const int32_t* offsets, const uint8_t* status, const float* wsum, int64_t n_rays,
+                     int64_t capacity, uint32_t* thin, cudaStream_t st);
 int launch_hier_setup(const tsdfs_grid* g, const float* ray_o, const float* ray_d, int64_t n_rays, float t_near,
                       float t_far, float* t0, float* te, uint8_t* status, float* tc, float* dc, int n_c,
                       cudaStream_t st);
@@ -422,9 +427,25 @@ extern "C" int render_rays(const tsdfs_mlp* mlp, const float* ray_o, const float
         rc = run_full_mlp(mlp, src, rec, max_samples, stash, st);
         if (rc) return rc;
     }
-    ProfScope ps("composite", st);
-    return launch_composite(rec, offsets, 0, status, n_rays, offsets + n_rays, max_samples, opacity_of(mlp),
-                            rgb, depth, wsum, normal, eik, st);
+    {
+        ProfScope ps("composite", st);
+        rc = launch_composite(rec, offsets, 0, status, n_rays, offsets + n_rays, max_samples, opacity_of(mlp), rgb, depth,
+                              wsum, normal, eik, st);
+        if (rc) return rc;
+    }
+    if (mlp->precision != TSDFS_PREC_F32 || mlp->arch != TSDFS_ARCH_ROOM || max_samples == 0) return TSDFS_OK;
+    // Rays of almost no weight (k_mark_thin): the two FP32 kernels' f differ by 1e-6 in the room networks,
+    // and a ray's depth and normal by as much as 3e-3 then.  The SIMT kernel evaluates their samples, so
+    // that its results for them are the results for them; without such rays three empty launches (5 us).  The
+    // tiny networks' f differ by 2e-7 and nothing comes of it.
+    ProfScope ps("thin_rays", st);
+    uint32_t* thin = reinterpret_cast<uint32_t*>(stash) + 1;
+    rc = launch_mark_thin(rec, offsets, status, wsum, n_rays, max_samples, thin, st);
+    if (rc) return rc;
+    rc = launch_mlp_full_simt<TSDFS_ARCH_ROOM>(net_params(mlp), src, rec, max_samples, thin, st);
+    if (rc) return rc;
+    return launch_composite_again(rec, offsets, 0, status, n_rays, offsets + n_rays, max_samples, opacity_of(mlp), rgb,
+                                  depth, wsum, normal, eik, thin, st);
 }
 
 extern "C" int tsdfs_autotune_network(const tsdfs_mlp* mlp, const float* ray_o, const float* ray_d, const float* t_n,

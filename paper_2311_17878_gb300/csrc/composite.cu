@@ -15,6 +15,7 @@ constexpr int kMaxHier = kMaxCoarse + kMaxFine;
 // ray: 999 rays 3.8 / 7.2, 4800 5.7 / 7.2, 10 800 9.0 / 7.3, 43 200 24 / 8.1; 96 samples a ray: 4800 rays
 // 10.7 / 48, 19 200 31 / 58.
 constexpr int64_t kCompWarpRays = 8192;
+constexpr float kThinRay = 1e-3f;   // see k_mark_thin
 
 
 // One thread per ray.  Uniform rays: samples offsets[r]..offsets[r+1]; explicit
@@ -25,7 +26,9 @@ __global__ void __launch_bounds__(kCompBlock) k_composite(const SampleRec* __res
                                                           const int32_t* total_dev, int64_t capacity, Opacity op,
                                                           float* __restrict__ rgb, float* __restrict__ depth,
                                                           float* __restrict__ wsum_out, float* __restrict__ normal,
-                                                          float* __restrict__ eik_out, const uint32_t* dev_status) {
+                                                          float* __restrict__ eik_out, const uint32_t* dev_status,
+                                                          const uint32_t* again) {
+    if (again && *again == 0) return;
     // outputs are zero when the samples overflowed the workspace, and while the device
     // status word holds a timeout of a network kernel (its records may be incomplete)
     const bool overflow = (total_dev && (int64_t)__ldg(total_dev) > capacity) ||
@@ -83,7 +86,9 @@ __global__ void __launch_bounds__(kCompBlock) k_composite_warp(const SampleRec* 
                                                                const int32_t* total_dev, int64_t capacity, Opacity op,
                                                                float* __restrict__ rgb, float* __restrict__ depth,
                                                                float* __restrict__ wsum_out, float* __restrict__ normal,
-                                                               float* __restrict__ eik_out, const uint32_t* dev_status) {
+                                                               float* __restrict__ eik_out, const uint32_t* dev_status,
+                                                               const uint32_t* again) {
+    if (again && *again == 0) return;
     __shared__ float rows[kCompWarps][9][33];   // w, r, g, b, t, normal, |grad f| - 1 of 32 samples
     const int lane = threadIdx.x & 31;
     float(*s)[33] = rows[threadIdx.x >> 5];
@@ -144,6 +149,22 @@ __global__ void __launch_bounds__(kCompBlock) k_composite_warp(const SampleRec* 
         else if (lane == 4) depth[r] = ok ? acc * inv : 0.0f;
         else if (lane < 8 && normal) normal[3 * r + lane - 5] = ok ? acc * inv : 0.0f;
         else if (lane == 8 && eik_out) eik_out[r] = st == TSDFS_BOUNDED && !overflow ? acc : 0.0f;
+    }
+}
+
+// Marks the groups of 16 samples of rays with a weight sum below kThinRay (pad of a group's first
+// record) and sets *thin if there is one.  Such a ray's opacities are differences of sigmoids near 1,
+// a few units in the last place each, and its depth and normal are divided by their sum: they hang on the last
+// bits of f.
+__global__ void k_mark_thin(SampleRec* __restrict__ rec, const int32_t* __restrict__ offsets,
+                            const uint8_t* __restrict__ status, const float* __restrict__ wsum, int64_t n_rays,
+                            int64_t capacity, uint32_t* thin) {
+    if ((int64_t)__ldg(offsets + n_rays) > capacity) return;
+    for (int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; r < n_rays; r += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t b = __ldg(offsets + r), e = __ldg(offsets + r + 1);
+        if (b >= e || !(wsum[r] < kThinRay) || (status && __ldg(status + r) == TSDFS_MISS)) continue;
+        for (int64_t g = b / 16; g <= (e - 1) / 16; ++g) rec[g * 16].pad = 1.0f;
+        *(volatile uint32_t*)thin = 1;
     }
 }
 
@@ -361,16 +382,31 @@ __global__ void k_recovery_merge(int64_t n_rays, const uint8_t* __restrict__ sta
 
 }  // namespace
 
-int launch_composite(const SampleRec* rec, const int32_t* offsets, int per_ray, const uint8_t* status, int64_t n_rays,
-                     const int32_t* total_dev, int64_t capacity, Opacity op, float* rgb, float* depth,
-                     float* wsum, float* normal, float* eik, cudaStream_t st) {
+// again: NULL, or a word in device memory that is 0 when nothing is to be done
+int launch_composite_again(const SampleRec* rec, const int32_t* offsets, int per_ray, const uint8_t* status,
+                           int64_t n_rays, const int32_t* total_dev, int64_t capacity, Opacity op, float* rgb,
+                           float* depth, float* wsum, float* normal, float* eik, const uint32_t* again, cudaStream_t st) {
     if (n_rays == 0) return TSDFS_OK;
     const bool warp = n_rays <= kCompWarpRays;
     auto composite = warp ? k_composite_warp : k_composite;
     composite<<<grid_1d(warp ? n_rays * 32 : n_rays, kCompBlock), kCompBlock, 0, st>>>(
         rec, offsets, per_ray, status, n_rays, total_dev, capacity, op, rgb, depth, wsum, normal, eik,
-        device_status_word());
+        device_status_word(), again);
     return cuda_check(cudaGetLastError(), "composite launch");
+}
+
+int launch_composite(const SampleRec* rec, const int32_t* offsets, int per_ray, const uint8_t* status, int64_t n_rays,
+                     const int32_t* total_dev, int64_t capacity, Opacity op, float* rgb, float* depth,
+                     float* wsum, float* normal, float* eik, cudaStream_t st) {
+    return launch_composite_again(rec, offsets, per_ray, status, n_rays, total_dev, capacity, op, rgb, depth, wsum, normal,
+                                  eik, nullptr, st);
+}
+
+int launch_mark_thin(SampleRec* rec, const int32_t* offsets, const uint8_t* status, const float* wsum, int64_t n_rays,
+                     int64_t capacity, uint32_t* thin, cudaStream_t st) {
+    if (n_rays == 0) return TSDFS_OK;
+    k_mark_thin<<<grid_1d(n_rays, 128), 128, 0, st>>>(rec, offsets, status, wsum, n_rays, capacity, thin);
+    return cuda_check(cudaGetLastError(), "mark thin rays launch");
 }
 
 int launch_hier_setup(const tsdfs_grid* g, const float* ray_o, const float* ray_d, int64_t n_rays, float t_near,

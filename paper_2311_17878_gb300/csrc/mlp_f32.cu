@@ -1006,13 +1006,13 @@ __global__ void __launch_bounds__(kThr, 1) k_mlp_f32(F32Params p) {
 }
 
 // Split the parameters into the items' hi and lo images (8 x 8 core matrices, K-major), one
-// 8-column row piece per thread; clears the redo word.  3 MB for the room networks, every call:
+// 8-column row piece per thread; clears the redo words.  3 MB for the room networks, every call:
 // the parameters may have changed since the last one.
 template <int ARCH>
 __global__ void k_split_weights(const float* __restrict__ sdf_w, const float* __restrict__ rgb_w,
                                 uint8_t* __restrict__ packed, uint32_t* __restrict__ redo) {
     using F = FArch<ARCH>;
-    if (blockIdx.x == 0 && threadIdx.x == 0) *redo = 0;
+    if (blockIdx.x == 0 && threadIdx.x == 0) redo[0] = redo[1] = 0;
     constexpr int64_t n8 = F::packed_bytes() / 32;   // 8 columns x 2 parts x 2 bytes
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n8; i += (int64_t)gridDim.x * blockDim.x) {
         int L = 0;

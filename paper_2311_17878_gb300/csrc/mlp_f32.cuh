@@ -5,7 +5,8 @@
 
 namespace tsdfs {
 
-// head of the path's scratch (the rest holds the split weights): word 0 is set when a tile is marked
+// head of the path's scratch (the rest holds the split weights): word 0 is set when a tile is marked by
+// the network kernel, word 1 when tiles are marked for a ray of almost no weight
 constexpr size_t kRedoBytes = 256;
 // first result of a marked group of 64 samples of a value pass
 constexpr uint32_t kRedoBits = 0x7fc5a5a5u;

@@ -138,3 +138,23 @@ def test_colour_layers_over_several_tiles(scene, counts, huge):
     compare(got, ref, depth_rel=DEPTH_REL_F32)
     rc, bits = T.tsdfs_sync_status()
     assert rc == 0, bits
+
+
+def test_rays_of_almost_no_weight():
+    """Room rays whose samples lie in free space keep the SIMT kernel's bits: those of a network scaled by a
+    power of two between two ReLU layers (the same FP32 function), all of whose tiles leave the parts' range."""
+    counts = [1, 16, 17, 40] * 25
+    o, d, b = rays("room", counts, seed=66)
+    free = np.arange(len(counts)) % 8 >= 4
+    b["t_f"] = np.where(free, b["t_n"] - 0.1, b["t_f"]).astype(np.float32)
+    b["t_n"] = np.where(free, 0.4 * b["t_f"], b["t_n"]).astype(np.float32)
+    spec = spec_of("room")
+    got = gpu_render(spec, o, d, b)
+    ref = gpu_render(scaled(spec, "rgb", 1, 2.0 ** 19, True), o, d, b)
+    thin = ref["wsum"] < 9e-4
+    assert 5 <= thin.sum() <= 60
+    for k in ("rgb", "depth", "wsum", "normal"):
+        assert np.array_equal(got[k][thin], ref[k][thin]), k
+    compare(got, ref, depth_rel=DEPTH_REL_F32)
+    rc, bits = T.tsdfs_sync_status()
+    assert rc == 0, bits
