@@ -45,19 +45,19 @@ WORKLOAD = WORKLOADS["view"]
 # over the 10 timed launches of `bench.py --only-main --no-graph --steps 10 --warmup 3` (room views 0-9,
 # network-fused grid, fp16 operands) in one ncu capture; reported only for that
 # configuration and while the kernel sources hash to the ones it was captured on
-MLP_TC_TRAFFIC = {"sha256": "f9a514cb2bb93e350029ef5ca1fd01644e13714e5f37fd6bb7e165b497660758", "bytes_per_launch": 262874086,
+MLP_TC_TRAFFIC = {"sha256": "508be6d8907a9f87b0215d8fba1172d1787711764664c78c763670091e89d4a9", "bytes_per_launch": 263375974,
                   "profile": "profiles/k_mlp_tc_room_view_traffic.md"}
 # the same for k_ray_bounds (the march of Alg. 1) on the same ten timed views
-MARCH_TRAFFIC = {"sha256": "c4307e3a56049f67dc00d5274645fbd858f05161b8c533815f880fbb3a07392b", "bytes_per_launch": 9989350,
+MARCH_TRAFFIC = {"sha256": "65df4dba21b44fef96a0b3ef24f0c80bf18050d138eae939e5ab46905f23370f", "bytes_per_launch": 10004685,
                  "profile": "profiles/k_ray_bounds_room_view_traffic.md"}
 ALGO_FLOP_PER_SAMPLE = 2.25e6   # SDF fwd + minimal reverse-mode grad + colour, 8x256 / 4x256 networks
 # what the tensor-core kernels issue per sample (value + 3 tangent rows through the SDF layers):
 # serial, 64-sample tiles in pairs: 4 rows per sample through SDF layers 0-6 and the folded
 # output layer's value column (N = 16), one row per sample through the colour layers (M = 128
 # over both tiles of a pair; the folded first colour layer with K = 256 + 48); pipelined,
-# 32-sample tiles: 4 rows per sample through both networks (M = 128 colour MMAs with 32 live
-# rows), the SDF MMAs twice with split operands
-EXEC_FLOP_PER_SAMPLE = {"serial": 3.77e6, "pipelined": 5.93e6, "pipelined-split": 9.63e6}
+# 32-sample tiles: 4 rows per sample through the SDF layers, one through the colour layers (M = 128
+# over up to four tiles of a CTA), the SDF MMAs twice with split operands
+EXEC_FLOP_PER_SAMPLE = {"serial": 3.77e6, "pipelined": 4.26e6, "pipelined-split": 7.96e6}
 N_VIEWS_TIMED = 10   # views cycled by the timed steps (4 for the panorama workload)
 QUALITY_PIXELS = 4096          # seeded pixels spread over every timed view (synth.quality_pixels)
 QUALITY_PIXELS_LIVE = 1024     # when the dense reference is rendered during the run (panorama workload)
