@@ -244,9 +244,9 @@ static size_t stash_bytes() {
     return a > b ? (a > c ? a : c) : (b > c ? b : c);
 }
 
-// the network evaluation of every render path
+// the network evaluation of every render path; simt: FP32 on the SIMT kernel alone
 static int run_full_mlp(const tsdfs_mlp* m, const SampleSource& src, SampleRec* rec, int64_t max_samples,
-                        uint8_t* stash, cudaStream_t st) {
+                        uint8_t* stash, cudaStream_t st, bool simt = false) {
     if (m->precision != TSDFS_PREC_F32) {
         if (netkernel_of(m->precision) == TSDFS_NETKERNEL_PIPELINED) {
             ProfScope ps("mlp_pipe", st);
@@ -259,23 +259,24 @@ static int run_full_mlp(const tsdfs_mlp* m, const SampleSource& src, SampleRec* 
     // mlp_f32.cu), at every size: one 32-sample tile takes less time than a SIMT tile of 16
     ProfScope ps("mlp_f32", st);
     const NetParams np = net_params(m);
-    const uint32_t* redo = reinterpret_cast<const uint32_t*>(stash);
-    int rc = launch_mlp_full_f32(m, src, rec, max_samples, stash, st);
+    const uint32_t* redo = simt ? nullptr : reinterpret_cast<const uint32_t*>(stash);
+    int rc = simt ? TSDFS_OK : launch_mlp_full_f32(m, src, rec, max_samples, stash, st);
     if (rc) return rc;
     return m->arch == TSDFS_ARCH_TINY ? launch_mlp_full_simt<TSDFS_ARCH_TINY>(np, src, rec, max_samples, redo, st)
                                       : launch_mlp_full_simt<TSDFS_ARCH_ROOM>(np, src, rec, max_samples, redo, st);
 }
 
 // SDF values only (the samplers' coarse passes)
-static int run_value_mlp(const tsdfs_mlp* m, const SampleSource& src, float* f_out, uint8_t* stash, cudaStream_t st) {
+static int run_value_mlp(const tsdfs_mlp* m, const SampleSource& src, float* f_out, uint8_t* stash, cudaStream_t st,
+                         bool simt = false) {
     if (m->precision != TSDFS_PREC_F32) {
         ProfScope ps("mlp_value_tc", st);
         return launch_mlp_value_tc(m, src, f_out, st);
     }
     ProfScope ps("mlp_value_f32", st);
     const NetParams np = net_params(m);
-    const uint32_t* redo = reinterpret_cast<const uint32_t*>(stash);
-    int rc = launch_mlp_value_f32(m, src, f_out, stash, st);
+    const uint32_t* redo = simt ? nullptr : reinterpret_cast<const uint32_t*>(stash);
+    int rc = simt ? TSDFS_OK : launch_mlp_value_f32(m, src, f_out, stash, st);
     if (rc) return rc;
     return m->arch == TSDFS_ARCH_TINY ? launch_mlp_value_simt<TSDFS_ARCH_TINY>(np, src, f_out, redo, st)
                                       : launch_mlp_value_simt<TSDFS_ARCH_ROOM>(np, src, f_out, redo, st);
@@ -571,7 +572,12 @@ extern "C" int render_rays_hier(const tsdfs_mlp* mlp, const tsdfs_grid* grid, co
     cs.per_ray = n_coarse;
     cs.total_host = n_rays * n_coarse;
     cs.capacity = n_rays * n_coarse;
-    rc = run_value_mlp(mlp, cs, w.fc, w.stash, st);
+    // With few coarse samples over the whole box a section is as long as the room networks' surfaces are sharp:
+    // where the fine samples fall, and the opacities there, hang on the last bits of f.  8 coarse samples:
+    // colours and normals of the FP32 kernels up to 4e-5 (2-norm) apart, and the SIMT kernel's 3e-5 to 4e-4
+    // from 64 bits; 33 and 64: below 2e-5.  So few stay with the SIMT kernel.
+    const bool simt = mlp->precision == TSDFS_PREC_F32 && mlp->arch == TSDFS_ARCH_ROOM && n_coarse < 32;
+    rc = run_value_mlp(mlp, cs, w.fc, w.stash, st, simt);
     if (rc) return rc;
     {
         ProfScope ps("hier_fine", st);
@@ -585,7 +591,7 @@ extern "C" int render_rays_hier(const tsdfs_mlp* mlp, const tsdfs_grid* grid, co
     fs.per_ray = n_h;
     fs.total_host = n_rays * n_h;
     fs.capacity = n_rays * n_h;
-    rc = run_full_mlp(mlp, fs, w.rec, n_rays * n_h, w.stash, st);
+    rc = run_full_mlp(mlp, fs, w.rec, n_rays * n_h, w.stash, st, simt);
     if (rc) return rc;
     ProfScope ps("composite", st);
     return launch_composite(w.rec, nullptr, n_h, w.status, n_rays, nullptr, n_rays * n_h, opacity_of(mlp),

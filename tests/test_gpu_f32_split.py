@@ -158,3 +158,30 @@ def test_rays_of_almost_no_weight():
     compare(got, ref, depth_rel=DEPTH_REL_F32)
     rc, bits = T.tsdfs_sync_status()
     assert rc == 0, bits
+
+
+@pytest.mark.parametrize("n_coarse", [8, 31, 32, 64])
+def test_sampler_with_few_coarse_samples(n_coarse):
+    """Room networks over the whole box: below 32 coarse samples the SIMT kernel's bits (those of a network
+    scaled by a power of two between two ReLU layers, the same FP32 function), from there the split's."""
+    o, d, _ = rays("room", [1] * 150, seed=67)
+    wl = synth.room_workload(with_views=False)
+    spec, bp = spec_of("room"), wl.bounds
+    g = T.Grid(wl.grid)
+
+    def render(spec):
+        out = T.HierRenderer(T.Mlp(spec), len(o), n_coarse=n_coarse, n_fine=4).render(g, dev(o), dev(d), bp.t_near, bp.t_far)
+        return {k: getattr(out, k).cpu().numpy() for k in ("rgb", "depth", "wsum", "normal")}
+
+    got = render(spec)
+    if n_coarse < 32:
+        ref = render(scaled(spec, "rgb", 1, 2.0 ** 19, True))
+        for k in got:
+            assert np.array_equal(got[k], ref[k]), k
+    else:
+        t0, te, ok = cgrid.clip_rays(wl.grid, o, d, bp.t_near, bp.t_far, "f32")
+        assert np.all(ok)
+        ref = orr.render_hier(orr.Net(spec), o, d, t0.astype(np.float64), te.astype(np.float64), n_coarse, 4)
+        compare(got, {k: ref[k].detach().numpy() for k in got}, depth_rel=DEPTH_REL_F32)
+    rc, bits = T.tsdfs_sync_status()
+    assert rc == 0, bits
