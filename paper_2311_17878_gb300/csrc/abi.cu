@@ -255,7 +255,7 @@ static int run_full_mlp(const tsdfs_mlp* m, const SampleSource& src, SampleRec* 
         ProfScope ps("mlp_tc", st);
         return launch_mlp_full_tc(m, src, rec, max_samples, stash, st);
     }
-    // FP32: the split tensor-core kernel, then the SIMT kernel over the tiles it marked (see
+    // FP32: the split tensor-core kernel, then the SIMT kernel over the samples it marked (see
     // mlp_f32.cu), at every size: one 32-sample tile takes less time than a SIMT tile of 16
     ProfScope ps("mlp_f32", st);
     const NetParams np = net_params(m);

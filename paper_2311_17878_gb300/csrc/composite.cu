@@ -152,8 +152,8 @@ __global__ void __launch_bounds__(kCompBlock) k_composite_warp(const SampleRec* 
     }
 }
 
-// Marks the groups of 16 samples of rays with a weight sum below kThinRay (pad of a group's first
-// record) and sets *thin if there is one.  Such a ray's opacities are differences of sigmoids near 1,
+// Marks the samples of rays with a weight sum below kThinRay (pad of their records) and sets *thin if there
+// is one.  Such a ray's opacities are differences of sigmoids near 1,
 // a few units in the last place each, and its depth and normal are divided by their sum: they hang on the last
 // bits of f.
 __global__ void k_mark_thin(SampleRec* __restrict__ rec, const int32_t* __restrict__ offsets,
@@ -163,7 +163,7 @@ __global__ void k_mark_thin(SampleRec* __restrict__ rec, const int32_t* __restri
     for (int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; r < n_rays; r += (int64_t)gridDim.x * blockDim.x) {
         const int64_t b = __ldg(offsets + r), e = __ldg(offsets + r + 1);
         if (b >= e || !(wsum[r] < kThinRay) || (status && __ldg(status + r) == TSDFS_MISS)) continue;
-        for (int64_t g = b / 16; g <= (e - 1) / 16; ++g) rec[g * 16].pad = 1.0f;
+        for (int64_t g = b; g < e; ++g) rec[g].pad = 1.0f;
         *(volatile uint32_t*)thin = 1;
     }
 }

@@ -47,10 +47,11 @@
 // VALUE: the samplers' coarse pass (SDF value only): 128 samples per tile, one row each, no
 // gradient and no colour network.
 //
-// Range: an operand beyond 2000, a non-finite value or a gradient below 1e-4 marks its tile (the
-// first record of each 16 samples gets pad = 1, a value tile's first results a NaN of a fixed
-// payload) and a launch of the SIMT kernel evaluates the marked tiles again: the split has no
-// exponent range to spare there.  Nothing is marked with networks of ordinary weights.
+// Range: an operand beyond 2000, a non-finite value or a gradient below 1e-4 marks its sample
+// (pad = 1 in its record; in the coarse pass a NaN of a fixed payload as its value) and a launch of
+// the SIMT kernel evaluates the marked samples again: the split has no exponent range to spare there.
+// Nothing is marked with networks of ordinary weights.  A sample's mark depends on its own rows only, so
+// that its results do not depend on which samples share its tile or its unit.
 //
 // Roles: warps 0-11 epilogue (TMEM lane quarter w % 4, column part w / 4), warp 12 MMA issue,
 // warps 13-15 weight producers.  Every wait is bounded; on timeout the kernel records
@@ -143,11 +144,11 @@ template <int ARCH> struct FArch {
     template <bool VALUE> __host__ __device__ static constexpr uint32_t table_floats() {
         return VALUE ? kTileV * (4 + 6 * A::kPeSdf) : kTile * (8 + 6 * (A::kPeSdf + A::kPeDir));
     }
-    // net_0's weights and partial sums (3 parts x 128 rows); the record's SDF half, the colour
-    // output's weights and partial sums (3 parts x 3 colours x 128 rows)
+    // net_0's weights and partial sums (3 parts x 128 rows), the samples' marks; the record's SDF half,
+    // the colour output's weights and partial sums (3 parts x 3 colours x 128 rows)
     static constexpr int kW0 = pad16(A::sdf(LS - 1).in), kWc = pad16(A::rgb(A::kRgbLayers - 1).in);
     template <bool VALUE> __host__ __device__ static constexpr uint32_t scratch_floats() {
-        return kW0 + kParts * 128 + (VALUE ? 0 : kTile * 8 + 3 * kWc + kParts * 3 * 128);
+        return kW0 + kParts * 128 + 128 + (VALUE ? 0 : kTile * 8 + 3 * kWc + kParts * 3 * 128);
     }
     // items of a tile's SDF layers, and of a unit's colour layers (the first one's phases take one
     // more each, the operand columns beyond the features)
@@ -250,7 +251,8 @@ __global__ void __launch_bounds__(kThr, 1) k_mlp_f32(F32Params p) {
     float* s_pd = s_pe + TS * A::kPeSdf * 6;   // of the direction
     float* s_w0 = s_x + F::template table_floats<VALUE>();
     float* s_dot = s_w0 + F::kW0;                  // [part][row]
-    float* s_out = s_dot + kParts * 128;           // [sample][8]
+    volatile uint32_t* s_bad = reinterpret_cast<uint32_t*>(s_dot + kParts * 128);   // [tile of the unit][sample]
+    float* s_out = s_dot + kParts * 128 + 128;     // [sample][8]
     float* s_wc = s_out + kTile * 8;               // [colour][input]
     float* s_cdot = s_wc + 3 * F::kWc;             // [part][colour][row]
     Item* items = reinterpret_cast<Item*>(s_w0 + F::template scratch_floats<VALUE>());
@@ -258,7 +260,6 @@ __global__ void __launch_bounds__(kThr, 1) k_mlp_f32(F32Params p) {
     // bars: full[2], empty[2], acc[2], drained[2], operand[2], epi, end, parked, back
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 14);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
-    volatile uint32_t* s_mark = tmem_slot + 2;
     const uint32_t bar_full = smem_u32(bars), bar_empty = smem_u32(bars + kStages);
     const uint32_t bar_acc = smem_u32(bars + 4), bar_drained = smem_u32(bars + 6), bar_op = smem_u32(bars + 8),
                    bar_epi = smem_u32(bars + 10), bar_end = smem_u32(bars + 11), bar_park = smem_u32(bars + 12),
@@ -286,7 +287,6 @@ __global__ void __launch_bounds__(kThr, 1) k_mlp_f32(F32Params p) {
         mbar_init(bar_park, kEpi);
         mbar_init(bar_back, 1);
         *abort_flag = 0;
-        *s_mark = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     // the items in order: layers, phases, chunks; a thread writes one layer's
@@ -334,6 +334,7 @@ __global__ void __launch_bounds__(kThr, 1) k_mlp_f32(F32Params p) {
             s_bias[F::bias_base(L) + i] = r >= 0 ? __ldg(b + r) : 0.0f;
         }
     });
+    for (int i = threadIdx.x; i < 128; i += kThr) s_bad[i] = 0;
     for (int i = threadIdx.x; i < F::kW0; i += kThr) {
         constexpr int K = A::sdf(LS - 1).in;
         s_w0[i] = i < K ? __ldg(p.sdf_w + F::param_offset(LS - 1) + i) : 0.0f;
@@ -463,8 +464,12 @@ __global__ void __launch_bounds__(kThr, 1) k_mlp_f32(F32Params p) {
         const int et = threadIdx.x;
         uint32_t phs = 0, epi_ph = 0, backs = 0;   // phases waited for, epilogue barriers, units fetched back
         uint32_t buf = 0, cor = 0;                // TMEM columns of the phase in hand: main, correction
-        __half2 big = __float2half2_rn(0.0f);     // largest |operand| (scaled high parts) of this thread, or NaN
-        const __half2 kHuge = __float2half2_rn(65504.0f);
+        // largest |operand| (scaled high parts) or NaN of the sample this thread works for; VALUE: of each of
+        // its four rows' samples
+        constexpr int kOwn = VALUE ? 4 : 1;
+        __half2 big[kOwn];
+#pragma unroll
+        for (int r = 0; r < kOwn; ++r) big[r] = __float2half2_rn(0.0f);
         bool ok = true;
         auto epi_sync = [&]() -> bool {
             __syncwarp();
@@ -515,20 +520,20 @@ __global__ void __launch_bounds__(kThr, 1) k_mlp_f32(F32Params p) {
             const int s = sample_of(r);
             return enc_tab(s_x + s * kXRow, s_pe + s * A::kPeSdf * 6, A::kPeSdf, j, VALUE ? 0 : r);
         };
-        auto split = [&](float a, float b, uint32_t& hi, uint32_t& lo) {
+        auto split = [&](float a, float b, uint32_t& hi, uint32_t& lo, __half2& most) {
             split_f32(a, b, hi, lo);
-            big = __hmax2_nan(big, __habs2(*reinterpret_cast<const __half2*>(&hi)));
+            most = __hmax2_nan(most, __habs2(*reinterpret_cast<const __half2*>(&hi)));
         };
         // split the four row groups' column pairs v (operands times kUp)
         auto split4 = [&](const float (&v)[8], uint32_t (&o)[8]) {
 #pragma unroll
-            for (int r = 0; r < 4; ++r) split(v[2 * r], v[2 * r + 1], o[r], o[4 + r]);
+            for (int r = 0; r < 4; ++r) split(v[2 * r], v[2 * r + 1], o[r], o[4 + r], big[VALUE ? r : 0]);
         };
-        // whether a value of this warp is out of the parts' range since the last call
-        auto out_of_range = [&]() {
-            const float2 m = __half22float2(big);
-            big = __float2half2_rn(0.0f);
-            return __any_sync(0xffffffffu, !(fmaxf(m.x, m.y) < kUp * kLimit && m.x == m.x && m.y == m.y)) != 0;
+        // whether a value since the last call was out of the parts' range
+        auto out_of_range = [&](__half2& most) {
+            const float2 m = __half22float2(most);
+            most = __float2half2_rn(0.0f);
+            return !(fmaxf(m.x, m.y) < kUp * kLimit && m.x == m.x && m.y == m.y);
         };
         auto store4 = [&](uint32_t rh, uint32_t rl, int c, const uint32_t (&o)[8]) {
             const uint32_t co = (uint32_t)(c >> 3) * 128u;
@@ -772,18 +777,18 @@ __global__ void __launch_bounds__(kThr, 1) k_mlp_f32(F32Params p) {
                     if constexpr (VALUE) {
                         if (last) {
                             // the SDF values, and the next tile's input
+#pragma unroll
+                            for (int r = 0; r < 4; ++r)
+                                if (out_of_range(big[r])) s_bad[sample_of(r)] = 1;
                             if (!epi_sync()) { ok = false; break; }
                             if (et < TS) {
                                 const float f = p.scale * (s_dot[et] + s_dot[128 + et] + s_dot[256 + et] + b0);
-                                if (!(fabsf(f) < __int_as_float(0x7f800000))) big = kHuge;
-                                if (tile * TS + et < total) p.f_out[tile * TS + et] = f;
-                            }
-                            if (out_of_range() && lane == 0) *s_mark = (uint32_t)(tile + 1);
-                            if (!epi_sync()) { ok = false; break; }
-                            if (et == 0 && *s_mark == (uint32_t)(tile + 1)) {
-                                for (int k = 0; k < TS / 64; ++k)
-                                    if (tile * TS + 64 * k < total) p.f_out[tile * TS + 64 * k] = __uint_as_float(kRedoBits);
-                                atomicExch(p.redo, 1u);
+                                const bool bad = s_bad[et] != 0 || !(fabsf(f) < __int_as_float(0x7f800000));
+                                s_bad[et] = 0;
+                                if (tile * TS + et < total) {
+                                    p.f_out[tile * TS + et] = bad ? __uint_as_float(kRedoBits) : f;
+                                    if (bad) atomicExch(p.redo, 1u);
+                                }
                             }
                             if (kt + 1 < mine) {
                                 if (!build_table(tile_of(kt + 1))) { ok = false; break; }
@@ -827,7 +832,7 @@ __global__ void __launch_bounds__(kThr, 1) k_mlp_f32(F32Params p) {
                                         z[e] = fmaf(z[e], kDown, bias[ph * kPh + c + fc + e]) * kUp;
                                     }
                                     uint32_t hi, lo;
-                                    split(z[0], z[1], hi, lo);
+                                    split(z[0], z[1], hi, lo, big[0]);
                                     uint32_t* at = reinterpret_cast<uint32_t*>(pf + (ph * kPh + c) / 8 * 128);
                                     at[0] = hi;
                                     at[F::kParkF / 4] = lo;
@@ -857,16 +862,20 @@ __global__ void __launch_bounds__(kThr, 1) k_mlp_f32(F32Params p) {
                                     R4[2] = make_float4(so[0], so[1], so[2], 0.0f);
                                     p.rec[g].gnorm = gn;
                                     const float inf = __int_as_float(0x7f800000);
-                                    if (!(gn >= kMinGrad && gn < inf) || !(fabsf(f) < inf)) big = kHuge;
+                                    if (!(gn >= kMinGrad && gn < inf) || !(fabsf(f) < inf)) s_bad[kTile * slot + s] = 1;
                                 }
                             }
                         }
                         if (!ok) break;
+                        // the tile's SDF operands and features (read and cleared by the unit's last thread for the
+                        // sample, an epi_sync before this tile's first mark)
+                        if (out_of_range(big[0])) s_bad[kTile * slot + sample_of(0)] = 1;
                         if (!epi_sync()) { ok = false; break; }
                         // x~, direction encoding, unit normal: one 8-column group of a sample per thread
                         if (et < kTile * (F::kXp / 8)) {
                             const int s = et / (F::kXp / 8), c = 8 * (et % (F::kXp / 8));
                             uint32_t o[8];
+                            __half2 most = __float2half2_rn(0.0f);
 #pragma unroll
                             for (int k = 0; k < 4; ++k) {
                                 float v[2];
@@ -879,8 +888,9 @@ __global__ void __launch_bounds__(kThr, 1) k_mlp_f32(F32Params p) {
                                         v[e] = enc_tab(s_x + s * 8 + 3, s_pd + s * A::kPeDir * 6, A::kPeDir, j - 3, 0);
                                     else if (j < F::kX) v[e] = s_out[s * 8 + j - 3 - A::kDirEnc];
                                 }
-                                split(v[0] * kUp, v[1] * kUp, o[k], o[4 + k]);
+                                split(v[0] * kUp, v[1] * kUp, o[k], o[4 + k], most);
                             }
+                            if (out_of_range(most)) s_bad[kTile * slot + s] = 1;
                             uint8_t* at = park + 2 * F::kParkF + a_off(32 * (s >> 3) + 8 * slot + (s & 7), c, F::kXp);
                             *reinterpret_cast<uint4*>(at) = make_uint4(o[0], o[1], o[2], o[3]);
                             *reinterpret_cast<uint4*>(at + F::kParkX) = make_uint4(o[4], o[5], o[6], o[7]);
@@ -908,6 +918,9 @@ __global__ void __launch_bounds__(kThr, 1) k_mlp_f32(F32Params p) {
                     const bool last = L == F::NL - 2;          // the colours' dot products are taken here
                     const uint32_t rh = row_at(a_hi, lane, Np), rl = row_at(a_lo, lane, Np);
                     float cd[3][4] = {};
+                    __half2 most[4];                           // of each row group
+#pragma unroll
+                    for (int r = 0; r < 4; ++r) most[r] = __float2half2_rn(0.0f);
                     auto act = [&](int c, const float (&z)[8], uint32_t (&o)[8]) {
                         float v[8];
                         const float2 b = *reinterpret_cast<const float2*>(bias + c + fc);
@@ -926,7 +939,8 @@ __global__ void __launch_bounds__(kThr, 1) k_mlp_f32(F32Params p) {
                                 for (int r = 0; r < 4; ++r) cd[k][r] = fmaf(v[2 * r + 1], w.y, fmaf(v[2 * r], w.x, cd[k][r]));
                             }
                         } else {
-                            split4(v, o);
+#pragma unroll
+                            for (int r = 0; r < 4; ++r) split(v[2 * r], v[2 * r + 1], o[r], o[4 + r], most[r]);
                         }
                     };
                     uint32_t held[kGrp][8];
@@ -954,6 +968,9 @@ __global__ void __launch_bounds__(kThr, 1) k_mlp_f32(F32Params p) {
                     drained();
                     if (!last) {
                         operand_done(two ? 1 : 0);
+#pragma unroll
+                        for (int r = 0; r < 4; ++r)
+                            if (out_of_range(most[r])) s_bad[kTile * r + 8 * q + sq] = 1;
                         continue;
                     }
                     // ---- the next unit's first layer-0 input (every MMA of this one is complete), the colours ----
@@ -965,15 +982,15 @@ __global__ void __launch_bounds__(kThr, 1) k_mlp_f32(F32Params p) {
                             cd[k][r] += __shfl_xor_sync(0xffffffffu, cd[k][r], 2);
                             if ((lane & 3) == 0) s_cdot[(pt * 3 + k) * 128 + 32 * q + 8 * r + sq] = cd[k][r] * (1.0f / kUp);
                         }
-                    if (out_of_range() && lane == 0) *s_mark = (uint32_t)(tile + 1);
                     if (!epi_sync()) { ok = false; break; }
                     if (kt + 1 < mine) write_input0();
                     if (et < 128) {
                         const float* bc = p.rgb_w + F::param_offset(F::NL - 1) + 3 * F::layer(F::NL - 1).in;
-                        const int j = (et >> 3) & 3;                       // tile of the unit
-                        const int64_t g = tile_of(kt - slot + j) * kTile + 8 * (et >> 5) + (et & 7);
+                        const int j = (et >> 3) & 3, s = 8 * (et >> 5) + (et & 7);   // tile of the unit, its sample
+                        const int64_t g = tile_of(kt - slot + j) * kTile + s;
+                        bool bad = s_bad[kTile * j + s] != 0;
+                        s_bad[kTile * j + s] = 0;
                         if (j <= slot && g < total) {
-                            bool bad = false;
                             float* R = reinterpret_cast<float*>(p.rec + g);
 #pragma unroll
                             for (int k = 0; k < 3; ++k) {
@@ -982,8 +999,8 @@ __global__ void __launch_bounds__(kThr, 1) k_mlp_f32(F32Params p) {
                                 bad = bad || !(fabsf(c3) < __int_as_float(0x7f800000));
                                 R[4 + k] = 1.0f / (1.0f + expf(-c3));
                             }
-                            if (bad || (*s_mark == (uint32_t)(tile + 1) && (g % 16) == 0)) {
-                                p.rec[g / 16 * 16].pad = 1.0f;
+                            if (bad) {
+                                p.rec[g].pad = 1.0f;
                                 atomicExch(p.redo, 1u);
                             }
                         }

@@ -229,7 +229,8 @@ __device__ void rgb_network(Smem& sm, const NetParams& np, int& cur) {
 #undef TSDFS_RGB
 }
 
-// Full evaluation: f, grad f, colour for each sample -> records.
+// Full evaluation: f, grad f, colour for each sample -> records.  With `redo`: the marked samples only
+// (pad != 0 in their records), a tile wherever it holds one.
 template <int ARCH>
 __global__ void __launch_bounds__(kThreads, 1) k_mlp_full(NetParams np, SampleSource src, SampleRec* __restrict__ rec,
                                                           const uint32_t* redo, uint32_t* dev_status) {
@@ -244,8 +245,13 @@ __global__ void __launch_bounds__(kThreads, 1) k_mlp_full(NetParams np, SampleSo
     }
     const int64_t n_tiles = (total + kTS - 1) / kTS;
     for (int64_t tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
+        bool mark = true;
+        if (redo) {
+            const int64_t g = tile * kTS + threadIdx.x;
+            mark = threadIdx.x < kTS && g < total && rec[g].pad != 0.0f;
+            if (!__syncthreads_or(mark)) continue;
+        }
         __syncthreads();
-        if (redo && rec[tile * kTS].pad == 0.0f) continue;   // not marked
         if (threadIdx.x < kTS) {
             const int s = threadIdx.x;
             const int64_t g = tile * kTS + s;
@@ -280,7 +286,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_mlp_full(NetParams np, SampleSo
             }
             sm.tval[s] = t;
             sm.dval[s] = dl;
-            sm.valid[s] = ok;
+            sm.valid[s] = ok && mark;
             sm.ray[s] = r;
         }
         __syncthreads();
@@ -361,7 +367,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_mlp_full(NetParams np, SampleSo
     }
 }
 
-// SDF values only (hierarchical coarse pass): 4*kTS samples per tile, one row each.
+// SDF values only (hierarchical coarse pass): 4*kTS samples per tile, one row each.  With `redo`: the
+// marked samples only (kRedoBits as their value).
 template <int ARCH>
 __global__ void __launch_bounds__(kThreads, 1) k_mlp_value(NetParams np, SampleSource src, float* __restrict__ f_out,
                                                            const uint32_t* redo, uint32_t* dev_status) {
@@ -377,8 +384,11 @@ __global__ void __launch_bounds__(kThreads, 1) k_mlp_value(NetParams np, SampleS
     constexpr int TS = 4 * kTS;
     const int64_t n_tiles = (total + TS - 1) / TS;
     for (int64_t tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
+        if (redo) {
+            const int64_t g = tile * TS + threadIdx.x;
+            if (!__syncthreads_or(threadIdx.x < TS && g < total && __float_as_uint(f_out[g]) == kRedoBits)) continue;
+        }
         __syncthreads();
-        if (redo && __float_as_uint(f_out[tile * TS]) != kRedoBits) continue;   // not marked
         if (threadIdx.x < TS) {
             const int s = threadIdx.x;
             const int64_t g = tile * TS + s;
@@ -419,7 +429,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_mlp_value(NetParams np, SampleS
             if (cg == 0) {
                 for (int r = 0; r < 4; ++r) {
                     const int64_t g = tile * TS + 4 * s + r;
-                    if (g < total) f_out[g] = np.scale * (acc[r][0] + __ldg(b));
+                    if (g < total && (!redo || __float_as_uint(f_out[g]) == kRedoBits))
+                        f_out[g] = np.scale * (acc[r][0] + __ldg(b));
                 }
             }
         }
