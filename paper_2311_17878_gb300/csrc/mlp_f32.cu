@@ -50,7 +50,10 @@
 // Range: an operand beyond 2000, a non-finite value or a gradient below 1e-4 marks its sample
 // (pad = 1 in its record; in the coarse pass a NaN of a fixed payload as its value) and a launch of
 // the SIMT kernel evaluates the marked samples again: the split has no exponent range to spare there.
-// Nothing is marked with networks of ordinary weights.  A sample's mark depends on its own rows only, so
+// So is, towards the floor, a sample with a hidden layer whose tangents (colours: activations) all lie
+// below 1.9e-6, where the scaled high part is subnormal and the two have fewer than 22 bits; a layer
+// whose weights do marks every sample.  Nothing is marked with networks of ordinary weights (the largest
+// tangent of a hidden layer of the fitted networks: 0.3 to 1).  A sample's mark depends on its own rows only, so
 // that its results do not depend on which samples share its tile or its unit.
 //
 // Roles: warps 0-11 epilogue (TMEM lane quarter w % 4, column part w / 4), warp 12 MMA issue,
@@ -82,6 +85,7 @@ constexpr float kDown = 1.0f / (kUp * kUp), kLoDown = 1.0f / kLoUp;
 constexpr float kLimit = 2000.0f;     // largest operand the high part is trusted with
 constexpr float kBias0 = 1.7e-8f, kBias1 = 1.58e-8f;   // what a main sum of n MMAs lacks: kBias0 + n kBias1
 constexpr float kMinGrad = 1e-4f;
+constexpr float kFloor = 1.0f / (16384.0f * kUp);   // 1.9e-6: the scaled high part of less is subnormal
 constexpr int kMaxCtas = 192;         // CTAs with a place to park
 constexpr float kRsqrt2 = 0.70710678118654752f;
 
@@ -144,11 +148,12 @@ template <int ARCH> struct FArch {
     template <bool VALUE> __host__ __device__ static constexpr uint32_t table_floats() {
         return VALUE ? kTileV * (4 + 6 * A::kPeSdf) : kTile * (8 + 6 * (A::kPeSdf + A::kPeDir));
     }
+    static constexpr int kChecked = NL - 2 - LS;   // colour layers whose outputs become operands
     // net_0's weights and partial sums (3 parts x 128 rows), the samples' marks; the record's SDF half,
-    // the colour output's weights and partial sums (3 parts x 3 colours x 128 rows)
+    // the colour output's weights and partial sums (3 parts x 3 colours x 128 rows), the floor's checks
     static constexpr int kW0 = pad16(A::sdf(LS - 1).in), kWc = pad16(A::rgb(A::kRgbLayers - 1).in);
     template <bool VALUE> __host__ __device__ static constexpr uint32_t scratch_floats() {
-        return kW0 + kParts * 128 + 128 + (VALUE ? 0 : kTile * 8 + 3 * kWc + kParts * 3 * 128);
+        return kW0 + kParts * 128 + 32 + (VALUE ? 0 : kTile * 8 + 3 * kWc + kParts * 3 * 128 + (kTile + kChecked * 128) / 4);
     }
     // items of a tile's SDF layers, and of a unit's colour layers (the first one's phases take one
     // more each, the operand columns beyond the features)
@@ -219,6 +224,8 @@ __device__ __forceinline__ void split_f32(float a, float b, uint32_t& hi, uint32
     lo = *reinterpret_cast<const uint32_t*>(&l);
 }
 
+__device__ __forceinline__ __half2 from_bits(uint32_t u) { return *reinterpret_cast<const __half2*>(&u); }
+
 // softplus_beta(z) = max(z, 0) + log(1 + e^{-beta |z|}) / beta and its slope sigma(beta z).  The
 // fast exponential and logarithm measure the same errors in f and grad f as expf and an FP32
 // series for the logarithm (|grad f| 6.3e-8 off through the tiny networks either way).
@@ -251,15 +258,20 @@ __global__ void __launch_bounds__(kThr, 1) k_mlp_f32(F32Params p) {
     float* s_pd = s_pe + TS * A::kPeSdf * 6;   // of the direction
     float* s_w0 = s_x + F::template table_floats<VALUE>();
     float* s_dot = s_w0 + F::kW0;                  // [part][row]
-    volatile uint32_t* s_bad = reinterpret_cast<uint32_t*>(s_dot + kParts * 128);   // [tile of the unit][sample]
-    float* s_out = s_dot + kParts * 128 + 128;     // [sample][8]
+    volatile uint8_t* s_bad = reinterpret_cast<volatile uint8_t*>(s_dot + kParts * 128);   // [tile of the unit][sample]
+    float* s_out = s_dot + kParts * 128 + 32;      // [sample][8]
     float* s_wc = s_out + kTile * 8;               // [colour][input]
     float* s_cdot = s_wc + 3 * F::kWc;             // [part][colour][row]
+    // whether the tangents of each sample of the tile reach the floor in every layer, and the activations of
+    // each sample of the unit in each colour layer
+    volatile uint8_t* s_tan = reinterpret_cast<volatile uint8_t*>(s_cdot + kParts * 3 * 128);
+    volatile uint8_t* s_act = s_tan + kTile;       // [colour layer][tile of the unit][sample]
     Item* items = reinterpret_cast<Item*>(s_w0 + F::template scratch_floats<VALUE>());
     uint64_t* bars = reinterpret_cast<uint64_t*>(items + NT);
     // bars: full[2], empty[2], acc[2], drained[2], operand[2], epi, end, parked, back
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 14);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+    volatile uint32_t* s_low = tmem_slot + 2;   // a layer's weights are all below the floor
     const uint32_t bar_full = smem_u32(bars), bar_empty = smem_u32(bars + kStages);
     const uint32_t bar_acc = smem_u32(bars + 4), bar_drained = smem_u32(bars + 6), bar_op = smem_u32(bars + 8),
                    bar_epi = smem_u32(bars + 10), bar_end = smem_u32(bars + 11), bar_park = smem_u32(bars + 12),
@@ -287,6 +299,9 @@ __global__ void __launch_bounds__(kThr, 1) k_mlp_f32(F32Params p) {
         mbar_init(bar_park, kEpi);
         mbar_init(bar_back, 1);
         *abort_flag = 0;
+        uint32_t low = 0;
+        for (int L = 0; L < NLr; ++L) low |= __ldg(p.redo + kLowWord + L);
+        *s_low = low;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     // the items in order: layers, phases, chunks; a thread writes one layer's
@@ -335,6 +350,8 @@ __global__ void __launch_bounds__(kThr, 1) k_mlp_f32(F32Params p) {
         }
     });
     for (int i = threadIdx.x; i < 128; i += kThr) s_bad[i] = 0;
+    if constexpr (!VALUE)
+        for (int i = threadIdx.x; i < kTile + F::kChecked * 128; i += kThr) s_tan[i] = 0;
     for (int i = threadIdx.x; i < F::kW0; i += kThr) {
         constexpr int K = A::sdf(LS - 1).in;
         s_w0[i] = i < K ? __ldg(p.sdf_w + F::param_offset(LS - 1) + i) : 0.0f;
@@ -470,6 +487,9 @@ __global__ void __launch_bounds__(kThr, 1) k_mlp_f32(F32Params p) {
         __half2 big[kOwn];
 #pragma unroll
         for (int r = 0; r < kOwn; ++r) big[r] = __float2half2_rn(0.0f);
+        // full evaluation: the same of its tangents in the layer in hand, and the smallest such of its layers
+        constexpr uint32_t kInf2 = 0x7c007c00u;
+        __half2 tang = __float2half2_rn(0.0f), least = from_bits(kInf2);
         bool ok = true;
         auto epi_sync = [&]() -> bool {
             __syncwarp();
@@ -527,8 +547,18 @@ __global__ void __launch_bounds__(kThr, 1) k_mlp_f32(F32Params p) {
         // split the four row groups' column pairs v (operands times kUp)
         auto split4 = [&](const float (&v)[8], uint32_t (&o)[8]) {
 #pragma unroll
-            for (int r = 0; r < 4; ++r) split(v[2 * r], v[2 * r + 1], o[r], o[4 + r], big[VALUE ? r : 0]);
+            for (int r = 0; r < 4; ++r) {
+                if constexpr (VALUE) split(v[2 * r], v[2 * r + 1], o[r], o[4 + r], big[r]);
+                else split(v[2 * r], v[2 * r + 1], o[r], o[4 + r], r > 0 ? tang : big[0]);
+            }
         };
+        // the tangents since the last call join what out_of_range tells of
+        auto fold_tangents = [&]() {
+            big[0] = __hmax2_nan(big[0], tang);
+            tang = __float2half2_rn(0.0f);
+        };
+        // whether one of two largest high parts is above the floor: a normal number
+        auto reaches = [](__half2 most) { return (*reinterpret_cast<const uint32_t*>(&most) & kInf2) != 0; };
         // whether a value since the last call was out of the parts' range
         auto out_of_range = [&](__half2& most) {
             const float2 m = __half22float2(most);
@@ -607,6 +637,7 @@ __global__ void __launch_bounds__(kThr, 1) k_mlp_f32(F32Params p) {
                 split4(v, o);
                 store4(rh, rl, 8 * gr, o);
             }
+            if constexpr (!VALUE) fold_tangents();
             operand_done(0);
         };
 
@@ -766,6 +797,17 @@ __global__ void __launch_bounds__(kThr, 1) k_mlp_f32(F32Params p) {
                            });
                     drained();
                     if (store) operand_done(two ? 1 : 0);
+                    if constexpr (!VALUE) {
+                        // (the last layer's tangents are summed in FP32.)  One thread with a tangent above the floor
+                        // in every layer will do
+                        if (!last) {
+                            least = __hmin2(least, tang);
+                        } else {
+                            if (reaches(least)) s_tan[sample_of(0)] = 1;
+                            least = from_bits(kInf2);
+                        }
+                        fold_tangents();
+                    }
                     if (last) {
 #pragma unroll
                         for (int r = 0; r < 4; ++r) {
@@ -783,7 +825,7 @@ __global__ void __launch_bounds__(kThr, 1) k_mlp_f32(F32Params p) {
                             if (!epi_sync()) { ok = false; break; }
                             if (et < TS) {
                                 const float f = p.scale * (s_dot[et] + s_dot[128 + et] + s_dot[256 + et] + b0);
-                                const bool bad = s_bad[et] != 0 || !(fabsf(f) < __int_as_float(0x7f800000));
+                                const bool bad = *s_low != 0 || s_bad[et] != 0 || !(fabsf(f) < __int_as_float(0x7f800000));
                                 s_bad[et] = 0;
                                 if (tile * TS + et < total) {
                                     p.f_out[tile * TS + et] = bad ? __uint_as_float(kRedoBits) : f;
@@ -855,6 +897,8 @@ __global__ void __launch_bounds__(kThr, 1) k_mlp_f32(F32Params p) {
                                 so[0] = gx * inv;
                                 so[1] = gy * inv;
                                 so[2] = gz * inv;
+                                if (s_tan[s] == 0) s_bad[kTile * slot + s] = 1;
+                                s_tan[s] = 0;
                                 const int64_t g = tile * kTile + s;
                                 if (g < total) {
                                     float4* R4 = reinterpret_cast<float4*>(p.rec + g);
@@ -969,8 +1013,11 @@ __global__ void __launch_bounds__(kThr, 1) k_mlp_f32(F32Params p) {
                     if (!last) {
                         operand_done(two ? 1 : 0);
 #pragma unroll
-                        for (int r = 0; r < 4; ++r)
-                            if (out_of_range(most[r])) s_bad[kTile * r + 8 * q + sq] = 1;
+                        for (int r = 0; r < 4; ++r) {
+                            const int at = kTile * r + 8 * q + sq;
+                            if (reaches(most[r])) s_act[(L - LS) * 128 + at] = 1;
+                            if (out_of_range(most[r])) s_bad[at] = 1;
+                        }
                         continue;
                     }
                     // ---- the next unit's first layer-0 input (every MMA of this one is complete), the colours ----
@@ -990,6 +1037,10 @@ __global__ void __launch_bounds__(kThr, 1) k_mlp_f32(F32Params p) {
                         const int64_t g = tile_of(kt - slot + j) * kTile + s;
                         bool bad = s_bad[kTile * j + s] != 0;
                         s_bad[kTile * j + s] = 0;
+                        for (int l = 0; l < F::kChecked; ++l) {
+                            bad = bad || s_act[l * 128 + kTile * j + s] == 0;
+                            s_act[l * 128 + kTile * j + s] = 0;
+                        }
                         if (j <= slot && g < total) {
                             float* R = reinterpret_cast<float*>(p.rec + g);
 #pragma unroll
@@ -999,7 +1050,7 @@ __global__ void __launch_bounds__(kThr, 1) k_mlp_f32(F32Params p) {
                                 bad = bad || !(fabsf(c3) < __int_as_float(0x7f800000));
                                 R[4 + k] = 1.0f / (1.0f + expf(-c3));
                             }
-                            if (bad) {
+                            if (bad || *s_low != 0) {
                                 p.rec[g].pad = 1.0f;
                                 atomicExch(p.redo, 1u);
                             }
@@ -1023,13 +1074,28 @@ __global__ void __launch_bounds__(kThr, 1) k_mlp_f32(F32Params p) {
 }
 
 // Split the parameters into the items' hi and lo images (8 x 8 core matrices, K-major), one
-// 8-column row piece per thread; clears the redo words.  3 MB for the room networks, every call:
+// 8-column row piece per thread; clears the redo words, and tells for each layer whether all its weights
+// are below kFloor (a block per layer, which looks at 256 of them with ordinary weights).  3 MB for the room networks, every call:
 // the parameters may have changed since the last one.
 template <int ARCH>
 __global__ void k_split_weights(const float* __restrict__ sdf_w, const float* __restrict__ rgb_w,
                                 uint8_t* __restrict__ packed, uint32_t* __restrict__ redo) {
     using F = FArch<ARCH>;
     if (blockIdx.x == 0 && threadIdx.x == 0) redo[0] = redo[1] = 0;
+    for (int L = blockIdx.x; L < F::NL - 1; L += gridDim.x) {
+        const Layer ly = F::layer(L);
+        const float* W = (L < F::LS ? sdf_w : rgb_w) + F::param_offset(L);
+        const int n = ly.out * ly.in;
+        int i = L == F::LS - 1 ? ly.in : 0;   // the SDF output's features: net_0's row is no operand
+        bool fine = false, some = false;      // a weight that reaches kFloor, one that is not 0
+        for (; i < n && !fine; i += blockDim.x) {
+            const float w = i + (int)threadIdx.x < n ? fabsf(__ldg(W + i + threadIdx.x)) : 0.0f;
+            some = some || w != 0.0f;
+            fine = __syncthreads_or(!(w < kFloor)) != 0;
+        }
+        if (!fine) some = __syncthreads_or(some) != 0;
+        if (threadIdx.x == 0) redo[kLowWord + L] = !fine && some ? 1u : 0u;
+    }
     constexpr int64_t n8 = F::packed_bytes() / 32;   // 8 columns x 2 parts x 2 bytes
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n8; i += (int64_t)gridDim.x * blockDim.x) {
         int L = 0;

@@ -8,6 +8,8 @@ namespace tsdfs {
 // head of the path's scratch (the rest holds the split weights): word 0 is set when a sample is marked by
 // the network kernel, word 1 when samples are marked for a ray of almost no weight
 constexpr size_t kRedoBytes = 256;
+// word of that head from which on a word per layer tells that its weights are below the parts' range
+constexpr int kLowWord = 8;
 // result of a marked sample of a value pass
 constexpr uint32_t kRedoBits = 0x7fc5a5a5u;
 

@@ -1,6 +1,9 @@
 """The samples that the split FP32 networks (mlp_f32.cu) hand to the SIMT kernel: which samples those are
-depends on the sample alone, so a ray has the same bits in every batch; and the coarse pass's marked
-values against the FP64 oracle, at totals around the halves of its 128-sample tiles."""
+depends on the sample alone, so a ray has the same bits in every batch; the coarse pass's marked
+values against the FP64 oracle, at totals around the halves of its 128-sample tiles; and networks whose
+operands come near the floor of the parts."""
+import dataclasses
+
 import numpy as np
 import pytest
 import torch
@@ -75,5 +78,59 @@ def test_marked_coarse_values(scene, n_rays, n_coarse):
     with torch.no_grad():
         ref = orr.render_hier(orr.Net(spec), o, d, t0.astype(np.float64), te.astype(np.float64), n_coarse, 4)
     compare(got, {k: ref[k].detach().numpy() for k in got}, depth_rel=DEPTH_REL_F32)
+    rc, bits = T.tsdfs_sync_status()
+    assert rc == 0, bits
+
+
+def near_the_floor(spec, case):
+    """The spec with operands of some layers so small that FP16 parts of a fixed scale have few bits left, and
+    the scale given back in the output layer, which takes no parts."""
+    nets = {"sdf": [(W.copy(), b.copy()) for W, b in spec.sdf], "rgb": [(W.copy(), b.copy()) for W, b in spec.rgb]}
+
+    def mul(net, layer, w, b):
+        W, bb = nets[net][layer]
+        nets[net][layer] = (W * np.float32(w), bb * np.float32(b))
+
+    n = len(nets["sdf"])
+    if case == "weights":            # of the last hidden layer: 1e-9 to 1e-7
+        mul("sdf", n - 2, 1e-7, 1e-7)
+        back = 1e7
+    elif case == "tangents":         # 2e-9 between two hidden layers whose weights are 1e-6 to 1e-4
+        for layer in ((0, 1) if n == 4 else (n - 4, n - 3)):
+            mul("sdf", layer, 1e-4, 1e-4)
+        back = 1e8
+    else:                            # colour activations of 1e-11; ReLU is homogeneous: the same function
+        for layer, (w, b) in enumerate([(1e-3, 1e-3), (1e-4, 1e-7), (1e-4, 1e-11), (1.0, 1e-11), (1e11, 1.0)]):
+            mul("rgb", layer, w, b)
+        return dataclasses.replace(spec, rgb=nets["rgb"])
+    W, b = nets["sdf"][-1]
+    W[0] *= np.float32(back)
+    return dataclasses.replace(spec, sdf=nets["sdf"])
+
+
+@pytest.mark.parametrize("scene,case", [("tiny", "weights"), ("tiny", "tangents"), ("room", "weights"), ("room", "tangents"),
+                                        ("room", "colours")])
+def test_operands_near_the_floor(scene, case):
+    """One sample to a ray, so that its normal and colour are the ray's; through the sampler without fine
+    samples, which has no rule for thin rays.  Every sample is handed over: the SDF cases have the SIMT kernel's
+    bits, those of a network scaled by a power of two between two ReLU layers (the same FP32 function), which is
+    out of range everywhere; the parts alone are 3e-5 to 1e-3 away in the normals, 1e-2 in the colours."""
+    o, d, b = rays(scene, [1] * 300, seed=74)
+    b["t_f"] = (b["t_n"] + np.linspace(0.02, 0.3, 300)).astype(np.float32)
+    spec = near_the_floor(spec_of(scene), case)
+    got = render_gpu(spec, o, d, bounds_on_device(b), 0)
+    if case == "colours":
+        with torch.no_grad():
+            ref = orr.render_hier_bounded(orr.Net(spec), o, d, b["t_n"].astype(np.float64), b["t_f"].astype(np.float64),
+                                          b["n"], 0)
+        ref = {k: ref[k].detach().numpy() for k in ("rgb", "wsum")}
+        live = ref["wsum"] > 1e-2
+        assert live.sum() > 20
+        off = np.abs(got["rgb"] / got["wsum"][:, None] - ref["rgb"] / ref["wsum"][:, None])[live]
+        assert off.max() < 2e-5
+    else:
+        ref = render_gpu(scaled(spec, "rgb", 1, 2.0 ** 19, True), o, d, bounds_on_device(b), 0)
+        for k in got:
+            assert got[k].tobytes() == ref[k].tobytes(), k
     rc, bits = T.tsdfs_sync_status()
     assert rc == 0, bits
