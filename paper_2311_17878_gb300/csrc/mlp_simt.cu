@@ -43,7 +43,8 @@ __device__ __forceinline__ float softplus_slope(float z, float beta) {
 }
 
 // acc[r][j] = sum_k in[row(r)][k] * W[col(j)][k] for this thread's RPT rows and
-// columns n = j*16 + cg (cg = thread % 16).  W is [N][K] row-major in global.
+// columns n = j*16 + cg (cg = thread % 16).  W is [N][K] row-major in global.  The next K chunk's
+// weights are loaded into registers while the current one's products are summed.
 template <int K, int N, int RPT>
 __device__ __forceinline__ void gemm(Smem& sm, const float (*in)[kLDA], int row0, const float* __restrict__ W,
                                      float (&acc)[RPT][(N + 15) / 16]) {
@@ -54,14 +55,25 @@ __device__ __forceinline__ void gemm(Smem& sm, const float (*in)[kLDA], int row0
     for (int r = 0; r < RPT; ++r)
 #pragma unroll
         for (int j = 0; j < NJ; ++j) acc[r][j] = 0.0f;
+    // element (kk, n0 + i * kRows) of a chunk: thread's i-th
+    constexpr int kRows = kThreads / kKC;
+    static_assert(NPAD % kRows == 0, "a thread stages whole rows");
+    const int wk = threadIdx.x % kKC, n0 = threadIdx.x / kKC;
+    float next[NPAD / kRows];
+    auto load = [&](int k0) {
+#pragma unroll
+        for (int i = 0; i < NPAD / kRows; ++i) {
+            const int n = n0 + i * kRows, k = k0 + wk;
+            next[i] = (n < N && k < K) ? __ldg(W + (int64_t)n * K + k) : 0.0f;
+        }
+    };
+    load(0);
     for (int k0 = 0; k0 < K; k0 += kKC) {
         __syncthreads();
-        for (int e = threadIdx.x; e < kKC * NPAD; e += kThreads) {
-            const int kk = e % kKC, n = e / kKC;
-            const int k = k0 + kk;
-            sm.wt[kk][n] = (n < N && k < K) ? __ldg(W + (int64_t)n * K + k) : 0.0f;
-        }
+#pragma unroll
+        for (int i = 0; i < NPAD / kRows; ++i) sm.wt[wk][n0 + i * kRows] = next[i];
         __syncthreads();
+        if (k0 + kKC < K) load(k0 + kKC);
         const int kmax = K - k0 < kKC ? K - k0 : kKC;
         for (int kk = 0; kk < kmax; ++kk) {
             float a[RPT];
