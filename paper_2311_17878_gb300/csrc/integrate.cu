@@ -56,6 +56,11 @@ constexpr int kCam = 20;
 // table once per block still costs less than that.  256^3, 100 views / 300 x 225 x 121, 3 views: 152 x 5
 // blocks 770 / 102 us, x 8 846 / 72, x 32 680 / 56, x 108 645 / 56, x 216 648 / 56.
 constexpr int kFuseBlocks = 152 * 5 * 20;
+// k_integrate_few (figures there): views staged at a time; the voxels up to which and the views above which it
+// is taken.  640 views' table is 52 KB: four blocks of k_integrate on an SM instead of five.
+constexpr int kViewChunk = 256;
+constexpr int64_t kFewVoxels = 64 * 64 * 64;
+constexpr int kManyViews = 640;
 
 // whether view P can see a voxel centre within h[3] of c[3]
 __device__ __forceinline__ bool brick_visible(const float* P, const float c[3], const float h[3], float fW, float fH) {
@@ -198,6 +203,108 @@ __global__ void __launch_bounds__(kFuseBlock) k_integrate(int nx, int ny, int nz
                     Vv = __fdiv_rn(__fadd_rn(__fmul_rn(Wf, Vv), sn), __fadd_rn(Wf, 1.0f));
                 if (Wv < 255) ++Wv;
             }
+            store_v(V, f16, q, Vv);
+            W[q] = (uint8_t)Wv;
+        }
+    }
+}
+
+// Few voxels, thin grids, many views: a brick of 2^lx x 2^ly x 2^(8 - lx - ly) voxels, one to a thread, shaped to
+// the grid (bricks of 8 x 8 x 8 leave 7 of 8 threads idle in a grid one voxel thick, and a grid of 16^3 is 8 of
+// them: then a voxel's chain of views is all there is to wait for); and at most kViewChunk views staged at a
+// time, so that their table does not cost resident blocks.  The pixel and the projection are taken at once by the
+// divisions: that chain is shorter than the approximations' with their branches, and the projection's is done
+// while the depth is on its way.
+// Measured (us, k_integrate / this; 100 views unless said otherwise; a sphere that all views see whole): 16^3 125 /
+// 53, 48^3 137 / 75, 64^3 174 / 152 and with 12 views 28.7 / 28.8, 512 x 512 x 1 182 / 144, 1 x 512 x 512 694 / 146,
+// 64^3 with 2048 views 6919 / 2877, 192^3 with 1000 38.5 / 31.8 ms; the room: 48^3 45 / 23, 64^3 47 / 30, 192^3 with
+// 1000 views 3.72 / 3.25 ms.  Above 64^3 voxels it depends on the views (80^3 of the room, 12 views 18.5 / 19.8,
+// 100 views 51 / 43), and soon no more: 96^3 with 12 views 22.6 / 28.7, 256^3 with 100 665 / 814.
+__global__ void __launch_bounds__(kFuseBlock) k_integrate_few(int nx, int ny, int nz, int lx, int ly, float ox, float oy,
+                                                              float oz, float vs, float trunc, void* V, int f16, uint8_t* W,
+                                                              const float* __restrict__ depth, int nv, int H, int Wd,
+                                                              const float* __restrict__ Kc, const float* __restrict__ c2w) {
+    __shared__ float cam[kViewChunk * 16];
+    __shared__ uint16_t list[kViewChunk];
+    __shared__ int s_warp[kFuseBlock / 32];
+    static_assert(kViewChunk == kFuseBlock, "a view per thread");
+    const int sx = 1 << lx, sy = 1 << ly, sz = kFuseBlock >> (lx + ly);
+    const int bx = (nx - 1) / sx + 1, by = (ny - 1) / sy + 1, bz = (nz - 1) / sz + 1;
+    const int64_t bricks = (int64_t)bx * by * bz;
+    const float fW = (float)Wd, fH = (float)H;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int64_t br = blockIdx.x; br < bricks; br += gridDim.x) {
+        const int i0 = (int)(br % bx) * sx, j0 = (int)((br / bx) % by) * sy, k0 = (int)(br / ((int64_t)bx * by)) * sz;
+        const float h[3] = {0.5f * (float)sx * vs, 0.5f * (float)sy * vs, 0.5f * (float)sz * vs};
+        const float c[3] = {ox + ((float)i0 + 0.5f * (float)sx) * vs, oy + ((float)j0 + 0.5f * (float)sy) * vs,
+                            oz + ((float)k0 + 0.5f * (float)sz) * vs};
+        const int i = i0 + ((int)threadIdx.x & (sx - 1)), j = j0 + (((int)threadIdx.x >> lx) & (sy - 1));
+        const int k = k0 + ((int)threadIdx.x >> (lx + ly));
+        const bool voxel = i < nx && j < ny && k < nz;
+        const int64_t q = ((int64_t)k * ny + j) * nx + i;
+        const float cx = __fadd_rn(ox, __fmul_rn(__fadd_rn((float)i, 0.5f), vs));
+        const float cy = __fadd_rn(oy, __fmul_rn(__fadd_rn((float)j, 0.5f), vs));
+        const float cz = __fadd_rn(oz, __fmul_rn(__fadd_rn((float)k, 0.5f), vs));
+        float Vv = 0.0f;
+        int Wv = 0;
+        bool seen = false;   // by a view; the voxel stays in registers from chunk to chunk
+        for (int v0 = 0; v0 < nv; v0 += kViewChunk) {
+            const int views = nv - v0 < kViewChunk ? nv - v0 : kViewChunk;
+            __syncthreads();   // the last list and its table; s_warp
+            if (nv > kViewChunk || br == blockIdx.x) {
+                for (int e = threadIdx.x; e < views * 16; e += kFuseBlock) {
+                    const int v = v0 + (e >> 4), a = e & 15;
+                    cam[e] = a < 12 ? c2w[v * 12 + a] : Kc[v * 4 + (a - 12)];
+                }
+                __syncthreads();
+            }
+            const bool keep = (int)threadIdx.x < views && brick_visible(cam + threadIdx.x * 16, c, h, fW, fH);
+            const unsigned m = __ballot_sync(0xffffffffu, keep);
+            if (lane == 0) s_warp[warp] = __popc(m);
+            __syncthreads();
+            int before = 0, n_list = 0;
+#pragma unroll
+            for (int w = 0; w < kFuseBlock / 32; ++w) {
+                const int n = s_warp[w];
+                before += w < warp ? n : 0;
+                n_list += n;
+            }
+            if (n_list == 0) continue;
+            if (keep) list[before + __popc(m & ((1u << lane) - 1u))] = (uint16_t)threadIdx.x;
+            __syncthreads();
+            if (voxel && !seen) {
+                Vv = load_v(V, f16, q);
+                Wv = W[q];
+            }
+            seen = true;
+            for (int l = 0; voxel && l < n_list; ++l) {
+                const int view = list[l];
+                const float* P = cam + view * 16;
+                const float dx = __fsub_rn(cx, P[3]), dy = __fsub_rn(cy, P[7]), dz = __fsub_rn(cz, P[11]);
+                const float zc = __fadd_rn(__fadd_rn(__fmul_rn(P[2], dx), __fmul_rn(P[6], dy)), __fmul_rn(P[10], dz));
+                if (!(zc > 0.0f)) continue;
+                const float xc = __fadd_rn(__fadd_rn(__fmul_rn(P[0], dx), __fmul_rn(P[4], dy)), __fmul_rn(P[8], dz));
+                const float yc = __fadd_rn(__fadd_rn(__fmul_rn(P[1], dx), __fmul_rn(P[5], dy)), __fmul_rn(P[9], dz));
+                const float fx = P[12], fy = P[13], ccx = P[14], ccy = P[15];
+                const float u = __fadd_rn(__fmul_rn(fx, __fdiv_rn(xc, zc)), ccx);
+                const float v = __fadd_rn(__fmul_rn(fy, __fdiv_rn(yc, zc)), ccy);
+                if (!(u >= 0.0f && u < fW && v >= 0.0f && v < fH)) continue;
+                const int px = min((int)floorf(u), Wd - 1), py = min((int)floorf(v), H - 1);
+                const float D = __ldg(depth + ((int64_t)(v0 + view) * H + py) * Wd + px);
+                const float a = __fdiv_rn(__fsub_rn(__fadd_rn((float)px, 0.5f), ccx), fx);
+                const float b = __fdiv_rn(__fsub_rn(__fadd_rn((float)py, 0.5f), ccy), fy);
+                const float nrm = __fsqrt_rn(__fadd_rn(__fadd_rn(__fmul_rn(a, a), __fmul_rn(b, b)), 1.0f));
+                const float proj = __fdiv_rn(__fadd_rn(__fadd_rn(__fmul_rn(a, xc), __fmul_rn(b, yc)), zc), nrm);
+                float s = __fsub_rn(D, proj);
+                if (s > trunc) s = trunc;
+                if (s < -trunc) s = -trunc;
+                if (!(s > -trunc)) continue;
+                const float sn = __fdiv_rn(s, trunc), Wf = (float)Wv;
+                Vv = __fdiv_rn(__fadd_rn(__fmul_rn(Wf, Vv), sn), __fadd_rn(Wf, 1.0f));
+                if (Wv < 255) ++Wv;
+            }
+        }
+        if (seen && voxel) {
             store_v(V, f16, q, Vv);
             W[q] = (uint8_t)Wv;
         }
@@ -469,6 +576,27 @@ extern "C" int tsdf_integrate(const tsdfs_grid* g, const float* depth, int32_t n
     if (n_views == 0) return TSDFS_OK;
     if (n_views > 2048) return fail(TSDFS_E_INVALID, "at most 2048 views per call (split larger sets)");
     if (!depth || !K || !c2w) return fail(TSDFS_E_INVALID, "depth, K and c2w must be non-NULL");
+    ProfScope ps("integrate", (cudaStream_t)stream);
+    const int n[3] = {g->nx, g->ny, g->nz};
+    const bool thin = n[0] < kBX || n[1] < kBY || n[2] < kBZ;
+    if (thin || n_views > kManyViews || (int64_t)n[0] * n[1] * n[2] <= kFewVoxels) {
+        // 8 x 8 x 4 voxels; an axis with fewer gives its share to those with the most bricks
+        int lg[3] = {3, 3, 2}, spare = 0;
+        for (int a = 0; a < 3; ++a)
+            for (; lg[a] > 0 && (1 << (lg[a] - 1)) >= n[a]; --lg[a]) ++spare;
+        for (; spare > 0; --spare) {
+            int most = 0;
+            for (int a = 1; a < 3; ++a)
+                if (n[a] >> lg[a] > n[most] >> lg[most]) most = a;
+            ++lg[most];
+        }
+        int64_t bricks = 1;
+        for (int a = 0; a < 3; ++a) bricks *= ((n[a] - 1) >> lg[a]) + 1;
+        k_integrate_few<<<grid_1d(bricks, 1, kFuseBlocks), kFuseBlock, 0, (cudaStream_t)stream>>>(
+            g->nx, g->ny, g->nz, lg[0], lg[1], g->origin[0], g->origin[1], g->origin[2], g->voxel_size, g->trunc, g->tsdf,
+            g->dtype == TSDFS_F16, g->weight, depth, n_views, H, W, K, c2w);
+        return cuda_check(cudaGetLastError(), "tsdf_integrate launch");
+    }
     const int64_t bricks = (int64_t)((g->nx + kBX - 1) / kBX) * ((g->ny + kBY - 1) / kBY) * ((g->nz + kBZ - 1) / kBZ);
     size_t smem = (size_t)n_views * (kCam * sizeof(float) + sizeof(uint16_t));
     if (smem > 48 * 1024) {
@@ -476,7 +604,6 @@ extern "C" int tsdf_integrate(const tsdfs_grid* g, const float* depth, int32_t n
                         "tsdf_integrate smem attribute");
         if (rc) return rc;
     }
-    ProfScope ps("integrate", (cudaStream_t)stream);
     k_integrate<<<grid_1d(bricks, 1, kFuseBlocks), kFuseBlock, smem, (cudaStream_t)stream>>>(
         g->nx, g->ny, g->nz, g->origin[0], g->origin[1], g->origin[2], g->voxel_size, g->trunc, g->tsdf,
         g->dtype == TSDFS_F16, g->weight, depth, n_views, H, W, K, c2w);

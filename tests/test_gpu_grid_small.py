@@ -1,0 +1,32 @@
+"""Fusion of small, thin and long grids, with few and many views, against the oracle bit for bit: the sizes at which
+its kernels change over."""
+import numpy as np
+import pytest
+
+from oracle import cgrid
+from paper_2311_17878_gb300 import build, synth
+from paper_2311_17878_gb300 import tsdfs as T
+from test_gpu_grid_kernels import bits, dev, random_views
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _lib():
+    build.build()
+    T.lib()
+
+
+@pytest.mark.parametrize("shape,n_views", [((1, 40, 37), 30), ((37, 1, 40), 30), ((40, 37, 1), 30), ((2, 300, 3), 90), ((1, 1, 700), 90),
+                                           ((16, 16, 16), 60), ((64, 64, 64), 4), ((65, 64, 64), 4), ((8, 9, 8), 256), ((24, 20, 16), 257),
+                                           ((24, 20, 16), 641), ((70, 66, 68), 640), ((70, 66, 68), 641), ((7, 200, 211), 3)])
+@pytest.mark.parametrize("dtype", ["f32", "f16"])
+def test_fusion(shape, n_views, dtype):
+    spec = synth.GridSpec(*shape, (-0.5, -0.4, -0.3), 1.0 / max(shape), 3.0 / max(shape), dtype)
+    views = random_views(n_views, 13, 11, n_views + shape[0], 1.1)
+    g = T.Grid(spec).init().integrate(dev(views.depth), dev(views.K), dev(views.c2w))
+    V, W = cgrid.integrate_projective(spec, views, "f32")
+    assert np.array_equal(g.W.cpu().numpy(), W)
+    got = g.V.cpu().numpy()
+    assert np.array_equal(bits(got), bits(V) if V.dtype != np.uint16 else V)
+    assert n_views < 9 or W.max() > 0
