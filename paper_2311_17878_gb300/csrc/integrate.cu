@@ -662,6 +662,7 @@ extern "C" int tsdfs_inside_mask(const tsdfs_grid* g, int32_t r, uint32_t* bits,
     if (rc) return rc;
     if (r < 0 || r > kMaxR) return fail(TSDFS_E_INVALID, "nb_radius must be in [0, %d]", kMaxR);
     if (!bits) return fail(TSDFS_E_INVALID, "mask_bits is NULL");
+    if (g->ny > 4 * 65535 || g->nz > 4 * 65535) return fail(TSDFS_E_INVALID, "grid too large for the mask kernel");
     int aligned = (g->nx % 32) == 0;
     if (!aligned) {
         rc = cuda_check(cudaMemsetAsync(bits, 0, (size_t)tsdfs_inside_mask_words(g) * 4, (cudaStream_t)stream),
@@ -669,7 +670,6 @@ extern "C" int tsdfs_inside_mask(const tsdfs_grid* g, int32_t r, uint32_t* bits,
         if (rc) return rc;
     }
     dim3 grid((g->nx + 32 * kMW - 1) / (32 * kMW), (g->ny + kMY - 1) / kMY, (g->nz + kMZ - 1) / kMZ);
-    if (grid.y > 65535 || grid.z > 65535) return fail(TSDFS_E_INVALID, "grid too large for the mask kernel");
     ProfScope ps("inside_mask", (cudaStream_t)stream);
     k_inside_mask<<<grid, kMThreads, 0, (cudaStream_t)stream>>>(g->tsdf, g->dtype == TSDFS_F16, g->nx, g->ny,
                                                                        g->nz, r, bits, aligned);

@@ -30,3 +30,12 @@ def test_fusion(shape, n_views, dtype):
     got = g.V.cpu().numpy()
     assert np.array_equal(bits(got), bits(V) if V.dtype != np.uint16 else V)
     assert n_views < 9 or W.max() > 0
+
+
+@pytest.mark.parametrize("ny,nz", [(262141, 1), (1, 262141)])
+def test_mask_refuses_what_it_refused(ny, nz):
+    """More than 262 140 rows along an axis."""
+    spec = synth.GridSpec(1, ny, nz, (0, 0, 0), 0.1, 0.3)
+    g = T.Grid(spec).init()
+    with pytest.raises(T.TsdfsError):
+        g.inside_mask(1)
