@@ -316,15 +316,22 @@ __global__ void __launch_bounds__(kFuseBlock) k_integrate_few(int nx, int ny, in
 // Only the signs matter, so the erosion runs on words of 32 voxels: a warp reads 32 voxels of a
 // row and one ballot makes their word; an x erosion is an AND of the word's shifts (with the
 // neighbour words' bits), the y and z erosions ANDs of whole words.  A block takes kMW words x
-// kMY x kMZ rows with a halo of r rows (and, at a tile's end inside the grid, one word); the volume is
+// kMY x kMZ rows (8 x 16, small grids 4 x 4) with a halo of r rows (and, at a tile's end inside the grid, one word); the volume is
 // read once from memory, the halo (1.9 x at r = 2) from L2.  Bound: the instructions of those reads.
 // 256^3 FP32, r = 2: 592 us as a running maximum of values over shared-memory tiles, 37 us so.  A NaN voxel
 // counts as negative unless its whole neighbourhood is NaN (a maximum of the values ignores a NaN):
 // a tile that has one goes through its neighbourhoods again.  Rows that are no multiple of 32 voxels
 // long put their words into the bit array with two atomic ORs each.
-constexpr int kMW = 8, kMY = 8, kMZ = 16, kMaxR = 4;
+constexpr int kMW = 8, kMaxR = 4;
 constexpr int kMThreads = 256;
+// Tiles of 4 x 4 rows where those of 8 x 16 would be fewer blocks than this (a block's rows are all there is to wait
+// for then), and in grids of at most 4 rows at r = 0, where half of a tile's are out of the grid.  Measured (us, 8 x 16 / 4 x
+// 4): 16^3, r = 2 19 / 8.4; 64^3, r = 0 10.3 / 7.1, r = 2 18.5 / 8.3; 96^3 (72 blocks), r = 4 28.7 / 24.6; 256 x 5 x 256 16.5 /
+// 7.2; 128^3 (128 blocks), r = 2 18.5 / 18.5, r = 4 28.7 / 36.9; 160^3, r = 2 22.6 / 26.7; 4 x 4 x 100000, r = 0 154 / 109, r = 2
+// 282 / 330.
+constexpr int64_t kSmallMask = 128;
 
+template <int kMY, int kMZ>
 __global__ void __launch_bounds__(kMThreads) k_inside_mask(const void* __restrict__ V, int f16, int nx, int ny, int nz,
                                                            int r, uint32_t* __restrict__ bits, int aligned_rows) {
     constexpr int RY = kMY + 2 * kMaxR, RZ = kMZ + 2 * kMaxR;
@@ -669,9 +676,14 @@ extern "C" int tsdfs_inside_mask(const tsdfs_grid* g, int32_t r, uint32_t* bits,
                         "tsdfs_inside_mask memset");
         if (rc) return rc;
     }
-    dim3 grid((g->nx + 32 * kMW - 1) / (32 * kMW), (g->ny + kMY - 1) / kMY, (g->nz + kMZ - 1) / kMZ);
+    const int64_t nx = g->nx, ny = g->ny, nz = g->nz;
+    const int64_t blocks = ((nx - 1) / (32 * kMW) + 1) * ((ny - 1) / 8 + 1) * ((nz - 1) / 16 + 1);
+    const bool small = blocks < kSmallMask || (ny <= 4 && r == 0);
+    const int my = small ? 4 : 8, mz = small ? 4 : 16;
+    dim3 grid((unsigned)((nx - 1) / (32 * kMW) + 1), (unsigned)((ny - 1) / my + 1), (unsigned)((nz - 1) / mz + 1));
     ProfScope ps("inside_mask", (cudaStream_t)stream);
-    k_inside_mask<<<grid, kMThreads, 0, (cudaStream_t)stream>>>(g->tsdf, g->dtype == TSDFS_F16, g->nx, g->ny,
-                                                                       g->nz, r, bits, aligned);
+    auto inside = small ? k_inside_mask<4, 4> : k_inside_mask<8, 16>;
+    inside<<<grid, kMThreads, 0, (cudaStream_t)stream>>>(g->tsdf, g->dtype == TSDFS_F16, g->nx, g->ny, g->nz, r, bits,
+                                                         aligned);
     return cuda_check(cudaGetLastError(), "tsdfs_inside_mask launch");
 }

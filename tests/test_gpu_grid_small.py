@@ -1,12 +1,13 @@
-"""Fusion of small, thin and long grids, with few and many views, against the oracle bit for bit: the sizes at which
-its kernels change over."""
+"""Fusion and inside mask of small, thin and long grids, with few and many views, against the oracle (the mask: a
+PyTorch restatement) bit for bit: the sizes at which their kernels change over."""
 import numpy as np
 import pytest
+import torch
 
 from oracle import cgrid
 from paper_2311_17878_gb300 import build, synth
 from paper_2311_17878_gb300 import tsdfs as T
-from test_gpu_grid_kernels import bits, dev, random_views
+from test_gpu_grid_kernels import bits, dev, mask_ref, random_views
 
 pytestmark = pytest.mark.gpu
 
@@ -30,6 +31,22 @@ def test_fusion(shape, n_views, dtype):
     got = g.V.cpu().numpy()
     assert np.array_equal(bits(got), bits(V) if V.dtype != np.uint16 else V)
     assert n_views < 9 or W.max() > 0
+
+
+@pytest.mark.parametrize("shape", [(4, 4, 700), (90, 4, 40), (121, 96, 130), (128, 128, 128), (130, 128, 127), (1, 65, 513), (2000, 3, 5)])
+@pytest.mark.parametrize("r", [0, 2, 4])
+def test_mask(shape, r):
+    gen = torch.Generator().manual_seed(r + shape[2])
+    V = -torch.rand(shape, generator=gen)
+    V = torch.where(torch.rand(shape, generator=gen) < 0.01, -V, V)
+    V[torch.rand(shape, generator=gen) < 0.002] = float("nan")
+    nz, ny, nx = shape
+    g = T.Grid(synth.GridSpec(nx, ny, nz, (0, 0, 0), 0.1, 0.3), V=V.cuda(), W=torch.zeros(shape, dtype=torch.uint8).cuda())
+    words = g.inside_mask(r).cpu().numpy().view(np.uint32)
+    got = np.unpackbits(words.view(np.uint8), bitorder="little")
+    ref = mask_ref(V, r).numpy().reshape(-1)
+    assert np.array_equal(got[:ref.size].astype(bool), ref)
+    assert not got[ref.size:].any()
 
 
 @pytest.mark.parametrize("ny,nz", [(262141, 1), (1, 262141)])
