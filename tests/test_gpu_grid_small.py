@@ -1,5 +1,5 @@
-"""Fusion and inside mask of small, thin and long grids, with few and many views, against the oracle (the mask: a
-PyTorch restatement) bit for bit: the sizes at which their kernels change over."""
+"""Fusion, inside mask and ray-casting fusion of small, thin and long grids, with few and many views, against the
+oracle (the mask: a PyTorch restatement) bit for bit: the sizes at which their kernels change over."""
 import numpy as np
 import pytest
 import torch
@@ -56,3 +56,17 @@ def test_mask_refuses_what_it_refused(ny, nz):
     g = T.Grid(spec).init()
     with pytest.raises(T.TsdfsError):
         g.inside_mask(1)
+
+
+@pytest.mark.parametrize("shape,w,h,spread", [((20, 21, 22), 9, 7, 3.0), ((20, 21, 22), 1, 70, 0.4), ((64, 64, 64), 100, 3, 2.0),
+                                              ((70, 69, 68), 90, 70, 0.9), ((90, 30, 100), 200, 150, 2.5), ((70, 70, 70), 33, 4, 0.3)])
+@pytest.mark.parametrize("dtype", ["f32", "f16"])
+def test_raycast(shape, w, h, spread, dtype):
+    """Cameras in the grid, near it and far from it, whose pixels' rays share voxels or do not."""
+    spec = synth.GridSpec(*shape, (-0.5, -0.4, -0.3), 1.0 / max(shape), 3.0 / max(shape), dtype)
+    views = random_views(7, w, h, w + shape[1], spread)
+    g = T.Grid(spec).init().integrate_raycast(dev(views.depth), dev(views.K), dev(views.c2w))
+    V, W = cgrid.integrate_raycast_batched(spec, views, "f32")
+    assert np.array_equal(g.W.cpu().numpy(), W)
+    got = g.V.cpu().numpy()
+    assert np.array_equal(bits(got), bits(V) if V.dtype != np.uint16 else V)
