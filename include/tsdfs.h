@@ -14,10 +14,13 @@
  *    allocates and frees nothing itself (no cudaMalloc / cudaFree in it; the
  *    layer-major backward's first call on a device creates a cuBLAS handle,
  *    whose state cuBLAS allocates).  The render workspaces (render_rays,
- *    render_rays_hier, render_rays_hier_bounded) include about 10 MB for the
- *    network kernels: the serial one parks the first tile of each pair of
- *    64-sample tiles there (256 CTAs x 38 KB), the FP32 one keeps the call's
- *    split weights there (3 MB).
+ *    render_rays_hier, render_rays_hier_bounded) include scratch of the network
+ *    kernels: parked tiles, and the FP32 path's split weights.  The
+ *    *_workspace_size functions ask for what mlp's precision and architecture
+ *    fill the GPU with (room networks: 33 MB in FP32, 15 MB in the others; tiny
+ *    networks: 10 MB); the calls take any workspace with 10 MB of it, whatever
+ *    the precision, run the FP32 and pipelined kernels on fewer SMs then, and
+ *    return TSDFS_E_WORKSPACE below that.  The results are the same.
  *  - Work is enqueued asynchronously on `stream` (a cudaStream_t; NULL = the
  *    legacy default stream); the calls that synchronise say so (the autotuners,
  *    the layer-major backward and training forward, which read the sample
@@ -47,7 +50,8 @@ typedef struct CUstream_st* tsdfs_stream_t; /* identical to cudaStream_t */
 #define TSDFS_OK 0
 #define TSDFS_E_INVALID (-1)     /* bad argument: null pointer, size, parameter  */
 #define TSDFS_E_CUDA (-2)        /* a CUDA runtime call failed                   */
-#define TSDFS_E_WORKSPACE (-3)   /* workspace smaller than the *_workspace_size  */
+#define TSDFS_E_WORKSPACE (-3)   /* workspace smaller than the *_workspace_size
+                                    (renders: than that with 10 MB of scratch)   */
 #define TSDFS_E_UNSUPPORTED (-4) /* architecture / precision combination         */
 #define TSDFS_E_DEVICE (-5)      /* tsdfs_sync_status: a device-side check fired */
 

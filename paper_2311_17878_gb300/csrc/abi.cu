@@ -4,6 +4,7 @@
 #include <cstdio>
 #include <cstring>
 #include <atomic>
+#include <algorithm>
 #include <mutex>
 
 #include "common.cuh"
@@ -191,8 +192,8 @@ int launch_mlp_full_tc(const tsdfs_mlp* mlp, const SampleSource& src, SampleRec*
                        uint8_t* stash, cudaStream_t st);
 size_t mlp_tc_stash_bytes();
 int launch_mlp_value_tc(const tsdfs_mlp* mlp, const SampleSource& src, float* f_out, cudaStream_t st);
-size_t mlp_pipe_stash_bytes();
-int launch_mlp_pipe(const tsdfs_mlp* mlp, const SampleSource& src, SampleRec* rec, int64_t max_samples, uint8_t* stash,
+size_t mlp_pipe_stash_bytes(int arch);
+int launch_mlp_pipe(const tsdfs_mlp* mlp, const SampleSource& src, SampleRec* rec, int64_t max_samples, Scratch stash,
                     cudaStream_t st);
 
 // network kernel per precision (tsdfs_set_network_kernel), index = TSDFS_PREC_*
@@ -237,29 +238,40 @@ static NetParams net_params(const tsdfs_mlp* m) {
     return np;
 }
 
-// scratch of the network kernels in the caller's workspace (256-byte aligned): the kernels'
-// parking space, the single-precision path's redo word and split weights
-static size_t stash_bytes() {
-    const size_t a = mlp_tc_stash_bytes(), b = mlp_f32_stash_bytes(), c = mlp_pipe_stash_bytes();
-    return a > b ? (a > c ? a : c) : (b > c ? b : c);
+// Scratch of the network kernels at the end of the caller's workspace (256-byte aligned): the kernels'
+// parking space, the single-precision path's redo words and split weights.  Every kernel runs in
+// least_stash(); the pipelined and the FP32 one take fewer CTAs then (128 and, room networks, 45), with the
+// same results.  The workspace sizes tell what the mlp's kernels fill the SMs with.
+static Scratch scratch_at(uintptr_t at, const void* ws, size_t ws_bytes) {
+    return Scratch{reinterpret_cast<uint8_t*>(at), (size_t)(reinterpret_cast<uintptr_t>(ws) + ws_bytes - at)};
+}
+static size_t least_stash() { return mlp_tc_stash_bytes(); }
+static size_t stash_bytes(const tsdfs_mlp* m) {
+    size_t most = least_stash();
+    for (int arch : {TSDFS_ARCH_TINY, TSDFS_ARCH_ROOM}) {
+        if (m && m->arch != arch && (m->arch == TSDFS_ARCH_TINY || m->arch == TSDFS_ARCH_ROOM)) continue;
+        if (!m || m->precision == TSDFS_PREC_F32) most = std::max(most, mlp_f32_stash_bytes(arch));
+        if (!m || m->precision != TSDFS_PREC_F32) most = std::max(most, mlp_pipe_stash_bytes(arch));
+    }
+    return most;
 }
 
 // the network evaluation of every render path; simt: FP32 on the SIMT kernel alone
 static int run_full_mlp(const tsdfs_mlp* m, const SampleSource& src, SampleRec* rec, int64_t max_samples,
-                        uint8_t* stash, cudaStream_t st, bool simt = false) {
+                        Scratch stash, cudaStream_t st, bool simt = false) {
     if (m->precision != TSDFS_PREC_F32) {
         if (netkernel_of(m->precision) == TSDFS_NETKERNEL_PIPELINED) {
             ProfScope ps("mlp_pipe", st);
             return launch_mlp_pipe(m, src, rec, max_samples, stash, st);
         }
         ProfScope ps("mlp_tc", st);
-        return launch_mlp_full_tc(m, src, rec, max_samples, stash, st);
+        return launch_mlp_full_tc(m, src, rec, max_samples, stash.at, st);
     }
     // FP32: the split tensor-core kernel, then the SIMT kernel over the samples it marked (see
     // mlp_f32.cu), at every size: one 32-sample tile takes less time than a SIMT tile of 16
     ProfScope ps("mlp_f32", st);
     const NetParams np = net_params(m);
-    const uint32_t* redo = simt ? nullptr : reinterpret_cast<const uint32_t*>(stash);
+    const uint32_t* redo = simt ? nullptr : reinterpret_cast<const uint32_t*>(stash.at);
     int rc = simt ? TSDFS_OK : launch_mlp_full_f32(m, src, rec, max_samples, stash, st);
     if (rc) return rc;
     return m->arch == TSDFS_ARCH_TINY ? launch_mlp_full_simt<TSDFS_ARCH_TINY>(np, src, rec, max_samples, redo, st)
@@ -267,7 +279,7 @@ static int run_full_mlp(const tsdfs_mlp* m, const SampleSource& src, SampleRec* 
 }
 
 // SDF values only (the samplers' coarse passes)
-static int run_value_mlp(const tsdfs_mlp* m, const SampleSource& src, float* f_out, uint8_t* stash, cudaStream_t st,
+static int run_value_mlp(const tsdfs_mlp* m, const SampleSource& src, float* f_out, Scratch stash, cudaStream_t st,
                          bool simt = false) {
     if (m->precision != TSDFS_PREC_F32) {
         ProfScope ps("mlp_value_tc", st);
@@ -275,7 +287,7 @@ static int run_value_mlp(const tsdfs_mlp* m, const SampleSource& src, float* f_o
     }
     ProfScope ps("mlp_value_f32", st);
     const NetParams np = net_params(m);
-    const uint32_t* redo = simt ? nullptr : reinterpret_cast<const uint32_t*>(stash);
+    const uint32_t* redo = simt ? nullptr : reinterpret_cast<const uint32_t*>(stash.at);
     int rc = simt ? TSDFS_OK : launch_mlp_value_f32(m, src, f_out, stash, st);
     if (rc) return rc;
     return m->arch == TSDFS_ARCH_TINY ? launch_mlp_value_simt<TSDFS_ARCH_TINY>(np, src, f_out, redo, st)
@@ -367,13 +379,14 @@ extern "C" int64_t tsdfs_rgb_param_count(int32_t arch) {
 }
 
 // render workspace: the per-sample records, then the ray index of every sample, then the
-// tensor-core network kernel's parking space
-extern "C" size_t tsdfs_render_workspace_size(const tsdfs_mlp* mlp, int64_t n_rays, int64_t max_samples) {
-    (void)mlp;
-    (void)n_rays;
-    if (max_samples < 0) return 0;
+// network kernels' scratch
+static size_t render_bytes(int64_t max_samples, size_t stash) {
     return align256((size_t)max_samples * sizeof(SampleRec)) + align256((size_t)max_samples * sizeof(int32_t)) +
-           align256(stash_bytes()) + 256;
+           align256(stash) + 256;
+}
+extern "C" size_t tsdfs_render_workspace_size(const tsdfs_mlp* mlp, int64_t n_rays, int64_t max_samples) {
+    (void)n_rays;
+    return max_samples < 0 ? 0 : render_bytes(max_samples, stash_bytes(mlp));
 }
 
 namespace tsdfs {
@@ -399,14 +412,14 @@ extern "C" int render_rays(const tsdfs_mlp* mlp, const float* ray_o, const float
     if (!ray_o || !ray_d || !t_n || !t_f || !offsets || !status || !rgb || !depth || !wsum)
         return fail(TSDFS_E_INVALID, "ray, bound and output pointers must be non-NULL (normal, eik may be NULL)");
     if (max_samples > (int64_t)INT32_MAX) return fail(TSDFS_E_INVALID, "max_samples must fit int32 offsets");
-    if (!ws || ws_bytes < tsdfs_render_workspace_size(mlp, n_rays, max_samples))
+    if (!ws || ws_bytes < render_bytes(max_samples, least_stash()))
         return fail(TSDFS_E_WORKSPACE, "render workspace too small");
     cudaStream_t st = (cudaStream_t)stream;
     SampleRec* rec = reinterpret_cast<SampleRec*>((reinterpret_cast<uintptr_t>(ws) + 255) & ~uintptr_t(255));
     int32_t* sample_ray = reinterpret_cast<int32_t*>(reinterpret_cast<uintptr_t>(rec) +
                                                      align256((size_t)max_samples * sizeof(SampleRec)));
-    uint8_t* stash = reinterpret_cast<uint8_t*>(reinterpret_cast<uintptr_t>(sample_ray) +
-                                                align256((size_t)max_samples * sizeof(int32_t)));
+    const Scratch stash = scratch_at(reinterpret_cast<uintptr_t>(sample_ray) + align256((size_t)max_samples * sizeof(int32_t)),
+                                     ws, ws_bytes);
     SampleSource src{};
     src.mode = kUniform;
     src.ray_o = ray_o;
@@ -440,7 +453,7 @@ extern "C" int render_rays(const tsdfs_mlp* mlp, const float* ray_o, const float
     // that its results for them are the results for them; without such rays three empty launches (5 us).  The
     // tiny networks' f differ by 2e-7 and nothing comes of it.
     ProfScope ps("thin_rays", st);
-    uint32_t* thin = reinterpret_cast<uint32_t*>(stash) + 1;
+    uint32_t* thin = reinterpret_cast<uint32_t*>(stash.at) + 1;
     rc = launch_mark_thin(rec, offsets, status, wsum, n_rays, max_samples, thin, st);
     if (rc) return rc;
     rc = launch_mlp_full_simt<TSDFS_ARCH_ROOM>(net_params(mlp), src, rec, max_samples, thin, st);
@@ -505,11 +518,11 @@ struct HierWs {
     float *t0, *te, *tc, *dc, *fc, *tf, *df;
     uint8_t* status;
     SampleRec* rec;
-    uint8_t* stash;
+    uintptr_t stash;   // the rest of the workspace
     size_t bytes;
 };
 
-static HierWs hier_layout(void* base, int64_t n, int n_c = 64, int n_f = 32) {
+static HierWs hier_layout(void* base, int64_t n, int n_c, int n_f, size_t stash) {
     HierWs w{};
     uintptr_t p = (reinterpret_cast<uintptr_t>(base) + 255) & ~uintptr_t(255);
     auto take = [&](size_t bytes) {
@@ -519,7 +532,6 @@ static HierWs hier_layout(void* base, int64_t n, int n_c = 64, int n_f = 32) {
     };
     const size_t n_h = (size_t)(n_c + n_f);
     w.rec = reinterpret_cast<SampleRec*>(take((size_t)n * n_h * sizeof(SampleRec)));
-    w.stash = reinterpret_cast<uint8_t*>(take(stash_bytes()));
     w.t0 = reinterpret_cast<float*>(take((size_t)n * 4));
     w.te = reinterpret_cast<float*>(take((size_t)n * 4));
     w.tc = reinterpret_cast<float*>(take((size_t)n * n_c * 4));
@@ -528,14 +540,13 @@ static HierWs hier_layout(void* base, int64_t n, int n_c = 64, int n_f = 32) {
     w.tf = reinterpret_cast<float*>(take((size_t)n * n_h * 4));
     w.df = reinterpret_cast<float*>(take((size_t)n * n_h * 4));
     w.status = reinterpret_cast<uint8_t*>(take((size_t)n));
+    w.stash = take(stash);
     w.bytes = p - reinterpret_cast<uintptr_t>(base) + 256;
     return w;
 }
 
 extern "C" size_t tsdfs_hier_workspace_size(const tsdfs_mlp* mlp, int64_t n_rays) {
-    (void)mlp;
-    if (n_rays < 0) return 0;
-    return hier_layout(nullptr, n_rays).bytes + 256;
+    return n_rays < 0 ? 0 : hier_layout(nullptr, n_rays, 64, 32, stash_bytes(mlp)).bytes + 256;
 }
 
 extern "C" int render_rays_hier(const tsdfs_mlp* mlp, const tsdfs_grid* grid, const float* ray_o, const float* ray_d,
@@ -555,9 +566,10 @@ extern "C" int render_rays_hier(const tsdfs_mlp* mlp, const tsdfs_grid* grid, co
     if (n_rays * 96 > (int64_t)INT32_MAX) return fail(TSDFS_E_INVALID, "too many rays");
     if (!ray_o || !ray_d || !rgb || !depth || !wsum) return fail(TSDFS_E_INVALID, "ray and output pointers must be non-NULL");
     if (!(t_near < t_far)) return fail(TSDFS_E_INVALID, "t_near must be < t_far");
-    if (!ws || ws_bytes < tsdfs_hier_workspace_size(mlp, n_rays)) return fail(TSDFS_E_WORKSPACE, "hier workspace too small");
+    if (!ws || ws_bytes < hier_layout(nullptr, n_rays, 64, 32, least_stash()).bytes + 256) return fail(TSDFS_E_WORKSPACE, "hier workspace too small");
     cudaStream_t st = (cudaStream_t)stream;
-    HierWs w = hier_layout(ws, n_rays, n_coarse, n_fine);
+    HierWs w = hier_layout(ws, n_rays, n_coarse, n_fine, least_stash());
+    const Scratch stash = scratch_at(w.stash, ws, ws_bytes);
     {
         ProfScope ps("hier_setup", st);
         rc = launch_hier_setup(grid, ray_o, ray_d, n_rays, t_near, t_far, w.t0, w.te, w.status, w.tc, w.dc, n_coarse, st);
@@ -577,7 +589,7 @@ extern "C" int render_rays_hier(const tsdfs_mlp* mlp, const tsdfs_grid* grid, co
     // colours and normals of the FP32 kernels up to 4e-5 (2-norm) apart, and the SIMT kernel's 3e-5 to 4e-4
     // from 64 bits; 33 and 64: below 2e-5.  So few stay with the SIMT kernel.
     const bool simt = mlp->precision == TSDFS_PREC_F32 && mlp->arch == TSDFS_ARCH_ROOM && n_coarse < 32;
-    rc = run_value_mlp(mlp, cs, w.fc, w.stash, st, simt);
+    rc = run_value_mlp(mlp, cs, w.fc, stash, st, simt);
     if (rc) return rc;
     {
         ProfScope ps("hier_fine", st);
@@ -591,7 +603,7 @@ extern "C" int render_rays_hier(const tsdfs_mlp* mlp, const tsdfs_grid* grid, co
     fs.per_ray = n_h;
     fs.total_host = n_rays * n_h;
     fs.capacity = n_rays * n_h;
-    rc = run_full_mlp(mlp, fs, w.rec, n_rays * n_h, w.stash, st, simt);
+    rc = run_full_mlp(mlp, fs, w.rec, n_rays * n_h, stash, st, simt);
     if (rc) return rc;
     ProfScope ps("composite", st);
     return launch_composite(w.rec, nullptr, n_h, w.status, n_rays, nullptr, n_rays * n_h, opacity_of(mlp),
@@ -611,11 +623,11 @@ struct BoundedHierWs {
     int32_t *ray_c, *n2, *off2, *sums, *ray2;
     float *fc, *t2, *d2;
     SampleRec* rec;
-    uint8_t* stash;
+    uintptr_t stash;   // the rest of the workspace
     size_t bytes;
 };
 
-static BoundedHierWs bounded_hier_layout(void* base, int64_t n, int64_t max_coarse, int64_t cap2) {
+static BoundedHierWs bounded_hier_layout(void* base, int64_t n, int64_t max_coarse, int64_t cap2, size_t stash) {
     BoundedHierWs w{};
     uintptr_t p = (reinterpret_cast<uintptr_t>(base) + 255) & ~uintptr_t(255);
     auto take = [&](size_t bytes) {
@@ -624,7 +636,6 @@ static BoundedHierWs bounded_hier_layout(void* base, int64_t n, int64_t max_coar
         return q;
     };
     w.rec = reinterpret_cast<SampleRec*>(take((size_t)cap2 * sizeof(SampleRec)));
-    w.stash = reinterpret_cast<uint8_t*>(take(stash_bytes()));
     w.ray_c = reinterpret_cast<int32_t*>(take((size_t)max_coarse * 4));
     w.fc = reinterpret_cast<float*>(take((size_t)max_coarse * 4));
     w.n2 = reinterpret_cast<int32_t*>(take((size_t)n * 4));
@@ -633,15 +644,15 @@ static BoundedHierWs bounded_hier_layout(void* base, int64_t n, int64_t max_coar
     w.t2 = reinterpret_cast<float*>(take((size_t)cap2 * 4));
     w.d2 = reinterpret_cast<float*>(take((size_t)cap2 * 4));
     w.ray2 = reinterpret_cast<int32_t*>(take((size_t)cap2 * 4));
+    w.stash = take(stash);
     w.bytes = p - reinterpret_cast<uintptr_t>(base) + 256;
     return w;
 }
 
 extern "C" size_t tsdfs_hier_bounded_workspace_size(const tsdfs_mlp* mlp, int64_t n_rays, int32_t n_fine,
                                                     int64_t max_coarse) {
-    (void)mlp;
     if (n_rays < 0 || max_coarse < 0 || n_fine < 0) return 0;
-    return bounded_hier_layout(nullptr, n_rays, max_coarse, max_coarse + n_rays * n_fine).bytes + 256;
+    return bounded_hier_layout(nullptr, n_rays, max_coarse, max_coarse + n_rays * n_fine, stash_bytes(mlp)).bytes + 256;
 }
 
 extern "C" int render_rays_hier_bounded(const tsdfs_mlp* mlp, const float* ray_o, const float* ray_d,
@@ -658,10 +669,11 @@ extern "C" int render_rays_hier_bounded(const tsdfs_mlp* mlp, const float* ray_o
     if (cap2 > (int64_t)INT32_MAX) return fail(TSDFS_E_INVALID, "max_coarse + n_rays * n_fine must fit int32 offsets");
     if (!ray_o || !ray_d || !t_n || !t_f || !offsets || !status || !rgb || !depth || !wsum)
         return fail(TSDFS_E_INVALID, "ray, bound and output pointers must be non-NULL (normal may be NULL)");
-    if (!ws || ws_bytes < tsdfs_hier_bounded_workspace_size(mlp, n_rays, n_fine, max_coarse))
+    if (!ws || ws_bytes < bounded_hier_layout(nullptr, n_rays, max_coarse, cap2, least_stash()).bytes + 256)
         return fail(TSDFS_E_WORKSPACE, "bounded hierarchical workspace too small");
     cudaStream_t st = (cudaStream_t)stream;
-    BoundedHierWs w = bounded_hier_layout(ws, n_rays, max_coarse, cap2);
+    BoundedHierWs w = bounded_hier_layout(ws, n_rays, max_coarse, cap2, least_stash());
+    const Scratch stash = scratch_at(w.stash, ws, ws_bytes);
     // coarse pass: SDF values at the midpoints of the bounds' ragged counts
     SampleSource cs{};
     cs.mode = kUniform;
@@ -681,7 +693,7 @@ extern "C" int render_rays_hier_bounded(const tsdfs_mlp* mlp, const float* ray_o
             if (rc) return rc;
         }
         cs.sample_ray = w.ray_c;  // the value kernels flag a coarse total above max_coarse
-        rc = run_value_mlp(mlp, cs, w.fc, w.stash, st);
+        rc = run_value_mlp(mlp, cs, w.fc, stash, st);
         if (rc) return rc;
     }
     // merged counts, their offsets, then the fine samples and the merged list
@@ -707,7 +719,7 @@ extern "C" int render_rays_hier_bounded(const tsdfs_mlp* mlp, const float* ray_o
     fs.total_dev = w.off2 + n_rays;
     fs.capacity = cap2;
     if (cap2 > 0) {
-        rc = run_full_mlp(mlp, fs, w.rec, cap2, w.stash, st);
+        rc = run_full_mlp(mlp, fs, w.rec, cap2, stash, st);
         if (rc) return rc;
     }
     ProfScope ps("composite", st);

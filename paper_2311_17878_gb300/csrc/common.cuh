@@ -161,6 +161,12 @@ struct SampleSource {
     int64_t capacity;  // records available in the workspace
 };
 
+// scratch of the network kernels in the caller's workspace
+struct Scratch {
+    uint8_t* at;
+    size_t bytes;
+};
+
 // opacity of a sample's section (Eq. 1 with the backbone's SDF-to-density transform)
 struct Opacity {
     int kind;     // TSDFS_OPACITY_NEUS / TSDFS_OPACITY_VOLSDF

@@ -86,7 +86,7 @@ constexpr float kLimit = 2000.0f;     // largest operand the high part is truste
 constexpr float kBias0 = 1.7e-8f, kBias1 = 1.58e-8f;   // what a main sum of n MMAs lacks: kBias0 + n kBias1
 constexpr float kMinGrad = 1e-4f;
 constexpr float kFloor = 1.0f / (16384.0f * kUp);   // 1.9e-6: the scaled high part of less is subnormal
-constexpr int kMaxCtas = 192;         // CTAs with a place to park
+constexpr int kMaxCtas = 192;         // CTAs that the workspace sizes have a place to park for
 constexpr float kRsqrt2 = 0.70710678118654752f;
 
 template <int ARCH> struct FArch {
@@ -1139,7 +1139,7 @@ __global__ void k_split_weights(const float* __restrict__ sdf_w, const float* __
 
 template <int ARCH, bool VALUE>
 int launch_f32(const tsdfs_mlp* m, const SampleSource& src, SampleRec* rec, float* f_out, int64_t max_samples,
-               uint8_t* stash, cudaStream_t st) {
+               Scratch stash, cudaStream_t st) {
     using F = FArch<ARCH>;
     constexpr size_t smem = F::template smem_bytes<VALUE>();
     static_assert(smem <= 232448, "k_mlp_f32 shared memory exceeds 227 KB");
@@ -1159,9 +1159,10 @@ int launch_f32(const tsdfs_mlp* m, const SampleSource& src, SampleRec* rec, floa
         }
     }
     F32Params p{};
-    p.packed = stash + kRedoBytes;
-    p.park = stash + kRedoBytes + F::packed_bytes();
-    p.redo = reinterpret_cast<uint32_t*>(stash);
+    constexpr size_t head = kRedoBytes + F::packed_bytes();
+    p.packed = stash.at + kRedoBytes;
+    p.park = stash.at + head;
+    p.redo = reinterpret_cast<uint32_t*>(stash.at);
     p.sdf_w = m->sdf_w;
     p.rgb_w = m->rgb_w;
     for (int a = 0; a < 3; ++a) p.center[a] = m->center[a];
@@ -1176,28 +1177,32 @@ int launch_f32(const tsdfs_mlp* m, const SampleSource& src, SampleRec* rec, floa
     p.withhold = test_withhold_chunk();
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const int64_t ts = VALUE ? kTileV : kTile, tiles = (max_samples + ts - 1) / ts;
-    if (sms > kMaxCtas) sms = kMaxCtas;
+    const int64_t places = (int64_t)((stash.bytes - head) / F::park_bytes());
+    if (!VALUE && sms > places) sms = (int)places;
     const unsigned blocks = (unsigned)(tiles < sms ? (tiles < 1 ? 1 : tiles) : sms);
     k_split_weights<ARCH><<<grid_1d(F::packed_bytes() / 32, 256), 256, 0, st>>>(m->sdf_w, m->rgb_w,
-                                                                               stash + kRedoBytes, p.redo);
+                                                                               stash.at + kRedoBytes, p.redo);
     k_mlp_f32<ARCH, VALUE><<<blocks, kThr, smem, st>>>(p);
     return cuda_check(cudaGetLastError(), "mlp_f32 launch");
 }
 
 }  // namespace
 
-size_t mlp_f32_stash_bytes() {
-    using F = FArch<TSDFS_ARCH_ROOM>;
-    return kRedoBytes + (size_t)F::packed_bytes() + kMaxCtas * F::park_bytes();
+size_t mlp_f32_stash_bytes(int arch) {
+    auto bytes = [](auto f) {
+        using F = decltype(f);
+        return kRedoBytes + (size_t)F::packed_bytes() + kMaxCtas * F::park_bytes();
+    };
+    return arch == TSDFS_ARCH_TINY ? bytes(FArch<TSDFS_ARCH_TINY>{}) : bytes(FArch<TSDFS_ARCH_ROOM>{});
 }
 
 int launch_mlp_full_f32(const tsdfs_mlp* m, const SampleSource& src, SampleRec* rec, int64_t max_samples,
-                        uint8_t* stash, cudaStream_t st) {
+                        Scratch stash, cudaStream_t st) {
     return m->arch == TSDFS_ARCH_TINY ? launch_f32<TSDFS_ARCH_TINY, false>(m, src, rec, nullptr, max_samples, stash, st)
                                       : launch_f32<TSDFS_ARCH_ROOM, false>(m, src, rec, nullptr, max_samples, stash, st);
 }
 
-int launch_mlp_value_f32(const tsdfs_mlp* m, const SampleSource& src, float* f_out, uint8_t* stash, cudaStream_t st) {
+int launch_mlp_value_f32(const tsdfs_mlp* m, const SampleSource& src, float* f_out, Scratch stash, cudaStream_t st) {
     const int64_t n = sample_bound(src);
     return m->arch == TSDFS_ARCH_TINY ? launch_f32<TSDFS_ARCH_TINY, true>(m, src, nullptr, f_out, n, stash, st)
                                       : launch_f32<TSDFS_ARCH_ROOM, true>(m, src, nullptr, f_out, n, stash, st);

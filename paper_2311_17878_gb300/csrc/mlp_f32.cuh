@@ -13,10 +13,10 @@ constexpr int kLowWord = 8;
 // result of a marked sample of a value pass
 constexpr uint32_t kRedoBits = 0x7fc5a5a5u;
 
-size_t mlp_f32_stash_bytes();
+size_t mlp_f32_stash_bytes(int arch);
 int launch_mlp_full_f32(const tsdfs_mlp* m, const SampleSource& src, SampleRec* rec, int64_t max_samples,
-                        uint8_t* stash, cudaStream_t st);
-int launch_mlp_value_f32(const tsdfs_mlp* m, const SampleSource& src, float* f_out, uint8_t* stash, cudaStream_t st);
+                        Scratch stash, cudaStream_t st);
+int launch_mlp_value_f32(const tsdfs_mlp* m, const SampleSource& src, float* f_out, Scratch stash, cudaStream_t st);
 
 // redo: NULL (every sample) or the word above (the marked samples only; none when it is 0)
 template <int ARCH>

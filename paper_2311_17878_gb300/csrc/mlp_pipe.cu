@@ -54,7 +54,7 @@ constexpr uint32_t kPABytes = 64 * 1024;        // 128 rows x 256 16-bit columns
 constexpr uint32_t kPXMax = 128 * 64 * 2;       // the colour input beyond column 256 (<= 64 columns)
 constexpr uint32_t kPBarBytes = 256;
 constexpr int kPUnit = 4;             // tiles per pass of the colour layers
-constexpr int kPMaxCtas = 192;        // CTAs with a place to park
+constexpr int kPMaxCtas = 192;        // CTAs that the workspace sizes have a place to park for
 constexpr int kPBatch = 4;            // 8-column groups an epilogue thread loads and computes together
 
 template <int MODE> struct PipeMode {
@@ -830,7 +830,7 @@ __global__ void __launch_bounds__(PipeMode<MODE>::kThreads, 1) k_mlp_pipe(PipePa
 }
 
 template <int ARCH, int MODE>
-int launch_pipe(const tsdfs_mlp* m, const SampleSource& src, SampleRec* rec, int64_t max_samples, uint8_t* stash,
+int launch_pipe(const tsdfs_mlp* m, const SampleSource& src, SampleRec* rec, int64_t max_samples, Scratch stash,
                 cudaStream_t st) {
     using TA = PipeArch<ARCH>;
     constexpr size_t smem = TA::template smem_bytes<MODE>();
@@ -858,17 +858,18 @@ int launch_pipe(const tsdfs_mlp* m, const SampleSource& src, SampleRec* rec, int
     p.status = device_status_word();
     p.spin = test_spin_limit(kMaxSpin);
     p.withhold = test_withhold_chunk();
-    p.park = stash;
+    p.park = stash.at;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const int64_t tiles = (max_samples + kPTile - 1) / kPTile;
-    if (sms > kPMaxCtas) sms = kPMaxCtas;
+    const int64_t places = (int64_t)(stash.bytes / (TA::kParkMain + TA::kParkX));
+    if (sms > places) sms = (int)places;
     const unsigned blocks = (unsigned)(tiles < sms ? (tiles < 1 ? 1 : tiles) : sms);
     k_mlp_pipe<ARCH, MODE><<<blocks, PipeMode<MODE>::kThreads, smem, st>>>(p);
     return cuda_check(cudaGetLastError(), "mlp_pipe launch");
 }
 
 template <int ARCH>
-int launch_pipe_arch(const tsdfs_mlp* m, const SampleSource& src, SampleRec* rec, int64_t max_samples, uint8_t* stash,
+int launch_pipe_arch(const tsdfs_mlp* m, const SampleSource& src, SampleRec* rec, int64_t max_samples, Scratch stash,
                      cudaStream_t st) {
     switch (m->precision) {
         case TSDFS_PREC_F16: return launch_pipe<ARCH, TSDFS_PREC_F16>(m, src, rec, max_samples, stash, st);
@@ -880,12 +881,12 @@ int launch_pipe_arch(const tsdfs_mlp* m, const SampleSource& src, SampleRec* rec
 
 }  // namespace
 
-size_t mlp_pipe_stash_bytes() {
-    using TA = PipeArch<TSDFS_ARCH_ROOM>;
-    return (size_t)kPMaxCtas * (TA::kParkMain + TA::kParkX);
+size_t mlp_pipe_stash_bytes(int arch) {
+    auto bytes = [](auto ta) { return (size_t)kPMaxCtas * (decltype(ta)::kParkMain + decltype(ta)::kParkX); };
+    return arch == TSDFS_ARCH_TINY ? bytes(PipeArch<TSDFS_ARCH_TINY>{}) : bytes(PipeArch<TSDFS_ARCH_ROOM>{});
 }
 
-int launch_mlp_pipe(const tsdfs_mlp* m, const SampleSource& src, SampleRec* rec, int64_t max_samples, uint8_t* stash,
+int launch_mlp_pipe(const tsdfs_mlp* m, const SampleSource& src, SampleRec* rec, int64_t max_samples, Scratch stash,
                     cudaStream_t st) {
     if ((reinterpret_cast<uintptr_t>(m->packed) & 15u) != 0) return fail(TSDFS_E_INVALID, "packed weights must be 16-byte aligned");
     if (m->arch == TSDFS_ARCH_TINY) return launch_pipe_arch<TSDFS_ARCH_TINY>(m, src, rec, max_samples, stash, st);
