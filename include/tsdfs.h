@@ -305,17 +305,18 @@ int render_rays_hier96(const tsdfs_mlp* mlp, const tsdfs_grid* grid, const float
 /* ---- launch shape of the march and its autotuner --------------------------
  * tsdf_ray_bounds and tsdf_recovery_bounds launch a grid-stride march of
  * `block` threads per block and at most `blocks_per_sm` blocks per SM (default
- * 128 and 64).  Outputs do not depend on the shape (rays are independent);
+ * 128 and 64): a warp per ray for few rays, a thread per ray above, each with a
+ * shape of its own.  Outputs do not depend on the shape (rays are independent);
  * speed does.  tsdfs_autotune_bounds times every candidate (block in {64, 128,
  * 256} x blocks_per_sm in {4, 8, 16, 32, 64}) with CUDA events on `stream`,
  * `reps` launches each of tsdf_ray_bounds on the caller's rays and buffers
  * (arguments as tsdf_ray_bounds; the outputs hold the last run's results), and
- * keeps the fastest as this device's shape; best_ms (host, or NULL) receives
- * its time per launch.  It synchronises the stream: call it at set-up, not
+ * keeps the fastest as this device's shape for the kernel that so many rays
+ * take; best_ms (host, or NULL) receives its time per launch.  It synchronises the stream: call it at set-up, not
  * inside a captured step.  tsdfs_set_bounds_launch_shape sets a shape
- * directly (0, 0 = the default; block a multiple of 32 in [32, 256],
- * blocks_per_sm in [1, 1024]); tsdfs_bounds_launch_shape reads it.  The shape
- * is per device and process-wide.                                            */
+ * for both directly (0, 0 = the default; block a multiple of 32 in [32, 256],
+ * blocks_per_sm in [1, 1024]); tsdfs_bounds_launch_shape reads the one last set
+ * or tuned.  The shapes are per device and process-wide.                     */
 int tsdfs_autotune_bounds(const tsdfs_grid* grid, const uint32_t* inside_mask, const float* ray_o, const float* ray_d,
                           int64_t n_rays, const tsdfs_bounds_params* params, float* t_n, float* t_f,
                           int32_t* n_samples, int32_t* offsets, float* t_zero, uint8_t* status, void* workspace,

@@ -552,21 +552,33 @@ __global__ void __launch_bounds__(kScanBlock) k_chunk_scan(const int32_t* __rest
 int64_t scan_chunks(int64_t n) { return (n + kScanChunk - 1) / kScanChunk; }
 
 // ---- launch shape of the march (threads per block, resident blocks per SM of the
-// grid-stride grid): the default, or what tsdfs_autotune_bounds measured, per device
+// grid-stride grid): the default, or what tsdfs_autotune_bounds measured, per device and per kernel (what
+// suits a thread per ray does not suit a warp per ray)
 namespace {
 struct MarchShape {
     int block = kBoundsBlock;
     int blocks_per_sm = 64;
 };
+struct MarchShapes {
+    MarchShape of[2];   // a thread per ray, a warp per ray
+    int last = 0;       // the one last set or tuned
+};
 std::mutex g_shape_mu;
-MarchShape g_shape[64];
+MarchShapes g_shape[64];
 
-MarchShape march_shape() {
+MarchShapes march_shapes() {
     int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return MarchShape{};
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return MarchShapes{};
     std::lock_guard<std::mutex> lk(g_shape_mu);
     return g_shape[dev];
 }
+
+// A warp per ray up to these many rays, with and without the inside mask.  Measured (us, warp /
+// thread, rays of a room view in 256^3 and of a sphere view in 64^3): with the mask 1728 rays 22 / 35 and
+// 20 / 78, 4800 39 / 35 and 25 / 78; without it 4800 80 / 190 and 47 / 550, 10 800 144 / 192 and 70 / 550;
+// a thread per ray takes the same up to 30 000 rays.
+constexpr int64_t kWarpRaysMask = 4096, kWarpRays = 16384;
+bool warp_per_ray(int64_t n_rays, const uint32_t* mask) { return n_rays <= (mask ? kWarpRaysMask : kWarpRays); }
 
 unsigned march_grid(int64_t n_rays, const MarchShape& sh) {
     int dev = 0, sms = 152;
@@ -595,16 +607,6 @@ int exclusive_scan(const int32_t* cnt, int64_t n, int32_t* offsets, int32_t* sum
 }  // namespace tsdfs
 
 using namespace tsdfs;
-
-namespace tsdfs {
-namespace {
-// A warp per ray up to these many rays, with and without the inside mask.  Measured (us, warp /
-// thread, rays of a room view in 256^3 and of a sphere view in 64^3): with the mask 1728 rays 22 / 35 and
-// 20 / 78, 4800 39 / 35 and 25 / 78; without it 4800 80 / 190 and 47 / 550, 10 800 144 / 192 and 70 / 550;
-// a thread per ray takes the same up to 30 000 rays.
-constexpr int64_t kWarpRaysMask = 4096, kWarpRays = 16384;
-}  // namespace
-}  // namespace tsdfs
 
 extern "C" size_t tsdfs_bounds_workspace_size(int64_t n_rays) {
     if (n_rays < 0) return 0;
@@ -639,9 +641,9 @@ extern "C" int tsdf_ray_bounds(const tsdfs_grid* g, const uint32_t* mask, const 
                    g->voxel_size, g->trunc};
         BoundsDev bd{p->d_s, p->t_near, p->t_far, p->step, p->nb_radius, p->m_confirm, p->n_max, p->n_fallback,
                      test_march_cap()};
-        const MarchShape sh = march_shape();
+        const bool warp = warp_per_ray(n_rays, mask), small = small_grid(gd.n);
+        const MarchShape sh = march_shapes().of[warp];
         ProfScope ps("ray_bounds", st);
-        const bool warp = n_rays <= (mask ? kWarpRaysMask : kWarpRays), small = small_grid(gd.n);
         auto march = warp ? (small ? k_ray_bounds_warp<true> : k_ray_bounds_warp<false>)
                           : (small ? k_ray_bounds<true> : k_ray_bounds<false>);
         march<<<march_grid(warp ? n_rays * 32 : n_rays, sh), sh.block, 0, st>>>(
@@ -675,7 +677,7 @@ extern "C" int tsdf_recovery_bounds(const tsdfs_grid* g, const float* ray_o, con
                    g->voxel_size, g->trunc};
         BoundsDev bd{p->d_s, p->t_near, p->t_far, p->step, p->nb_radius, p->m_confirm, p->n_max, p->n_fallback,
                      test_march_cap()};
-        const MarchShape sh = march_shape();
+        const MarchShape sh = march_shapes().of[0];
         ProfScope ps("recovery_bounds", st);
         k_recovery_bounds<<<march_grid(n_rays, sh), sh.block, 0, st>>>(
             gd, ray_o, ray_d, n_rays, bd, tau, wsum, status, t_n2, t_f2, n2, status2);
@@ -885,7 +887,8 @@ constexpr int kTunePerSm[] = {4, 8, 16, 32, 64};
 
 extern "C" int tsdfs_bounds_launch_shape(int32_t* block, int32_t* blocks_per_sm) {
     if (!block || !blocks_per_sm) return fail(TSDFS_E_INVALID, "block and blocks_per_sm must be non-NULL");
-    const MarchShape sh = march_shape();
+    const MarchShapes all = march_shapes();
+    const MarchShape sh = all.of[all.last];
     *block = sh.block;
     *blocks_per_sm = sh.blocks_per_sm;
     return TSDFS_OK;
@@ -904,8 +907,8 @@ extern "C" int tsdfs_set_bounds_launch_shape(int32_t block, int32_t blocks_per_s
     if (rc) return rc;
     if (dev < 0 || dev >= 64) return fail(TSDFS_E_UNSUPPORTED, "device index %d out of range", dev);
     std::lock_guard<std::mutex> lk(g_shape_mu);
-    g_shape[dev].block = block;
-    g_shape[dev].blocks_per_sm = blocks_per_sm;
+    for (MarchShape& sh : g_shape[dev].of) sh = MarchShape{block, blocks_per_sm};
+    g_shape[dev].last = 0;
     return TSDFS_OK;
 }
 
@@ -915,14 +918,13 @@ extern "C" int tsdfs_autotune_bounds(const tsdfs_grid* g, const uint32_t* mask, 
                                      size_t ws_bytes, int32_t reps, float* best_ms, tsdfs_stream_t stream) {
     if (reps < 1 || reps > 1000) return fail(TSDFS_E_INVALID, "reps must be in [1, 1000]");
     if (n_rays < 1) return fail(TSDFS_E_INVALID, "autotuning needs at least one ray");
-    int32_t b0 = 0, s0 = 0;
-    tsdfs_bounds_launch_shape(&b0, &s0);
+    MarchShapes shapes = march_shapes();
     cudaStream_t st = (cudaStream_t)stream;
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     int rc = cuda_check(cudaEventCreate(&e0), "autotune event");
     if (!rc) rc = cuda_check(cudaEventCreate(&e1), "autotune event");
     float best = 1e30f;
-    int best_b = b0, best_s = s0;
+    MarchShape fastest;
     for (int bi = 0; !rc && bi < (int)(sizeof(kTuneBlocks) / sizeof(int)); ++bi)
         for (int si = 0; !rc && si < (int)(sizeof(kTunePerSm) / sizeof(int)); ++si) {
             rc = tsdfs_set_bounds_launch_shape(kTuneBlocks[bi], kTunePerSm[si]);
@@ -939,13 +941,22 @@ extern "C" int tsdfs_autotune_bounds(const tsdfs_grid* g, const uint32_t* mask, 
             if (!rc) rc = cuda_check(cudaEventElapsedTime(&ms, e0, e1), "autotune elapsed");
             if (!rc && ms < best) {
                 best = ms;
-                best_b = kTuneBlocks[bi];
-                best_s = kTunePerSm[si];
+                fastest = MarchShape{kTuneBlocks[bi], kTunePerSm[si]};
             }
         }
     if (e0) cudaEventDestroy(e0);
     if (e1) cudaEventDestroy(e1);
-    const int rc2 = tsdfs_set_bounds_launch_shape(rc ? b0 : best_b, rc ? s0 : best_s);
+    // the kernel that these rays take keeps the fastest shape, the other one its own
+    if (!rc) {
+        shapes.last = warp_per_ray(n_rays, mask);
+        shapes.of[shapes.last] = fastest;
+    }
+    int dev = 0;
+    const int rc2 = cuda_check(cudaGetDevice(&dev), "cudaGetDevice");
+    if (!rc2 && dev >= 0 && dev < 64) {
+        std::lock_guard<std::mutex> lk(g_shape_mu);
+        g_shape[dev] = shapes;
+    }
     if (rc) return rc;
     if (best_ms) *best_ms = best / (float)reps;
     return rc2;
