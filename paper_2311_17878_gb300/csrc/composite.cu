@@ -158,8 +158,10 @@ __global__ void __launch_bounds__(kCompBlock) k_composite_warp(const SampleRec* 
 // bits of f.
 __global__ void k_mark_thin(SampleRec* __restrict__ rec, const int32_t* __restrict__ offsets,
                             const uint8_t* __restrict__ status, const float* __restrict__ wsum, int64_t n_rays,
-                            int64_t capacity, uint32_t* thin) {
+                            int64_t capacity, uint32_t* thin, const uint32_t* dev_status) {
+    // all weights are 0 then (k_composite)
     if ((int64_t)__ldg(offsets + n_rays) > capacity) return;
+    if (dev_status && (*(const volatile uint32_t*)dev_status & TSDFS_DEV_TIMEOUT)) return;
     for (int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; r < n_rays; r += (int64_t)gridDim.x * blockDim.x) {
         const int64_t b = __ldg(offsets + r), e = __ldg(offsets + r + 1);
         if (b >= e || !(wsum[r] < kThinRay) || (status && __ldg(status + r) == TSDFS_MISS)) continue;
@@ -405,7 +407,8 @@ int launch_composite(const SampleRec* rec, const int32_t* offsets, int per_ray, 
 int launch_mark_thin(SampleRec* rec, const int32_t* offsets, const uint8_t* status, const float* wsum, int64_t n_rays,
                      int64_t capacity, uint32_t* thin, cudaStream_t st) {
     if (n_rays == 0) return TSDFS_OK;
-    k_mark_thin<<<grid_1d(n_rays, 128), 128, 0, st>>>(rec, offsets, status, wsum, n_rays, capacity, thin);
+    k_mark_thin<<<grid_1d(n_rays, 128), 128, 0, st>>>(rec, offsets, status, wsum, n_rays, capacity, thin,
+                                                      device_status_word());
     return cuda_check(cudaGetLastError(), "mark thin rays launch");
 }
 
