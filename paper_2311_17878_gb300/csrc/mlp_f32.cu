@@ -73,6 +73,11 @@ constexpr int kParts = 3;
 constexpr int kMma = 12;              // MMA warp
 constexpr int kStages = 2;
 constexpr int kProd = 3;               // weight producers (16 warps in all leave 128 registers a thread)
+constexpr int kItemParts = 2;          // copies of an item (hi and lo), each by the next producer in turn
+// A producer waits for the release of the item kStages before its own by a parity, so the release before that
+// one must be behind it: its last part was kProd parts ago, and it waited then for a release at most kStages
+// items further back.  That also takes the MMA warp to release the stages in the items' order.
+static_assert(kProd <= kItemParts * kStages, "a producer would wait a phase ahead of its stage");
 constexpr int kThr = 32 * (kMma + 1 + kProd);
 constexpr int kPh = 128;              // outputs per phase
 constexpr int kGrp = 6;               // 8-column groups of a phase per part, at most
@@ -288,7 +293,7 @@ __global__ void __launch_bounds__(kThr, 1) k_mlp_f32(F32Params p) {
 
     if (threadIdx.x == 0) {
         for (int i = 0; i < kStages; ++i) {
-            mbar_init(bar_full + 8 * i, 2);
+            mbar_init(bar_full + 8 * i, kItemParts);
             mbar_init(bar_empty + 8 * i, 1);
             mbar_init(bar_acc + 8 * i, 1);
             mbar_init(bar_drained + 8 * i, kEpi);
@@ -388,7 +393,7 @@ __global__ void __launch_bounds__(kThr, 1) k_mlp_f32(F32Params p) {
             bool ok = true;
             auto item = [&](int j) {
                 const bool operand = (items[j].edge & 32u) != 0;
-                for (uint32_t part = 0; part < 2; ++part, --turn) {
+                for (uint32_t part = 0; part < kItemParts; ++part, --turn) {
                     if (turn != 0) continue;
                     turn = kProd;
                     const uint32_t stage = (uint32_t)g & 1u;
@@ -455,7 +460,7 @@ __global__ void __launch_bounds__(kThr, 1) k_mlp_f32(F32Params p) {
                 if (it.steps == kKChunk / 16) static_for<0, kKChunk / 16>([&](auto k) { step(decltype(k)::value); });
                 else
                     for (int k = 0; k < it.steps; ++k) step(k);
-                if (it.edge & 64u) commit_el(el, bar_empty + 8 * (stage ^ 1u));
+                if (it.edge & 64u) commit_el(el, bar_empty + 8 * (stage ^ 1u));   // the operand item is the earlier one
                 commit_el(el, bar_empty + 8 * stage);
                 if (it.edge & 2u) commit_el(el, bar_acc + 8 * (ph++ & 1u));
             }
