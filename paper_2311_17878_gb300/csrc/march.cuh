@@ -19,13 +19,6 @@ struct GridDev {
     float trunc;
 };
 
-__device__ __forceinline__ float gval(const GridDev& g, int i, int j, int k) {
-    if (i < 0 || j < 0 || k < 0 || i >= g.n[0] || j >= g.n[1] || k >= g.n[2]) return -1.0f;
-    const int64_t idx = ((int64_t)k * g.n[1] + j) * g.n[0] + i;
-    return g.f16 ? __half2float(__ldg(reinterpret_cast<const __half*>(g.V) + idx))
-                 : __ldg(reinterpret_cast<const float*>(g.V) + idx);
-}
-
 // V at a voxel of the grid by its linear index
 __device__ __forceinline__ float vat(const GridDev& g, int64_t idx) {
     return g.f16 ? __half2float(__ldg(reinterpret_cast<const __half*>(g.V) + idx))

@@ -19,11 +19,8 @@ struct TcLayer {
 };
 
 __host__ __device__ constexpr int pad16(int x) { return (x + 15) / 16 * 16; }
-// column range [lo, hi) of a K-wide operand row written by column half hf:
-// the split is rounded up to 16 so every 16-column block stays inside K
-__host__ __device__ constexpr int half_lo(int K, int hf) { return hf ? pad16(K / 2) : 0; }
-__host__ __device__ constexpr int half_hi(int K, int hf) { return hf ? K : pad16(K / 2); }
-// the same for `parts` parts of whole 16-column blocks (K a multiple of 16)
+// column range [lo, hi) of a K-wide operand row written by part pt of `parts` parts of whole 16-column
+// blocks (K a multiple of 16)
 __host__ __device__ constexpr int part_lo(int K, int pt, int parts) { return ((K / 16) * pt / parts) * 16; }
 __host__ __device__ constexpr int part_hi(int K, int pt, int parts) { return pt + 1 == parts ? K : part_lo(K, pt + 1, parts); }
 // the same in 8-column groups (K a multiple of 8): parts differ by at most one group, the
@@ -380,19 +377,6 @@ __device__ __forceinline__ void static_for(F&& f) {
     }
 }
 
-// positional encoding entry j of coordinate vector xt, and its derivative along axis a
-__device__ __forceinline__ float enc_val(const float* xt, int j, int pe, int a, bool deriv) {
-    if (j < 3) return deriv ? (j == a ? 1.0f : 0.0f) : xt[j];
-    const int q = j - 3;
-    const int oct = q / 6, part = (q % 6) / 3, b = q % 3;
-    if (oct >= pe) return 0.0f;
-    if (deriv && b != a) return 0.0f;
-    const float f = (float)(1 << oct);
-    float sn, cs;
-    sincosf(f * xt[b], &sn, &cs);
-    if (!deriv) return part == 0 ? sn : cs;
-    return part == 0 ? f * cs : -f * sn;
-}
 
 // the same entry from the per-tile tables: sx = the 3 coordinates, spe = sin / cos of
 // 2^oct x_b at ((oct * 3 + b) * 2 + {0: sin, 1: cos}); comp 0 = value, comp a + 1 =
