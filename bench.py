@@ -13,7 +13,7 @@ Fusion runs once before the timed region and is reported separately.
     python bench.py [--steps K] [--warmup W] [--precision bf16|f32]
     python bench.py --impl reference     # the CPU oracle on a bounded sample
 
-One JSON line on stdout (rank 0).
+On stdout (rank 0) a line "detail: {...}" with every leg's figures, then the result: one short JSON line.
 """
 from __future__ import annotations
 
@@ -1322,6 +1322,26 @@ def run_reference(args, ws, rank):
             "e2e": {"value": value, "unit": UNIT, "h2d_bytes_per_step": 0, "d2h_bytes_per_step": 0}}
 
 
+HEADLINE = ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling",
+            "vs_baseline", "dtype", "data", "impl", "config", "e2e", "gpu_launches", "clocks", "psnr_gate")
+HEADLINE_CONFIG = ("workload", "rays_per_step", "views", "samples_per_step", "grid", "grid_source", "fusion_form",
+                   "ray_subset", "cuda_graph", "network_kernel", "recovery_tau", "networks", "l2", "parallelism")
+
+
+def headline(line):
+    """The line's result: what a reader of the last kilobytes of the output needs, without the per-view and
+    per-leg diagnostics (some 20 KB)."""
+    out = {k: line[k] for k in HEADLINE if line.get(k) is not None or k == "vs_baseline"}
+    out["config"] = {k: line["config"][k] for k in HEADLINE_CONFIG if k in line["config"]}
+    return out
+
+
+def report(line):
+    """The whole line first, marked as not being the result line, then the result as one short JSON line."""
+    print("detail: " + json.dumps(line), flush=True)
+    print(json.dumps(headline(line)), flush=True)
+
+
 def main():
     global WORKLOAD, N_VIEWS_TIMED
     args = parse()
@@ -1340,7 +1360,7 @@ def main():
     ws, rank, local = dist_setup()
     line = run_ours(args, ws, rank, local)
     if rank == 0:
-        print(json.dumps(line), flush=True)
+        report(line)
     if ws > 1:
         import torch.distributed as dist
         dist.destroy_process_group()
