@@ -121,8 +121,12 @@ typedef struct {
 #define TSDFS_ARCH_TINY 0
 #define TSDFS_ARCH_ROOM 1
 #define TSDFS_PREC_F32 0  /* FP32 networks: tcgen05 with every operand split into two FP16
-                             * parts (22 bits) and FP32 sums; samples whose operands leave
-                             * the parts' range (|x| > 2000) on FP32 SIMT cores           */
+                             * parts (22 bits) and FP32 sums.  On FP32 SIMT cores: samples
+                             * whose operands leave the parts' range (one above 2000, or a
+                             * layer's all below 2e-6), or with |grad f| < 1e-4; with the
+                             * room networks also rays of render_rays whose weights sum to
+                             * less than 1e-3, and render_rays_hier with less than 32 coarse
+                             * samples.  A ray's results do not depend on its batch.        */
 #define TSDFS_PREC_BF16 1 /* BF16 tcgen05 networks, FP32 accumulate (packed required) */
 #define TSDFS_PREC_F16 2  /* FP16 operands on the same tcgen05 path (packed required)  */
 #define TSDFS_PREC_BF16X2 3 /* BF16 tcgen05 networks with every SDF layer's operand split

@@ -449,9 +449,12 @@ extern "C" int render_rays(const tsdfs_mlp* mlp, const float* ray_o, const float
     }
     if (mlp->precision != TSDFS_PREC_F32 || mlp->arch != TSDFS_ARCH_ROOM || max_samples == 0) return TSDFS_OK;
     // Rays of almost no weight (k_mark_thin): the two FP32 kernels' f differ by 1e-6 in the room networks,
-    // and a ray's depth and normal by as much as 3e-3 then.  The SIMT kernel evaluates their samples, so
-    // that its results for them are the results for them; without such rays three empty launches (5 us).  The
-    // tiny networks' f differ by 2e-7 and nothing comes of it.
+    // and a ray's depth and normal by as much as 3e-3 then.  The SIMT kernel evaluates their samples (theirs
+    // alone: a ray's results do not depend on its neighbours), so that its results for them are the results for
+    // them; without such rays three empty launches (5 us).  The tiny networks' f differ by 2e-7 and nothing
+    // comes of it.  The samplers have no such rule: over views of the room the two kernels' normals are 1e-5
+    // (2-norm; largest 9e-4) apart inside the bound and 2e-5 (5e-4) over the box from 33 coarse samples, with
+    // neither nearer to 64 bits than this kernel's.
     ProfScope ps("thin_rays", st);
     uint32_t* thin = reinterpret_cast<uint32_t*>(stash.at) + 1;
     rc = launch_mark_thin(rec, offsets, status, wsum, n_rays, max_samples, thin, st);
@@ -585,9 +588,11 @@ extern "C" int render_rays_hier(const tsdfs_mlp* mlp, const tsdfs_grid* grid, co
     cs.total_host = n_rays * n_coarse;
     cs.capacity = n_rays * n_coarse;
     // With few coarse samples over the whole box a section is as long as the room networks' surfaces are sharp:
-    // where the fine samples fall, and the opacities there, hang on the last bits of f.  8 coarse samples:
-    // colours and normals of the FP32 kernels up to 4e-5 (2-norm) apart, and the SIMT kernel's 3e-5 to 4e-4
-    // from 64 bits; 33 and 64: below 2e-5.  So few stay with the SIMT kernel.
+    // where the fine samples fall, and the opacities there, hang on the last bits of f.  Depths and normals of the
+    // two FP32 kernels over four views, 2-norm / largest difference: 8 coarse samples 4e-5 / 7e-4, 12 1e-4 / 4e-3, 16
+    // 3e-5 / 9e-4, 20 to 31 1e-5 / 3e-4, 33 2e-5 / 5e-4, 64 6e-6 / 1e-4 (the SIMT kernel itself is as far from 64 bits,
+    // the split one no further).  So few stay with the SIMT kernel, whose results are what they were; the line
+    // stands at 32, on the safe side of 20.
     const bool simt = mlp->precision == TSDFS_PREC_F32 && mlp->arch == TSDFS_ARCH_ROOM && n_coarse < 32;
     rc = run_value_mlp(mlp, cs, w.fc, stash, st, simt);
     if (rc) return rc;
