@@ -45,10 +45,10 @@ WORKLOAD = WORKLOADS["view"]
 # over the 10 timed launches of `bench.py --only-main --no-graph --steps 10 --warmup 3` (room views 0-9,
 # network-fused grid, fp16 operands) in one ncu capture; reported only for that
 # configuration and while the kernel sources hash to the ones it was captured on
-MLP_TC_TRAFFIC = {"sha256": "508be6d8907a9f87b0215d8fba1172d1787711764664c78c763670091e89d4a9", "bytes_per_launch": 263375974,
+MLP_TC_TRAFFIC = {"sha256": "f5c7570156f8a72954bff9a0e789964c9be650d248b872466390d78fa4c794cf", "bytes_per_launch": 263191168,
                   "profile": "profiles/k_mlp_tc_room_view_traffic.md"}
 # the same for k_ray_bounds (the march of Alg. 1) on the same ten timed views
-MARCH_TRAFFIC = {"sha256": "65df4dba21b44fef96a0b3ef24f0c80bf18050d138eae939e5ab46905f23370f", "bytes_per_launch": 10004685,
+MARCH_TRAFFIC = {"sha256": "f13a7a98ef5bc0528bbca149585eece7ff9ace6d9a58063255f00a8440bf57c2", "bytes_per_launch": 9994291,
                  "profile": "profiles/k_ray_bounds_room_view_traffic.md"}
 ALGO_FLOP_PER_SAMPLE = 2.25e6   # SDF fwd + minimal reverse-mode grad + colour, 8x256 / 4x256 networks
 # what the tensor-core kernels issue per sample (value + 3 tangent rows through the SDF layers):
