@@ -453,8 +453,7 @@ extern "C" int render_rays(const tsdfs_mlp* mlp, const float* ray_o, const float
     // alone: a ray's results do not depend on its neighbours), so that its results for them are the results for
     // them; without such rays three empty launches (5 us).  The tiny networks' f differ by 2e-7 and nothing
     // comes of it.  The samplers have no such rule: over views of the room the two kernels' normals are 1e-5
-    // (2-norm; largest 9e-4) apart inside the bound and 2e-5 (5e-4) over the box from 33 coarse samples, with
-    // neither nearer to 64 bits than this kernel's.
+    // (2-norm; largest 9e-4) apart inside the bound and 2e-5 (5e-4) over the box from 33 coarse samples.
     ProfScope ps("thin_rays", st);
     uint32_t* thin = reinterpret_cast<uint32_t*>(stash.at) + 1;
     rc = launch_mark_thin(rec, offsets, status, wsum, n_rays, max_samples, thin, st);
@@ -590,8 +589,8 @@ extern "C" int render_rays_hier(const tsdfs_mlp* mlp, const tsdfs_grid* grid, co
     // With few coarse samples over the whole box a section is as long as the room networks' surfaces are sharp:
     // where the fine samples fall, and the opacities there, hang on the last bits of f.  Depths and normals of the
     // two FP32 kernels over four views, 2-norm / largest difference: 8 coarse samples 4e-5 / 7e-4, 12 1e-4 / 4e-3, 16
-    // 3e-5 / 9e-4, 20 to 31 1e-5 / 3e-4, 33 2e-5 / 5e-4, 64 6e-6 / 1e-4 (the SIMT kernel itself is as far from 64 bits,
-    // the split one no further).  So few stay with the SIMT kernel, whose results are what they were; the line
+    // 3e-5 / 9e-4, 20 to 31 1e-5 / 3e-4, 33 2e-5 / 5e-4, 64 6e-6 / 1e-4 (each is as far from 64 bits itself, and neither
+    // nearer on the whole).  So few stay with the SIMT kernel, whose results are what they were; the line
     // stands at 32, on the safe side of 20.
     const bool simt = mlp->precision == TSDFS_PREC_F32 && mlp->arch == TSDFS_ARCH_ROOM && n_coarse < 32;
     rc = run_value_mlp(mlp, cs, w.fc, stash, st, simt);
