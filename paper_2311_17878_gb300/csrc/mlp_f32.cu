@@ -1080,8 +1080,8 @@ __global__ void __launch_bounds__(kThr, 1) k_mlp_f32(F32Params p) {
 
 // Split the parameters into the items' hi and lo images (8 x 8 core matrices, K-major), one
 // 8-column row piece per thread; clears the redo words, and tells for each layer whether all its weights
-// are below kFloor (a block per layer, which looks at 256 of them with ordinary weights).  3 MB for the room networks, every call:
-// the parameters may have changed since the last one.
+// are below kFloor (a block per layer, which looks at 256 of them with ordinary weights).  3 MB for the
+// room networks, every call: the parameters may have changed since the last one.
 template <int ARCH>
 __global__ void k_split_weights(const float* __restrict__ sdf_w, const float* __restrict__ rgb_w,
                                 uint8_t* __restrict__ packed, uint32_t* __restrict__ redo) {
