@@ -1,6 +1,8 @@
 // Volume-rendering compositing (Eq. 1, Eq. 2, the rendered normal) with NeuS
 // opacity, and the per-ray steps of the hierarchical comparator (n_c coarse +
 // n_f inverse-CDF fine samples; 64 + 32 is the comparator of Tab. 2).
+#include <type_traits>
+
 #include "common.cuh"
 
 namespace tsdfs {
@@ -124,12 +126,20 @@ __global__ void __launch_bounds__(kCompBlock) k_composite_warp(const SampleRec* 
                 s[7][lane] = q2.z;
                 s[8][lane] = q1.w - 1.0f;
             }
+            // The sums before each lane, in the samples' order; the lanes from n on are nobody's, so few samples
+            // take few steps.  8192 rays, 31 steps always / as here (us): 1 sample a ray 7.4 / 6.2, 2 7.5 / 6.3,
+            // 8 7.6 / 6.6, 32 8.5 / 8.7.
             float lt = logT;
+            auto before = [&](auto count) {
 #pragma unroll
-            for (int i = 0; i < 31; ++i) {
-                const float v = __shfl_sync(0xffffffffu, l, i);
-                if (i < lane) lt += v;
-            }
+                for (int i = 0; i < decltype(count)::value; ++i) {
+                    const float v = __shfl_sync(0xffffffffu, l, i);
+                    if (i < lane) lt += v;
+                }
+            };
+            if (n <= 2) before(std::integral_constant<int, 1>{});
+            else if (n <= 8) before(std::integral_constant<int, 7>{});
+            else before(std::integral_constant<int, 31>{});
             logT = __shfl_sync(0xffffffffu, lt + l, n - 1);
             s[0][lane] = expf(lt) * alpha;
             __syncwarp();
